@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_big_plan(BigCtl* __restrict__ 
     ctl->R = R;
     ctl->ncounters = G ? cnt0 : 0ull;
     ctl->next_big = cur ^ 1u;
-    for (int k = 0; k < 4; ++k) ctl->next_item[k] = 0;
+    for (int k = 0; k < 2; ++k) ctl->next_item[k] = 0;
     if (G) {
       *c.big[cur ^ 1u].count = 0;  // the list the round's new big subsets go to
       ctl->cur = cur ^ 1u;
@@ -266,65 +266,175 @@ struct ItemStream {
   __device__ __forceinline__ uint32_t next() { return share(ahead); }
 };
 
+// Threads of a sampling block: one per sampled key.  A round waits for its
+// sampling blocks (often a single one: the root's), so their latency counts,
+// not their throughput.  With 256 threads of 4 keys each and every key ranked
+// in the 7 other warps' runs by binary search (196 dependent shared-memory
+// loads) a block took 36 us; one key per thread, warp-sorted and then merged
+// run by run (35 dependent loads), takes 18.5 us (1 M URLs, per round).
 template <int LOGV>
-__global__ void __launch_bounds__(kBlock) k_big_sample(const BigCtl* __restrict__ ctl, uint32_t* __restrict__ work) {
-  __shared__ __align__(16) Splitters<LOGV, u128> sp;
-  __shared__ __align__(16) BuildScratch<LOGV, u128> bs;
+constexpr uint32_t kSampleThreads = Geo<LOGV>::S;
+
+// Shared memory of a sampling block.  The merge alternates between `sample`
+// and the room of the splitters, which are only written once it is done.
+template <int LOGV>
+struct SampleSmem {
+  static_assert(sizeof(u128) * Geo<LOGV>::S <= sizeof(Splitters<LOGV, u128>), "the merge's second buffer");
+  union {
+    Splitters<LOGV, u128> sp;
+    u128 merge[Geo<LOGV>::S];
+  };
+  u128 sample[Geo<LOGV>::S];
+  uint16_t lo[Geo<LOGV>::S];   // first sample position with a key >= sample[i]
+  uint16_t hi[Geo<LOGV>::S];   // first sample position with a key >  sample[i]
+  uint32_t heads[32];          // bit i of word w: position 32 w + i starts a run of equal keys
+};
+
+// The sampling steps of Algorithm 4.1 as in build_splitters_k, by a block of
+// one thread per sampled key (`key`: this thread's, in any order).  Ends with
+// __syncthreads().
+template <int LOGV>
+__device__ void build_splitters_wide(u128 key, SampleSmem<LOGV>& sm, uint32_t dna) {
+  using G = Geo<LOGV>;
+  constexpr uint32_t S = G::S;
+  constexpr uint32_t NW = S / 32;
+  constexpr int kLevels = LOGV + 1 - 5;  // merge levels from runs of 32 to S
+  const uint32_t tid = threadIdx.x, w = tid >> 5, lane = lane_id();
+  u128 v[1] = {key};
+  warp_bitonic<1, u128>(v);
+  u128* src = (kLevels & 1) ? sm.merge : sm.sample;  // the last level writes sample
+  u128* dst = (kLevels & 1) ? sm.sample : sm.merge;
+  src[tid] = v[0];
+  __syncthreads();
+#pragma unroll 1
+  for (uint32_t run = 32; run < S; run <<= 1) {
+    // each key's place in the merged pair of runs: its own index plus the
+    // partner's keys before it (a left key goes before an equal right one)
+    const u128 k = src[tid];
+    const uint32_t i = tid & (run - 1);
+    const u128* other = src + (tid ^ i ^ run);
+    const bool right = (tid & run) != 0;
+    uint32_t a = 0;
+    for (uint32_t half = run >> 1; half > 0; half >>= 1) {
+      const u128 o = other[a + half - 1];
+      a += (right ? o <= k : o < k) ? half : 0u;
+    }
+    const u128 o = other[a];
+    a += (right ? o <= k : o < k) ? 1u : 0u;
+    dst[(tid & ~(2 * run - 1)) + i + a] = k;
+    __syncthreads();
+    u128* t = src;
+    src = dst;
+    dst = t;
+  }
+  const u128* s = sm.sample;
+  // runs of equal keys, from one bit per position that starts one
+  const bool head = tid == 0 || s[tid - 1] != s[tid];
+  const uint32_t hb = __ballot_sync(0xFFFFFFFFu, head);
+  if (lane == 0) sm.heads[w] = hb;
+  __syncthreads();
+  const uint32_t some = __ballot_sync(0xFFFFFFFFu, lane < NW && sm.heads[lane < NW ? lane : 0] != 0);
+  {
+    const uint32_t own = hb & ((2u << lane) - 1);  // lane 31: all bits
+    const uint32_t wl = own ? w : 31 - __clz(some & ((1u << w) - 1));  // position 0 starts a run
+    const uint32_t hl = own ? own : sm.heads[wl];
+    sm.lo[tid] = (uint16_t)(wl * 32 + 31 - __clz(hl));
+    const uint32_t above = lane == 31 ? 0u : hb & ~((2u << lane) - 1);
+    const uint32_t wa = w == 31 ? 0u : some & ~((2u << w) - 1);
+    const uint32_t wh = above ? w : (wa ? __ffs(wa) - 1 : NW);
+    sm.hi[tid] = (uint16_t)(wh == NW ? S : wh * 32 + __ffs(above ? above : sm.heads[wh]) - 1);
+  }
+  __syncthreads();
+  u128 val = 0;
+  uint32_t slot = 0;
+  if (tid < G::V) {
+    const uint32_t i = tid + 1;             // level-order index
+    const int l = 31 - __clz(i);            // its level
+    uint32_t a = 0, b = S;                  // its range of the sorted sample
+    for (int d = l - 1; d >= 0; --d) {
+      if (a < b) {
+        const uint32_t m = (a + b) >> 1;
+        if (((i >> d) & 1u) == 0) {
+          const uint32_t le = sm.lo[m];
+          b = le > a ? le : a;              // left of the run of keys equal to s[m]
+        } else {
+          const uint32_t rs = sm.hi[m];
+          a = rs < b ? rs : b;              // right of that run
+        }
+      } else {
+        a = b;
+      }
+    }
+    val = a < b ? s[(a + b) >> 1] : (b < S ? s[b] : KeyOps<u128>::ones());
+    slot = (2 * (i - (1u << l)) + 1) * (1u << (LOGV - 1 - l)) - 1;
+    sm.sp.tree[i] = val;
+    sm.sp.x[slot] = val;
+  }
+  if (tid == 0) sm.sp.tree[0] = 0;
+  if (tid == G::V) sm.sp.x[G::V] = 0;
+  __syncthreads();
+  if (tid <= G::V)
+    sm.sp.hp[tid] = (tid == 0 || tid == G::V) ? 0 : (uint8_t)KeyOps<u128>::lcp(sm.sp.x[tid - 1], sm.sp.x[tid], dna);
+  __syncthreads();
+}
+
+template <int LOGV>
+__global__ void __launch_bounds__(kSampleThreads<LOGV>) k_big_sample(const BigCtl* __restrict__ ctl) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  SampleSmem<LOGV>& sm = *reinterpret_cast<SampleSmem<LOGV>*>(smem);
   __shared__ uint64_t ref[kPjWindows];
+  __shared__ uint32_t s_min;
   const uint32_t G = ctl->G;
   const SortCtx& c = ctl->c;
   BigSplitters<LOGV>* out = reinterpret_cast<BigSplitters<LOGV>*>(ctl->splitters);
   unsigned long long bytes = 0;
-  ItemStream items{work, 0u};
-  for (uint32_t gi = items.first(); gi < G; gi = items.next()) {
-    items.claim();
+  for (uint32_t gi = blockIdx.x; gi < G; gi += gridDim.x) {
     const GenTask g = ctl->gt[gi];
     const uint32_t par = task_par(g.t);
-    const Rec* recs = c.rec[par] + g.t.begin;
-    const uint2* wids = c.wid[par] + g.t.begin;
     const SetDesc sd = c.sets[task_set(g.t)];
     const uint64_t hseed = mix64(c.seed ^ ((uint64_t)g.t.begin << 20) ^ g.t.depth);
-    build_splitters_k<LOGV, u128>([&](uint32_t pos) { return load_wkey(recs + pos); }, g.t.len, hseed, sp, bs,
-                                  sd.dna);
-    const uint4* src = reinterpret_cast<const uint4*>(&sp);
+    auto sample_pos = [&](uint32_t i) {
+      return g.t.begin + (uint32_t)(((mix64(hseed + i) >> 32) * (uint64_t)g.t.len) >> 32);
+    };
+    if (threadIdx.x == 0) s_min = 0xFFFFFFFFu;
+    build_splitters_wide<LOGV>(load_wkey(c.rec[par] + sample_pos(threadIdx.x)), sm, sd.dna);
+    const uint4* src = reinterpret_cast<const uint4*>(&sm.sp);
     uint4* dst = reinterpret_cast<uint4*>(&out[gi].sp);
-    for (uint32_t i = threadIdx.x; i < sizeof(sp) / 16; i += blockDim.x) dst[i] = src[i];
-    if (threadIdx.x == 0) bytes += Geo<LOGV>::S * 16ull + sizeof(sp);
+    for (uint32_t i = threadIdx.x; i < sizeof(sm.sp) / 16; i += blockDim.x) dst[i] = src[i];
+    if (threadIdx.x == 0) bytes += Geo<LOGV>::S * 16ull + sizeof(sm.sp);
     // prefix jump: a one-key sample whose strings agree beyond kPjMinSample
-    // characters turns on the check of the whole subset
-    const u128 k0 = bs.sample[0];  // the sorted sample
-    const bool one_key = !sd.dna && k0 == bs.sample[Geo<LOGV>::S - 1] && !KeyOps<u128>::end(k0, 0u);
-    uint32_t on = 0;
+    // characters turns on the check of the whole subset; the first sampled
+    // string is the reference
+    const u128 k0 = sm.sample[0];  // the sorted sample
+    const bool one_key = !sd.dna && k0 == sm.sample[Geo<LOGV>::S - 1] && !KeyOps<u128>::end(k0, 0u);
     uint64_t ref_off = 0;
     if (one_key) {  // uniform over the block
-      auto sample_pos = [&](uint32_t i) {
-        return (uint32_t)(((mix64(hseed + i) >> 32) * (uint64_t)g.t.len) >> 32);
-      };
-      const uint32_t wide = c.wide[task_set(g.t)];
-      auto off_of = [&](uint32_t i) {
-        const uint2 w = wids[sample_pos(i)];
-        return rec_offset(sd, wide, w.x, w.y);
-      };
-      ref_off = off_of(0);
-      if (threadIdx.x == 0) {
-        uint64_t w[kPjWindows];
-        load_pj_windows(sd.chars, ref_off, g.t.depth, sd.cap, w);
-        for (int j = 0; j < kPjWindows; ++j) ref[j] = w[j];
+      uint64_t w[kPjWindows];
+      if (threadIdx.x < kPjSampleChecks) {
+        const uint2 id = c.wid[par][sample_pos(threadIdx.x)];
+        const uint64_t off = rec_offset(sd, c.wide[task_set(g.t)], id.x, id.y);
+        load_pj_windows(sd.chars, off, g.t.depth, sd.cap, w);
+        bytes += 8 + 8 * kPjWindows;
+        if (threadIdx.x == 0) {
+          ref_off = off;
+          for (int j = 0; j < kPjWindows; ++j) ref[j] = w[j];
+        }
       }
       __syncthreads();
-      const uint32_t agree = block_min_agreement(sd, g.t.depth, kPjSampleChecks, off_of, ref, bytes);
-      on = agree > kPjMinSample && agree != 0xFFFFFFFFu ? 1u : 0u;
+      if (threadIdx.x < kPjSampleChecks) atomicMin(&s_min, window_lcp(w, ref));
+      __syncthreads();
     }
     if (threadIdx.x == 0) {
-      out[gi].pj_on = on;
+      out[gi].pj_on = one_key && s_min > kPjMinSample ? 1u : 0u;
       out[gi].pj_lcp = 0xFFFFFFFFu;
       out[gi].pj_ref = ref_off;
     }
     if (c.classifier == kClassifyUIJ) {
       for (uint32_t p = threadIdx.x; p < kJumpSize; p += blockDim.x)
-        out[gi].jump[p] = (uint16_t)jump_entry<LOGV, u128>(p, sp.tree);
+        out[gi].jump[p] = (uint16_t)jump_entry<LOGV, u128>(p, sm.sp.tree);
       if (threadIdx.x == 0) bytes += 2ull * kJumpSize;
     }
+    __syncthreads();  // the next subset reuses the shared arrays
   }
   // sample reads + splitter (and jump table) writes
   account(c, kKBigSample, bytes);
@@ -401,22 +511,27 @@ __global__ void __launch_bounds__(kBlock, 4) k_big_classify(const BigCtl* __rest
   account(c, kKBigClassify, bytes);
 }
 
+// Buckets of one subset handled by one block of k_big_emit: one per thread.
+// The kernel is a chain of dependent loads and counter atomics per bucket, so
+// a subset's buckets are spread over KP / 256 blocks instead of four rounds of
+// one block (1 M URLs: 15-22 us -> 7-8 us a round).
 template <int LOGV>
-__global__ void __launch_bounds__(kBlock) k_big_emit(const BigCtl* __restrict__ ctl, uint32_t* __restrict__ work) {
+__global__ void __launch_bounds__(kBlock) k_big_emit(const BigCtl* __restrict__ ctl) {
   using Gm = Geo<LOGV>;
-  const uint32_t G = ctl->G;
+  constexpr uint32_t kParts = Gm::KP / kBlock;
+  const uint32_t items = ctl->G * kParts;
   const SortCtx& c = ctl->c;
   const BigSplitters<LOGV>* spl = reinterpret_cast<const BigSplitters<LOGV>*>(ctl->splitters);
   const uint32_t next_big = ctl->next_big;
   unsigned long long bytes = 0;
-  ItemStream items{work, 0u};
-  for (uint32_t gi = items.first(); gi < G; gi = items.next()) {
-    items.claim();
+  for (uint32_t it = blockIdx.x; it < items; it += gridDim.x) {
+    const uint32_t gi = it / kParts;
+    const uint32_t b = (it % kParts) * kBlock + threadIdx.x;
     const GenTask g = ctl->gt[gi];
     const Splitters<LOGV, u128>& sp = spl[gi].sp;
     const SetDesc sd = c.sets[task_set(g.t)];
     const uint32_t* sc = ctl->counters + cnt_base(g);
-    for (uint32_t b = threadIdx.x; b < Gm::K; b += blockDim.x) {
+    if (b < Gm::K) {
       bytes += 16;  // two bucket offsets read, start and descriptor written
       const uint32_t s = sc[(uint64_t)b * g.tiles] - g.rec_base;
       const uint32_t e = (b + 1 < Gm::K) ? sc[(uint64_t)(b + 1) * g.tiles] - g.rec_base : g.t.len;
@@ -665,17 +780,22 @@ static cudaError_t launch_big_round_t(BigCtl* ctl, uint32_t R_max, uint32_t sms,
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(k_big_scatter<LOGV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)big_scatter_smem(LOGV, kMaxRounds));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_big_sample<LOGV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)sizeof(SampleSmem<LOGV>));
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
   // fixed grids (the work of a round is only known on the device): blocks
   // loop over subsets, tiles or counter chunks and return when there are none
-  hook.run("big_sample", [&] { k_big_sample<LOGV><<<sms * 8, kBlock, 0, st>>>(ctl, &ctl->next_item[0]); });
-  hook.run("big_classify", [&] { k_big_classify<LOGV><<<sms * 8, kBlock, 0, st>>>(ctl, &ctl->next_item[1]); });
+  hook.run("big_sample", [&] { 
+    k_big_sample<LOGV><<<sms * (2048 / kSampleThreads<LOGV>), kSampleThreads<LOGV>, sizeof(SampleSmem<LOGV>), st>>>(ctl);
+  });
+  hook.run("big_classify", [&] { k_big_classify<LOGV><<<sms * 8, kBlock, 0, st>>>(ctl, &ctl->next_item[0]); });
   hook.run("scan", [&] { k_scan_reduce<<<sms * 8, kBlock, 0, st>>>(ctl); });
   hook.run("scan", [&] { k_scan_down<<<sms * 8, kBlock, 0, st>>>(ctl); });
-  hook.run("big_emit", [&] { k_big_emit<LOGV><<<sms * 8, kBlock, 0, st>>>(ctl, &ctl->next_item[2]); });
-  hook.run("big_scatter", [&] { k_big_scatter<LOGV><<<sms * 3, kBlock, smem, st>>>(ctl, &ctl->next_item[3]); });
+  hook.run("big_emit", [&] { k_big_emit<LOGV><<<sms * 8, kBlock, 0, st>>>(ctl); });
+  hook.run("big_scatter", [&] { k_big_scatter<LOGV><<<sms * 3, kBlock, smem, st>>>(ctl, &ctl->next_item[1]); });
   return cudaGetLastError();
 }
 

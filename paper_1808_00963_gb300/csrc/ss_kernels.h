@@ -46,8 +46,8 @@ struct BigCtl {
   uint32_t R;             // tile = 256 * R records
   uint64_t ncounters;
   // work counters of the round's kernels (zeroed by the plan): blocks take
-  // the next subset or tile from them, so that uneven tiles balance out
-  uint32_t next_item[4];  // sample, classify, emit, scatter
+  // the next tile from them, so that uneven tiles balance out
+  uint32_t next_item[2];  // classify, scatter
 };
 
 // Most rounds of multi-block steps one sort may take (each advances every big
