@@ -127,12 +127,10 @@ __device__ uint32_t block_min_agreement(const SetDesc& sd, uint32_t depth, uint3
 
 __device__ unsigned long long g_graph_launches;  // kernels launched by loop graphs (this device)
 
-constexpr uint32_t kPlanThreads = 1024;
-
-// Exclusive scan of one 64-bit value per thread of a kPlanThreads block;
-// returns the block total.
+// Exclusive scan of one 64-bit value per thread of a kBlock block; returns
+// the block total.
 __device__ uint64_t plan_scan(uint64_t v, uint64_t& excl) {
-  __shared__ uint64_t wsum[kPlanThreads / 32];
+  __shared__ uint64_t wsum[kWarps];
   const uint32_t w = threadIdx.x >> 5, lane = lane_id();
   uint64_t inc = v;
 #pragma unroll
@@ -142,35 +140,30 @@ __device__ uint64_t plan_scan(uint64_t v, uint64_t& excl) {
   }
   if (lane == 31) wsum[w] = inc;
   __syncthreads();
-  if (w == 0) {
-    uint64_t x = wsum[lane];
+  uint64_t before = 0, total = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint64_t t = __shfl_up_sync(0xFFFFFFFFu, x, o);
-      if (lane >= (uint32_t)o) x += t;
-    }
-    wsum[lane] = x;
+  for (uint32_t k = 0; k < kWarps; ++k) {
+    before += k < w ? wsum[k] : 0ull;
+    total += wsum[k];
   }
   __syncthreads();
-  excl = inc - v + (w ? wsum[w - 1] : 0ull);
-  const uint64_t total = wsum[kPlanThreads / 32 - 1];
-  __syncthreads();
+  excl = inc - v + before;
   return total;
 }
 
-// Turns the big subsets left by the previous round (list ctl->cur) into the
-// task table of this round: for every subset its tiles, its first tile, its
-// first record among the round's records and its first counter (the host
-// plan of a multi-block step, done on the device).  With use_cond it sets the
-// loop graph's condition: 1 while there is a round to run.
-__global__ void __launch_bounds__(kPlanThreads) k_big_plan(BigCtl* __restrict__ ctl,
-                                                           cudaGraphConditionalHandle h, uint32_t use_cond) {
+// Turns the big subsets on list `list` into the task table and plan of the
+// next round (ctl->cur), by one kBlock block: for every subset its tiles, its
+// first tile, its first record among the round's records and its first
+// counter (the host plan of a multi-block step, done on the device).  Empties
+// the other list, which that round's big children go to.  Every thread
+// returns whether there is a round to run.
+__device__ bool plan_round(BigCtl* ctl, uint32_t list, GenTask* gt) {
+  constexpr uint32_t kPer = 4;  // tasks per thread and pass
   __shared__ uint32_t s_G;
   const SortCtx& c = ctl->c;
-  const uint32_t cur = ctl->cur;
   if (threadIdx.x == 0) {
-    uint32_t g = min(*c.big[cur].count, ctl->cap_big);
-    if (g && (*c.status != 0 || ctl->round >= kMaxBigRounds)) {
+    uint32_t g = min(__ldcg(c.big[list].count), ctl->cap_big);
+    if (g && (__ldcg(c.status) != 0 || ctl->round >= kMaxBigRounds)) {
       if (ctl->round >= kMaxBigRounds) latch_status(c.status, kStTooDeep);
       g = 0;  // stop: this sort has latched an error, or the loop ran too long
     }
@@ -178,66 +171,72 @@ __global__ void __launch_bounds__(kPlanThreads) k_big_plan(BigCtl* __restrict__ 
   }
   __syncthreads();
   uint32_t G = s_G;
-  // strings in this round's subsets, for the tile size
+  const Task* items = c.big[list].items;
+  auto task_at = [&](uint32_t g) {
+    const uint4 v = __ldcg(reinterpret_cast<const uint4*>(items + g));
+    return Task{v.x, v.y, v.z, v.w};
+  };
+  // strings in the round's subsets, for the tile size
   uint64_t mine = 0;
-  for (uint32_t g = threadIdx.x; g < G; g += kPlanThreads) mine += c.big[cur].items[g].len;
+  for (uint32_t g = threadIdx.x; g < G; g += kBlock) mine += task_at(g).len;
   uint64_t ex;
   const uint64_t total = plan_scan(mine, ex);
-  uint32_t R = ctl->R_fixed;
-  if (!R) {
-    const uint64_t per = total / ((uint64_t)ctl->sms * 2 * kBlock) + 1;
-    R = (uint32_t)(per < 8 ? 8 : (per > kMaxRounds ? kMaxRounds : per));
-  }
-  const uint32_t T = kBlock * R;
   const uint64_t K = ctl->K;
-  uint64_t tiles0 = 0, rec0 = 0, cnt0 = 0;
-  for (uint32_t g0 = 0; g0 < G; g0 += kPlanThreads) {
-    const uint32_t g = g0 + threadIdx.x;
-    Task t{0, 0, 0, 0};
-    if (g < G) t = c.big[cur].items[g];
-    const uint32_t tl = (t.len + T - 1) / T;
-    uint64_t e_tiles, e_rec, e_cnt;
-    const uint64_t s_tiles = plan_scan(tl, e_tiles);
-    const uint64_t s_rec = plan_scan(t.len, e_rec);
-    const uint64_t s_cnt = plan_scan(K * tl, e_cnt);
-    if (g < G) {
-      GenTask x;
-      x.t = t;
-      x.tile_start = (uint32_t)(tiles0 + e_tiles);
-      x.tiles = tl;
-      x.rec_base = (uint32_t)(rec0 + e_rec);
-      const uint64_t cb = cnt0 + e_cnt;
-      x.cnt_base_lo = (uint32_t)cb;
-      x.cnt_base_hi = (uint32_t)(cb >> 32);
-      x.pad[0] = x.pad[1] = x.pad[2] = 0;
-      ctl->gt[g] = x;
+  const uint32_t R = tile_rounds(total, G, ctl->sms, (uint32_t)K, ctl->ncounters_max, ctl->R_fixed);
+  const uint32_t T = kBlock * R;
+  uint64_t base = 0;  // tiles (high half) and records (low half) of the passes before
+  for (uint32_t g0 = 0; g0 < G; g0 += kPer * kBlock) {
+    Task t[kPer];
+    uint64_t sum = 0;
+#pragma unroll
+    for (uint32_t u = 0; u < kPer; ++u) {
+      const uint32_t g = g0 + threadIdx.x * kPer + u;
+      t[u] = g < G ? task_at(g) : Task{0, 0, 0, 0};
+      sum += (uint64_t)((t[u].len + T - 1) / T) << 32 | t[u].len;
     }
-    tiles0 += s_tiles;
-    rec0 += s_rec;
-    cnt0 += s_cnt;
+    const uint64_t all = plan_scan(sum, ex);
+    uint64_t at = base + ex;
+#pragma unroll
+    for (uint32_t u = 0; u < kPer; ++u) {
+      const uint32_t g = g0 + threadIdx.x * kPer + u;
+      if (g < G) {
+        GenTask x;
+        x.t = t[u];
+        x.tile_start = (uint32_t)(at >> 32);
+        x.tiles = (t[u].len + T - 1) / T;
+        x.rec_base = (uint32_t)at;
+        const uint64_t cb = K * x.tile_start;
+        x.cnt_base_lo = (uint32_t)cb;
+        x.cnt_base_hi = (uint32_t)(cb >> 32);
+        x.pad[0] = x.pad[1] = x.pad[2] = 0;
+        gt[g] = x;
+        at += (uint64_t)x.tiles << 32 | x.t.len;
+      }
+    }
+    base += all;
   }
+  const uint64_t ncounters = K * (base >> 32);
+  if (ncounters > ctl->ncounters_max) G = 0;  // cannot happen: the counters are sized for the largest round
   if (threadIdx.x == 0) {
-    if (cnt0 > ctl->ncounters_max) {  // cannot happen: the counters are sized for the largest round
-      latch_status(c.status, kStQueueFull);
-      G = 0;
-    }
-    ctl->G = G;
-    ctl->tiles = G ? (uint32_t)tiles0 : 0u;
-    ctl->R = R;
-    ctl->ncounters = G ? cnt0 : 0ull;
-    ctl->next_big = cur ^ 1u;
-    for (int k = 0; k < 2; ++k) ctl->next_item[k] = 0;
+    if (ncounters > ctl->ncounters_max) latch_status(c.status, kStQueueFull);
+    BigPlan p;
+    p.gt = gt;
+    p.G = G;
+    p.tiles = G ? (uint32_t)(base >> 32) : 0u;
+    p.R = R;
+    p.list = list;
+    p.ncounters = G ? ncounters : 0ull;
+    p.next_tile = 0;
+    ctl->cur = p;
     if (G) {
-      *c.big[cur ^ 1u].count = 0;  // the list the round's new big subsets go to
-      ctl->cur = cur ^ 1u;
+      *c.big[list ^ 1u].count = 0;
       ctl->round += 1;
     }
-    if (use_cond) {
-      atomicAdd(&g_graph_launches, 1ull + (G ? kBigRoundKernels : 0ull));
-      cudaGraphSetConditional(h, G ? 1u : 0u);
-    }
   }
+  return G != 0;
 }
+
+__global__ void __launch_bounds__(kBlock) k_big_plan(BigCtl* ctl) { plan_round(ctl, 0, ctl->gtbuf[0]); }
 
 // ---- the kernels of one round -----------------------------------------------------------
 
@@ -384,12 +383,12 @@ __global__ void __launch_bounds__(kSampleThreads<LOGV>) k_big_sample(const BigCt
   SampleSmem<LOGV>& sm = *reinterpret_cast<SampleSmem<LOGV>*>(smem);
   __shared__ uint64_t ref[kPjWindows];
   __shared__ uint32_t s_min;
-  const uint32_t G = ctl->G;
+  const uint32_t G = ctl->cur.G;
   const SortCtx& c = ctl->c;
   BigSplitters<LOGV>* out = reinterpret_cast<BigSplitters<LOGV>*>(ctl->splitters);
   unsigned long long bytes = 0;
   for (uint32_t gi = blockIdx.x; gi < G; gi += gridDim.x) {
-    const GenTask g = ctl->gt[gi];
+    const GenTask g = ctl->cur.gt[gi];
     const uint32_t par = task_par(g.t);
     const SetDesc sd = c.sets[task_set(g.t)];
     const uint64_t hseed = mix64(c.seed ^ ((uint64_t)g.t.begin << 20) ^ g.t.depth);
@@ -450,9 +449,9 @@ __global__ void __launch_bounds__(kBlock, 4) k_big_classify(const BigCtl* __rest
   __shared__ uint64_t ref[kPjWindows];
   __shared__ uint32_t s_g;
   __shared__ uint32_t ts[kTileStartsMax];
-  const uint32_t G = ctl->G, tiles = ctl->tiles, R = ctl->R;
+  const uint32_t G = ctl->cur.G, tiles = ctl->cur.tiles, R = ctl->cur.R;
   const SortCtx& c = ctl->c;
-  const GenTask* __restrict__ gt = ctl->gt;
+  const GenTask* __restrict__ gt = ctl->cur.gt;
   BigSplitters<LOGV>* spl = reinterpret_cast<BigSplitters<LOGV>*>(ctl->splitters);
   const bool use_jump = c.classifier == kClassifyUIJ;
   load_tile_starts(gt, G, ts);
@@ -512,22 +511,26 @@ __global__ void __launch_bounds__(kBlock, 4) k_big_classify(const BigCtl* __rest
 }
 
 // Buckets of one subset handled by one block of k_big_emit: one per thread.
-// The kernel is a chain of dependent loads and counter atomics per bucket, so
+// This part of the kernel is a chain of dependent loads and counter atomics per bucket, so
 // a subset's buckets are spread over KP / 256 blocks instead of four rounds of
 // one block (1 M URLs: 15-22 us -> 7-8 us a round).
 template <int LOGV>
-__global__ void __launch_bounds__(kBlock) k_big_emit(const BigCtl* __restrict__ ctl) {
+__global__ void __launch_bounds__(kBlock) k_big_emit(BigCtl* ctl, cudaGraphConditionalHandle h,
+                                                           uint32_t use_cond) {
   using Gm = Geo<LOGV>;
   constexpr uint32_t kParts = Gm::KP / kBlock;
-  const uint32_t items = ctl->G * kParts;
+  const BigPlan plan = ctl->cur;
+  const uint32_t items = plan.G * kParts;
+  const uint32_t blocks = max(1u, min(items, gridDim.x));  // blocks with work (or the one that ends the loop)
+  if (blockIdx.x >= blocks) return;
   const SortCtx& c = ctl->c;
   const BigSplitters<LOGV>* spl = reinterpret_cast<const BigSplitters<LOGV>*>(ctl->splitters);
-  const uint32_t next_big = ctl->next_big;
+  const uint32_t next_big = plan.list ^ 1u;
   unsigned long long bytes = 0;
   for (uint32_t it = blockIdx.x; it < items; it += gridDim.x) {
     const uint32_t gi = it / kParts;
     const uint32_t b = (it % kParts) * kBlock + threadIdx.x;
-    const GenTask g = ctl->gt[gi];
+    const GenTask g = plan.gt[gi];
     const Splitters<LOGV, u128>& sp = spl[gi].sp;
     const SetDesc sd = c.sets[task_set(g.t)];
     const uint32_t* sc = ctl->counters + cnt_base(g);
@@ -558,6 +561,24 @@ __global__ void __launch_bounds__(kBlock) k_big_emit(const BigCtl* __restrict__ 
     }
   }
   account(c, kKBigEmit, bytes);
+  // the last block to finish plans the next round
+  __shared__ uint32_t s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&ctl->emitted, 1u) == blocks - 1 ? 1u : 0u;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (threadIdx.x == 0) {
+    ctl->emitted = 0;
+    ctl->mv = plan;
+    ctl->mv.next_tile = 0;
+  }
+  const bool more = plan_round(ctl, next_big, ctl->gtbuf[plan.gt == ctl->gtbuf[0] ? 1 : 0]);
+  if (use_cond && threadIdx.x == 0) {
+    if (plan.G) atomicAdd(&g_graph_launches, (unsigned long long)kBigRoundKernels);
+    cudaGraphSetConditional(h, more ? 1u : 0u);
+  }
 }
 
 template <int LOGV>
@@ -571,9 +592,9 @@ __global__ void __launch_bounds__(kBlock, 3) k_big_scatter(const BigCtl* __restr
   uint16_t* tb = reinterpret_cast<uint16_t*>(bfirst + Gm::KP);
   __shared__ uint32_t s_g;
   __shared__ uint32_t ts[kTileStartsMax];
-  const uint32_t G = ctl->G, tiles = ctl->tiles, R = ctl->R;
+  const uint32_t G = ctl->mv.G, tiles = ctl->mv.tiles, R = ctl->mv.R;
   const SortCtx& c = ctl->c;
-  const GenTask* __restrict__ gt = ctl->gt;
+  const GenTask* __restrict__ gt = ctl->mv.gt;
   load_tile_starts(gt, G, ts);
   unsigned long long bytes = 0;
   uint32_t loaded = 0xFFFFFFFFu;
@@ -677,9 +698,9 @@ __device__ __forceinline__ void load_scan_items(const uint32_t* __restrict__ a, 
 }
 
 // Phase 1: the total of every chunk of kScanChunk counters of the round
-// (ctl->ncounters values).
+// (ctl->cur.ncounters values).
 __global__ void __launch_bounds__(kBlock) k_scan_reduce(const BigCtl* __restrict__ ctl) {
-  const uint64_t n = ctl->ncounters;
+  const uint64_t n = ctl->cur.ncounters;
   const uint32_t* __restrict__ a = ctl->counters;
   uint32_t* __restrict__ part = ctl->partials;
   const uint64_t nb = (n + kScanChunk - 1) / kScanChunk;
@@ -707,7 +728,7 @@ __global__ void __launch_bounds__(kBlock) k_scan_reduce(const BigCtl* __restrict
 // (carried from one of its chunks to its next), so no third kernel scans the
 // totals.
 __global__ void __launch_bounds__(kBlock) k_scan_down(const BigCtl* __restrict__ ctl) {
-  const uint64_t n = ctl->ncounters;
+  const uint64_t n = ctl->cur.ncounters;
   uint32_t* __restrict__ a = ctl->counters;
   const uint32_t* __restrict__ part = ctl->partials;
   const uint64_t nb = (n + kScanChunk - 1) / kScanChunk;
@@ -764,17 +785,14 @@ size_t big_scatter_smem(int logv, uint32_t R) {
   return (size_t)(kWarps * KP + 3 * KP) * 4 + (size_t)kBlock * R * 2;
 }
 
-cudaError_t launch_big_plan(BigCtl* ctl, uint64_t cond_handle, bool use_cond, cudaStream_t st,
-                            const LaunchHook& hook) {
-  hook.run("big_sample", [&] {
-    k_big_plan<<<1, kPlanThreads, 0, st>>>(ctl, (cudaGraphConditionalHandle)cond_handle, use_cond ? 1u : 0u);
-  });
+cudaError_t launch_big_plan(BigCtl* ctl, cudaStream_t st, const LaunchHook& hook) {
+  hook.run("big_sample", [&] { k_big_plan<<<1, kBlock, 0, st>>>(ctl); });
   return cudaGetLastError();
 }
 
 template <int LOGV>
-static cudaError_t launch_big_round_t(BigCtl* ctl, uint32_t R_max, uint32_t sms, cudaStream_t st,
-                                      const LaunchHook& hook) {
+static cudaError_t launch_big_round_t(BigCtl* ctl, uint32_t R_max, uint32_t sms, uint64_t cond, bool use_cond,
+                                      cudaStream_t st, const LaunchHook& hook) {
   const size_t smem = big_scatter_smem(LOGV, R_max);
   static bool attr_set = false;
   if (!attr_set) {
@@ -791,19 +809,21 @@ static cudaError_t launch_big_round_t(BigCtl* ctl, uint32_t R_max, uint32_t sms,
   hook.run("big_sample", [&] { 
     k_big_sample<LOGV><<<sms * (2048 / kSampleThreads<LOGV>), kSampleThreads<LOGV>, sizeof(SampleSmem<LOGV>), st>>>(ctl);
   });
-  hook.run("big_classify", [&] { k_big_classify<LOGV><<<sms * 8, kBlock, 0, st>>>(ctl, &ctl->next_item[0]); });
+  hook.run("big_classify", [&] { k_big_classify<LOGV><<<sms * 8, kBlock, 0, st>>>(ctl, &ctl->cur.next_tile); });
   hook.run("scan", [&] { k_scan_reduce<<<sms * 8, kBlock, 0, st>>>(ctl); });
   hook.run("scan", [&] { k_scan_down<<<sms * 8, kBlock, 0, st>>>(ctl); });
-  hook.run("big_emit", [&] { k_big_emit<LOGV><<<sms * 8, kBlock, 0, st>>>(ctl); });
-  hook.run("big_scatter", [&] { k_big_scatter<LOGV><<<sms * 3, kBlock, smem, st>>>(ctl, &ctl->next_item[1]); });
+  hook.run("big_emit", [&] {
+    k_big_emit<LOGV><<<sms * 8, kBlock, 0, st>>>(ctl, (cudaGraphConditionalHandle)cond, use_cond ? 1u : 0u);
+  });
+  hook.run("big_scatter", [&] { k_big_scatter<LOGV><<<sms * 3, kBlock, smem, st>>>(ctl, &ctl->mv.next_tile); });
   return cudaGetLastError();
 }
 
-cudaError_t launch_big_round(int logv, BigCtl* ctl, uint32_t R_max, uint32_t sms, cudaStream_t st,
-                             const LaunchHook& hook) {
+cudaError_t launch_big_round(int logv, BigCtl* ctl, uint32_t R_max, uint32_t sms, uint64_t cond_handle, bool use_cond,
+                             cudaStream_t st, const LaunchHook& hook) {
   switch (logv) {
-    case 8: return launch_big_round_t<8>(ctl, R_max, sms, st, hook);
-    case 9: return launch_big_round_t<9>(ctl, R_max, sms, st, hook);
+    case 8: return launch_big_round_t<8>(ctl, R_max, sms, cond_handle, use_cond, st, hook);
+    case 9: return launch_big_round_t<9>(ctl, R_max, sms, cond_handle, use_cond, st, hook);
     default: return cudaErrorInvalidValue;  // 2^10 wide splitters exceed static shared memory
   }
 }

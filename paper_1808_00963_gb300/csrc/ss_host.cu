@@ -230,7 +230,11 @@ static Layout make_layout(uint64_t M, uint32_t num_sets, const Opts& o, bool big
   L.cap_sc = (uint32_t)(M / 33 + 2);
   L.cap_scw = (uint32_t)(M / (kSmallCtaNarrowMax + 1) + 2);
   const uint64_t KP = 2ull << o.logv_big;
-  const uint64_t tiles_max = big ? M / (kBlock * 8) + L.cap_big : 0;
+  // tiles of the largest round: tile_rounds gives one over all strings the
+  // tile of a GPU of kSizingSms SMs if its counters fit, else up to 8 rounds
+  constexpr uint32_t kSizingSms = 152;
+  const uint32_t R0 = tile_rounds(M, 1, kSizingSms, (2u << o.logv_big) - 1, ~0ull, 0);
+  const uint64_t tiles_max = big ? M / (kBlock * std::min(R0, 8u)) + L.cap_big : 0;
   L.ncounters_max = big ? KP * (tiles_max + L.cap_big) : 0;
   L.ctrl = take(kCtrlBytes);
   L.sets = take((size_t)num_sets * sizeof(SetDesc));
@@ -242,7 +246,7 @@ static Layout make_layout(uint64_t M, uint32_t num_sets, const Opts& o, bool big
   L.bucket_of = take(M * 2);
   L.big0 = take((size_t)L.cap_big * sizeof(Task));
   L.big1 = take((size_t)L.cap_big * sizeof(Task));
-  L.gen = take((size_t)L.cap_big * sizeof(GenTask));
+  L.gen = take(2 * (size_t)L.cap_big * sizeof(GenTask));
   L.spl = take((size_t)L.cap_big * big_splitters_bytes(o.logv_big));
   L.counters = take(L.ncounters_max * 4);
   L.partials = take((L.ncounters_max / 4096 + 2) * 4);
@@ -344,8 +348,12 @@ static cudaError_t zero_fill(void* dst, size_t bytes, cudaStream_t st, const Lau
 // neither stages it nor waits for a copy before enqueuing the sort.
 __global__ void k_set_desc(SetDesc* dst, SetDesc v) { *dst = v; }
 
-// Writes the control block of the multi-block loop (same reason).
-__global__ void k_set_ctl(BigCtl* dst, BigCtl v) { *dst = v; }
+// Writes the control block of the multi-block loop (same reason), and the
+// task of the first round where the host knows it (one set: its root).
+__global__ void k_set_ctl(BigCtl* dst, BigCtl v, GenTask root) {
+  *dst = v;
+  if (v.cur.G) v.cur.gt[0] = root;
+}
 
 // A batch's set descriptors, up to kDescChunk per launch (kernel parameters).
 constexpr uint32_t kDescChunk = 128;
@@ -358,11 +366,11 @@ __global__ void k_set_descs(SetDesc* dst, uint32_t count, SetDescChunk v) {
 
 // ---- the multi-block loop as a CUDA graph -------------------------------------------------
 //
-// One round of multi-block steps is a plan kernel plus the round's kernels, all
-// reading the control block in device memory.  The rounds run in a graph with
-// a conditional WHILE node: the plan before the loop and the plan at the end
-// of each round set the condition to 1 while big subsets remain, so the host
-// enqueues the whole loop with one graph launch and never waits for it.  The
+// The kernels of one round of multi-block steps all read the control block in
+// device memory.  The rounds run in a graph with a conditional WHILE node: the
+// emit kernel of each round plans the next one and sets the condition to 1
+// while big subsets remain, so the host enqueues the whole loop with one graph
+// launch and never waits for it.  The
 // graph depends only on the control block's address and the step geometry;
 // it is built once per stream (whose control block every sort and batch run
 // on that stream uses) and reused.  A run inside a caller's stream capture
@@ -403,14 +411,14 @@ static cudaError_t capture_streams(CaptureStreams*& out) {
   return cudaSuccess;
 }
 
-// Adds the loop to the graph being captured on `st`: the first plan, then a
-// WHILE node whose body is one round and the next plan.  Work captured on st
-// afterwards depends on the loop.
+// Adds the loop to the graph being captured on `st`: a WHILE node whose body
+// is one round (its emit plans the next one and sets the condition; the first
+// round always runs, the plan for it is in the control block).  Work captured
+// on st afterwards depends on the loop.
 static cudaError_t add_loop(cudaStream_t st, BigCtl* ctl, int logv, uint32_t R_max, uint32_t sms) {
   CaptureStreams* cs = nullptr;
   cudaError_t e = capture_streams(cs);
   if (e != cudaSuccess) return e;
-  const LaunchHook hook{st};
   cudaStreamCaptureStatus status;
   cudaGraph_t graph = nullptr;
   const cudaGraphNode_t* deps = nullptr;
@@ -418,9 +426,7 @@ static cudaError_t add_loop(cudaStream_t st, BigCtl* ctl, int logv, uint32_t R_m
   if ((e = cudaStreamGetCaptureInfo(st, &status, nullptr, &graph, &deps, nullptr, &ndeps)) != cudaSuccess) return e;
   if (status != cudaStreamCaptureStatusActive) return cudaErrorStreamCaptureInvalidated;
   cudaGraphConditionalHandle h;
-  if ((e = cudaGraphConditionalHandleCreate(&h, graph, 0, cudaGraphCondAssignDefault)) != cudaSuccess) return e;
-  if ((e = launch_big_plan(ctl, (uint64_t)h, true, st, hook)) != cudaSuccess) return e;
-  if ((e = cudaStreamGetCaptureInfo(st, &status, nullptr, &graph, &deps, nullptr, &ndeps)) != cudaSuccess) return e;
+  if ((e = cudaGraphConditionalHandleCreate(&h, graph, 1, cudaGraphCondAssignDefault)) != cudaSuccess) return e;
   cudaGraphNodeParams p{};
   p.type = cudaGraphNodeTypeConditional;
   p.conditional.handle = h;
@@ -433,12 +439,10 @@ static cudaError_t add_loop(cudaStream_t st, BigCtl* ctl, int logv, uint32_t R_m
       cudaSuccess)
     return e;
   const LaunchHook bhook{cs->body};
-  cudaError_t e1 = launch_big_round(logv, ctl, R_max, sms, cs->body, bhook);
-  cudaError_t e2 = launch_big_plan(ctl, (uint64_t)h, true, cs->body, bhook);
+  cudaError_t e1 = launch_big_round(logv, ctl, R_max, sms, (uint64_t)h, true, cs->body, bhook);
   cudaGraph_t done = nullptr;
   e = cudaStreamEndCapture(cs->body, &done);
   if (e1 != cudaSuccess) return e1;
-  if (e2 != cudaSuccess) return e2;
   if (e != cudaSuccess) return e;
   return cudaStreamUpdateCaptureDependencies(st, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
 }
@@ -524,7 +528,8 @@ static ss_status run_sort(uint8_t* ws, const Layout& L, SortCtx c, const Opts& o
     if (!ctl) return SS_ERR_INVALID;
     BigCtl v{};
     v.c = c;
-    v.gt = reinterpret_cast<GenTask*>(ws + L.gen);
+    v.gtbuf[0] = reinterpret_cast<GenTask*>(ws + L.gen);
+    v.gtbuf[1] = v.gtbuf[0] + L.cap_big;
     v.splitters = ws + L.spl;
     v.counters = reinterpret_cast<uint32_t*>(ws + L.counters);
     v.partials = reinterpret_cast<uint32_t*>(ws + L.partials);
@@ -535,10 +540,21 @@ static ss_status run_sort(uint8_t* ws, const Layout& L, SortCtx c, const Opts& o
     v.R_fixed = o.R;
     v.sms = (uint32_t)dev.sms;
     v.K = (2u << o.logv_big) - 1;
-    v.cur = 0;
-    v.round = 0;
-    hook.run("init", [&] { k_set_ctl<<<1, 1, 0, st>>>(ctl, v); });
+    GenTask root{};
+    if (c.num_sets == 1) {  // the first round's plan: one subset, the whole set
+      const uint32_t R = tile_rounds(c.total, 1, v.sms, v.K, v.ncounters_max, o.R);
+      root.t = Task{0, c.total, 0, make_meta(0, 0)};
+      root.tiles = (c.total + kBlock * R - 1) / (kBlock * R);
+      v.cur.gt = v.gtbuf[0];
+      v.cur.G = 1;
+      v.cur.tiles = root.tiles;
+      v.cur.R = R;
+      v.cur.ncounters = (uint64_t)v.K * root.tiles;
+      v.round = 1;
+    }
+    hook.run("init", [&] { k_set_ctl<<<1, 1, 0, st>>>(ctl, v, root); });
     SS_CUDA(cudaGetLastError());
+    if (c.num_sets > 1) SS_CUDA(launch_big_plan(ctl, st, hook));
     const uint32_t R_max = o.R ? o.R : kMaxRounds;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     SS_CUDA(cudaStreamIsCapturing(st, &cs));
@@ -549,14 +565,12 @@ static ss_status run_sort(uint8_t* ws, const Layout& L, SortCtx c, const Opts& o
       // launch by launch (timed, or for a profiler): the host runs the rounds, reading each plan
       if (t_down.reserve(64) != SS_OK) return SS_ERR_OOM;
       uint32_t* hG = static_cast<uint32_t*>(t_down.p);
-      while (true) {
-        SS_CUDA(launch_big_plan(ctl, 0, false, st, hook));
-        SS_CUDA(cudaMemcpyAsync(hG, &ctl->G, 4, cudaMemcpyDeviceToHost, st));
+      do {
+        SS_CUDA(launch_big_round(o.logv_big, ctl, R_max, (uint32_t)dev.sms, 0, false, st, hook));
+        SS_CUDA(cudaMemcpyAsync(hG, &ctl->cur.G, 4, cudaMemcpyDeviceToHost, st));
         SS_CUDA(cudaStreamSynchronize(st));
         collect_profile();
-        if (*hG == 0) break;
-        SS_CUDA(launch_big_round(o.logv_big, ctl, R_max, (uint32_t)dev.sms, st, hook));
-      }
+      } while (*hG);
     } else {
       cudaGraphExec_t exec = nullptr;
       SS_CUDA(loop_exec(ctl, o.logv_big, R_max, (uint32_t)dev.sms, &exec));

@@ -19,14 +19,27 @@ struct LaunchHook {
   void run(const char* name, const std::function<void()>& launch) const;
 };
 
+// Plan of one round of multi-block steps: its task table and geometry.
+struct BigPlan {
+  GenTask* gt;            // the round's subsets
+  uint32_t G;             // how many (0: the loop ends)
+  uint32_t tiles;         // tiles over them
+  uint32_t R;             // tile = 256 * R records
+  uint32_t list;          // big list they came from; their big children go to the other one
+  uint64_t ncounters;
+  uint32_t next_tile;     // work counter: blocks take the next tile from it, so that uneven tiles balance out
+};
+
 // Control block of the multi-block steps in device memory.  The host fills
-// the first part once per sort; k_big_plan writes the plan of each round from
-// the list of big subsets the previous round left, and every kernel of the
-// round reads it there, so rounds follow one another with no host in the loop
-// (Section 4.2.8: the fully parallel levels need no sequential coordinator).
+// the first part once per sort (and the first round's plan, if it knows it:
+// a single set is one subset); the last block of each round's k_big_emit
+// writes the plan of the next round from the list of big subsets this round
+// leaves (a planning kernel before each round took 6-8 us), so rounds follow
+// one another with no host in between (Section 4.2.8: the fully parallel levels need no sequential
+// coordinator).  The scatter, which runs after that, reads the copy in `mv`.
 struct BigCtl {
   SortCtx c;
-  GenTask* gt;            // cap_big tasks of the current round
+  GenTask* gtbuf[2];      // cap_big tasks each, for two successive rounds
   void* splitters;        // cap_big * big_splitters_bytes(logv)
   uint32_t* counters;     // [task][bucket][tile] counters of the round
   uint32_t* partials;     // ncounters_max / 4096 + 2
@@ -37,37 +50,47 @@ struct BigCtl {
   uint32_t R_fixed;       // tile rounds; 0: chosen per round from the strings in big subsets
   uint32_t sms;
   uint32_t K;             // buckets per step, 2^(logv + 1) - 1
-  // the plan of the current round (k_big_plan)
-  uint32_t cur;           // big list the next plan reads
-  uint32_t next_big;      // big list the current round's new big subsets go to
   uint32_t round;
-  uint32_t G;             // big subsets of the round (0: the loop ends)
-  uint32_t tiles;         // tiles over them
-  uint32_t R;             // tile = 256 * R records
-  uint64_t ncounters;
-  // work counters of the round's kernels (zeroed by the plan): blocks take
-  // the next tile from them, so that uneven tiles balance out
-  uint32_t next_item[2];  // classify, scatter
+  uint32_t emitted;       // blocks of the round's k_big_emit that are done
+  BigPlan cur;            // the round's plan, as all its kernels but the scatter read it
+  BigPlan mv;             // the same, for the scatter (k_big_emit has put the next round's into cur by then)
 };
+
+// Rounds of 256 strings in a tile of a round over `total` strings in G
+// subsets: two tiles per SM where there are that many strings, at least
+// kMinTileRounds (a tile's fixed work is its 2^(logv + 1) counters; with a
+// minimum of 8, 100 k strings filled 49 of 152 SMs: classification 17.3 ->
+// 12.8 us, scatter 22.9 -> 15.4 us), at most kMaxTileRounds, and more where
+// the tiles' counters would not fit.
+constexpr uint32_t kMinTileRounds = 2, kMaxTileRounds = 32;
+__host__ __device__ inline uint32_t tile_rounds(uint64_t total, uint64_t G, uint32_t sms, uint32_t K,
+                                                uint64_t ncounters_max, uint32_t fixed) {
+  if (fixed) return fixed;
+  const uint64_t per = total / ((uint64_t)sms * 2 * 256) + 1;
+  uint32_t R = (uint32_t)(per < kMinTileRounds ? kMinTileRounds : (per > kMaxTileRounds ? kMaxTileRounds : per));
+  while (R < 8 && K * (total / (256ull * R) + G) > ncounters_max) ++R;
+  return R;
+}
 
 // Most rounds of multi-block steps one sort may take (each advances every big
 // subset by at least one character; a subset sharing more than about 2^20
 // characters is reported as SS_ERR_TOO_LARGE).
 constexpr uint32_t kMaxBigRounds = 1u << 20;
 
-// Kernel launches of one multi-block round after its plan: sample, classify,
-// the two prefix-sum kernels, emit and scatter.
+// Kernel launches of one multi-block round: sample, classify, the two
+// prefix-sum kernels, emit and scatter.
 constexpr uint32_t kBigRoundKernels = 6;
 
 size_t big_splitters_bytes(int logv);
 size_t big_scatter_smem(int logv, uint32_t R);
-// The plan of the next round; with use_cond it also sets the loop graph's
-// condition (1 while big subsets remain).
-cudaError_t launch_big_plan(BigCtl* ctl, uint64_t cond_handle, bool use_cond, cudaStream_t st,
-                            const LaunchHook& hook);
-// The kernels of one round (they do nothing when the plan found no subset).
-cudaError_t launch_big_round(int logv, BigCtl* ctl, uint32_t R_max, uint32_t sms, cudaStream_t st,
-                             const LaunchHook& hook);
+// The plan of the first round from list 0 (for several sets; a single set's
+// is written by the host).
+cudaError_t launch_big_plan(BigCtl* ctl, cudaStream_t st, const LaunchHook& hook);
+// The kernels of one round (they do nothing when its plan holds no subset);
+// with use_cond it also sets the loop graph's condition (1 while big subsets
+// remain).
+cudaError_t launch_big_round(int logv, BigCtl* ctl, uint32_t R_max, uint32_t sms, uint64_t cond_handle, bool use_cond,
+                             cudaStream_t st, const LaunchHook& hook);
 // Kernels the loop graphs of this device have launched so far (their plan
 // kernels count them on the device; reading the count waits for the device).
 uint64_t graph_launch_count();
