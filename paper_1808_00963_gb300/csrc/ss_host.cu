@@ -555,7 +555,7 @@ static ss_status run_sort(uint8_t* ws, const Layout& L, SortCtx c, const Opts& o
     hook.run("init", [&] { k_set_ctl<<<1, 1, 0, st>>>(ctl, v, root); });
     SS_CUDA(cudaGetLastError());
     if (c.num_sets > 1) SS_CUDA(launch_big_plan(ctl, st, hook));
-    const uint32_t R_max = o.R ? o.R : kMaxRounds;
+    const uint32_t R_max = o.R ? o.R : kMaxTileRounds;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     SS_CUDA(cudaStreamIsCapturing(st, &cs));
     if (cs == cudaStreamCaptureStatusActive) {

@@ -61,8 +61,11 @@ struct BigCtl {
 // kMinTileRounds (a tile's fixed work is its 2^(logv + 1) counters; with a
 // minimum of 8, 100 k strings filled 49 of 152 SMs: classification 17.3 ->
 // 12.8 us, scatter 22.9 -> 15.4 us), at most kMaxTileRounds, and more where
-// the tiles' counters would not fit.
-constexpr uint32_t kMinTileRounds = 2, kMaxTileRounds = 32;
+// the tiles' counters would not fit.  With at most 16 the scatter's shared
+// memory lets three blocks share an SM instead of two (20 M URLs 4820 -> 4415
+// us, 4 M DNA suffixes 1270 -> 1201 us; at most 8: 4401 / 1164 us, but the
+// batch of 512 sets 2637 instead of 2620 us and twice the counters).
+constexpr uint32_t kMinTileRounds = 2, kMaxTileRounds = 16;
 __host__ __device__ inline uint32_t tile_rounds(uint64_t total, uint64_t G, uint32_t sms, uint32_t K,
                                                 uint64_t ncounters_max, uint32_t fixed) {
   if (fixed) return fixed;

@@ -9,7 +9,7 @@ namespace ss {
 
 constexpr uint32_t kBlock = 256;
 constexpr uint32_t kWarps = kBlock / 32;
-constexpr uint32_t kMaxRounds = 32;                  // tile = 256 * rounds records (kMaxTileRounds)
+constexpr uint32_t kMaxRounds = 32;                  // tile = 256 * rounds records
 constexpr uint32_t kMaxTile = kBlock * kMaxRounds;
 constexpr uint32_t kFin = 1u << 31;                  // bucket descriptor: finished
 constexpr uint32_t kNulEq = 1u << 30;                // ... all members equal strings
