@@ -22,9 +22,9 @@
  *                         out_perm[j-1] and out_perm[j].  Two equal strings
  *                         have lcp = their length.
  * Reads of a string stay inside the 4 KiB-aligned blocks that hold a byte of
- * the string or its terminator: the library loads aligned 8-byte words, and
- * when it looks ahead along a long common prefix it may read bytes past a
- * terminator inside such a block (they are ignored).  Memory is mapped in
+ * the string or its terminator: the library loads aligned words of 8 or 16
+ * bytes and may read bytes before a string or past its terminator inside such
+ * a block (they are ignored).  Memory is mapped in
  * blocks of at least 4 KiB, so these reads never leave mapped memory.
  *
  * Streams: `stream` is a cudaStream_t passed as void* (NULL = legacy default

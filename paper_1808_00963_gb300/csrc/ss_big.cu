@@ -25,8 +25,9 @@ __device__ __forceinline__ uint32_t find_gen_task(const GenTask* gt, uint32_t G,
 // The first tile of every subset of the round, for up to kTileStartsMax
 // subsets, copied into shared memory when a kernel starts: a block then finds
 // the subset of each tile it takes with a shared-memory search instead of a
-// chain of dependent global loads.
-constexpr uint32_t kTileStartsMax = 4096;
+// chain of dependent global loads.  1024 subsets: the table shares an SM's
+// shared memory with three scatter blocks' counters (see kMaxTileRounds).
+constexpr uint32_t kTileStartsMax = 1024;
 
 __device__ __forceinline__ void load_tile_starts(const GenTask* gt, uint32_t G, uint32_t* ts) {
   const uint32_t m = G < kTileStartsMax ? G : kTileStartsMax;

@@ -188,119 +188,161 @@ __device__ __forceinline__ uint64_t load_cache(const uint8_t* chars, uint64_t of
   return bswap64(v);
 }
 
-// load_cache with both words issued at once: when the window is unaligned and
-// the second aligned word lies in the same 4 KiB block as byte h, it is loaded
-// together with the first (one memory round trip instead of two; bytes past
-// the terminator are discarded); across a block boundary it is loaded only if
-// the first word holds no terminator, as in load_cache.  Same result and
-// precondition as load_cache.
-__device__ __forceinline__ uint64_t load_cache_2w(const uint8_t* chars, uint64_t off, uint32_t h,
+// Position (0..7) of the first zero byte of a cache (first character most
+// significant), 8 if none.  Exact per byte: no borrow runs between bytes.
+__device__ __forceinline__ uint32_t first_nul(uint64_t w) {
+  constexpr uint64_t k7F = 0x7F7F7F7F7F7F7F7Full;
+  const uint64_t z = ~(((w & k7F) + k7F) | w | k7F);
+  return z ? (uint32_t)__clzll((long long)z) >> 3 : 8u;
+}
+
+// A cache cut to its first `keep` characters (0..8).
+__device__ __forceinline__ uint64_t keep_chars(uint64_t w, uint32_t keep) {
+  return keep >= 8 ? w : (keep ? w & (~0ull << (64 - 8 * keep)) : 0ull);
+}
+
+// Character reads with 16-byte loads.  The 16 characters at an address lie in
+// at most two aligned 16-byte words, against three 8-byte ones; gathers from
+// random strings are bound by the number of such requests a warp has to issue
+// and wait for, and by the instructions around them (with 8-byte words and a
+// mask per word: 20 M URLs 4711 us, with these 4381; 4 M DNA suffixes 1211 /
+// 1126, 1 M records under a 200-character prefix 1097 / 940, a 16-way merge of
+// 20 M URLs 4128 / 3867).  Only words inside the 4 KiB-aligned block that holds
+// the first byte are read: memory is mapped in blocks of at least 4 KiB, so
+// these reads cannot fault, and bytes past the terminator are discarded.  A window that runs past that block is read word
+// by word instead, while the string continues (load_cache).
+//
+// Two phases, so that a thread can have the reads of several strings in
+// flight before it uses any of them: issue_chars loads the words,
+// finish_chars8 / finish_chars16 turn them into the 8 or 16 characters from
+// depth h (first character most significant, zero at / after the terminator
+// or the cap).  Precondition: the string has no terminator before h, so the
+// byte at h belongs to the string (or is its terminator).
+struct CharWords {
+  uint4 a, b;
+};
+
+__device__ __forceinline__ bool chars_in_block(uintptr_t at) { return (at & 4095u) <= 4096u - 16u; }
+
+// Bytes [at, at + 32) rounded down to 16; the second word only if bytes
+// [at, at + need) reach it.  need: 8 or 16.
+__device__ __forceinline__ void issue_chars(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap,
+                                            uint32_t need, CharWords& w) {
+  const uintptr_t at = (uintptr_t)(chars + off + h);
+  w.a = make_uint4(0, 0, 0, 0);
+  w.b = make_uint4(0, 0, 0, 0);
+  if (h < cap && chars_in_block(at)) {
+    const uint4* p = reinterpret_cast<const uint4*>(at & ~(uintptr_t)15);
+    w.a = __ldg(p);
+    if ((uint32_t)(at & 15u) + need > 16u) w.b = __ldg(p + 1);
+  }
+}
+
+// Bytes [sh, sh + 4 N) (sh < 16) of a sequence of 32-bit words x, as N words
+// with the first byte most significant.
+template <int N>
+__device__ __forceinline__ void take_words(const uint32_t (&x)[N + 4], uint32_t sh, uint32_t (&out)[N]) {
+  const bool s8 = sh & 8u, s4 = sh & 4u;
+  uint32_t t[N + 2], y[N + 1];
+#pragma unroll
+  for (int i = 0; i < N + 2; ++i) t[i] = s8 ? x[i + 2] : x[i];
+#pragma unroll
+  for (int i = 0; i < N + 1; ++i) y[i] = s4 ? t[i + 1] : t[i];
+  const uint32_t sel = 0x0123u + 0x1111u * (sh & 3u);
+#pragma unroll
+  for (int i = 0; i < N; ++i) out[i] = __byte_perm(y[i], y[i + 1], sel);
+}
+
+__device__ __forceinline__ uint64_t finish_chars8(const CharWords& w, const uint8_t* chars, uint64_t off, uint32_t h,
                                                   uint32_t cap) {
   if (h >= cap) return 0;
-  const uintptr_t a = (uintptr_t)(chars + off + h);
-  const uint64_t* p = (const uint64_t*)(a & ~(uintptr_t)7);
-  const uint32_t sh = (uint32_t)(a & 7);
-  const bool same_block = (((uintptr_t)(p + 1)) & 4095u) != 0;
-  const uint64_t w0 = __ldg(p);
-  uint64_t w1 = (sh && same_block) ? __ldg(p + 1) : 0ull;
-  uint64_t v = w0 >> (8 * sh);
-  const uint32_t room = cap - h;
-  uint32_t z;
-  if (sh == 0) {
-    z = first_zero_byte(v);
-  } else {
-    const uint32_t nb0 = 8 - sh;
-    z = first_zero_byte(v | (~0ull << (8 * nb0)));
-    if (z >= nb0 && room > nb0) {
-      if (!same_block) w1 = __ldg(p + 1);
-      v |= w1 << (8 * nb0);
-      z = first_zero_byte(v);
-    }
+  const uintptr_t at = (uintptr_t)(chars + off + h);
+  if (!chars_in_block(at)) return load_cache(chars, off, h, cap);
+  const uint32_t x[6] = {w.a.x, w.a.y, w.a.z, w.a.w, w.b.x, w.b.y};
+  uint32_t o[2];
+  take_words<2>(x, (uint32_t)(at & 15u), o);
+  const uint64_t k = ((uint64_t)o[0] << 32) | o[1];
+  return keep_chars(k, min(first_nul(k), cap - h));
+}
+
+__device__ __forceinline__ void finish_chars16(const CharWords& w, const uint8_t* chars, uint64_t off, uint32_t h,
+                                               uint32_t cap, uint64_t& hi, uint64_t& lo) {
+  hi = 0;
+  lo = 0;
+  if (h >= cap) return;
+  const uintptr_t at = (uintptr_t)(chars + off + h);
+  if (!chars_in_block(at)) {
+    hi = load_cache(chars, off, h, cap);
+    if (hi & 0xFFu) lo = load_cache(chars, off, h + 8, cap);
+    return;
   }
-  uint32_t keep = z < room ? z : room;
-  if (keep < 8) v &= (keep == 0) ? 0ull : (~0ull >> (64 - 8 * keep));
-  return bswap64(v);
+  const uint32_t x[8] = {w.a.x, w.a.y, w.a.z, w.a.w, w.b.x, w.b.y, w.b.z, w.b.w};
+  uint32_t o[4];
+  take_words<4>(x, (uint32_t)(at & 15u), o);
+  hi = ((uint64_t)o[0] << 32) | o[1];
+  lo = ((uint64_t)o[2] << 32) | o[3];
+  const uint32_t room = cap - h;
+  const uint32_t k0 = min(first_nul(hi), room);
+  hi = keep_chars(hi, k0);
+  lo = k0 < 8 ? 0ull : keep_chars(lo, min(first_nul(lo), room - 8));
+}
+
+// The 8 characters of the string at `off` from depth h (as load_cache, both
+// words requested at once).
+__device__ __forceinline__ uint64_t load_chars8(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap) {
+  CharWords w;
+  issue_chars(chars, off, h, cap, 8, w);
+  return finish_chars8(w, chars, off, h, cap);
 }
 
 constexpr int kLookWindows = 8;  // look-ahead: 8 windows = 64 characters per round
 
 // Look-ahead read for the refinement of long common prefixes: the KW windows
 // of 8 characters at depths h, h + 8, ..., h + 8(KW-1) (first character most
-// significant, zero at/after the terminator or the cap).  Precondition: the
-// string has no terminator before h, so the byte at h belongs to the string
-// (or is its terminator).  All KW + 1 aligned words are issued at once, but
-// only words inside the 4 KiB-aligned block that holds byte h are read: memory
-// is mapped in blocks of at least 4 KiB, so these reads cannot fault, and bytes
-// past the terminator are discarded.  Returns how many leading windows are
-// fully determined (windows past the block, before a terminator was seen, are
-// not).
-//
-// Two phases, so that a thread can have the reads of several strings in
-// flight before it uses any of them: issue_windows loads the words,
-// finish_windows turns them into the windows.
-template <int KW>
-struct WindowWords {
-  uint64_t word[KW + 1];
-};
-
-// Loads the first `words` (<= KW + 1) of the words; a caller that uses only
-// the first window may ask for 2 (the rest read as 0, and their windows are
-// not to be used).
-template <int KW>
-__device__ __forceinline__ void issue_windows(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap,
-                                              WindowWords<KW>& ww, uint32_t words = KW + 1) {
-  const uintptr_t a = (uintptr_t)(chars + off + h);
-  const uintptr_t blk_end = (a & ~(uintptr_t)4095) + 4096;
-  const uintptr_t p0 = a & ~(uintptr_t)7;
-#pragma unroll
-  for (int i = 0; i <= KW; ++i) {
-    const uintptr_t q = p0 + 8 * (uintptr_t)i;
-    ww.word[i] = ((uint32_t)i < words && h < cap && q < blk_end) ? __ldg(reinterpret_cast<const uint64_t*>(q)) : 0ull;
-  }
-}
-
-// The same string and depth as the issue_windows call that filled ww.
-template <int KW>
-__device__ __forceinline__ uint32_t finish_windows(const WindowWords<KW>& ww, const uint8_t* chars, uint64_t off,
-                                                   uint32_t h, uint32_t cap, uint64_t (&w)[KW]) {
-#pragma unroll
-  for (int j = 0; j < KW; ++j) w[j] = 0;
-  if (h >= cap) return KW;
-  const uintptr_t a = (uintptr_t)(chars + off + h);
-  const uintptr_t blk_end = (a & ~(uintptr_t)4095) + 4096;
-  const uint32_t sh = (uint32_t)(a & 7);
-  const uint64_t known_total = (uint64_t)(blk_end - a);  // bytes from h that may be read (>= 1)
-  const uint64_t room_total = (uint64_t)cap - h;         // bytes from h before the cap (>= 1)
-  uint32_t nwin = KW;
-  bool ended = false;
-#pragma unroll
-  for (int j = 0; j < KW; ++j) {
-    if (ended || (uint32_t)j >= nwin) continue;
-    uint64_t v = sh ? ((ww.word[j] >> (8 * sh)) | (ww.word[j + 1] << (64 - 8 * sh))) : ww.word[j];
-    const uint64_t ws = 8ull * j;
-    const uint32_t known = known_total > ws ? (known_total - ws >= 8 ? 8u : (uint32_t)(known_total - ws)) : 0u;
-    const uint32_t room = room_total > ws ? (room_total - ws >= 8 ? 8u : (uint32_t)(room_total - ws)) : 0u;
-    const uint32_t z = first_zero_byte(known < 8 ? (v | (~0ull << (8 * known))) : v);
-    if (z < known || room <= known) {
-      const uint32_t keep = z < room ? z : room;
-      if (keep < 8) {
-        v &= keep ? (~0ull >> (64 - 8 * keep)) : 0ull;
-        ended = true;
-      }
-      w[j] = bswap64(v);
-    } else {
-      nwin = (uint32_t)j;  // bytes past the block decide this window
-    }
-  }
-  return nwin;
-}
-
+// significant, zero at/after the terminator or the cap), from KW / 2 + 1
+// aligned 16-byte words issued at once (precondition and reads as
+// issue_chars).  Returns how many leading windows are determined: those that
+// lie in the 4 KiB block of byte h, or all of them if the string (or the cap)
+// ends in one of these.
 template <int KW>
 __device__ __forceinline__ uint32_t load_windows(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap,
                                                  uint64_t (&w)[KW]) {
-  WindowWords<KW> ww;
-  issue_windows<KW>(chars, off, h, cap, ww);
-  return finish_windows<KW>(ww, chars, off, h, cap, w);
+  static_assert(KW % 2 == 0, "whole 16-byte words");
+  constexpr int kWords = KW / 2 + 1;
+#pragma unroll
+  for (int j = 0; j < KW; ++j) w[j] = 0;
+  if (h >= cap) return KW;
+  const uintptr_t at = (uintptr_t)(chars + off + h);
+  const uint32_t left = 4096u - (uint32_t)(at & 4095u);  // bytes from h inside the block (>= 1)
+  const uint32_t sh = (uint32_t)(at & 15u);
+  const uint4* p = reinterpret_cast<const uint4*>(at & ~(uintptr_t)15);
+  uint32_t x[4 * kWords];
+#pragma unroll
+  for (int i = 0; i < kWords; ++i) {
+    const uint4 v = 16u * i < left + sh ? __ldg(p + i) : make_uint4(0, 0, 0, 0);
+    x[4 * i] = v.x;
+    x[4 * i + 1] = v.y;
+    x[4 * i + 2] = v.z;
+    x[4 * i + 3] = v.w;
+  }
+  uint32_t o[2 * KW];
+  {
+    uint32_t y[2 * KW + 4];
+#pragma unroll
+    for (int i = 0; i < 2 * KW + 4; ++i) y[i] = x[i];
+    take_words<2 * KW>(y, sh, o);
+  }
+  const uint32_t room = cap - h;
+  bool ended = false;
+#pragma unroll
+  for (int j = 0; j < KW; ++j) {
+    if (ended || 8u * (j + 1) > left) continue;
+    const uint64_t k = ((uint64_t)o[2 * j] << 32) | o[2 * j + 1];
+    const uint32_t keep = min(first_nul(k), room > 8u * j ? room - 8u * j : 0u);
+    w[j] = keep_chars(k, keep);
+    ended = keep < 8;
+  }
+  return ended ? (uint32_t)KW : min((uint32_t)KW, left / 8);
 }
 
 // Offset of a record's string.
@@ -382,7 +424,7 @@ __device__ __forceinline__ uint32_t key_nnz(uint64_t c, uint32_t dna) {
 
 __device__ __forceinline__ uint64_t load_key(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap,
                                              uint32_t dna) {
-  return dna ? dna_key(chars, off, h, cap) : load_cache(chars, off, h, cap);
+  return dna ? dna_key(chars, off, h, cap) : load_chars8(chars, off, h, cap);
 }
 
 // The KW keys at depths h, h + w, ..., h + (KW - 1) w (w = key_width) and how
@@ -461,9 +503,7 @@ struct KeyOps<u128> {
 };
 
 // The wide key of the string at `off` from depth h (precondition as
-// load_cache).  Bytes: the 16 characters are fetched with the three aligned
-// words that cover them in one round trip when they lie in the 4 KiB block of
-// byte h (load_windows); otherwise word by word while the string continues.
+// load_cache).
 __device__ __forceinline__ u128 load_key128(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap,
                                             uint32_t dna) {
   if (dna) {
@@ -471,11 +511,11 @@ __device__ __forceinline__ u128 load_key128(const uint8_t* chars, uint64_t off, 
     const uint64_t lo = key_end(hi, 1) ? 0ull : dna_key(chars, off, h + kDnaWidth, cap);
     return make_k(hi, lo);
   }
-  uint64_t w[2];
-  const uint32_t nw = load_windows<2>(chars, off, h, cap, w);
-  if (nw == 0) w[0] = load_cache(chars, off, h, cap);
-  if (nw < 2) w[1] = has_nul(w[0]) ? 0ull : load_cache(chars, off, h + 8, cap);
-  return make_k(w[0], w[1]);
+  CharWords w;
+  issue_chars(chars, off, h, cap, 16, w);
+  uint64_t hi, lo;
+  finish_chars16(w, chars, off, h, cap, hi, lo);
+  return make_k(hi, lo);
 }
 
 // The narrow key (8 characters) d characters into a byte-encoded wide key,

@@ -41,7 +41,7 @@ constexpr uint32_t kMergeBlock = 128;
 constexpr uint32_t kNoSample = 0xFFFFFFFFu;
 
 __device__ __forceinline__ uint64_t cache_at(const uint8_t* chars, uint32_t cap, uint64_t off, uint32_t h) {
-  return load_cache_2w(chars, off, h, cap);
+  return load_chars8(chars, off, h, cap);
 }
 
 // Compares string a (index ia, at offset oa) with string b (ib, ob); both
@@ -105,24 +105,12 @@ __device__ __forceinline__ uint32_t first_zero_char(uint64_t w0, uint64_t w1) {
   return z0 ? (uint32_t)__clzll((long long)z0) >> 3 : (z1 ? 8u + ((uint32_t)__clzll((long long)z1) >> 3) : 16u);
 }
 
-// The 16 characters of a string from depth h (no terminator before h): the
-// three aligned words that cover them in one round trip when they lie in the
-// 4 KiB block of byte h, otherwise word by word while the string continues.
-__device__ __forceinline__ void finish_words(const WindowWords<2>& ww, const uint8_t* chars, uint32_t cap,
-                                             uint64_t off, uint32_t h, uint64_t& w0, uint64_t& w1) {
-  uint64_t w[2];
-  const uint32_t nw = finish_windows<2>(ww, chars, off, h, cap, w);
-  if (nw == 0) w[0] = cache_at(chars, cap, off, h);
-  if (nw < 2) w[1] = has_nul(w[0]) ? 0ull : cache_at(chars, cap, off, h + 8);
-  w0 = w[0];
-  w1 = w[1];
-}
-
+// The 16 characters of a string from depth h (no terminator before h).
 __device__ __forceinline__ void load_words(const uint8_t* chars, uint32_t cap, uint64_t off, uint32_t h,
                                            uint64_t& w0, uint64_t& w1) {
-  WindowWords<2> ww;
-  issue_windows<2>(chars, off, h, cap, ww);
-  finish_words(ww, chars, cap, off, h, w0, w1);
+  CharWords ww;
+  issue_chars(chars, off, h, cap, 16, ww);
+  finish_chars16(ww, chars, off, h, cap, w0, w1);
 }
 
 // Index of the last range whose start is <= i (starts non-decreasing).
@@ -146,7 +134,7 @@ __global__ void __launch_bounds__(256) k_merge_prep(MergePrepArgs a) {
   for (uint32_t g0 = blockIdx.x * blockDim.x + threadIdx.x; g0 < a.total; g0 += stride * kPrepBatch) {
     uint32_t idx[kPrepBatch], h[kPrepBatch];
     uint64_t off[kPrepBatch];
-    WindowWords<2> ww[kPrepBatch];
+    CharWords ww[kPrepBatch];
 #pragma unroll
     for (int u = 0; u < kPrepBatch; ++u) {
       const uint32_t g = g0 + u * stride;
@@ -163,7 +151,7 @@ __global__ void __launch_bounds__(256) k_merge_prep(MergePrepArgs a) {
     for (int u = 0; u < kPrepBatch; ++u) off[u] = g0 + u * stride < a.total ? a.offsets[idx[u]] : 0ull;
 #pragma unroll
     for (int u = 0; u < kPrepBatch; ++u)
-      if (g0 + u * stride < a.total) issue_windows<2>(a.chars, off[u], h[u], a.cap, ww[u]);
+      if (g0 + u * stride < a.total) issue_chars(a.chars, off[u], h[u], a.cap, 16, ww[u]);
 #pragma unroll
     for (int u = 0; u < kPrepBatch; ++u) {
       const uint32_t g = g0 + u * stride;
@@ -173,7 +161,7 @@ __global__ void __launch_bounds__(256) k_merge_prep(MergePrepArgs a) {
       r.h = h[u];
       r.off = off[u];
       r.miss = 0;
-      finish_words(ww[u], a.chars, a.cap, off[u], h[u], r.w0, r.w1);
+      finish_chars16(ww[u], a.chars, off[u], h[u], a.cap, r.w0, r.w1);
       store_mrec(a.dst + g, r);
     }
   }
@@ -348,8 +336,8 @@ __global__ void __launch_bounds__(kMergeBlock) k_merge_round(MergeRoundArgs a) {
       // is reloaded at lw
       const bool moved = both && eqh;
       const uint64_t loff = take_a ? fb.off : fa.off;
-      WindowWords<2> ww;
-      if (slow) issue_windows<2>(a.chars, loff, lw, a.cap, ww);
+      CharWords ww;
+      if (slow) issue_chars(a.chars, loff, lw, a.cap, 16, ww);
       // the winner is output; its run moves on
       const MRec w = take_a ? fa : fb;
       if (act) {
@@ -372,7 +360,7 @@ __global__ void __launch_bounds__(kMergeBlock) k_merge_round(MergeRoundArgs a) {
       uint64_t r0 = lo.w0, r1 = lo.w1;
       uint32_t rmiss = lo.miss;
       if (slow) {
-        finish_words(ww, a.chars, a.cap, loff, lw, r0, r1);
+        finish_chars16(ww, a.chars, loff, lw, a.cap, r0, r1);
         rmiss = 0;
       } else if (moved) {
         const uint32_t d = lw - lo.h;  // < m: the cache keeps at least one valid character

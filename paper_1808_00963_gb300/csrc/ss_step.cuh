@@ -483,13 +483,13 @@ __device__ __forceinline__ uint32_t move_batch(const SortCtx& c, const SetDesc& 
   }
   // the characters of every byte-string reload are requested before any of
   // them is used (one memory round trip for the batch)
-  WindowWords<1> ww[kMoveBatch];
+  CharWords ww[kMoveBatch];
 #pragma unroll
   for (int u = 0; u < kMoveBatch; ++u) {
     off[u] = 0;
     if (pp[u] != kInvalid && !(ds[u] & kFin) && (ds[u] & kLow30) != depth) {
       off[u] = rec_offset(sd, wide, id[u], o32[u]);
-      if (!sd.dna) issue_windows<1>(sd.chars, off[u], ds[u] & kLow30, sd.cap, ww[u]);
+      if (!sd.dna) issue_chars(sd.chars, off[u], ds[u] & kLow30, sd.cap, 8, ww[u]);
     }
   }
 #pragma unroll
@@ -510,13 +510,7 @@ __device__ __forceinline__ uint32_t move_batch(const SortCtx& c, const SetDesc& 
     uint64_t k = key[u];
     bytes += 34;
     if (nd != depth) {
-      if (sd.dna) {
-        k = load_key(sd.chars, off[u], nd, sd.cap, 1u);
-      } else {
-        uint64_t w[1];
-        // bytes past the 4 KiB block of the first character decide: word by word
-        k = finish_windows<1>(ww[u], sd.chars, off[u], nd, sd.cap, w) ? w[0] : load_cache(sd.chars, off[u], nd, sd.cap);
-      }
+      k = sd.dna ? dna_key(sd.chars, off[u], nd, sd.cap) : finish_chars8(ww[u], sd.chars, off[u], nd, sd.cap);
       bytes += 8;
     }
     store_rec(c.rec[par ^ 1] + dest, k, id[u], o32[u]);
@@ -559,7 +553,7 @@ __device__ __forceinline__ uint32_t move_batch_wide(const SortCtx& c, const SetD
   }
   // what each record needs; the characters of every byte-string gather are
   // requested before any of them is used (one memory round trip for the batch)
-  WindowWords<2> ww[MB];
+  CharWords ww[MB];
 #pragma unroll
   for (int u = 0; u < MB; ++u) {
     how[u] = kSkip;
@@ -575,9 +569,8 @@ __device__ __forceinline__ uint32_t move_batch_wide(const SortCtx& c, const SetD
     to_wide[u] = c.big_enabled && size > c.big_threshold;
     const bool derive = to_wide[u] ? adv == 0 : (sd.dna ? (adv == 0 || adv == kDnaWidth) : adv <= 8);
     how[u] = derive ? kKeep : kGather;
-    if (!derive && !sd.dna)  // a narrow key needs the first window only: two words, not three
-      issue_windows<2>(sd.chars, rec_offset(sd, wide, wi[u].x, wi[u].y), d & kLow30, sd.cap, ww[u],
-                       to_wide[u] ? 3u : 2u);
+    if (!derive && !sd.dna)
+      issue_chars(sd.chars, rec_offset(sd, wide, wi[u].x, wi[u].y), d & kLow30, sd.cap, to_wide[u] ? 16 : 8, ww[u]);
   }
 #pragma unroll
   for (int u = 0; u < MB; ++u) {
@@ -600,13 +593,11 @@ __device__ __forceinline__ uint32_t move_batch_wide(const SortCtx& c, const SetD
         const uint64_t o = rec_offset(sd, wide, wi[u].x, wi[u].y);
         k = to_wide[u] ? load_key128(sd.chars, o, nd, sd.cap, 1u) : make_k(dna_key(sd.chars, o, nd, sd.cap), 0);
       } else {
-        uint64_t w[2];
         const uint64_t o = rec_offset(sd, wide, wi[u].x, wi[u].y);
-        const uint32_t nw = finish_windows<2>(ww[u], sd.chars, o, nd, sd.cap, w);
-        // bytes past the 4 KiB block of the first character decide: word by word
-        if (nw == 0) w[0] = load_cache(sd.chars, o, nd, sd.cap);
-        if (to_wide[u] && nw < 2) w[1] = has_nul(w[0]) ? 0ull : load_cache(sd.chars, o, nd + 8, sd.cap);
-        k = make_k(w[0], w[1]);
+        uint64_t hi, lo = 0;
+        if (to_wide[u]) finish_chars16(ww[u], sd.chars, o, nd, sd.cap, hi, lo);
+        else hi = finish_chars8(ww[u], sd.chars, o, nd, sd.cap);
+        k = make_k(hi, lo);
       }
       bytes += to_wide[u] ? 16 : 8;
     }
