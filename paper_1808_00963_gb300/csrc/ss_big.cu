@@ -268,120 +268,15 @@ struct ItemStream {
 
 // Threads of a sampling block: one per sampled key.  A round waits for its
 // sampling blocks (often a single one: the root's), so their latency counts,
-// not their throughput.  With 256 threads of 4 keys each and every key ranked
-// in the 7 other warps' runs by binary search (196 dependent shared-memory
-// loads) a block took 36 us; one key per thread, warp-sorted and then merged
-// run by run (35 dependent loads), takes 18.5 us (1 M URLs, per round).
+// not their throughput: 36 us with 256 threads of 4 keys each, 18.5 us now
+// (1 M URLs, per round).
 template <int LOGV>
 constexpr uint32_t kSampleThreads = Geo<LOGV>::S;
-
-// Shared memory of a sampling block.  The merge alternates between `sample`
-// and the room of the splitters, which are only written once it is done.
-template <int LOGV>
-struct SampleSmem {
-  static_assert(sizeof(u128) * Geo<LOGV>::S <= sizeof(Splitters<LOGV, u128>), "the merge's second buffer");
-  union {
-    Splitters<LOGV, u128> sp;
-    u128 merge[Geo<LOGV>::S];
-  };
-  u128 sample[Geo<LOGV>::S];
-  uint16_t lo[Geo<LOGV>::S];   // first sample position with a key >= sample[i]
-  uint16_t hi[Geo<LOGV>::S];   // first sample position with a key >  sample[i]
-  uint32_t heads[32];          // bit i of word w: position 32 w + i starts a run of equal keys
-};
-
-// The sampling steps of Algorithm 4.1 as in build_splitters_k, by a block of
-// one thread per sampled key (`key`: this thread's, in any order).  Ends with
-// __syncthreads().
-template <int LOGV>
-__device__ void build_splitters_wide(u128 key, SampleSmem<LOGV>& sm, uint32_t dna) {
-  using G = Geo<LOGV>;
-  constexpr uint32_t S = G::S;
-  constexpr uint32_t NW = S / 32;
-  constexpr int kLevels = LOGV + 1 - 5;  // merge levels from runs of 32 to S
-  const uint32_t tid = threadIdx.x, w = tid >> 5, lane = lane_id();
-  u128 v[1] = {key};
-  warp_bitonic<1, u128>(v);
-  u128* src = (kLevels & 1) ? sm.merge : sm.sample;  // the last level writes sample
-  u128* dst = (kLevels & 1) ? sm.sample : sm.merge;
-  src[tid] = v[0];
-  __syncthreads();
-#pragma unroll 1
-  for (uint32_t run = 32; run < S; run <<= 1) {
-    // each key's place in the merged pair of runs: its own index plus the
-    // partner's keys before it (a left key goes before an equal right one)
-    const u128 k = src[tid];
-    const uint32_t i = tid & (run - 1);
-    const u128* other = src + (tid ^ i ^ run);
-    const bool right = (tid & run) != 0;
-    uint32_t a = 0;
-    for (uint32_t half = run >> 1; half > 0; half >>= 1) {
-      const u128 o = other[a + half - 1];
-      a += (right ? o <= k : o < k) ? half : 0u;
-    }
-    const u128 o = other[a];
-    a += (right ? o <= k : o < k) ? 1u : 0u;
-    dst[(tid & ~(2 * run - 1)) + i + a] = k;
-    __syncthreads();
-    u128* t = src;
-    src = dst;
-    dst = t;
-  }
-  const u128* s = sm.sample;
-  // runs of equal keys, from one bit per position that starts one
-  const bool head = tid == 0 || s[tid - 1] != s[tid];
-  const uint32_t hb = __ballot_sync(0xFFFFFFFFu, head);
-  if (lane == 0) sm.heads[w] = hb;
-  __syncthreads();
-  const uint32_t some = __ballot_sync(0xFFFFFFFFu, lane < NW && sm.heads[lane < NW ? lane : 0] != 0);
-  {
-    const uint32_t own = hb & ((2u << lane) - 1);  // lane 31: all bits
-    const uint32_t wl = own ? w : 31 - __clz(some & ((1u << w) - 1));  // position 0 starts a run
-    const uint32_t hl = own ? own : sm.heads[wl];
-    sm.lo[tid] = (uint16_t)(wl * 32 + 31 - __clz(hl));
-    const uint32_t above = lane == 31 ? 0u : hb & ~((2u << lane) - 1);
-    const uint32_t wa = w == 31 ? 0u : some & ~((2u << w) - 1);
-    const uint32_t wh = above ? w : (wa ? __ffs(wa) - 1 : NW);
-    sm.hi[tid] = (uint16_t)(wh == NW ? S : wh * 32 + __ffs(above ? above : sm.heads[wh]) - 1);
-  }
-  __syncthreads();
-  u128 val = 0;
-  uint32_t slot = 0;
-  if (tid < G::V) {
-    const uint32_t i = tid + 1;             // level-order index
-    const int l = 31 - __clz(i);            // its level
-    uint32_t a = 0, b = S;                  // its range of the sorted sample
-    for (int d = l - 1; d >= 0; --d) {
-      if (a < b) {
-        const uint32_t m = (a + b) >> 1;
-        if (((i >> d) & 1u) == 0) {
-          const uint32_t le = sm.lo[m];
-          b = le > a ? le : a;              // left of the run of keys equal to s[m]
-        } else {
-          const uint32_t rs = sm.hi[m];
-          a = rs < b ? rs : b;              // right of that run
-        }
-      } else {
-        a = b;
-      }
-    }
-    val = a < b ? s[(a + b) >> 1] : (b < S ? s[b] : KeyOps<u128>::ones());
-    slot = (2 * (i - (1u << l)) + 1) * (1u << (LOGV - 1 - l)) - 1;
-    sm.sp.tree[i] = val;
-    sm.sp.x[slot] = val;
-  }
-  if (tid == 0) sm.sp.tree[0] = 0;
-  if (tid == G::V) sm.sp.x[G::V] = 0;
-  __syncthreads();
-  if (tid <= G::V)
-    sm.sp.hp[tid] = (tid == 0 || tid == G::V) ? 0 : (uint8_t)KeyOps<u128>::lcp(sm.sp.x[tid - 1], sm.sp.x[tid], dna);
-  __syncthreads();
-}
 
 template <int LOGV>
 __global__ void __launch_bounds__(kSampleThreads<LOGV>) k_big_sample(const BigCtl* __restrict__ ctl) {
   extern __shared__ __align__(16) uint8_t smem[];
-  SampleSmem<LOGV>& sm = *reinterpret_cast<SampleSmem<LOGV>*>(smem);
+  SampleSmem<LOGV, u128>& sm = *reinterpret_cast<SampleSmem<LOGV, u128>*>(smem);
   __shared__ uint64_t ref[kPjWindows];
   __shared__ uint32_t s_min;
   const uint32_t G = ctl->cur.G;
@@ -397,7 +292,8 @@ __global__ void __launch_bounds__(kSampleThreads<LOGV>) k_big_sample(const BigCt
       return g.t.begin + (uint32_t)(((mix64(hseed + i) >> 32) * (uint64_t)g.t.len) >> 32);
     };
     if (threadIdx.x == 0) s_min = 0xFFFFFFFFu;
-    build_splitters_wide<LOGV>(load_wkey(c.rec[par] + sample_pos(threadIdx.x)), sm, sd.dna);
+    build_splitters<LOGV, u128, kSampleThreads<LOGV>>(
+        [&](uint32_t pos) { return load_wkey(c.rec[par] + g.t.begin + pos); }, g.t.len, hseed, sm, sd.dna);
     const uint4* src = reinterpret_cast<const uint4*>(&sm.sp);
     uint4* dst = reinterpret_cast<uint4*>(&out[gi].sp);
     for (uint32_t i = threadIdx.x; i < sizeof(sm.sp) / 16; i += blockDim.x) dst[i] = src[i];
@@ -484,7 +380,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_big_classify(const BigCtl* __rest
     const uint32_t par = task_par(g.t);
     const Rec* recs = c.rec[par] + g.t.begin + t0;
     uint16_t* bo = c.bucket_of + g.t.begin + t0;
-    const uint32_t mine = classify_count_k<LOGV, u128>([&](uint32_t p) { return load_wkey(recs + p); }, bo, tl,
+    const uint32_t mine = classify_count_k<LOGV, u128, kBlock>([&](uint32_t p) { return load_wkey(recs + p); }, bo, tl,
                                                        tree, x, hist, c.classifier, use_jump ? jump : nullptr);
     __syncthreads();
     uint32_t* cnt = ctl->counters + cnt_base(g) + tile;
@@ -636,7 +532,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_big_scatter(const BigCtl* __restr
     const uint32_t depth = g.t.depth;
     const uint32_t wide = c.wide[task_set(g.t)];
     if (threadIdx.x == 0) bytes += (fresh ? 12ull : 4ull) * Gm::K;  // per-bucket tile offsets (+ descriptors and starts)
-    tile_scatter<LOGV, kWideMoveBatch>(
+    tile_scatter<LOGV, kBlock, kWideMoveBatch>(
         tb, tl, R, base, cntw,
         [&](const uint32_t(&pp)[kWideMoveBatch], const uint32_t(&bb)[kWideMoveBatch],
             const uint32_t(&dd)[kWideMoveBatch]) {
@@ -801,14 +697,14 @@ static cudaError_t launch_big_round_t(BigCtl* ctl, uint32_t R_max, uint32_t sms,
                                          (int)big_scatter_smem(LOGV, kMaxRounds));
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_big_sample<LOGV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)sizeof(SampleSmem<LOGV>));
+                               (int)sizeof(SampleSmem<LOGV, u128>));
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
   // fixed grids (the work of a round is only known on the device): blocks
   // loop over subsets, tiles or counter chunks and return when there are none
   hook.run("big_sample", [&] { 
-    k_big_sample<LOGV><<<sms * (2048 / kSampleThreads<LOGV>), kSampleThreads<LOGV>, sizeof(SampleSmem<LOGV>), st>>>(ctl);
+    k_big_sample<LOGV><<<sms * (2048 / kSampleThreads<LOGV>), kSampleThreads<LOGV>, sizeof(SampleSmem<LOGV, u128>), st>>>(ctl);
   });
   hook.run("big_classify", [&] { k_big_classify<LOGV><<<sms * 8, kBlock, 0, st>>>(ctl, &ctl->cur.next_tile); });
   hook.run("scan", [&] { k_scan_reduce<<<sms * 8, kBlock, 0, st>>>(ctl); });

@@ -552,13 +552,24 @@ __device__ __forceinline__ void list_push(const TaskList& l, const Task& t, uint
   else latch_status(status, kStQueueFull);
 }
 
+// Loads and stores of the work queue's flags that order the task they guard:
+// what was written before a release store is visible after an acquire load
+// that sees it (also writes of other threads of the block, before a barrier).
+__device__ __forceinline__ uint32_t load_acquire(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void store_release(uint32_t* p, uint32_t v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
 // Waits (bounded by wait_ns) until *flag == want; false if the wait expired.
 __device__ __forceinline__ bool wait_flag(const uint32_t* flag, uint32_t want, uint64_t wait_ns) {
-  volatile const uint32_t* f = flag;
-  if (*f == want) return true;
+  if (load_acquire(flag) == want) return true;
   const uint64_t t0 = globaltimer_ns();
   uint32_t ns = 32;
-  while (*f != want) {
+  while (load_acquire(flag) != want) {
     if (globaltimer_ns() - t0 > wait_ns) return false;
     __nanosleep(ns);
     ns = ns < 1024 ? ns * 2 : ns;
@@ -578,10 +589,8 @@ __device__ __forceinline__ void queue_put(const WorkQueue& q, uint32_t k, const 
     atomicSub(q.pending, 1u);
     return;
   }
-  __threadfence();
   q.items[slot] = t;
-  __threadfence();
-  atomicExch(q.ready + slot, 2 * lap + 1);
+  store_release(q.ready + slot, 2 * lap + 1);
 }
 
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }

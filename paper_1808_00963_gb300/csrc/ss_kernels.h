@@ -101,8 +101,7 @@ uint64_t graph_launch_count();
 // Persistent work-queue kernel (single-block S^5 steps).
 size_t queue_smem(int logv);
 cudaError_t queue_occupancy(int logv, int* blocks_per_sm);
-cudaError_t launch_queue(int logv, const SortCtx& c, uint32_t grid, uint32_t R, cudaStream_t st,
-                         const LaunchHook& hook);
+cudaError_t launch_queue(int logv, const SortCtx& c, uint32_t grid, cudaStream_t st, const LaunchHook& hook);
 
 // Small subsets, set-up and LCP fix-up.
 size_t small_cta_smem(uint32_t pmax);

@@ -17,24 +17,36 @@ namespace ss {
 
 namespace {
 
+// Threads of a block.  Most subsets are a few thousand strings and the last
+// ones to be split decide when the kernel ends (blocks of the 1 M URL sort
+// were idle for 4/5 of it), so a step is built for latency: 16 warps at 64
+// registers, two blocks per SM.  Cycles of an average step (2600 strings, 20 M
+// URLs) with three 256-thread blocks per SM / now: sample and splitters
+// 24.5k / 12.7k, classification 13.6k / 11.5k, scatter 53k / 29k.  1 M URLs 788
+// -> 726 us, suffix array of 4 M characters 1791 -> 1742, 20 M URLs 4370 -> 4281;
+// four records per lane and move batch spill: 740 / 1809 / 4355 us.
+constexpr uint32_t kQueueThreads = 512;
+constexpr uint32_t kQueueWarps = kQueueThreads / 32;
+constexpr uint32_t kQueueBlocks = 2;                      // per SM
+constexpr uint32_t kQueueRounds = kMaxTile / kQueueThreads;  // tile = kQueueThreads * rounds records
+constexpr int kQueueMoveBatch = 2;                        // records per lane moved together
+
 template <int LOGV>
 struct QueueSmem {
-  Splitters<LOGV> sp;
+  SampleSmem<LOGV, uint64_t> sm;
   uint32_t hist[Geo<LOGV>::KP];    // bucket sizes, then running destinations
   uint32_t bstart[Geo<LOGV>::KP];  // bucket starts relative to the task (KP >= K + 1)
   uint32_t desc[Geo<LOGV>::KP];
-  union U {
-    BuildScratch<LOGV> bs;
+  union {
     struct {
-      unsigned long long bmin[Geo<LOGV>::KP];  // smallest / largest key of each even bucket
-      unsigned long long bmax[Geo<LOGV>::KP];
-      uint32_t prev[Geo<LOGV>::KP];            // last non-empty bucket before each bucket, + 1 (0: none)
-    } mm;
-    struct {
-      uint32_t cntw[kWarps * Geo<LOGV>::KP];
-      uint16_t tb[kMaxTile];
-    } sc;
+      // largest LCP of an even bucket's keys with the splitter below / above it
+      uint32_t below[Geo<LOGV>::V + 1];
+      uint32_t above[Geo<LOGV>::V + 1];
+      uint32_t used[64];           // bit i of word w: bucket 32 w + i is not empty
+    } lc;
+    uint32_t cntw[kQueueWarps * Geo<LOGV>::KP];
   } u;
+  uint16_t tb[kMaxTile];           // bucket of each record of a tile
   Task task;
   uint32_t got;
 };
@@ -46,15 +58,12 @@ __device__ bool claim_task(const WorkQueue& q, Task* out, uint32_t* status, uint
   const uint32_t slot = k % q.cap, lap = k / q.cap;
   const uint64_t t0 = globaltimer_ns();
   uint32_t ns = 64;
-  volatile uint32_t* ready = q.ready;
   volatile uint32_t* pending = q.pending;
   while (true) {
-    if (ready[slot] == 2 * lap + 1) {
-      __threadfence();
+    if (load_acquire(q.ready + slot) == 2 * lap + 1) {
       const uint4 v = __ldcg(reinterpret_cast<const uint4*>(q.items + slot));
       *out = Task{v.x, v.y, v.z, v.w};
-      __threadfence();  // the task is read before the slot is handed to the next lap
-      atomicExch(q.ready + slot, 2 * lap + 2);
+      store_release(q.ready + slot, 2 * lap + 2);  // the task is read before the slot goes to the next lap
       return true;
     }
     if (*pending == 0) return false;
@@ -67,13 +76,13 @@ __device__ bool claim_task(const WorkQueue& q, Task* out, uint32_t* status, uint
   }
 }
 
-// Exclusive scan of n (a multiple of the block size) counters in shared memory.
+// Exclusive scan of n counters in shared memory.
 __device__ void block_excl_scan_smem(const uint32_t* in, uint32_t* out, uint32_t n) {
-  __shared__ uint32_t wsum[kWarps];
-  const uint32_t per = n / kBlock;
-  const uint32_t b0 = threadIdx.x * per;
+  __shared__ uint32_t wsum[kQueueWarps];
+  const uint32_t per = (n + kQueueThreads - 1) / kQueueThreads;
+  const uint32_t b0 = min(n, threadIdx.x * per), b1 = min(n, b0 + per);
   uint32_t s = 0;
-  for (uint32_t j = 0; j < per; ++j) s += in[b0 + j];
+  for (uint32_t j = b0; j < b1; ++j) s += in[j];
   uint32_t inc = s;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -83,57 +92,13 @@ __device__ void block_excl_scan_smem(const uint32_t* in, uint32_t* out, uint32_t
   const uint32_t w = threadIdx.x >> 5;
   if (lane_id() == 31) wsum[w] = inc;
   __syncthreads();
-  if (w == 0) {
-    uint32_t v = lane_id() < kWarps ? wsum[lane_id()] : 0;
+  uint32_t run = inc - s;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      uint32_t t = __shfl_up_sync(0xFFFFFFFFu, v, o);
-      if (lane_id() >= (uint32_t)o) v += t;
-    }
-    if (lane_id() < kWarps) wsum[lane_id()] = v;
-  }
-  __syncthreads();
-  uint32_t run = inc - s + (w ? wsum[w - 1] : 0);
-  for (uint32_t j = 0; j < per; ++j) {
-    const uint32_t v = in[b0 + j];
-    out[b0 + j] = run;
+  for (uint32_t k = 0; k < kQueueWarps; ++k) run += k < w ? wsum[k] : 0u;
+  for (uint32_t j = b0; j < b1; ++j) {
+    const uint32_t v = in[j];
+    out[j] = run;
     run += v;
-  }
-  __syncthreads();
-}
-
-// Inclusive max-scan of n (a multiple of the block size) values in shared memory.
-__device__ void block_max_scan_smem(uint32_t* a, uint32_t n) {
-  __shared__ uint32_t wmax[kWarps];
-  const uint32_t per = n / kBlock;
-  const uint32_t b0 = threadIdx.x * per;
-  uint32_t m = 0;
-  for (uint32_t j = 0; j < per; ++j) m = max(m, a[b0 + j]);
-  uint32_t inc = m;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-    if (lane_id() >= (uint32_t)o) inc = max(inc, t);
-  }
-  const uint32_t w = threadIdx.x >> 5;
-  if (lane_id() == 31) wmax[w] = inc;
-  __syncthreads();
-  if (w == 0) {
-    uint32_t v = lane_id() < kWarps ? wmax[lane_id()] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, v, o);
-      if (lane_id() >= (uint32_t)o) v = max(v, t);
-    }
-    if (lane_id() < kWarps) wmax[lane_id()] = v;
-  }
-  __syncthreads();
-  uint32_t run = __shfl_up_sync(0xFFFFFFFFu, inc, 1);
-  if (lane_id() == 0) run = 0;
-  run = max(run, w ? wmax[w - 1] : 0u);
-  for (uint32_t j = 0; j < per; ++j) {
-    run = max(run, a[b0 + j]);
-    a[b0 + j] = run;
   }
   __syncthreads();
 }
@@ -143,54 +108,76 @@ __device__ void block_max_scan_smem(uint32_t* a, uint32_t n) {
 // cache 8 read + bucket index 2 written per record while classifying, and the
 // bytes of each record's move.
 template <int LOGV>
-__device__ unsigned long long queue_step(const SortCtx& c, const Task& t, QueueSmem<LOGV>& s, uint32_t R) {
+__device__ unsigned long long queue_step(const SortCtx& c, const Task& t, QueueSmem<LOGV>& s) {
   using Gm = Geo<LOGV>;
+  constexpr uint32_t NT = kQueueThreads;
   const SetDesc sd = c.sets[task_set(t)];
   const uint32_t par = task_par(t);
   const Rec* recs = c.rec[par] + t.begin;
   const uint32_t wide = c.wide[task_set(t)];
-  build_splitters<LOGV>(recs, t.len, mix64(c.seed ^ ((uint64_t)t.begin << 20) ^ t.depth), s.sp, s.u.bs, sd.dna);
+  Splitters<LOGV>& sp = s.sm.sp;
+  const bool with_lcp = sd.lcp != nullptr;
+  for (uint32_t b = threadIdx.x; b < Gm::KP; b += NT) {
+    s.hist[b] = 0;
+    if (b <= Gm::V) s.u.lc.below[b] = s.u.lc.above[b] = 0;
+  }
+  build_splitters<LOGV, uint64_t, NT>([&](uint32_t pos) { return recs[pos].key; }, t.len,
+                                      mix64(c.seed ^ ((uint64_t)t.begin << 20) ^ t.depth), s.sm, sd.dna);
   unsigned long long bytes = threadIdx.x == 0 ? Gm::S * 8ull : 0ull;
 
-  // classification (Algorithm 4.1): classify into the array o and count; with
-  // an LCP output also the smallest and largest key of each even bucket
-  const bool with_lcp = sd.lcp != nullptr;
-  for (uint32_t b = threadIdx.x; b < Gm::KP; b += kBlock) {
-    s.hist[b] = 0;
-    s.u.mm.bmin[b] = ~0ull;
-    s.u.mm.bmax[b] = 0ull;
-  }
-  __syncthreads();
-  uint16_t* bo = c.bucket_of + t.begin;
-  bytes += 10ull * classify_count_k<LOGV, uint64_t>([&](uint32_t p) { return recs[p].key; }, bo, t.len, s.sp.tree,
-                                                    s.sp.x, s.hist, c.classifier, nullptr,
-                                                    with_lcp ? s.u.mm.bmin : nullptr,
-                                                    with_lcp ? s.u.mm.bmax : nullptr);
+  // classification (Algorithm 4.1): classify into the array o and count.  With
+  // an LCP output also how far each even bucket's keys agree with the
+  // splitters around it: its smallest key x has the largest LCP with the
+  // splitter below, its largest key with the one above.  These are small
+  // numbers, raised with 32-bit atomics where they grow (minima and maxima of
+  // the 64-bit keys themselves took a compare-and-swap loop per key).
+  // A subset of at most one tile keeps its bucket indices in shared memory.
+  const bool one_tile = t.len <= kMaxTile;
+  uint16_t* bo = one_tile ? s.tb : c.bucket_of + t.begin;
+  bytes += 10ull * classify_count_k<LOGV, uint64_t, NT>(
+      [&](uint32_t p) { return recs[p].key; }, bo, t.len, sp.tree, sp.x, s.hist, c.classifier, nullptr,
+      [&](uint32_t b, uint64_t k) {
+        if (!with_lcp || (b & 1u)) return;
+        const uint32_t r = b >> 1;
+        if (r > 0) {
+          const uint32_t l = key_lcp(k, sp.x[r - 1], sd.dna);
+          if (l > s.u.lc.below[r]) atomicMax(&s.u.lc.below[r], l);
+        }
+        if (r < Gm::V) {
+          const uint32_t l = key_lcp(k, sp.x[r], sd.dna);
+          if (l > s.u.lc.above[r]) atomicMax(&s.u.lc.above[r], l);
+        }
+      });
   __syncthreads();
 
   // prefix sum over the bucket sizes; bucket outcomes
+  for (uint32_t b = threadIdx.x; b < Gm::KP; b += NT) {  // whole warps: KP is a multiple of 32
+    const uint32_t used = __ballot_sync(0xFFFFFFFFu, b < Gm::K && s.hist[b] != 0);
+    if (lane_id() == 0) s.u.lc.used[b >> 5] = used;
+  }
   block_excl_scan_smem(s.hist, s.bstart, Gm::KP);  // bstart[K] = len (hist[K] is 0)
   if (with_lcp) {
     // LCP at each bucket boundary (Section 4.2.3 "LCP via XOR", Section 4.2.8
-    // "LCP Calculation"): the last string of the previous non-empty bucket
-    // and the first string of this one are the largest key of the one and
-    // the smallest of the other, which differ within the step's 8 characters
-    for (uint32_t b = threadIdx.x; b < Gm::KP; b += kBlock) s.u.mm.prev[b] = (b < Gm::K && s.hist[b]) ? b + 1 : 0u;
-    __syncthreads();
-    block_max_scan_smem(s.u.mm.prev, Gm::KP);  // prev[b] - 1: last non-empty bucket <= b
-    for (uint32_t b = threadIdx.x + 1; b < Gm::K; b += kBlock) {
-      const uint32_t q = s.u.mm.prev[b - 1];
-      if (!s.hist[b] || q == 0) continue;
-      const uint32_t pb = q - 1;
-      const uint64_t hi = (pb & 1u) ? s.sp.x[pb >> 1] : s.u.mm.bmax[pb];
-      const uint64_t lo = (b & 1u) ? s.sp.x[b >> 1] : s.u.mm.bmin[b];
-      sd.lcp[t.begin + s.bstart[b] - sd.base] = t.depth + key_lcp(hi, lo, sd.dna);
+    // "LCP Calculation"): between the last string of the previous non-empty
+    // bucket and the first string of this one lie the splitters x_a <= ... <=
+    // x_b, and for keys u <= v <= w lcp(u, w) is the smaller of lcp(u, v) and
+    // lcp(v, w).  An equality bucket's key is its splitter.
+    const uint64_t some = nonzero_words(s.u.lc.used, Gm::KP / 32);
+    for (uint32_t b = threadIdx.x; b < Gm::K; b += NT) {
+      if (!s.hist[b]) continue;
+      const uint32_t pb = last_set_before(s.u.lc.used, some, b);
+      if (pb == kNone) continue;
+      const uint32_t ra = pb >> 1, rb = (b & 1u) ? b >> 1 : (b >> 1) - 1;
+      uint32_t l = key_lcp(sp.x[ra], sp.x[rb], sd.dna);
+      if (!(pb & 1u)) l = min(l, s.u.lc.above[ra]);
+      if (!(b & 1u)) l = min(l, s.u.lc.below[b >> 1]);
+      sd.lcp[t.begin + s.bstart[b] - sd.base] = t.depth + l;
     }
     __syncthreads();  // hist is overwritten below
   }
-  for (uint32_t b = threadIdx.x; b < Gm::K; b += kBlock) {
+  for (uint32_t b = threadIdx.x; b < Gm::K; b += NT) {
     const uint32_t size = s.hist[b];
-    s.desc[b] = size ? bucket_desc<LOGV>(b, size, t.depth, s.sp, sd.dna) : kFin;
+    s.desc[b] = size ? bucket_desc<LOGV>(b, size, t.depth, sp, sd.dna) : kFin;
     s.hist[b] = t.begin + s.bstart[b];
   }
   __syncthreads();
@@ -198,25 +185,28 @@ __device__ unsigned long long queue_step(const SortCtx& c, const Task& t, QueueS
   // redistribution: stable and out of place, tile by tile; a subset that fits
   // one tile is spread over all warps (each warp owns 32 * R consecutive
   // records of a tile)
-  R = min(R, (t.len + kBlock - 1) / kBlock);
-  const uint32_t T = kBlock * R;
+  const uint32_t R = min(kQueueRounds, (t.len + NT - 1) / NT);
+  const uint32_t T = NT * R;
   for (uint32_t t0 = 0; t0 < t.len; t0 += T) {
     const uint32_t tl = min(T, t.len - t0);
-    for (uint32_t p = threadIdx.x; p < tl; p += kBlock) s.u.sc.tb[p] = bo[t0 + p];
-    __syncthreads();
+    if (!one_tile) {
+      for (uint32_t p = threadIdx.x; p < tl; p += NT) s.tb[p] = bo[t0 + p];
+      __syncthreads();
+    }
     const uint32_t src0 = t.begin + t0;
-    tile_scatter<LOGV>(s.u.sc.tb, tl, R, s.hist, s.u.sc.cntw,
-                       [&](const uint32_t(&pp)[kMoveBatch], const uint32_t(&bb)[kMoveBatch],
-                           const uint32_t(&dd)[kMoveBatch]) {
-                         bytes += move_batch(c, sd, wide, par, src0, t.depth, s.desc,
-                                             [&](uint32_t b) { return t.begin + s.bstart[b]; }, pp, bb, dd);
-                       });
+    tile_scatter<LOGV, NT, kQueueMoveBatch>(
+        s.tb, tl, R, s.hist, s.u.cntw,
+        [&](const uint32_t(&pp)[kQueueMoveBatch], const uint32_t(&bb)[kQueueMoveBatch],
+            const uint32_t(&dd)[kQueueMoveBatch]) {
+          bytes += move_batch<kQueueMoveBatch>(c, sd, wide, par, src0, t.depth, s.desc,
+                                               [&](uint32_t b) { return t.begin + s.bstart[b]; }, pp, bb, dd);
+        });
   }
-  __threadfence();
   __syncthreads();
 
-  // new subsets become visible only after their records have been moved
-  for (uint32_t b = threadIdx.x; b < Gm::K; b += kBlock) {
+  // new subsets become visible only after their records have been moved (the
+  // push releases what the block wrote before the barrier)
+  for (uint32_t b = threadIdx.x; b < Gm::K; b += NT) {
     const uint32_t start = s.bstart[b];
     const uint32_t size = s.bstart[b + 1] - start;
     if (size) emit_bucket(c, sd, t, start, size, s.desc[b], 0, 0u);  // boundary LCPs are written already
@@ -225,7 +215,7 @@ __device__ unsigned long long queue_step(const SortCtx& c, const Task& t, QueueS
 }
 
 template <int LOGV>
-__global__ void __launch_bounds__(kBlock, 3) k_queue(SortCtx c, uint32_t R) {
+__global__ void __launch_bounds__(kQueueThreads, kQueueBlocks) k_queue(SortCtx c) {
   extern __shared__ __align__(16) uint8_t smem[];
   QueueSmem<LOGV>& s = *reinterpret_cast<QueueSmem<LOGV>*>(smem);
   unsigned long long bytes = 0;
@@ -234,7 +224,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_queue(SortCtx c, uint32_t R) {
     __syncthreads();
     if (!s.got) break;
     const Task t = s.task;
-    bytes += queue_step<LOGV>(c, t, s, R);
+    bytes += queue_step<LOGV>(c, t, s);
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
@@ -266,38 +256,37 @@ cudaError_t queue_occupancy(int logv, int* blocks_per_sm) {
   switch (logv) {
     case 7:
       if (cudaError_t e = set_queue_attr<7>()) return e;
-      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_queue<7>, kBlock, sizeof(QueueSmem<7>));
+      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_queue<7>, kQueueThreads, sizeof(QueueSmem<7>));
     case 8:
       if (cudaError_t e = set_queue_attr<8>()) return e;
-      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_queue<8>, kBlock, sizeof(QueueSmem<8>));
+      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_queue<8>, kQueueThreads, sizeof(QueueSmem<8>));
     case 9:
       if (cudaError_t e = set_queue_attr<9>()) return e;
-      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_queue<9>, kBlock, sizeof(QueueSmem<9>));
+      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_queue<9>, kQueueThreads, sizeof(QueueSmem<9>));
     default:
       if (cudaError_t e = set_queue_attr<10>()) return e;
-      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_queue<10>, kBlock,
+      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_queue<10>, kQueueThreads,
                                                            sizeof(QueueSmem<10>));
   }
 }
 
-cudaError_t launch_queue(int logv, const SortCtx& c, uint32_t grid, uint32_t R, cudaStream_t st,
-                         const LaunchHook& hook) {
+cudaError_t launch_queue(int logv, const SortCtx& c, uint32_t grid, cudaStream_t st, const LaunchHook& hook) {
   switch (logv) {
     case 7:
       if (cudaError_t e = set_queue_attr<7>()) return e;
-      hook.run("queue", [&] { k_queue<7><<<grid, kBlock, sizeof(QueueSmem<7>), st>>>(c, R); });
+      hook.run("queue", [&] { k_queue<7><<<grid, kQueueThreads, sizeof(QueueSmem<7>), st>>>(c); });
       break;
     case 8:
       if (cudaError_t e = set_queue_attr<8>()) return e;
-      hook.run("queue", [&] { k_queue<8><<<grid, kBlock, sizeof(QueueSmem<8>), st>>>(c, R); });
+      hook.run("queue", [&] { k_queue<8><<<grid, kQueueThreads, sizeof(QueueSmem<8>), st>>>(c); });
       break;
     case 9:
       if (cudaError_t e = set_queue_attr<9>()) return e;
-      hook.run("queue", [&] { k_queue<9><<<grid, kBlock, sizeof(QueueSmem<9>), st>>>(c, R); });
+      hook.run("queue", [&] { k_queue<9><<<grid, kQueueThreads, sizeof(QueueSmem<9>), st>>>(c); });
       break;
     default:
       if (cudaError_t e = set_queue_attr<10>()) return e;
-      hook.run("queue", [&] { k_queue<10><<<grid, kBlock, sizeof(QueueSmem<10>), st>>>(c, R); });
+      hook.run("queue", [&] { k_queue<10><<<grid, kQueueThreads, sizeof(QueueSmem<10>), st>>>(c); });
       break;
   }
   return cudaGetLastError();

@@ -32,157 +32,171 @@ struct Splitters {
   uint8_t hp[Geo<LOGV>::V + 1];     // h'_0..h'_v: lcp of neighbouring splitters
 };
 
-// Scratch of the splitter construction (may alias other shared memory).
-template <int LOGV, typename K = uint64_t>
-struct BuildScratch {
+// Shared memory of the splitter construction.  The merge alternates between
+// `sample` and the room of the splitters, which are only written once it is
+// done.
+template <int LOGV, typename K>
+struct SampleSmem {
+  static_assert(sizeof(K) * Geo<LOGV>::S <= sizeof(Splitters<LOGV, K>), "the merge's second buffer");
+  union {
+    Splitters<LOGV, K> sp;
+    K merge[Geo<LOGV>::S];
+  };
   K sample[Geo<LOGV>::S];
   uint16_t lo[Geo<LOGV>::S];   // first sample position with a key >= sample[i]
   uint16_t hi[Geo<LOGV>::S];   // first sample position with a key >  sample[i]
+  uint32_t heads[64];          // bit i of word w: position 32 w + i starts a run of equal keys
 };
 
-// Ascending bitonic sort of the 32 * E keys a warp holds, E per lane in
-// index order lane * E + e: partners closer than E sit in the same lane,
-// farther ones are exchanged with shuffles.
-template <int E, typename K>
-__device__ __forceinline__ void warp_bitonic(K (&v)[E]) {
-  constexpr uint32_t N = 32 * E;
-  const uint32_t lane = threadIdx.x & 31;
-#pragma unroll
-  for (uint32_t k = 2; k <= N; k <<= 1) {
-#pragma unroll
-    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-      if (j >= E) {
-        const uint32_t lj = j / E;
-        const bool lower = (lane & lj) == 0;
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-          const K o = KeyOps<K>::shfl_xor(v[e], (int)lj);
-          const bool up = ((lane * E + e) & k) == 0;
-          const bool take_min = lower == up;
-          v[e] = take_min ? (o < v[e] ? o : v[e]) : (o > v[e] ? o : v[e]);
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-          if ((e & j) == 0) {
-            const int f = e | (int)j;
-            const bool up = ((lane * E + e) & k) == 0;
-            if ((v[e] > v[f]) == up) {
-              const K t = v[e];
-              v[e] = v[f];
-              v[f] = t;
-            }
-          }
-        }
-      }
-    }
-  }
+// Which of a bitmap's up to 64 words hold a set bit (bit w: word w); every
+// lane of the warp calls it.
+__device__ __forceinline__ uint64_t nonzero_words(const uint32_t* words, uint32_t nw) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t b0 = __ballot_sync(0xFFFFFFFFu, lane < nw && words[lane] != 0);
+  const uint32_t b1 = __ballot_sync(0xFFFFFFFFu, lane + 32 < nw && words[lane + 32] != 0);
+  return (uint64_t)b1 << 32 | b0;
 }
 
-// The sampling steps of Algorithm 4.1 for the len keys at `keys`: draw a sample of
-// alpha * (v + 1) keys at pseudo-random positions, sort it, select the
-// splitters with the recursive duplicate-skipping rule of Section 4.2.3
-// ("Sampling"): the middle sample of a range becomes the splitter, the ranges
-// left and right of the run of samples equal to it are split recursively.
-// A node whose range is empty takes the sample just above its range (the
-// nearest splitter on the right among its ancestors), or all-ones past the
-// end, which keeps t a search tree.  Finally h'_i = lcp(x_{i-1}, x_i) with
-// h'_0 = h'_v = 0, the splitter LCPs of Algorithm 4.1.
-// The sample is sorted warp by warp in registers and merged by computing each
-// key's rank (its position in its chunk plus, in every other chunk, the keys
-// before it: <= for earlier chunks, < for later ones).  With the run of equal
-// keys around every sample position known, each tree node finds its range by
-// walking from the root along its level-order index, so the recursion needs
-// no step-by-step synchronisation.  Ends with __syncthreads().
-// key_at(pos) gives the key of the subset's record pos.
-template <int LOGV, typename K, typename KeyAt>
-__device__ void build_splitters_k(KeyAt&& key_at, uint32_t len, uint64_t hseed, Splitters<LOGV, K>& sp,
-                                  BuildScratch<LOGV, K>& bs, uint32_t dna) {
-  using G = Geo<LOGV>;
-  constexpr uint32_t C = G::S / kWarps;  // keys per warp
-  constexpr int E = (int)(C / 32);       // keys per lane
-  static_assert(E >= 1 && C % 32 == 0, "sample does not split into whole warps");
-  const uint32_t w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  K v[E];
+// The last set bit before / the first one after position p of such a bitmap
+// (kNone: there is none); some: its nonzero_words.
+constexpr uint32_t kNone = 0xFFFFFFFFu;
+
+__device__ __forceinline__ uint32_t last_set_before(const uint32_t* words, uint64_t some, uint32_t p) {
+  const uint32_t w = p >> 5;
+  const uint32_t own = words[w] & ((1u << (p & 31u)) - 1);
+  if (own) return w * 32 + 31 - __clz(own);
+  const uint64_t below = some & ((1ull << w) - 1);
+  if (!below) return kNone;
+  const uint32_t v = 63 - __clzll((long long)below);
+  return v * 32 + 31 - __clz(words[v]);
+}
+
+__device__ __forceinline__ uint32_t first_set_after(const uint32_t* words, uint64_t some, uint32_t p) {
+  const uint32_t w = p >> 5;
+  const uint32_t own = words[w] & ~((2u << (p & 31u)) - 1);  // bit 31: none above
+  if (own) return w * 32 + __ffs(own) - 1;
+  const uint64_t above = w == 63 ? 0ull : some & ~((2ull << w) - 1);
+  if (!above) return kNone;
+  const uint32_t v = __ffsll((long long)above) - 1;
+  return v * 32 + __ffs(words[v]) - 1;
+}
+
+// Ascending bitonic sort of the 32 keys a warp holds, one per lane.
+template <typename K>
+__device__ __forceinline__ K warp_bitonic(K v) {
+  const uint32_t lane = threadIdx.x & 31;
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const uint32_t i = w * C + lane * E + e;
-    const uint64_t h = mix64(hseed + i);
-    const uint32_t pos = (uint32_t)(((h >> 32) * (uint64_t)len) >> 32);
-    v[e] = key_at(pos);
-  }
-  warp_bitonic<E, K>(v);
-  K* s = bs.sample;
+  for (uint32_t k = 2; k <= 32; k <<= 1) {
 #pragma unroll
-  for (int e = 0; e < E; ++e) s[w * C + lane * E + e] = v[e];
-  __syncthreads();
-  uint32_t rank[E];
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    uint32_t r = lane * E + e;
-#pragma unroll
-    for (uint32_t ww = 0; ww < kWarps; ++ww) {
-      if (ww == w) continue;
-      const K* ch = s + ww * C;
-      uint32_t a = 0, b = C;
-      if (ww < w) {
-        while (a < b) { const uint32_t m = (a + b) >> 1; if (ch[m] <= v[e]) a = m + 1; else b = m; }
-      } else {
-        while (a < b) { const uint32_t m = (a + b) >> 1; if (ch[m] < v[e]) a = m + 1; else b = m; }
-      }
-      r += a;
+    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+      const K o = KeyOps<K>::shfl_xor(v, (int)j);
+      const bool take_min = ((lane & j) == 0) == ((lane & k) == 0);
+      v = take_min ? (o < v ? o : v) : (o > v ? o : v);
     }
-    rank[e] = r;
+  }
+  return v;
+}
+
+// The sampling steps of Algorithm 4.1 for a subset of len keys, by a block of
+// NT threads: draw a sample of alpha * (v + 1) keys at pseudo-random positions,
+// sort it, select the splitters with the recursive duplicate-skipping rule of
+// Section 4.2.3 ("Sampling"): the middle sample of a range becomes the
+// splitter, the ranges left and right of the run of samples equal to it are
+// split recursively.  A node whose range is empty takes the sample just above
+// its range (the nearest splitter on the right among its ancestors), or
+// all-ones past the end, which keeps t a search tree.  Finally h'_i =
+// lcp(x_{i-1}, x_i) with h'_0 = h'_v = 0, the splitter LCPs of Algorithm 4.1.
+//
+// A step waits for its sample, so this is built for latency: warps sort runs
+// of 32 keys in registers, the runs are merged pairwise, each key finding its
+// place with a binary search in the partner run (30 dependent shared loads
+// for 512 keys; ranking every key in every other warp's run took 84 in
+// a 256-thread block, then 36 more to find the runs of equal keys, which now
+// come from a bitmap of run starts).  With the run of equal keys around every
+// sample position known, each tree node finds its range by walking from the
+// root along its level-order index, so the recursion needs no step-by-step
+// synchronisation.  Ends with __syncthreads().
+// key_at(pos) gives the key of the subset's record pos.
+template <int LOGV, typename K, uint32_t NT, typename KeyAt>
+__device__ void build_splitters(KeyAt&& key_at, uint32_t len, uint64_t hseed, SampleSmem<LOGV, K>& sm, uint32_t dna) {
+  using G = Geo<LOGV>;
+  constexpr uint32_t S = G::S;
+  constexpr int kLevels = LOGV + 1 - 5;  // merge levels from runs of 32 to S
+  const uint32_t tid = threadIdx.x;
+  K* src = (kLevels & 1) ? sm.merge : sm.sample;  // the last level writes sample
+  K* dst = (kLevels & 1) ? sm.sample : sm.merge;
+  for (uint32_t p = tid; p < S; p += NT) {  // whole warps: S is a multiple of 32
+    const uint64_t h = mix64(hseed + p);
+    src[p] = warp_bitonic<K>(key_at((uint32_t)(((h >> 32) * (uint64_t)len) >> 32)));
   }
   __syncthreads();
-#pragma unroll
-  for (int e = 0; e < E; ++e) s[rank[e]] = v[e];
-  __syncthreads();
-  for (uint32_t i = threadIdx.x; i < G::S; i += blockDim.x) {
-    const K val = s[i];
-    uint32_t a = 0, b = i;
-    while (a < b) { const uint32_t m = (a + b) >> 1; if (s[m] < val) a = m + 1; else b = m; }
-    bs.lo[i] = (uint16_t)a;
-    a = i + 1;
-    b = G::S;
-    while (a < b) { const uint32_t m = (a + b) >> 1; if (s[m] <= val) a = m + 1; else b = m; }
-    bs.hi[i] = (uint16_t)a;
+#pragma unroll 1
+  for (uint32_t run = 32; run < S; run <<= 1) {
+    // each key's place in the merged pair of runs: its own index plus the
+    // partner's keys before it (a left key goes before an equal right one)
+    for (uint32_t p = tid; p < S; p += NT) {
+      const K k = src[p];
+      const uint32_t i = p & (run - 1);
+      const K* other = src + (p ^ i ^ run);
+      const bool right = (p & run) != 0;
+      uint32_t a = 0;
+      for (uint32_t half = run >> 1; half > 0; half >>= 1) {
+        const K o = other[a + half - 1];
+        a += (right ? o <= k : o < k) ? half : 0u;
+      }
+      const K o = other[a];
+      a += (right ? o <= k : o < k) ? 1u : 0u;
+      dst[(p & ~(2 * run - 1)) + i + a] = k;
+    }
+    __syncthreads();
+    K* t = src;
+    src = dst;
+    dst = t;
+  }
+  const K* s = sm.sample;
+  // runs of equal keys, from one bit per position that starts one
+  for (uint32_t p = tid; p < S; p += NT) {
+    const uint32_t hb = __ballot_sync(0xFFFFFFFFu, p == 0 || s[p - 1] != s[p]);
+    if ((tid & 31u) == 0) sm.heads[p >> 5] = hb;
   }
   __syncthreads();
-  for (uint32_t q = threadIdx.x; q < G::V; q += blockDim.x) {
+  const uint64_t some = nonzero_words(sm.heads, S / 32);
+  for (uint32_t p = tid; p < S; p += NT) {
+    const bool head = (sm.heads[p >> 5] >> (p & 31u)) & 1u;
+    sm.lo[p] = (uint16_t)(head ? p : last_set_before(sm.heads, some, p));  // position 0 starts a run
+    sm.hi[p] = (uint16_t)min(S, first_set_after(sm.heads, some, p));
+  }
+  __syncthreads();
+  for (uint32_t q = tid; q < G::V; q += NT) {
     const uint32_t i = q + 1;               // level-order index
     const int l = 31 - __clz(i);            // its level
-    uint32_t a = 0, b = G::S;               // its range of the sorted sample
+    uint32_t a = 0, b = S;                  // its range of the sorted sample
     for (int d = l - 1; d >= 0; --d) {
       if (a < b) {
         const uint32_t m = (a + b) >> 1;
         if (((i >> d) & 1u) == 0) {
-          const uint32_t le = bs.lo[m];
+          const uint32_t le = sm.lo[m];
           b = le > a ? le : a;              // left of the run of keys equal to s[m]
         } else {
-          const uint32_t rs = bs.hi[m];
+          const uint32_t rs = sm.hi[m];
           a = rs < b ? rs : b;              // right of that run
         }
       } else {
         a = b;
       }
     }
-    const K val = a < b ? s[(a + b) >> 1] : (b < G::S ? s[b] : KeyOps<K>::ones());
-    sp.tree[i] = val;
-    sp.x[(2 * (i - (1u << l)) + 1) * (1u << (LOGV - 1 - l)) - 1] = val;
+    const K val = a < b ? s[(a + b) >> 1] : (b < S ? s[b] : KeyOps<K>::ones());
+    sm.sp.tree[i] = val;
+    sm.sp.x[(2 * (i - (1u << l)) + 1) * (1u << (LOGV - 1 - l)) - 1] = val;
+  }
+  if (tid == 0) {
+    sm.sp.tree[0] = 0;
+    sm.sp.x[G::V] = 0;
   }
   __syncthreads();
-  for (uint32_t r = threadIdx.x; r <= G::V; r += blockDim.x)
-    sp.hp[r] = (r == 0 || r == G::V) ? 0 : (uint8_t)KeyOps<K>::lcp(sp.x[r - 1], sp.x[r], dna);
-  if (threadIdx.x == 0) sp.tree[0] = 0;
+  for (uint32_t r = tid; r <= G::V; r += NT)
+    sm.sp.hp[r] = (r == 0 || r == G::V) ? 0 : (uint8_t)KeyOps<K>::lcp(sm.sp.x[r - 1], sm.sp.x[r], dna);
   __syncthreads();
-}
-
-// The sampling steps for a subset of narrow records.
-template <int LOGV>
-__device__ __forceinline__ void build_splitters(const Rec* __restrict__ recs, uint32_t len, uint64_t hseed,
-                                                Splitters<LOGV>& sp, BuildScratch<LOGV>& bs, uint32_t dna) {
-  build_splitters_k<LOGV, uint64_t>([&](uint32_t pos) { return recs[pos].key; }, len, hseed, sp, bs, dna);
 }
 
 // Lemma 4.1: one-based level-order index l <-> one-based pre-order index p
@@ -296,55 +310,46 @@ __device__ __forceinline__ void classify_batch(const K (&k)[U], uint32_t (&b)[U]
 // Classifies n keys (the classification loop of Algorithm 4.1): writes the bucket of
 // keys[p] to bo[p] and counts it in hist (one shared-memory atomic per key:
 // cheaper than grouping a warp's equal buckets with __match_any_sync first).  Each thread loads 8 keys before descending the tree for them,
-// so that the loads of a batch overlap.  Returns this thread's records.
-template <int LOGV, typename K, typename KeyAt>
-__device__ __forceinline__ uint32_t classify_count_k(KeyAt&& key_at, uint16_t* __restrict__ bo, uint32_t n,
-                                                     const K* tree, const K* x, uint32_t* hist, uint32_t variant,
-                                                     const uint16_t* jump, unsigned long long* bmin = nullptr,
-                                                     unsigned long long* bmax = nullptr) {
-  constexpr int U = sizeof(K) == 8 ? 8 : 4;  // keys per thread in flight (wide keys take 4 registers)
-  uint32_t mine = 0;
-  const uint32_t lim = (n + kBlock - 1) / kBlock * kBlock;
-  for (uint32_t p0 = threadIdx.x; p0 < lim; p0 += U * kBlock) {
-    K k[U];
+// so that the loads of a batch overlap.  seen(b, key) is called for every key
+// after its bucket is known.  Returns this thread's records.
+struct NothingSeen {
+  template <typename K>
+  __device__ __forceinline__ void operator()(uint32_t, K) const {}
+};
+template <int LOGV, typename K, uint32_t NT, int U, typename KeyAt, typename Seen>
+__device__ __forceinline__ void classify_some(KeyAt&& key_at, uint16_t* __restrict__ bo, uint32_t p0, uint32_t n,
+                                              const K* tree, const K* x, uint32_t* hist, uint32_t variant,
+                                              const uint16_t* jump, Seen&& seen) {
+  K k[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const uint32_t p = p0 + u * kBlock;
-      k[u] = p < n ? key_at(p) : (K)0;
-    }
-    uint32_t bb[U];
-    classify_batch<LOGV, U, K>(k, bb, tree, x, variant, jump);
+  for (int u = 0; u < U; ++u) {
+    const uint32_t p = p0 + u * NT;
+    k[u] = p < n ? key_at(p) : (K)0;
+  }
+  uint32_t bb[U];
+  classify_batch<LOGV, U, K>(k, bb, tree, x, variant, jump);
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const uint32_t p = p0 + u * kBlock;
-      if (p >= lim) break;  // uniform across the block
-      const bool valid = p < n;
-      const uint32_t b = valid ? bb[u] : 0xFFFFu;
-      if (valid) {
-        bo[p] = (uint16_t)b;
-        ++mine;
-      }
-      if (valid) atomicAdd(&hist[b], 1u);
-      if constexpr (sizeof(K) == 8) {
-        // smallest and largest key of each even bucket (an equality bucket's
-        // keys all equal its splitter), for the LCPs at bucket boundaries
-        if (bmin && valid && !(b & 1u)) {
-          atomicMin(&bmin[b], (unsigned long long)k[u]);
-          atomicMax(&bmax[b], (unsigned long long)k[u]);
-        }
-      }
+  for (int u = 0; u < U; ++u) {
+    const uint32_t p = p0 + u * NT;
+    if (p < n) {
+      bo[p] = (uint16_t)bb[u];
+      atomicAdd(&hist[bb[u]], 1u);
+      seen(bb[u], k[u]);
     }
   }
-  return mine;
 }
 
-template <int LOGV>
-__device__ __forceinline__ uint32_t classify_count(const Rec* __restrict__ recs, uint16_t* __restrict__ bo,
-                                                   uint32_t n, const uint64_t* tree, const uint64_t* x,
-                                                   uint32_t* hist, uint32_t variant,
-                                                   const uint16_t* jump = nullptr) {
-  return classify_count_k<LOGV, uint64_t>([&](uint32_t p) { return recs[p].key; }, bo, n, tree, x, hist, variant,
-                                          jump);
+template <int LOGV, typename K, uint32_t NT, typename KeyAt, typename Seen = NothingSeen>
+__device__ __forceinline__ uint32_t classify_count_k(KeyAt&& key_at, uint16_t* __restrict__ bo, uint32_t n,
+                                                     const K* tree, const K* x, uint32_t* hist, uint32_t variant,
+                                                     const uint16_t* jump, Seen&& seen = NothingSeen()) {
+  constexpr int U = sizeof(K) == 8 ? 8 : 4;  // keys per thread in flight (wide keys take 4 registers)
+  uint32_t p0 = threadIdx.x, left = (n + NT - 1) / NT;  // keys per thread
+  for (; left > U / 2; left -= min(left, (uint32_t)U), p0 += U * NT)
+    classify_some<LOGV, K, NT, U>(key_at, bo, p0, n, tree, x, hist, variant, jump, seen);
+  // the rest (or a subset of few keys per thread) without idle descents
+  if (left) classify_some<LOGV, K, NT, U / 2>(key_at, bo, p0, n, tree, x, hist, variant, jump, seen);
+  return threadIdx.x < n ? (n - 1 - threadIdx.x) / NT + 1 : 0u;
 }
 
 // What happens to bucket b of a step at depth h (Output of Algorithm 4.1 and
@@ -366,11 +371,6 @@ __device__ __forceinline__ uint32_t bucket_desc(uint32_t b, uint32_t size, uint3
   return depth + sp.hp[r];
 }
 
-// Records moved per batch of one warp in the distribution: the loads of a
-// batch are issued together so that each warp keeps kMoveBatch rounds of
-// memory accesses in flight.  4 (not 8) keeps the multi-block distribution at
-// 64 registers, 4 blocks per SM: more warps in flight beat deeper batches.
-constexpr int kMoveBatch = 4;
 constexpr uint32_t kInvalid = 0xFFFFFFFFu;
 
 // The lanes of the warp whose record falls into the same bucket b as this
@@ -395,18 +395,19 @@ __device__ __forceinline__ uint32_t bucket_peers(uint32_t b, bool valid) {
 //   tb[0..tl)    bucket of each record of the tile (shared memory)
 //   base[b]      in: destination of the tile's first record of bucket b;
 //                out: base[b] + number of the tile's records in bucket b
-//   cntw         shared scratch, kWarps * KP uint32
+//   cntw         shared scratch, NT / 32 * KP uint32
 // Warp w owns records [w * 32R, (w + 1) * 32R) of the tile; inside a warp
 // ranks come from the lanes with the same bucket (bucket_peers), so equal
 // buckets keep input order.
-// move(p[], b[], dest[]) is called with kMoveBatch rounds of one warp at a time
+// move(p[], b[], dest[]) is called with MB rounds of one warp at a time
 // (p = kInvalid for lanes without a record).  Ends with __syncthreads().
-template <int LOGV, int MB = kMoveBatch, typename Move>
+template <int LOGV, uint32_t NT, int MB, typename Move>
 __device__ void tile_scatter(const uint16_t* tb, uint32_t tl, uint32_t R, uint32_t* base,
                              uint32_t* cntw, Move&& move) {
   using G = Geo<LOGV>;
+  constexpr uint32_t kWarps = NT / 32;
   const uint32_t w = threadIdx.x >> 5, lane = lane_id();
-  for (uint32_t i = threadIdx.x; i < kWarps * G::KP; i += blockDim.x) cntw[i] = 0;
+  for (uint32_t i = threadIdx.x; i < kWarps * G::KP; i += NT) cntw[i] = 0;
   __syncthreads();
   uint32_t* mine = cntw + w * G::KP;
   const uint32_t p0 = w * 32 * R;
@@ -415,7 +416,7 @@ __device__ void tile_scatter(const uint16_t* tb, uint32_t tl, uint32_t R, uint32
     if (p < tl) atomicAdd(&mine[tb[p]], 1u);  // counts only: no need to group equal buckets
   }
   __syncthreads();
-  for (uint32_t b = threadIdx.x; b < G::K; b += blockDim.x) {
+  for (uint32_t b = threadIdx.x; b < G::K; b += NT) {
     uint32_t run = base[b];
 #pragma unroll
     for (uint32_t ww = 0; ww < kWarps; ++ww) {
@@ -459,16 +460,16 @@ __device__ void tile_scatter(const uint16_t* tb, uint32_t tl, uint32_t R, uint32
 // + record 16 read (the record carries the string's offset); finished: perm 4
 // (+ lcp 4) written; open: record 16 written, plus 8 characters read when the
 // cache is reloaded.
-template <typename First>
+template <int MB, typename First>
 __device__ __forceinline__ uint32_t move_batch(const SortCtx& c, const SetDesc& sd, uint32_t wide, uint32_t par,
                                                uint32_t src0, uint32_t depth, const uint32_t* desc,
-                                               First&& bucket_first, const uint32_t (&pp)[kMoveBatch],
-                                               const uint32_t (&bb)[kMoveBatch], const uint32_t (&dd)[kMoveBatch]) {
-  uint32_t id[kMoveBatch], ds[kMoveBatch], o32[kMoveBatch];
-  uint64_t key[kMoveBatch], off[kMoveBatch];
+                                               First&& bucket_first, const uint32_t (&pp)[MB],
+                                               const uint32_t (&bb)[MB], const uint32_t (&dd)[MB]) {
+  uint32_t id[MB], ds[MB], o32[MB];
+  uint64_t key[MB], off[MB];
   uint32_t bytes = 0;
 #pragma unroll
-  for (int u = 0; u < kMoveBatch; ++u) {
+  for (int u = 0; u < MB; ++u) {
     id[u] = 0;
     o32[u] = 0;
     ds[u] = kFin;
@@ -483,9 +484,9 @@ __device__ __forceinline__ uint32_t move_batch(const SortCtx& c, const SetDesc& 
   }
   // the characters of every byte-string reload are requested before any of
   // them is used (one memory round trip for the batch)
-  CharWords ww[kMoveBatch];
+  CharWords ww[MB];
 #pragma unroll
-  for (int u = 0; u < kMoveBatch; ++u) {
+  for (int u = 0; u < MB; ++u) {
     off[u] = 0;
     if (pp[u] != kInvalid && !(ds[u] & kFin) && (ds[u] & kLow30) != depth) {
       off[u] = rec_offset(sd, wide, id[u], o32[u]);
@@ -493,7 +494,7 @@ __device__ __forceinline__ uint32_t move_batch(const SortCtx& c, const SetDesc& 
     }
   }
 #pragma unroll
-  for (int u = 0; u < kMoveBatch; ++u) {
+  for (int u = 0; u < MB; ++u) {
     if (pp[u] == kInvalid) continue;
     const uint32_t d = ds[u];
     const uint32_t dest = dd[u];
