@@ -579,7 +579,7 @@ static ss_status run_sort(uint8_t* ws, const Layout& L, SortCtx c, const Opts& o
   }
   const uint32_t qgrid = (uint32_t)(dev.sms * dev.queue_blocks[o.logv]);
   SS_CUDA(launch_queue(o.logv, c, qgrid, st, hook));
-  SS_CUDA(launch_small(c, pmax_of(o.cutoff), (uint32_t)dev.sms * 8, (uint32_t)dev.sms * 4, st, hook));
+  SS_CUDA(launch_small(c, pmax_of(o.cutoff), (uint32_t)dev.sms, st, hook));
   const uint32_t fgrid = std::max(1u, std::min<uint32_t>((c.total + kBlock - 1) / kBlock, (uint32_t)dev.sms * 16));
   SS_CUDA(launch_lcp_fix(c, fgrid, st, hook));
   return SS_OK;

@@ -106,8 +106,7 @@ cudaError_t launch_queue(int logv, const SortCtx& c, uint32_t grid, cudaStream_t
 // Small subsets, set-up and LCP fix-up.
 size_t small_cta_smem(uint32_t pmax);
 cudaError_t launch_init(const SortCtx& c, cudaStream_t st, const LaunchHook& hook);
-cudaError_t launch_small(const SortCtx& c, uint32_t pmax, uint32_t grid_warp, uint32_t grid_cta,
-                         cudaStream_t st, const LaunchHook& hook);
+cudaError_t launch_small(const SortCtx& c, uint32_t pmax, uint32_t sms, cudaStream_t st, const LaunchHook& hook);
 cudaError_t launch_lcp_fix(const SortCtx& c, uint32_t grid, cudaStream_t st, const LaunchHook& hook);
 // Packs bytes over {A, C, G, T, 0} into 3-bit codes (dna_key's layout).
 // Copies bytes (a multiple of 4, 4-byte aligned) from pinned host memory

@@ -285,335 +285,412 @@ __global__ void __launch_bounds__(kBlock) k_small_warp(SortCtx c, TaskList list,
 }
 
 // ---- block-level refinement -------------------------------------------------------
+//
+// A subset of 33..small_cutoff strings is sorted by one block in shared memory.
+// These sorts are bound by instruction issue (their data is on chip), so the
+// design minimises the instructions per string: one more splitting by 32 or 64
+// sampled keys, after which a string finds its rank by comparing itself with
+// the few others of its bucket.  Both launches, 20 M URLs 700 -> 571 us, 1 M
+// URLs 190 -> 139, batch of 512 sets 930 -> 700, 4 M DNA suffixes 171 -> 126
+// against a block merge sort (runs of 32 by warp networks, merge paths) in 64-
+// and 256-thread blocks; merging by binary searches in the partner run took as
+// many instructions as the merge paths (794 us on 20 M URLs), one-warp blocks
+// for the small subsets 570 / 220 / 834 / 124 us, 128-thread ones 713 / 168 /
+// 789 / 173.
 
-// Element tags of the block sort: handed (1 bit) << 25 | segment (12 bits)
-// << 13 | original position (12 bits) << 1 | open (1 bit).  Sorting by (segment, cache, tag)
-// orders each segment by cache and, among equal caches, by original position
-// (= ascending index).  Index and offset stay at the original position.
-__device__ __forceinline__ uint32_t tag_seg(uint32_t t) { return (t >> 13) & 0xFFFu; }
-constexpr uint32_t kHanded = 1u << 25;  // run passed on to the warp list
-__device__ __forceinline__ uint32_t tag_pos(uint32_t t) { return (t >> 1) & 0xFFFu; }
-__device__ __forceinline__ uint32_t make_tag(uint32_t seg, uint32_t pos, uint32_t open) {
-  return (seg << 13) | (pos << 1) | open;
-}
+constexpr uint32_t kSmallNarrowThreads = 64, kSmallWideThreads = 256;
 
-struct CtaSmem {  // carved from dynamic shared memory, pmax elements
-  uint64_t* key;    // cache, in sorted position
-  uint64_t* key2;   // second buffer of the merge sort
-  uint32_t* tag2;
-  uint64_t* off;    // string offset, by original position
-  uint32_t* tag;    // in sorted position
-  uint32_t* idx;    // index, by original position
-  uint32_t* aux;    // segment sizes
-  uint16_t* nseg;   // segment start of each position
+// Sampled keys, all of them splitters: 2 * S + 1 buckets (bucket 2r + 1: the
+// keys equal to splitter r; bucket 2r: those between splitters r - 1 and r).
+template <uint32_t NT>
+constexpr uint32_t kSmallSample = NT == kSmallNarrowThreads ? 32 : 64;
+
+// Equality buckets of more strings than this get their places in string order
+// right away instead of a rank by comparing positions.
+constexpr uint32_t kSmallEqual = 64;
+
+template <uint32_t NT>
+struct SmallSplit {
+  uint64_t key[kSmallSample<NT>];           // the sorted sample
+  uint32_t first[2 * kSmallSample<NT> + 2]; // bucket sizes, then bucket starts
+  uint8_t big[2 * kSmallSample<NT> + 2];    // number of a large equality bucket, kNotBig for the others
+  uint32_t nbig;
+};
+constexpr uint32_t kNotBig = 255;
+
+struct SmallSmem {    // carved from dynamic shared memory, for subsets of up to pmax strings
+  uint64_t* key;      // cache: in the order before a sort, in sorted order after it
+  uint64_t* gkey;     // cache, grouped by bucket
+  uint2* open;        // ranges still to be sorted deeper: (start | length << 16, depth)
+  uint32_t* idx;      // index, by original position
+  uint32_t* off;      // low offset word, by original position
+  uint32_t* tmp;      // bucket | place in it << 16; after the sort: runs to hand on, start | length << 16
+  uint32_t* heads;    // bit i of word w: sorted position lo + 32 w + i starts a run of equal caches
+  uint16_t* pos[2];   // original position, in sorted order (two buffers)
+  uint16_t* gpos;     // position before the sort, grouped by bucket
 };
 
-// Order of the block sort: (segment, cache, tag), evaluated without branches.
-// OneSeg: every element is in segment 0 and none is handed on (the first pass
-// over a subset, which does nearly all of the block sorts' work), so the tags
-// compare as original positions and the segment test drops out.
-template <bool OneSeg>
-__device__ __forceinline__ bool elem_less(uint64_t ka, uint32_t ta, uint64_t kb, uint32_t tb) {
-  if (OneSeg) return (ka < kb) | ((ka == kb) & (ta < tb));
-  const uint32_t sa = tag_seg(ta), sb = tag_seg(tb);
-  return (sa < sb) | ((sa == sb) & ((ka < kb) | ((ka == kb) & (ta < tb))));
+__host__ __device__ inline uint32_t small_words(uint32_t pmax) { return pmax / 32 + 1; }
+
+__device__ __forceinline__ SmallSmem small_smem(uint8_t* smem, uint32_t pmax) {
+  SmallSmem m;
+  m.key = reinterpret_cast<uint64_t*>(smem);
+  m.gkey = m.key + pmax;
+  m.open = reinterpret_cast<uint2*>(m.gkey + pmax);
+  m.idx = reinterpret_cast<uint32_t*>(m.open + small_words(pmax));
+  m.off = m.idx + pmax;
+  m.tmp = m.off + pmax;
+  m.heads = m.tmp + pmax;
+  m.pos[0] = reinterpret_cast<uint16_t*>(m.heads + small_words(pmax));
+  m.pos[1] = m.pos[0] + pmax;
+  m.gpos = m.pos[1] + pmax;
+  return m;
 }
 
-// Slots past the end of a subset: after every real element in elem_less order.
-constexpr uint32_t kPadTag = 0xFFFFFFFFu;
-
-// Bitonic sort of one (key, tag) per lane by elem_less, ascending in lane order.
-// The stages of each merge level run as a loop: the smaller code was faster
-// than the fully unrolled network in the block sort kernels.
-template <bool OneSeg>
-__device__ __forceinline__ void warp_sort_elems(uint64_t& key, uint32_t& tag) {
-  const uint32_t lane = lane_id();
-#pragma unroll
-  for (uint32_t k = 2; k <= 32; k <<= 1) {
-#pragma unroll 1
-    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-      const uint32_t ot = __shfl_xor_sync(kFull, tag, j);
-      const uint64_t ok = __shfl_xor_sync(kFull, key, j);
-      const bool up = (lane & k) == 0;
-      const bool lower = (lane & j) == 0;
-      const bool take = (lower == up) ? elem_less<OneSeg>(ok, ot, key, tag) : elem_less<OneSeg>(key, tag, ok, ot);
-      tag = take ? ot : tag;
-      key = take ? ok : key;
-    }
-  }
-}
-
-// Stable block merge sort of (key, tag) at positions [0, n), n <= pmax.
-// Each warp first sorts runs of 32 positions with a bitonic network in
-// registers; then every merge pass doubles the run length, each thread
-// producing ipt (<= 32) outputs of one merged pair of runs: it finds where its
-// outputs start with a binary search along the merge path and merges
-// sequentially.  Uses (key2, tag2) as the second buffer; the result ends in
-// (m.key, m.tag).
-template <uint32_t NT, bool OneSeg>
-__device__ void block_sort(CtaSmem& m, uint32_t n) {
-  uint32_t ipt = 1;
-  while (ipt * NT < n) ipt <<= 1;
-  for (uint32_t c0 = threadIdx.x & ~31u; c0 < n; c0 += NT) {
-    const uint32_t p = c0 + lane_id();
-    uint64_t k = p < n ? m.key[p] : ~0ull;
-    uint32_t t = p < n ? m.tag[p] : kPadTag;
-    warp_sort_elems<OneSeg>(k, t);
-    if (p < n) {
-      m.key[p] = k;
-      m.tag[p] = t;
-    }
-  }
-  __syncthreads();
-  uint64_t* sk = m.key;
-  uint32_t* st = m.tag;
-  uint64_t* dk = m.key2;
-  uint32_t* dt = m.tag2;
-  for (uint32_t run = 32; run < n; run <<= 1) {
-    const uint32_t out = threadIdx.x * ipt;
-    if (out < n) {
-      const uint32_t base = (out / (2 * run)) * (2 * run);
-      const uint32_t la = min(run, n - base);
-      const uint32_t lb = base + run < n ? min(run, n - base - run) : 0u;
-      const uint64_t* ak = sk + base;
-      const uint32_t* at = st + base;
-      const uint64_t* bk = sk + base + run;
-      const uint32_t* bt = st + base + run;
-      const uint32_t d = out - base;
-      uint32_t lo = d > lb ? d - lb : 0u, hi = min(d, la);
-      while (lo < hi) {  // number of A elements among the first d outputs
-        const uint32_t mid = (lo + hi) >> 1;
-        if (!elem_less<OneSeg>(bk[d - mid - 1], bt[d - mid - 1], ak[mid], at[mid])) lo = mid + 1;
-        else hi = mid;
-      }
-      uint32_t i = lo, j = d - lo;
-      const uint32_t cnt = min(ipt, n - out);
-      for (uint32_t q = 0; q < cnt; ++q) {
-        const bool take_a = i < la && (j >= lb || !elem_less<OneSeg>(bk[j], bt[j], ak[i], at[i]));
-        if (take_a) {
-          dk[out + q] = ak[i];
-          dt[out + q] = at[i];
-          ++i;
-        } else {
-          dk[out + q] = bk[j];
-          dt[out + q] = bt[j];
-          ++j;
-        }
-      }
-    }
-    __syncthreads();
-    uint64_t* tk = sk; sk = dk; dk = tk;
-    uint32_t* tt = st; st = dt; dt = tt;
-  }
-  if (sk != m.key) {
-    for (uint32_t j = threadIdx.x; j < n; j += NT) {
-      m.key[j] = sk[j];
-      m.tag[j] = st[j];
-    }
-    __syncthreads();
-  }
-}
-
-// Inclusive max-scan of a[0..n) in place.
+// Sorts the n elements whose caches are key[0, n) by (cache, place before the
+// sort): key becomes sorted, pos_out[i] is pos_in[place of the i-th] (null: the
+// place itself).  pos_out must not be pos_in.  Ends with a barrier; the caller
+// has written key before a barrier.
 template <uint32_t NT>
-__device__ void block_max_scan(uint16_t* a, uint32_t n) {
-  constexpr uint32_t NW = NT / 32;
-  __shared__ uint32_t wmax[NW];
-  const uint32_t per = (n + NT - 1) / NT;
-  const uint32_t b0 = threadIdx.x * per;
-  uint32_t m = 0;
-  for (uint32_t j = 0; j < per && b0 + j < n; ++j) m = max(m, (uint32_t)a[b0 + j]);
-  uint32_t inc = m;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    uint32_t t = __shfl_up_sync(kFull, inc, o);
-    if (lane_id() >= (uint32_t)o) inc = max(inc, t);
+__device__ void small_sort(const SmallSmem& m, SmallSplit<NT>& sp, uint64_t* key, uint32_t n, const uint16_t* pos_in,
+                           uint16_t* pos_out) {
+  constexpr uint32_t S = kSmallSample<NT>;
+  const uint32_t tid = threadIdx.x, lane = lane_id();
+  // the sample, from evenly spaced places, put in order by counting
+  for (uint32_t b = tid; b < 2 * S + 2; b += NT) sp.first[b] = 0;
+  if (tid == 0) sp.nbig = 0;
+  if (tid < S) {
+    const uint64_t mine = key[tid * n / S];
+    uint32_t r = 0;
+#pragma unroll 8
+    for (uint32_t i = 0; i < S; ++i) {
+      const uint64_t o = key[i * n / S];  // the same word for every lane
+      r += (o < mine || (o == mine && i < tid)) ? 1u : 0u;
+    }
+    sp.key[r] = mine;
   }
-  const uint32_t w = threadIdx.x >> 5;
-  if (lane_id() == 31) wmax[w] = inc;
   __syncthreads();
-  if (w == 0) {
-    uint32_t v = lane_id() < NW ? wmax[lane_id()] : 0;
+  // bucket of every element, and its place in the bucket (in no particular order)
+  for (uint32_t j = tid; j < n; j += NT) {
+    const uint64_t k = key[j];
+    uint32_t a = 0;
+#pragma unroll
+    for (uint32_t half = S / 2; half > 0; half >>= 1) a += sp.key[a + half - 1] < k ? half : 0u;
+    a += sp.key[a] < k ? 1u : 0u;
+    const uint32_t b = 2 * a + ((a < S && sp.key[a] == k) ? 1u : 0u);
+    m.tmp[j] = b | atomicAdd(&sp.first[b], 1u) << 16;
+  }
+  __syncthreads();
+  if (tid < 32) {  // bucket starts
+    constexpr uint32_t kPer = (2 * S + 2 + 31) / 32;
+    uint32_t v[kPer], sum = 0;
+#pragma unroll
+    for (uint32_t u = 0; u < kPer; ++u) {
+      const uint32_t b = lane * kPer + u;
+      v[u] = b < 2 * S + 2 ? sp.first[b] : 0u;
+      sum += v[u];
+    }
+    uint32_t inc = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      uint32_t t = __shfl_up_sync(kFull, v, o);
-      if (lane_id() >= (uint32_t)o) v = max(v, t);
+      const uint32_t t = __shfl_up_sync(kFull, inc, o);
+      if (lane >= (uint32_t)o) inc += t;
     }
-    if (lane_id() < NW) wmax[lane_id()] = v;
+    uint32_t run = inc - sum;
+#pragma unroll
+    for (uint32_t u = 0; u < kPer; ++u) {
+      const uint32_t b = lane * kPer + u;
+      if (b < 2 * S + 2) {
+        sp.first[b] = run;
+        sp.big[b] = (b & 1u) && v[u] > kSmallEqual ? (uint8_t)atomicAdd(&sp.nbig, 1u) : (uint8_t)kNotBig;
+      }
+      run += v[u];
+    }
   }
   __syncthreads();
-  uint32_t excl = __shfl_up_sync(kFull, inc, 1);
-  if (lane_id() == 0) excl = 0;
-  uint32_t run = max(excl, w ? wmax[w - 1] : 0u);
-  for (uint32_t j = 0; j < per && b0 + j < n; ++j) {
-    run = max(run, (uint32_t)a[b0 + j]);
-    a[b0 + j] = (uint16_t)run;
+  const uint32_t nbig = sp.nbig;
+  if (nbig) {
+    // stable places in the large equality buckets: the strings of each in every
+    // 32 consecutive ones, by ballots, and the sums of these counts before them
+    uint16_t* cnt = reinterpret_cast<uint16_t*>(m.gkey);  // nbig * chunks <= n / 65 * (n / 32 + 1) counts
+    const uint32_t chunks = (n + 31) / 32;
+    for (uint32_t c0 = tid >> 5; c0 < chunks; c0 += NT / 32) {
+      const uint32_t j = 32 * c0 + lane;
+      const uint32_t t = j < n ? m.tmp[j] : 0u;
+      const uint32_t id = j < n ? sp.big[t & 0xFFFFu] : kNotBig;
+      uint32_t place = t >> 16;
+      for (uint32_t g = 0; g < nbig; ++g) {
+        const uint32_t mask = __ballot_sync(kFull, id == g);
+        if (id == g) place = __popc(mask & lanemask_lt());
+        if (lane == 0) cnt[g * chunks + c0] = (uint16_t)__popc(mask);
+      }
+      if (j < n) m.tmp[j] = (t & 0xFFFFu) | place << 16;
+    }
+    __syncthreads();
+    for (uint32_t g = tid; g < nbig; g += NT) {
+      uint32_t run = 0;
+      for (uint32_t c0 = 0; c0 < chunks; ++c0) {
+        const uint32_t v = cnt[g * chunks + c0];
+        cnt[g * chunks + c0] = (uint16_t)run;
+        run += v;
+      }
+    }
+    __syncthreads();
+    for (uint32_t j = tid; j < n; j += NT) {
+      const uint32_t id = sp.big[m.tmp[j] & 0xFFFFu];
+      if (id != kNotBig) m.tmp[j] += (uint32_t)cnt[id * chunks + j / 32] << 16;
+    }
+    __syncthreads();
+  }
+  for (uint32_t j = tid; j < n; j += NT) {
+    const uint32_t t = m.tmp[j];
+    const uint32_t q = sp.first[t & 0xFFFFu] + (t >> 16);
+    m.gkey[q] = key[j];
+    m.gpos[q] = (uint16_t)j;
+  }
+  __syncthreads();
+  for (uint32_t q = tid; q < n; q += NT) {
+    const uint64_t k = m.gkey[q];
+    const uint32_t j = m.gpos[q];
+    const uint32_t b = m.tmp[j] & 0xFFFFu;
+    const uint32_t s = sp.first[b], e = sp.first[b + 1];
+    uint32_t r = s;
+    if (b & 1u) {  // equal keys
+      if (e - s > kSmallEqual) r = q;  // in string order already
+      else
+        for (uint32_t i = s; i < e; ++i) r += m.gpos[i] < j ? 1u : 0u;
+    } else {
+      for (uint32_t i = s; i < e; ++i) {
+        const uint64_t o = m.gkey[i];
+        r += (o < k || (o == k && m.gpos[i] < j)) ? 1u : 0u;
+      }
+    }
+    __syncwarp(__activemask());
+    key[r] = k;  // the unsorted keys are not needed any more
+    pos_out[r] = pos_in ? pos_in[j] : (uint16_t)j;
   }
   __syncthreads();
 }
 
-// The narrow launch (narrow = 1) sorts the subsets of c.small_cta, the wide
-// one those of c.small_cta_wide; while there are fewer than min_count subsets
-// in all, the narrow launch leaves every subset to the wide one.  Each block
-// claims one subset at a time from its launch's counter (subset sizes vary
-// several-fold, so a fixed share per block left many SMs idle at the end).
+// Sorts the subsets of one list: c.small_cta (64-thread blocks) or
+// c.small_cta_wide (256 threads; it runs first, and passes runs that the
+// 64-thread blocks can take on to them).  While there are fewer than min_count
+// subsets in all, the wide launch takes both lists and passes nothing on: a
+// larger block is done with a subset sooner, and the GPU is not full anyway.
+// Each block claims one subset at a time from its launch's counter (subset sizes vary several-fold, so a fixed share
+// per block left many SMs idle at the end); the next subset is claimed, and
+// its task read, while the current one sorts.
 template <uint32_t NT, bool DNA>
-__global__ void __launch_bounds__(NT) k_small_cta(SortCtx c, uint32_t pmax, uint32_t min_count, uint32_t narrow) {
+__global__ void __launch_bounds__(NT) k_small_cta(SortCtx c, uint32_t pmax, uint32_t min_count) {
   constexpr uint32_t dna = DNA ? 1u : 0u;  // the character encoding, fixed per instance
+  constexpr uint32_t NW = NT / 32;
+  constexpr bool kWide = NT == kSmallWideThreads;
   extern __shared__ __align__(16) uint8_t smem[];
-  CtaSmem m;
-  m.key = reinterpret_cast<uint64_t*>(smem);
-  m.key2 = m.key + pmax;
-  m.off = m.key2 + pmax;
-  m.tag = reinterpret_cast<uint32_t*>(m.off + pmax);
-  m.tag2 = m.tag + pmax;
-  m.idx = m.tag2 + pmax;
-  m.aux = m.idx + pmax;
-  m.nseg = reinterpret_cast<uint16_t*>(m.aux + pmax);
-  __shared__ uint32_t s_max_open, s_jstop, s_neq;
+  const SmallSmem m = small_smem(smem, pmax);
+  __shared__ SmallSplit<NT> split;
+  __shared__ uint32_t s_ti, s_open, s_jstop, s_neq, s_runs, s_base;
+  __shared__ Task s_task;
   __shared__ uint64_t s_lead[kLookWindows];
+  const uint32_t tid = threadIdx.x, lane = lane_id(), w = tid >> 5;
   unsigned long long bytes = 0;
+  // Subsets passed on while this launch runs only raise n_narrow from at
+  // least min_count - n_wide, so every block of both launches finds the same `few`.
   const uint32_t n_narrow = min(*c.small_cta.count, c.small_cta.cap);
   const uint32_t n_wide = min(*c.small_cta_wide.count, c.small_cta_wide.cap);
   const bool few = n_narrow + n_wide < min_count;
-  if (narrow && few) return;
+  if (!kWide && few) return;
   // this launch's subsets: the first na of the narrow list, then the wide list
-  const uint32_t na = (narrow || few) ? n_narrow : 0u;
-  const uint32_t count = narrow ? n_narrow : na + n_wide;
-  uint32_t* claim = c.small_claim + (narrow ? 0 : 1);
-  __shared__ uint32_t s_ti;
-  if (threadIdx.x == 0) s_ti = atomicAdd(claim, 1u);
-  __syncthreads();
-  for (uint32_t ti = s_ti; ti < count; ti = s_ti) {
-    const Task t = ti < na ? c.small_cta.items[ti] : c.small_cta_wide.items[ti - na];
-    __syncthreads();  // every thread has read s_ti
-    if (threadIdx.x == 0) s_ti = atomicAdd(claim, 1u);  // the next subset, claimed while this one sorts
+  const uint32_t na = !kWide || few ? n_narrow : 0u;
+  const uint32_t count = kWide ? na + n_wide : na;
+  const uint32_t hand_max = kWide && !few ? kSmallCtaNarrowMax : 32u;
+  auto task_of = [&](uint32_t i) { return i < na ? c.small_cta.items[i] : c.small_cta_wide.items[i - na]; };
+  uint32_t* claim = c.small_claim + (kWide ? 1 : 0);
+  uint32_t next = 0;  // thread 0: the claimed subset, kept in registers until it is needed
+  Task next_task{0, 0, 0, 0};
+  if (tid == 0) {
+    next = atomicAdd(claim, 1u);
+    if (next < count) next_task = task_of(next);
+  }
+  while (true) {
+    if (tid == 0) {
+      s_ti = next;
+      s_task = next_task;
+      s_open = 0;
+      s_neq = 0;
+      s_runs = 0;
+    }
+    __syncthreads();
+    if (s_ti >= count) break;
+    const Task t = s_task;
+    if (tid == 0) next = atomicAdd(claim, 1u);
+    __syncwarp();  // lane 0 would run on by itself, and every shuffle below would wait for it
     if (t.len > pmax) {  // cannot happen: a list holds only sizes its launch's shared arrays take
-      if (threadIdx.x == 0) latch_status(c.status, kStQueueFull);
-      __syncthreads();
-      continue;
+      if (tid == 0) latch_status(c.status, kStQueueFull);
+      break;
     }
     const SetDesc sd = c.sets[task_set(t)];
     const uint32_t kw = key_width(dna);  // characters per key
-    const uint32_t par = task_par(t);
-    const uint32_t n = t.len;
-    const uint32_t wide = c.wide[task_set(t)];
-    for (uint32_t j = threadIdx.x; j < n; j += NT) {
-      const Rec r = load_rec(c.rec[par] + t.begin + j);
-      m.key[j] = r.key;
-      m.idx[j] = r.idx;
-      m.off[j] = rec_offset(sd, wide, r.idx, r.off);
-      m.tag[j] = make_tag(0, j, 1);
-    }
+    Rec* recs = c.rec[task_par(t)] + t.begin;
     uint32_t* lcp = sd.lcp ? sd.lcp + (t.begin - sd.base) : nullptr;
-    uint32_t depth = t.depth;
+    uint32_t* perm = sd.perm + (t.begin - sd.base);
+    const uint32_t wide = c.wide[task_set(t)];
+    uint32_t lo = 0, n = t.len, depth = t.depth;
+    // the range being sorted: the whole subset first, then runs of more than
+    // 32 strings whose caches were equal (rare), one at a time
+    const uint64_t k0 = recs[0].key;
+    bool neq = false;
+    for (uint32_t j = tid; j < n; j += NT) {
+      const Rec r = load_rec(recs + j);
+      m.idx[j] = r.idx;
+      m.off[j] = r.off;
+      m.key[j] = r.key;
+      neq = neq || r.key != k0;
+    }
+    if (neq) s_neq = 1;
     __syncthreads();
-
-    // While every string of the subset has the same cache (and it holds no
-    // terminator), jump over the common prefix: compare each string's next 64
-    // characters with the first string's and continue at the first window
-    // where some string differs or ends.
-    while (true) {
-      if (threadIdx.x == 0) s_neq = 0;
-      __syncthreads();
-      const uint64_t k0 = m.key[0];
-      for (uint32_t j = threadIdx.x; j < n; j += NT)
-        if (m.key[j] != k0) s_neq = 1;
-      __syncthreads();
-      if (s_neq || key_end(k0, dna) || depth + kw * kLookWindows > kMaxDepth) break;
-      if (threadIdx.x == 0) {
-        uint64_t w[kLookWindows];
-        const uint32_t nwin = load_key_windows<kLookWindows>(sd.chars, m.off[0], depth + kw, sd.cap, dna, w);
-        uint32_t js = kLookWindows - 1;
-        for (int j = kLookWindows - 1; j >= 0; --j) {
-          s_lead[j] = w[j];
-          if ((uint32_t)j >= nwin || key_end(w[j], dna)) js = (uint32_t)j;
-        }
-        s_jstop = js;
+    auto off_at = [&](uint32_t j) {  // string offset of the element at sorted position j
+      const uint32_t q = m.pos[0][j];
+      return rec_offset(sd, wide, m.idx[q], m.off[q]);
+    };
+    // one run: jump over the prefix all its strings share
+    bool sorted = s_neq || key_end(k0, dna);
+    if (s_neq) {
+      small_sort<NT>(m, split, m.key, n, nullptr, m.pos[0]);
+    } else {
+      for (uint32_t j = tid; j < n; j += NT) m.pos[0][j] = (uint16_t)j;
+      if (tid == 0 && !sorted) {
+        m.open[0] = make_uint2(n << 16, depth);
+        s_open = 1;
       }
-      __syncthreads();
-      for (uint32_t j = threadIdx.x + 1; j < n; j += NT) {
-        uint64_t w[kLookWindows];
-        const uint32_t nwin = load_key_windows<kLookWindows>(sd.chars, m.off[j], depth + kw, sd.cap, dna, w);
-        uint32_t js = kLookWindows;
-#pragma unroll
-        for (int q = kLookWindows - 1; q >= 0; --q)
-          if ((uint32_t)q >= nwin || w[q] != s_lead[q]) js = (uint32_t)q;
-        if (js < kLookWindows) atomicMin(&s_jstop, js);
-      }
-      __syncthreads();
-      const uint32_t nd = depth + kw * (s_jstop + 1);
-      for (uint32_t j = threadIdx.x; j < n; j += NT) {
-        m.key[j] = load_key(sd.chars, m.off[j], nd, sd.cap, dna);
-        bytes += 8ull * (s_jstop + 1);
-      }
-      depth = nd;
       __syncthreads();
     }
-
-    bool first_pass = true;  // every tag is make_tag(0, position, 1)
+    if (tid == 0 && next < count) next_task = task_of(next);
+    __syncwarp();
     while (true) {
-      if (first_pass) block_sort<NT, true>(m, n);
-      else block_sort<NT, false>(m, n);
-      first_pass = false;
-      if (threadIdx.x == 0) s_max_open = 0;
-      for (uint32_t j = threadIdx.x; j < n; j += NT) {
-        const uint32_t tg = m.tag[j];
-        const bool st = j == 0 || tag_seg(tg) != tag_seg(m.tag[j - 1]) || m.key[j] != m.key[j - 1];
-        if (lcp && (tg & 1u) && j > 0 && tag_seg(tg) == tag_seg(m.tag[j - 1]) && m.key[j] != m.key[j - 1])
-          lcp[j] = depth + key_lcp(m.key[j - 1], m.key[j], dna);
-        m.nseg[j] = st ? (uint16_t)j : 0;
-        m.aux[j] = 0;
-      }
-      __syncthreads();
-      block_max_scan<NT>(m.nseg, n);
-      for (uint32_t j = threadIdx.x; j < n; j += NT) atomicAdd(&m.aux[m.nseg[j]], 1u);
-      __syncthreads();
-      // Runs of one string or of equal strings are finished; runs of at most
-      // 32 strings go back to the record buffer as new warp tasks (a warp
-      // finishes them without holding this block); larger runs continue here.
-      for (uint32_t j = threadIdx.x; j < n; j += NT) {
-        const uint32_t s0 = m.nseg[j];
-        uint32_t tg = m.tag[j];
-        uint32_t open = tg & 1u, handed = tg & kHanded;
-        if (open) {
-          const uint32_t size = m.aux[s0];
-          if (size == 1) {
-            open = 0;
-          } else if (key_end(m.key[j], dna)) {
-            open = 0;
-            if (lcp && j != s0) lcp[j] = depth + key_nnz(m.key[j], dna);
-          } else if (size <= 32) {
-            open = 0;
-            handed = kHanded;
-            store_rec(c.rec[par] + t.begin + j, m.key[j], m.idx[tag_pos(tg)], (uint32_t)m.off[tag_pos(tg)]);
-            bytes += 16;
-            if (j == s0) list_push(c.small_warp, Task{t.begin + j, size, depth, t.meta}, c.status);
-          } else {
-            atomicMax(&s_max_open, size);
-          }
+      if (sorted) {
+        // LCPs between neighbours with different caches, run starts
+        const uint64_t* key = m.key;
+        const uint32_t nw = (n + 31) / 32;
+        for (uint32_t q = w; q < nw; q += NW) {
+          const uint32_t j = lo + 32 * q + lane;
+          const bool in = 32 * q + lane < n;
+          const uint64_t k = in ? key[j] : 0ull;
+          const uint64_t pk = in && j > lo ? key[j - 1] : 0ull;
+          const bool differs = in && j > lo && k != pk;
+          if (differs && lcp) lcp[j] = depth + key_lcp(pk, k, dna);
+          const uint32_t hb = __ballot_sync(kFull, differs || j == lo);
+          if (lane == 0) m.heads[q] = hb;
         }
-        m.tag[j] = handed | make_tag(s0, tag_pos(tg), open);
+        __syncthreads();
+        // Runs of one string or of equal strings are finished; runs of at most
+        // 32 strings go back to the record buffer as new warp tasks (a warp
+        // finishes them without holding this block); larger ones are sorted
+        // deeper here.
+        for (uint32_t q = w; q < nw; q += NW) {
+          const uint32_t j = lo + 32 * q + lane;
+          const bool in = 32 * q + lane < n;
+          const uint32_t own = m.heads[q];
+          uint32_t ws = q, hs = own & ((2u << lane) - 1);  // lane 31: all bits
+          while (!hs) hs = m.heads[--ws];                  // position lo starts a run
+          const uint32_t s0 = lo + 32 * ws + 31 - __clz(hs);
+          uint32_t wn = q, hn = own & ~((2u << lane) - 1);
+          while (!hn && ++wn < nw) hn = m.heads[wn];
+          const uint32_t size = (hn ? lo + 32 * wn + __ffs(hn) - 1 : lo + n) - s0;
+          const uint64_t k = in ? key[j] : 0ull;
+          const bool ended = key_end(k, dna);
+          const bool fin = in && (size == 1 || ended);
+          const bool hand = in && !fin && size <= hand_max;
+          const uint32_t src = in ? m.pos[0][j] : 0u;
+          const uint32_t id = m.idx[src];
+          if (fin) {
+            perm[j] = id;
+            if (lcp && j != s0) lcp[j] = depth + key_nnz(k, dna);
+          } else if (hand) {
+            store_rec(recs + j, k, id, m.off[src]);
+            bytes += 16;
+          }
+          if (in && !fin && j == s0) {
+            if (size <= 32) m.tmp[atomicAdd(&s_runs, 1u)] = j | size << 16;
+            else if (hand) list_push(c.small_cta, Task{t.begin + j, size, depth, t.meta}, c.status);
+            else m.open[atomicAdd(&s_open, 1u)] = make_uint2(s0 | size << 16, depth);
+          }
+          __syncwarp();
+        }
+        __syncthreads();
+        // the runs for the warp list, with one counter update for all of them:
+        // every block of the launch appends to the same counter
+        const uint32_t runs = s_runs;
+        if (runs) {
+          if (tid == 0) s_base = atomicAdd(c.small_warp.count, runs);
+          __syncthreads();
+          for (uint32_t q = tid; q < runs; q += NT) {
+            const uint32_t r = m.tmp[q], slot = s_base + q;
+            if (slot < c.small_warp.cap) c.small_warp.items[slot] = Task{t.begin + (r & 0xFFFFu), r >> 16, depth, t.meta};
+            else latch_status(c.status, kStQueueFull);
+          }
+          __syncthreads();
+          if (tid == 0) s_runs = 0;
+        }
+      }
+      sorted = true;
+      const uint32_t left = s_open;
+      if (left == 0) break;
+      // the next open range: all its caches are equal and hold no terminator;
+      // compare each string's next 64 characters with the first one's and
+      // continue at the first window where some string differs or ends
+      const uint2 r = m.open[left - 1];
+      lo = r.x & 0xFFFFu;
+      n = r.x >> 16;
+      depth = r.y;
+      const bool look = depth + kw * kLookWindows <= kMaxDepth;  // else one window only
+      __syncthreads();
+      if (tid == 0) {
+        s_open = left - 1;
+        s_jstop = look ? kLookWindows - 1 : 0u;
+      }
+      uint64_t x[kLookWindows];
+      uint32_t nwin = 0;
+      for (uint32_t j0 = 0; j0 < n; j0 += NT) {  // the same code for the leader and the others: it is
+        const uint32_t j = j0 + tid;             // run rarely, so fetching it is part of what it costs
+        if (look && j < n) nwin = load_key_windows<kLookWindows>(sd.chars, off_at(lo + j), depth + kw, sd.cap, dna, x);
+        if (j == 0) {
+#pragma unroll
+          for (int q = 0; q < kLookWindows; ++q) s_lead[q] = x[q];
+        }
+        if (j0 == 0) __syncthreads();
+        uint32_t js = kLookWindows;
+        if (look && j < n) {
+#pragma unroll
+          for (int q = kLookWindows - 1; q >= 0; --q)
+            if ((uint32_t)q >= nwin || x[q] != s_lead[q] || key_end(x[q], dna)) js = (uint32_t)q;
+        }
+        js = __reduce_min_sync(kFull, js);
+        if (lane == 0 && js < kLookWindows) atomicMin(&s_jstop, js);
       }
       __syncthreads();
-      if (s_max_open == 0) break;
-      if (depth + kw > kMaxDepth) {
-        if (threadIdx.x == 0) latch_status(c.status, kStTooDeep);
+      const uint32_t jstop = s_jstop;
+      depth += kw * (jstop + 1);
+      if (depth > kMaxDepth) {
+        if (tid == 0) latch_status(c.status, kStTooDeep);
         break;
       }
-      depth += kw;
-      for (uint32_t j = threadIdx.x; j < n; j += NT)
-        if (m.tag[j] & 1u) {
-          m.key[j] = load_key(sd.chars, m.off[tag_pos(m.tag[j])], depth, sd.cap, dna);
-          bytes += 8;
+      for (uint32_t j = tid; j < n; j += NT) {
+        if (n <= NT && jstop < nwin) {  // the windows are still at hand
+          uint64_t k = x[0];
+#pragma unroll
+          for (int q = 1; q < kLookWindows; ++q) k = (uint32_t)q == jstop ? x[q] : k;
+          m.key[lo + j] = k;
+        } else {
+          m.key[lo + j] = load_key(sd.chars, off_at(lo + j), depth, sd.cap, dna);
         }
+        bytes += 8ull * (jstop + 1);
+      }
+      __syncthreads();
+      small_sort<NT>(m, split, m.key + lo, n, m.pos[0] + lo, m.pos[1] + lo);
+      for (uint32_t j = tid; j < n; j += NT) m.pos[0][lo + j] = m.pos[1][lo + j];
       __syncthreads();
     }
-    for (uint32_t j = threadIdx.x; j < n; j += NT) {
-      const uint32_t tg = m.tag[j];
-      if (!(tg & kHanded)) sd.perm[t.begin - sd.base + j] = m.idx[tag_pos(tg)];
-      bytes += sd.lcp ? 24 : 20;  // record 16 read; perm 4 (+ lcp 4) written
-    }
+    for (uint32_t j = tid; j < t.len; j += NT) bytes += sd.lcp ? 24 : 20;  // record 16 read; perm 4 (+ lcp 4) written
     __syncthreads();
   }
   account(c, kKSmallCta, bytes);
@@ -725,7 +802,12 @@ __global__ void k_pack_dna(const uint8_t* __restrict__ chars, uint64_t len, uint
   }
 }
 
-size_t small_cta_smem(uint32_t pmax) { return (size_t)pmax * (8 + 8 + 8 + 4 + 4 + 4 + 4 + 2); }
+// Blocks per SM of the two block-sort launches.
+constexpr uint32_t kSmallNarrowBlocks = 16, kSmallWideBlocks = 4;
+
+size_t small_cta_smem(uint32_t pmax) {
+  return (size_t)pmax * (8 + 8 + 4 + 4 + 4 + 2 + 2 + 2) + (size_t)small_words(pmax) * (8 + 4);
+}
 
 cudaError_t launch_init(const SortCtx& c, cudaStream_t st, const LaunchHook& hook) {
   const uint32_t grid = max(1u, min((c.total + kBlock - 1) / kBlock, 152u * 16u));
@@ -735,34 +817,28 @@ cudaError_t launch_init(const SortCtx& c, cudaStream_t st, const LaunchHook& hoo
 }
 
 template <bool DNA>
-static cudaError_t launch_small_t(const SortCtx& c, uint32_t pmax, uint32_t grid_warp, uint32_t grid_cta,
-                                  cudaStream_t st, const LaunchHook& hook) {
+static cudaError_t launch_small_t(const SortCtx& c, uint32_t pmax, uint32_t sms, cudaStream_t st,
+                                  const LaunchHook& hook) {
   static uint32_t attr_pmax = 0;
   if (pmax > attr_pmax) {
-    cudaError_t e = cudaFuncSetAttribute(k_small_cta<kBlock, DNA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_small_cta<kSmallWideThreads, DNA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)small_cta_smem(pmax));
     if (e != cudaSuccess) return e;
     attr_pmax = pmax;
   }
-  // subsets of up to kSmallCtaNarrowMax strings: 64-thread blocks with small
-  // shared arrays, many per SM (a subset's sort is latency-bound, so more of
-  // them in flight beats more threads on each); larger ones: 256 threads
-  // (when there are enough subsets to fill the GPU with them)
-  const uint32_t min_count = 2 * grid_cta;
-  if (pmax <= kSmallCtaNarrowMax) {
+  // subsets of more than kSmallCtaNarrowMax strings, then smaller ones
+  const uint32_t min_count = 2 * sms * kSmallWideBlocks;
+  if (pmax > kSmallCtaNarrowMax)
     hook.run("small_cta", [&] {
-      k_small_cta<64, DNA><<<grid_cta * 4, 64, small_cta_smem(pmax), st>>>(c, pmax, 0u, 1u);
+      k_small_cta<kSmallWideThreads, DNA>
+          <<<sms * kSmallWideBlocks, kSmallWideThreads, small_cta_smem(pmax), st>>>(c, pmax, min_count);
     });
-  } else {
-    hook.run("small_cta", [&] {
-      k_small_cta<64, DNA><<<grid_cta * 4, 64, small_cta_smem(kSmallCtaNarrowMax), st>>>(
-          c, kSmallCtaNarrowMax, min_count, 1u);
-    });
-    hook.run("small_cta", [&] {
-      k_small_cta<kBlock, DNA><<<grid_cta, kBlock, small_cta_smem(pmax), st>>>(
-          c, pmax, min_count, 0u);
-    });
-  }
+  const uint32_t narrow_max = min(pmax, kSmallCtaNarrowMax);
+  hook.run("small_cta", [&] {
+    k_small_cta<kSmallNarrowThreads, DNA>
+        <<<sms * kSmallNarrowBlocks, kSmallNarrowThreads, small_cta_smem(narrow_max), st>>>(
+            c, narrow_max, pmax > kSmallCtaNarrowMax ? min_count : 0u);
+  });
   // the lists alternate: a pass reads one and defers into the other, emptied first
   for (uint32_t p = 0; p < kWarpPasses; ++p) {
     const TaskList in = (p & 1) ? c.small_deep : c.small_warp;
@@ -771,15 +847,14 @@ static cudaError_t launch_small_t(const SortCtx& c, uint32_t pmax, uint32_t grid
       const cudaError_t e = launch_upload(nullptr, out.count, 4, st, hook);
       if (e != cudaSuccess) return e;
     }
-    hook.run("small_warp", [&] { k_small_warp<<<grid_warp, kBlock, 0, st>>>(c, in, out, kWarpPassJumps[p]); });
+    hook.run("small_warp", [&] { k_small_warp<<<sms * 8, kBlock, 0, st>>>(c, in, out, kWarpPassJumps[p]); });
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_small(const SortCtx& c, uint32_t pmax, uint32_t grid_warp, uint32_t grid_cta,
-                         cudaStream_t st, const LaunchHook& hook) {
-  return c.dna ? launch_small_t<true>(c, pmax, grid_warp, grid_cta, st, hook)
-               : launch_small_t<false>(c, pmax, grid_warp, grid_cta, st, hook);
+cudaError_t launch_small(const SortCtx& c, uint32_t pmax, uint32_t sms, cudaStream_t st, const LaunchHook& hook) {
+  return c.dna ? launch_small_t<true>(c, pmax, sms, st, hook)
+               : launch_small_t<false>(c, pmax, sms, st, hook);
 }
 
 cudaError_t launch_pack_dna(const uint8_t* chars, uint64_t len, uint64_t* out, uint64_t words, uint32_t* bad,
