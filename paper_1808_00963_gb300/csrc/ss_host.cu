@@ -276,7 +276,8 @@ static SortCtx make_ctx(uint8_t* ws, const Layout& L, uint32_t num_sets, uint32_
   c.wid[1] = reinterpret_cast<uint2*>(ws + L.wid1);
   c.bucket_of = reinterpret_cast<uint16_t*>(ws + L.bucket_of);
   c.status = ctrl + kCStatus;
-  c.abytes = reinterpret_cast<unsigned long long*>(ctrl + kCtrlWords);
+  // counted for ss_kernel_stats only (the updates of all warps queue up at one counter)
+  c.abytes = g_profiling.load() ? reinterpret_cast<unsigned long long*>(ctrl + kCtrlWords) : nullptr;
   c.big[0] = TaskList{reinterpret_cast<Task*>(ws + L.big0), ctrl + kCBig0, L.cap_big};
   c.big[1] = TaskList{reinterpret_cast<Task*>(ws + L.big1), ctrl + kCBig1, L.cap_big};
   c.mq = WorkQueue{reinterpret_cast<Task*>(ws + L.mq_items), reinterpret_cast<uint32_t*>(ws + L.mq_ready),

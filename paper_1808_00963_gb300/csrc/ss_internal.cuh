@@ -120,7 +120,7 @@ struct SortCtx {
   uint32_t* wide;          // per set: 1 if some offset is 2^32 or more (then off is not enough)
   uint16_t* bucket_of;     // bucket index of each record (array o of Algorithm 4.1)
   uint32_t* status;
-  unsigned long long* abytes;  // [kKClasses] algorithmic bytes moved, per kernel class
+  unsigned long long* abytes;  // [kKClasses] algorithmic bytes moved, per kernel class (null: not counted)
   TaskList big[2];         // multi-block tasks, ping-pong by step
   WorkQueue mq;            // tasks for the persistent single-block kernel
   TaskList small_warp;     // 2..32 records
@@ -659,6 +659,7 @@ __device__ __forceinline__ uint32_t warp_slot(uint32_t* counter, bool pred) {
 // Adds a thread's algorithmic byte count to its kernel class (one atomic per
 // warp; every lane of the warp must call it).
 __device__ __forceinline__ void account(const SortCtx& c, uint32_t cls, unsigned long long bytes) {
+  if (!c.abytes) return;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) bytes += __shfl_xor_sync(0xFFFFFFFFu, bytes, o);
   if ((threadIdx.x & 31u) == 0 && bytes) atomicAdd(c.abytes + cls, bytes);
