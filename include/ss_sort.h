@@ -130,8 +130,8 @@ typedef struct ss_options {
  * graph per stream, built on the first such call); the rest is a fixed
  * sequence of launches.  The return value reports argument and launch errors;
  * device-side errors go to the stream's status word (ss_stream_status).
- * The first call on a stream allocates that stream's status word and loop
- * control block (4 KiB, kept until exit).  Without a caller workspace the
+ * The first call on a stream allocates that stream's status word (pinned host
+ * memory) and loop control block (device memory; both kept until exit).  Without a caller workspace the
  * workspace is stream-ordered memory, freed on `stream` after the sort.
  * The caller's buffers must stay valid until the stream has run the sort.
  * n = 0 is a no-op; n = 1 gives perm = [0], lcp = [0].  Returns

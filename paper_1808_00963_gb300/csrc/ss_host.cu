@@ -331,30 +331,7 @@ struct Pinned {
     return SS_OK;
   }
 };
-static thread_local Pinned t_down, t_up;
-
-// Small uploads and zero fills of the sort: on the copy engines, except while
-// a large copy on another stream holds them (the overlapped host path), when
-// a kernel that reads the pinned staging memory does them instead.  (A kernel
-// reading host memory costs 6-55 us per launch on the GB300 machine, more than
-// the copy engine when it is free.)
-static thread_local bool t_kernel_copies = false;
-
-static cudaError_t zero_fill(void* dst, size_t bytes, cudaStream_t st, const LaunchHook& hook) {
-  if (t_kernel_copies) return launch_upload(nullptr, dst, bytes, st, hook);
-  return cudaMemsetAsync(dst, 0, bytes, st);
-}
-
-// Writes a set descriptor into the workspace: a kernel parameter, so the host
-// neither stages it nor waits for a copy before enqueuing the sort.
-__global__ void k_set_desc(SetDesc* dst, SetDesc v) { *dst = v; }
-
-// Writes the control block of the multi-block loop (same reason), and the
-// task of the first round where the host knows it (one set: its root).
-__global__ void k_set_ctl(BigCtl* dst, BigCtl v, GenTask root) {
-  *dst = v;
-  if (v.cur.G) v.cur.gt[0] = root;
-}
+static thread_local Pinned t_down;
 
 // A batch's set descriptors, up to kDescChunk per launch (kernel parameters).
 constexpr uint32_t kDescChunk = 128;
@@ -482,19 +459,22 @@ static cudaError_t loop_exec(BigCtl* ctl, int logv, uint32_t R_max, uint32_t sms
 
 // ---- per-stream state of asynchronous sorts ---------------------------------------------
 
-// Device memory of one (device, stream): the status word the stream's sorts
-// fold their device status into, and the multi-block loop's control block.
+// One (device, stream): the status word the stream's sorts fold their device
+// status into, in pinned host memory that the kernels reach directly (reading
+// it takes no copy and second wait after the wait for the stream; with the
+// fewer launches of k_begin, 1 M URLs 698 -> 653 us), and the multi-block
+// loop's control block in device memory.
 struct StreamSlot {
-  uint32_t status;
-  uint32_t pad[63];
-  BigCtl ctl;
+  uint32_t* status = nullptr;      // host address
+  uint32_t* status_dev = nullptr;  // the same word for kernels
+  BigCtl* ctl = nullptr;
 };
 
 static std::mutex g_slot_mu;
-static std::map<std::pair<int, void*>, StreamSlot*> g_slots;
+static std::map<std::pair<int, void*>, StreamSlot> g_slots;
 
-static ss_status stream_slot(cudaStream_t st, bool create, StreamSlot** out) {
-  *out = nullptr;
+static ss_status stream_slot(cudaStream_t st, bool create, StreamSlot* out) {
+  *out = StreamSlot();
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return SS_ERR_NO_DEVICE;
   std::lock_guard<std::mutex> lk(g_slot_mu);
@@ -505,10 +485,18 @@ static ss_status stream_slot(cudaStream_t st, bool create, StreamSlot** out) {
     return SS_OK;
   }
   if (!create) return SS_OK;
-  StreamSlot* p = nullptr;
-  if (cudaMalloc(reinterpret_cast<void**>(&p), sizeof(StreamSlot)) != cudaSuccess) return SS_ERR_OOM;
-  if (cudaMemsetAsync(p, 0, sizeof(StreamSlot), st) != cudaSuccess) {  // ordered before the stream's first use
-    cudaFree(p);
+  StreamSlot p;
+  constexpr size_t kStatusBytes = 64;
+  if (cudaMalloc(reinterpret_cast<void**>(&p.ctl), sizeof(BigCtl)) != cudaSuccess) return SS_ERR_OOM;
+  if (cudaHostAlloc(reinterpret_cast<void**>(&p.status), kStatusBytes, cudaHostAllocMapped | cudaHostAllocPortable) !=
+      cudaSuccess) {
+    cudaFree(p.ctl);
+    return SS_ERR_OOM;
+  }
+  *p.status = 0;
+  if (cudaHostGetDevicePointer(reinterpret_cast<void**>(&p.status_dev), p.status, 0) != cudaSuccess) {
+    cudaFreeHost(p.status);
+    cudaFree(p.ctl);
     return SS_ERR_CUDA;
   }
   g_slots[key] = p;
@@ -516,18 +504,28 @@ static ss_status stream_slot(cudaStream_t st, bool create, StreamSlot** out) {
   return SS_OK;
 }
 
-// Enqueues everything after the set descriptors are in place.  ctl: where the
-// multi-block loop's control block lives (needed when big).
+// Enqueues a sort.  sd: the descriptor of its only set (null: a batch, whose
+// descriptors are in place already).  ctl: where the multi-block loop's control
+// block lives (needed when big).
 static ss_status run_sort(uint8_t* ws, const Layout& L, SortCtx c, const Opts& o, const DevInfo& dev,
-                          bool big, cudaStream_t st, BigCtl* ctl = nullptr) {
+                          bool big, cudaStream_t st, const SetDesc* sd, BigCtl* ctl = nullptr) {
   const LaunchHook hook{st};
-  SS_CUDA(zero_fill(ws + L.ctrl, kCtrlBytes, st, hook));
-  SS_CUDA(zero_fill(ws + L.mq_ready, (size_t)L.cap_mq * 4, st, hook));
-  SS_CUDA(zero_fill(ws + L.wide, (size_t)c.num_sets * 4, st, hook));
-  SS_CUDA(launch_init(c, st, hook));
+  BeginArgs a{};
+  a.ctrl = reinterpret_cast<uint32_t*>(ws + L.ctrl);
+  a.ctrl_words = (uint32_t)(kCtrlBytes / 4);
+  a.ready = reinterpret_cast<uint32_t*>(ws + L.mq_ready);
+  const bool queue = c.total > o.cutoff;  // else no subset can need the work queue
+  a.ready_words = queue ? L.cap_mq : 0u;
+  a.wide = c.wide;
+  a.num_sets = c.num_sets;
+  if (sd) {
+    a.set = reinterpret_cast<SetDesc*>(ws + L.sets);
+    a.sd = *sd;
+  }
   if (big) {
     if (!ctl) return SS_ERR_INVALID;
-    BigCtl v{};
+    a.ctl = ctl;
+    BigCtl& v = a.v;
     v.c = c;
     v.gtbuf[0] = reinterpret_cast<GenTask*>(ws + L.gen);
     v.gtbuf[1] = v.gtbuf[0] + L.cap_big;
@@ -541,20 +539,21 @@ static ss_status run_sort(uint8_t* ws, const Layout& L, SortCtx c, const Opts& o
     v.R_fixed = o.R;
     v.sms = (uint32_t)dev.sms;
     v.K = (2u << o.logv_big) - 1;
-    GenTask root{};
     if (c.num_sets == 1) {  // the first round's plan: one subset, the whole set
       const uint32_t R = tile_rounds(c.total, 1, v.sms, v.K, v.ncounters_max, o.R);
-      root.t = Task{0, c.total, 0, make_meta(0, 0)};
-      root.tiles = (c.total + kBlock * R - 1) / (kBlock * R);
+      a.root.t = Task{0, c.total, 0, make_meta(0, 0)};
+      a.root.tiles = (c.total + kBlock * R - 1) / (kBlock * R);
       v.cur.gt = v.gtbuf[0];
       v.cur.G = 1;
-      v.cur.tiles = root.tiles;
+      v.cur.tiles = a.root.tiles;
       v.cur.R = R;
-      v.cur.ncounters = (uint64_t)v.K * root.tiles;
+      v.cur.ncounters = (uint64_t)v.K * a.root.tiles;
       v.round = 1;
     }
-    hook.run("init", [&] { k_set_ctl<<<1, 1, 0, st>>>(ctl, v, root); });
-    SS_CUDA(cudaGetLastError());
+  }
+  SS_CUDA(launch_begin(a, st, hook));
+  SS_CUDA(launch_init(c, st, hook));
+  if (big) {
     if (c.num_sets > 1) SS_CUDA(launch_big_plan(ctl, st, hook));
     const uint32_t R_max = o.R ? o.R : kMaxTileRounds;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -578,10 +577,10 @@ static ss_status run_sort(uint8_t* ws, const Layout& L, SortCtx c, const Opts& o
       SS_CUDA(cudaGraphLaunch(exec, st));
     }
   }
-  const uint32_t qgrid = (uint32_t)(dev.sms * dev.queue_blocks[o.logv]);
-  SS_CUDA(launch_queue(o.logv, c, qgrid, st, hook));
+  if (queue) SS_CUDA(launch_queue(o.logv, c, (uint32_t)(dev.sms * dev.queue_blocks[o.logv]), st, hook));
   SS_CUDA(launch_small(c, pmax_of(o.cutoff), (uint32_t)dev.sms, st, hook));
-  const uint32_t fgrid = std::max(1u, std::min<uint32_t>((c.total + kBlock - 1) / kBlock, (uint32_t)dev.sms * 16));
+  // (without multi-block steps there are no marks to resolve)
+  const uint32_t fgrid = std::max(1u, std::min<uint32_t>((c.total + kBlock - 1) / kBlock, (uint32_t)dev.sms * (big ? 16 : 1)));
   SS_CUDA(launch_lcp_fix(c, fgrid, st, hook));
   return SS_OK;
 }
@@ -622,19 +621,16 @@ static ss_status sort_device(const uint8_t* chars, const uint64_t* offsets, uint
     if (cudaMallocAsync(reinterpret_cast<void**>(&ws), L.total, st) != cudaSuccess) return SS_ERR_OOM;
     owned = true;
   }
-  StreamSlot* slot = nullptr;
+  StreamSlot slot;
   if ((s = stream_slot(st, true, &slot)) != SS_OK) {
     if (owned) cudaFreeAsync(ws, st);
     return s;
   }
   SetDesc sd{chars, offsets, perm, lcp, (uint32_t)n, o.cap, 0, dna};
-  ss_status r = SS_OK;
-  LaunchHook{st}.run("init", [&] { k_set_desc<<<1, 1, 0, st>>>(reinterpret_cast<SetDesc*>(ws + L.sets), sd); });
-  if (cudaGetLastError() != cudaSuccess) r = SS_ERR_CUDA;
   SortCtx ctx = make_ctx(ws, L, 1, (uint32_t)n, o, big);
   ctx.dna = dna;
-  ctx.fold_status = &slot->status;  // the device status goes to the stream's status word
-  if (r == SS_OK) r = run_sort(ws, L, ctx, o, dev, big, st, &slot->ctl);
+  ctx.fold_status = slot.status_dev;  // the device status goes to the stream's status word
+  const ss_status r = run_sort(ws, L, ctx, o, dev, big, st, &sd, slot.ctl);
   if (g_profiling.load()) read_status(ws, L, st);  // waits: per-kernel times and bytes
   if (owned) cudaFreeAsync(ws, st);
   return r;
@@ -643,20 +639,14 @@ static ss_status sort_device(const uint8_t* chars, const uint64_t* offsets, uint
 // Waits for the stream and returns the device status its sorts have left in
 // its status word since it was last read (clearing it).
 static ss_status take_stream_status(cudaStream_t st) {
-  StreamSlot* slot = nullptr;
+  StreamSlot slot;
   stream_slot(st, false, &slot);
   if (cudaStreamSynchronize(st) != cudaSuccess) return SS_ERR_CUDA;
   collect_profile();
-  if (!slot) return SS_OK;
-  if (t_down.reserve(64) != SS_OK) return SS_ERR_OOM;
-  uint32_t* h = static_cast<uint32_t*>(t_down.p);
-  SS_CUDA(cudaMemcpyAsync(h, &slot->status, 4, cudaMemcpyDeviceToHost, st));
-  SS_CUDA(cudaStreamSynchronize(st));
-  const uint32_t v = *h;
-  if (v) {
-    SS_CUDA(cudaMemsetAsync(&slot->status, 0, 4, st));
-    SS_CUDA(cudaStreamSynchronize(st));
-  }
+  if (!slot.status) return SS_OK;
+  volatile uint32_t* word = slot.status;
+  const uint32_t v = *word;
+  if (v) *word = 0;
   return map_status(v);
 }
 
@@ -1181,16 +1171,11 @@ static ss_status sort_host_parts(const uint8_t* chars, uint64_t chars_len, const
   CopyLane* lane = nullptr;
   ss_status s = copy_lane(lane);
   if (s != SS_OK) return s;
-  // whatever happens below, no copy is still writing the buffers on return,
-  // and the sort's small uploads are back on the copy engines
+  // whatever happens below, no copy is still writing the buffers on return
   struct Drain {
     cudaStream_t cs;
-    ~Drain() {
-      cudaStreamSynchronize(cs);
-      t_kernel_copies = false;
-    }
+    ~Drain() { cudaStreamSynchronize(cs); }
   } drain{lane->cs};
-  t_kernel_copies = true;
   const LaunchHook hook{st};
   const uint32_t sms = (uint32_t)dev.sms;
   const size_t recb = align256(n * sizeof(MergeRec));
@@ -1398,13 +1383,13 @@ ss_status ss_batch_run(ss_batch* b, void* stream) {
     if (cs == cudaStreamCaptureStatusActive) {
       ctl = reinterpret_cast<BigCtl*>(b->ws + b->L.bigctl);
     } else {
-      StreamSlot* slot = nullptr;
+      StreamSlot slot;
       ss_status s = stream_slot(st, true, &slot);
       if (s != SS_OK) return s;
-      ctl = &slot->ctl;
+      ctl = slot.ctl;
     }
   }
-  return run_sort(b->ws, b->L, c, b->o, b->dev, b->big, st, ctl);
+  return run_sort(b->ws, b->L, c, b->o, b->dev, b->big, st, nullptr, ctl);
 }
 
 ss_status ss_batch_status(ss_batch* b, void* stream) {
@@ -1507,12 +1492,9 @@ extern "C" ss_status ss_sort_noalloc(const uint8_t* chars, const uint64_t* offse
   if ((s = noalloc_scratch(&ws)) != SS_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const SetDesc sd{chars, offsets, out_perm, out_lcp, (uint32_t)n, o.cap, 0, 0};
-  const LaunchHook hook{st};
-  hook.run("init", [&] { k_set_desc<<<1, 1, 0, st>>>(reinterpret_cast<SetDesc*>(ws + L.sets), sd); });
-  if (cudaGetLastError() != cudaSuccess) return SS_ERR_CUDA;
   // run_sort clears the control words and the queue flags, the only scratch
   // that must start at zero; everything else is written before it is read.
-  s = run_sort(ws, L, make_ctx(ws, L, 1, (uint32_t)n, o, false), o, dev, false, st);
+  s = run_sort(ws, L, make_ctx(ws, L, 1, (uint32_t)n, o, false), o, dev, false, st, &sd);
   if (s != SS_OK) return s;
   uint32_t status = 0;
   if (cudaMemcpyAsync(&status, ws + L.ctrl, sizeof(status), cudaMemcpyDeviceToHost, st) != cudaSuccess ||

@@ -104,7 +104,19 @@ cudaError_t queue_occupancy(int logv, int* blocks_per_sm);
 cudaError_t launch_queue(int logv, const SortCtx& c, uint32_t grid, cudaStream_t st, const LaunchHook& hook);
 
 // Small subsets, set-up and LCP fix-up.
+struct BeginArgs {
+  uint32_t* ctrl;
+  uint32_t* ready;
+  uint32_t* wide;
+  uint32_t ctrl_words, ready_words, num_sets;
+  SetDesc* set;   // where the set descriptor goes, or null
+  SetDesc sd;
+  BigCtl* ctl;    // where the multi-block loop's control block goes, or null
+  BigCtl v;
+  GenTask root;   // the first round's task, where the host knows it (v.cur.G)
+};
 size_t small_cta_smem(uint32_t pmax);
+cudaError_t launch_begin(const BeginArgs& a, cudaStream_t st, const LaunchHook& hook);
 cudaError_t launch_init(const SortCtx& c, cudaStream_t st, const LaunchHook& hook);
 cudaError_t launch_small(const SortCtx& c, uint32_t pmax, uint32_t sms, cudaStream_t st, const LaunchHook& hook);
 cudaError_t launch_lcp_fix(const SortCtx& c, uint32_t grid, cudaStream_t st, const LaunchHook& hook);
