@@ -20,7 +20,7 @@ LIB_PATH = os.path.join(_BUILD, "libss_sort.so")
 ROOT = os.path.dirname(_HERE)
 HEADER = os.path.join(ROOT, "include", "ss_sort.h")
 
-SOURCES = ["ss_host.cu", "ss_big.cu", "ss_queue.cu", "ss_small.cu", "ss_merge.cu", "ss_sa.cu"]
+SOURCES = ["ss_host.cu", "ss_big.cu", "ss_queue.cu", "ss_small.cu", "ss_rank.cu", "ss_merge.cu", "ss_sa.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
                      "-Xcompiler", "-Wall"]

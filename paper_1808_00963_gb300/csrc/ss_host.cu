@@ -157,6 +157,7 @@ struct Opts {
   uint32_t big_thr = SS_TUNED_BIG_THRESHOLD;
   uint32_t seed = 0x5EED;
   uint32_t classifier = 0;
+  bool plain_steps = true;  // no option selects or sizes the distribution steps
   uint32_t host_parts = 0;  // ss_sort_host: 0 = automatic
   uint64_t wait_ns = kDefaultWaitNs;
 };
@@ -190,6 +191,8 @@ static ss_status resolve_opts(const ss_options* o, Opts& r) {
   if (o->seed) r.seed = o->seed;
   if (o->classifier > 3) return SS_ERR_INVALID;
   r.classifier = o->classifier;
+  r.plain_steps = !(o->splitters_log2 || o->big_splitters_log2 || o->tile_rounds || o->small_cutoff ||
+                    o->big_threshold || o->classifier);
   if (o->workspace && ((uintptr_t)o->workspace & 255)) return SS_ERR_INVALID;
   if (o->wait_limit_us) r.wait_ns = (uint64_t)o->wait_limit_us * 1000;
   return SS_OK;
@@ -207,16 +210,20 @@ constexpr uint32_t kCtrlWords = 64;                          // status and list 
 constexpr size_t kCtrlBytes = kCtrlWords * 4 + kKClasses * 8;  // + algorithmic byte counters
 enum Ctrl : uint32_t { kCStatus = 0, kCBig0 = 1, kCBig1 = 2, kCHead = 3, kCTail = 4, kCPending = 5,
                        kCSmallW = 6, kCSmallC = 7, kCSmallD = 8, kCMarks = 9, kCSmallCW = 10,
-                       kCClaim = 11 /* and 12 */ };
+                       kCClaim = 11 /* and 12 */, kCDone = 13 };
 
 struct Layout {
   size_t ctrl, sets, wide, rec0, rec1, wid0, wid1, bucket_of, big0, big1, gen, spl, counters, partials, gstart,
-      gdesc, bigctl, marks, mq_items, mq_ready, sw_items, sc_items, scw_items, total;
+      gdesc, bigctl, marks, mq_items, mq_ready, sw_items, sc_items, scw_items, rank_keys, rank, total;
   uint32_t cap_big, cap_mq, cap_sw, cap_sc, cap_scw;
   uint64_t ncounters_max;
 };
 
-static Layout make_layout(uint64_t M, uint32_t num_sets, const Opts& o, bool big) {
+// Plain sorts of this many strings are ranked by counting, unless an option
+// asks for particular distribution steps.
+static bool by_rank(uint64_t n, const Opts& o) { return o.plain_steps && n >= kRankMin && n <= kRankMax; }
+
+static Layout make_layout(uint64_t M, uint32_t num_sets, const Opts& o, bool big, bool rank = false) {
   Layout L{};
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t at = off; off += align256(bytes); return at; };
@@ -259,6 +266,8 @@ static Layout make_layout(uint64_t M, uint32_t num_sets, const Opts& o, bool big
   L.sw_items = take(2 * (size_t)L.cap_sw * sizeof(Task));
   L.sc_items = take((size_t)L.cap_sc * sizeof(Task));
   L.scw_items = take((size_t)L.cap_scw * sizeof(Task));
+  L.rank_keys = take(rank ? M * 2 * sizeof(ulonglong2) : 0);
+  L.rank = take(rank ? M * 4 : 0);
   L.total = off;
   return L;
 }
@@ -287,6 +296,7 @@ static SortCtx make_ctx(uint8_t* ws, const Layout& L, uint32_t num_sets, uint32_
   c.small_cta = TaskList{reinterpret_cast<Task*>(ws + L.sc_items), ctrl + kCSmallC, L.cap_sc};
   c.small_cta_wide = TaskList{reinterpret_cast<Task*>(ws + L.scw_items), ctrl + kCSmallCW, L.cap_scw};
   c.small_claim = ctrl + kCClaim;
+  c.done = ctrl + kCDone;
   c.marks = reinterpret_cast<uint32_t*>(ws + L.marks);
   c.marks_count = ctrl + kCMarks;
   c.marks_cap = big ? total : 0u;
@@ -551,8 +561,15 @@ static ss_status run_sort(uint8_t* ws, const Layout& L, SortCtx c, const Opts& o
       v.round = 1;
     }
   }
-  SS_CUDA(launch_begin(a, st, hook));
-  SS_CUDA(launch_init(c, st, hook));
+  // (a set sorted by counting is small enough to end in the warp sorts)
+  const bool rank = sd && !big && by_rank(c.total, o);
+  if (rank) {
+    const RankArgs r{reinterpret_cast<ulonglong2*>(ws + L.rank_keys), reinterpret_cast<uint32_t*>(ws + L.rank)};
+    SS_CUDA(launch_rank(a, r, c, st, hook));
+  } else {
+    SS_CUDA(launch_begin(a, st, hook));
+    SS_CUDA(launch_init(c, st, hook));
+  }
   if (big) {
     if (c.num_sets > 1) SS_CUDA(launch_big_plan(ctl, st, hook));
     const uint32_t R_max = o.R ? o.R : kMaxTileRounds;
@@ -578,7 +595,8 @@ static ss_status run_sort(uint8_t* ws, const Layout& L, SortCtx c, const Opts& o
     }
   }
   if (queue) SS_CUDA(launch_queue(o.logv, c, (uint32_t)(dev.sms * dev.queue_blocks[o.logv]), st, hook));
-  SS_CUDA(launch_small(c, pmax_of(o.cutoff), (uint32_t)dev.sms, st, hook));
+  SS_CUDA(launch_small(c, pmax_of(o.cutoff), (uint32_t)dev.sms, rank, st, hook));
+  if (rank) return SS_OK;
   // (without multi-block steps there are no marks to resolve)
   const uint32_t fgrid = std::max(1u, std::min<uint32_t>((c.total + kBlock - 1) / kBlock, (uint32_t)dev.sms * (big ? 16 : 1)));
   SS_CUDA(launch_lcp_fix(c, fgrid, st, hook));
@@ -611,7 +629,7 @@ static ss_status sort_device(const uint8_t* chars, const uint64_t* offsets, uint
   DevInfo dev;
   if ((s = device_info(dev)) != SS_OK) return s;
   const bool big = n > o.big_thr;
-  const Layout L = make_layout(n, 1, o, big);
+  const Layout L = make_layout(n, 1, o, big, by_rank(n, o));
   uint8_t* ws = nullptr;
   bool owned = false;
   if (opt && opt->workspace) {
@@ -939,8 +957,10 @@ ss_status ss_suffix_array(const uint8_t* text, uint64_t n, uint32_t* out_sa, uin
   if (ok) {
     ss_options o{};
     o.max_len = h0;
-    o.small_cutoff = kSaSmallCutoff;
-    o.big_threshold = kSaBigThreshold;
+    if (n > kRankMax) {
+      o.small_cutoff = kSaSmallCutoff;
+      o.big_threshold = kSaBigThreshold;
+    }
     s = sort_device(text, off, n, out_sa, lcp0, &o, st);
     ok = s == SS_OK;
   }
@@ -971,8 +991,10 @@ ss_status ss_suffix_array(const uint8_t* text, uint64_t n, uint32_t* out_sa, uin
     ok = sa_launch(SaKernel::kEncode, r, grid_for(M), st, hook) == cudaSuccess;
     if (ok) {
       ss_options o2{};
-      o2.small_cutoff = kSaSmallCutoff;
-      o2.big_threshold = kSaBigThreshold;
+      if (M > kRankMax) {  // (smaller sets are ranked by counting)
+        o2.small_cutoff = kSaSmallCutoff;
+        o2.big_threshold = kSaBigThreshold;
+      }
       s = sort_device(enc, eoff, M, perm2, lcp2, &o2, st);
       ok = s == SS_OK;
     }
@@ -1026,7 +1048,7 @@ ss_status ss_suffix_array(const uint8_t* text, uint64_t n, uint32_t* out_sa, uin
 size_t ss_workspace_size(uint64_t n, const ss_options* opt) {
   Opts o;
   if (resolve_opts(opt, o) != SS_OK || n >= 0xFFFFFFFFull) return 0;
-  return make_layout(n, 1, o, n > o.big_thr).total;
+  return make_layout(n, 1, o, n > o.big_thr, by_rank(n, o)).total;
 }
 
 ss_status ss_sort_ex(const uint8_t* chars, const uint64_t* offsets, uint64_t n, uint32_t* out_perm,
@@ -1483,7 +1505,7 @@ extern "C" ss_status ss_sort_noalloc(const uint8_t* chars, const uint64_t* offse
   if (g_profiling.load()) return SS_ERR_INVALID;  // profiling would create CUDA events
   Opts o;
   if (max_len) o.cap = max_len;
-  const Layout L = make_layout(n, 1, o, false);
+  const Layout L = make_layout(n, 1, o, false, by_rank(n, o));
   if (L.total > SS_NOALLOC_SCRATCH_BYTES) return SS_ERR_TOO_LARGE;
   DevInfo dev;
   ss_status s = device_info(dev);

@@ -139,6 +139,7 @@ struct SortCtx {
   uint32_t big_cur;        // which big[] list the current step reads
   uint32_t dna;            // every set holds 3-bit character codes (SetDesc::dna)
   uint64_t wait_ns;        // bound on every device-side wait (then kStTimeout)
+  uint32_t* done;          // blocks of the sort's last kernel that have finished
   uint32_t* fold_status;   // if set: the last kernel ORs *status into it (the stream's status word)
 };
 
@@ -441,6 +442,35 @@ __device__ __forceinline__ uint32_t load_key_windows(const uint8_t* chars, uint6
     ended = ended || key_end(w[j], 1);
   }
   return KW;
+}
+
+// The key at depth h, out of line: for windows past the 4 KiB block of a
+// look-ahead, which are rare.
+static __device__ __noinline__ uint64_t load_key_far(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap,
+                                              uint32_t dna) {
+  return load_key(chars, off, h, cap, dna);
+}
+
+// load_key_windows with every window determined: those past the 4 KiB block of
+// the first character (1 string in 64 has some) are read one by one while the
+// string continues.  A group of strings that looks ahead together would
+// otherwise stop at the first block edge any of them meets: 1000 strings
+// sharing 200 characters took 17 look-aheads instead of 4 (352 -> 107 us).  The
+// warp sorts, whose groups are small, do without (their code grew by more than
+// they gained: 4 M DNA suffixes 348 -> 379 us).
+template <int KW>
+__device__ __forceinline__ void load_all_windows(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap,
+                                                 uint32_t dna, uint64_t (&w)[KW]) {
+  const uint32_t n = load_key_windows<KW>(chars, off, h, cap, dna, w);
+  bool more = n < (uint32_t)KW;
+  if (more) {
+#pragma unroll
+    for (int j = 0; j < KW; ++j)
+      if (more && (uint32_t)j >= n) {
+        w[j] = load_key_far(chars, off, h + key_width(dna) * (uint32_t)j, cap, dna);
+        more = !key_end(w[j], dna);
+      }
+  }
 }
 
 // ---------------------------------------------------------------------------

@@ -115,10 +115,22 @@ struct BeginArgs {
   BigCtl v;
   GenTask root;   // the first round's task, where the host knows it (v.cur.G)
 };
+// Sets of kRankMin..kRankMax strings are ranked by counting (ss_rank.cu).
+constexpr uint32_t kRankMin = 33, kRankMax = 4096;
+struct RankArgs {
+  ulonglong2* keys;   // [n][2]: the first 4 keys of each string
+  uint32_t* rank;     // [n]
+};
+cudaError_t launch_rank(const BeginArgs& a, const RankArgs& r, const SortCtx& c, cudaStream_t st,
+                        const LaunchHook& hook);
+
 size_t small_cta_smem(uint32_t pmax);
 cudaError_t launch_begin(const BeginArgs& a, cudaStream_t st, const LaunchHook& hook);
 cudaError_t launch_init(const SortCtx& c, cudaStream_t st, const LaunchHook& hook);
-cudaError_t launch_small(const SortCtx& c, uint32_t pmax, uint32_t sms, cudaStream_t st, const LaunchHook& hook);
+// With `last`, the warp sorts are the sort's last kernel and do what
+// launch_lcp_fix does otherwise (there are no marks to resolve then).
+cudaError_t launch_small(const SortCtx& c, uint32_t pmax, uint32_t sms, bool last, cudaStream_t st,
+                         const LaunchHook& hook);
 cudaError_t launch_lcp_fix(const SortCtx& c, uint32_t grid, cudaStream_t st, const LaunchHook& hook);
 // Packs bytes over {A, C, G, T, 0} into 3-bit codes (dna_key's layout).
 // Copies bytes (a multiple of 4, 4-byte aligned) from pinned host memory

@@ -78,6 +78,23 @@ __global__ void __launch_bounds__(kBlock) k_init(SortCtx c) {
   account(c, kKInit, bytes);
 }
 
+// What the last kernel of a sort does about its status: it goes into the
+// stream's status word, and if a device-side error stopped the sort part way,
+// positions it did not reach hold whatever the output buffers held, so every
+// set gets the identity permutation and zero LCPs instead and no later kernel
+// (this one, or a caller's) follows an index that is out of range.  Called by
+// `stride` threads numbered by `thread`; returns whether there was an error.
+__device__ __forceinline__ bool end_sort(const SortCtx& c, uint32_t status, uint32_t thread, uint32_t stride) {
+  if (!status) return false;
+  if (c.fold_status && thread == 0) atomicOr_system(c.fold_status, status);
+  for (uint32_t r = thread; r < c.total; r += stride) {
+    const SetDesc sd = c.sets[c.num_sets == 1 ? 0 : find_set(c, r)];
+    sd.perm[r - sd.base] = r - sd.base;
+    if (sd.lcp) sd.lcp[r - sd.base] = 0;
+  }
+  return true;
+}
+
 // ---- warp-level refinement ----------------------------------------------------
 
 constexpr uint32_t kFull = 0xFFFFFFFFu;
@@ -251,6 +268,8 @@ static_assert(kWarpPassJumps[kWarpPasses - 1] == 0, "the last pass finishes ever
 // One pass over a list of warp tasks.  With max_jumps > 0, runs with long
 // common prefixes are deferred to the list `out`: their records go back to
 // the record buffer at their current positions, and each run becomes a task.
+// Last: this is the sort's last kernel.
+template <bool Last>
 __global__ void __launch_bounds__(kBlock) k_small_warp(SortCtx c, TaskList list, TaskList out, uint32_t max_jumps) {
   const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -300,6 +319,14 @@ __global__ void __launch_bounds__(kBlock) k_small_warp(SortCtx c, TaskList list,
     });
   }
   account(c, kKSmallWarp, bytes);
+  if constexpr (Last) {  // the last block ends the sort
+    __shared__ uint32_t s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(c.done, 1u) == gridDim.x - 1 ? 1u : 0u;
+    __syncthreads();
+    if (s_last) end_sort(c, __ldcg(c.status), threadIdx.x, kBlock);
+  }
 }
 
 // ---- block-level refinement -------------------------------------------------------
@@ -667,10 +694,10 @@ __global__ void __launch_bounds__(NT) k_small_cta(SortCtx c, uint32_t pmax, uint
         s_jstop = look ? kLookWindows - 1 : 0u;
       }
       uint64_t x[kLookWindows];
-      uint32_t nwin = 0;
       for (uint32_t j0 = 0; j0 < n; j0 += NT) {  // the same code for the leader and the others: it is
         const uint32_t j = j0 + tid;             // run rarely, so fetching it is part of what it costs
-        if (look && j < n) nwin = load_key_windows<kLookWindows>(sd.chars, off_at(lo + j), depth + kw, sd.cap, dna, x);
+        if (look && j < n) load_all_windows<kLookWindows>(sd.chars, off_at(lo + j), depth + kw, sd.cap, dna, x);
+        __syncwarp();
         if (j == 0) {
 #pragma unroll
           for (int q = 0; q < kLookWindows; ++q) s_lead[q] = x[q];
@@ -680,7 +707,7 @@ __global__ void __launch_bounds__(NT) k_small_cta(SortCtx c, uint32_t pmax, uint
         if (look && j < n) {
 #pragma unroll
           for (int q = kLookWindows - 1; q >= 0; --q)
-            if ((uint32_t)q >= nwin || x[q] != s_lead[q] || key_end(x[q], dna)) js = (uint32_t)q;
+            if (x[q] != s_lead[q] || key_end(x[q], dna)) js = (uint32_t)q;
         }
         js = __reduce_min_sync(kFull, js);
         if (lane == 0 && js < kLookWindows) atomicMin(&s_jstop, js);
@@ -693,7 +720,7 @@ __global__ void __launch_bounds__(NT) k_small_cta(SortCtx c, uint32_t pmax, uint
         break;
       }
       for (uint32_t j = tid; j < n; j += NT) {
-        if (n <= NT && jstop < nwin) {  // the windows are still at hand
+        if (n <= NT && look) {  // the windows are still at hand
           uint64_t k = x[0];
 #pragma unroll
           for (int q = 1; q < kLookWindows; ++q) k = (uint32_t)q == jstop ? x[q] : k;
@@ -721,22 +748,8 @@ __global__ void __launch_bounds__(NT) k_small_cta(SortCtx c, uint32_t pmax, uint
 __global__ void __launch_bounds__(kBlock) k_lcp_fix(SortCtx c) {
   const uint32_t stride = gridDim.x * blockDim.x;
   unsigned long long bytes = 0;
-  // the last kernel of a sort: every other one has finished, so the sort's
-  // status is final and goes into the stream's status word
-  const uint32_t status = *c.status;
-  if (c.fold_status && blockIdx.x == 0 && threadIdx.x == 0 && status) atomicOr_system(c.fold_status, status);
-  if (status) {
-    // a device-side error stopped the sort part way: positions it did not
-    // reach hold whatever the output buffers held.  Give every set the
-    // identity permutation and zero LCPs instead, so that no later kernel
-    // (this one, or a caller's) follows an index that is out of range.
-    for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < c.total; r += stride) {
-      const SetDesc sd = c.sets[c.num_sets == 1 ? 0 : find_set(c, r)];
-      sd.perm[r - sd.base] = r - sd.base;
-      if (sd.lcp) sd.lcp[r - sd.base] = 0;
-    }
-    return;
-  }
+  // every other kernel of the sort has finished, so its status is final
+  if (end_sort(c, *c.status, blockIdx.x * blockDim.x + threadIdx.x, stride)) return;
   const uint32_t nm = min(*c.marks_count, c.marks_cap);
   for (uint32_t m = blockIdx.x * blockDim.x + threadIdx.x; m < nm; m += stride) {
     const uint32_t r = c.marks[m];
@@ -840,7 +853,7 @@ cudaError_t launch_init(const SortCtx& c, cudaStream_t st, const LaunchHook& hoo
 }
 
 template <bool DNA>
-static cudaError_t launch_small_t(const SortCtx& c, uint32_t pmax, uint32_t sms, cudaStream_t st,
+static cudaError_t launch_small_t(const SortCtx& c, uint32_t pmax, uint32_t sms, bool last, cudaStream_t st,
                                   const LaunchHook& hook) {
   static uint32_t attr_pmax = 0;
   if (pmax > attr_pmax) {
@@ -864,6 +877,11 @@ static cudaError_t launch_small_t(const SortCtx& c, uint32_t pmax, uint32_t sms,
         <<<sms * kSmallNarrowBlocks, kSmallNarrowThreads, small_cta_smem(narrow_max), st>>>(
             c, narrow_max, pmax > kSmallCtaNarrowMax ? min_count : 0u);
   });
+  const uint32_t grid = max(1u, min(sms * 8, (c.total / 2 + kWarps - 1) / kWarps));  // tasks hold at least 2 strings
+  if (last) {  // few strings: one pass, there is nothing to gain from packing deferred runs
+    hook.run("small_warp", [&] { k_small_warp<true><<<grid, kBlock, 0, st>>>(c, c.small_warp, c.small_deep, 0u); });
+    return cudaGetLastError();
+  }
   // the lists alternate: a pass reads one and defers into the other, emptied first
   for (uint32_t p = 0; p < kWarpPasses; ++p) {
     const TaskList in = (p & 1) ? c.small_deep : c.small_warp;
@@ -872,15 +890,15 @@ static cudaError_t launch_small_t(const SortCtx& c, uint32_t pmax, uint32_t sms,
       const cudaError_t e = launch_upload(nullptr, out.count, 4, st, hook);
       if (e != cudaSuccess) return e;
     }
-    const uint32_t grid = max(1u, min(sms * 8, (c.total / 2 + kWarps - 1) / kWarps));  // tasks hold at least 2 strings
-    hook.run("small_warp", [&] { k_small_warp<<<grid, kBlock, 0, st>>>(c, in, out, kWarpPassJumps[p]); });
+    hook.run("small_warp", [&] { k_small_warp<false><<<grid, kBlock, 0, st>>>(c, in, out, kWarpPassJumps[p]); });
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_small(const SortCtx& c, uint32_t pmax, uint32_t sms, cudaStream_t st, const LaunchHook& hook) {
-  return c.dna ? launch_small_t<true>(c, pmax, sms, st, hook)
-               : launch_small_t<false>(c, pmax, sms, st, hook);
+cudaError_t launch_small(const SortCtx& c, uint32_t pmax, uint32_t sms, bool last, cudaStream_t st,
+                         const LaunchHook& hook) {
+  return c.dna ? launch_small_t<true>(c, pmax, sms, last, st, hook)
+               : launch_small_t<false>(c, pmax, sms, last, st, hook);
 }
 
 cudaError_t launch_pack_dna(const uint8_t* chars, uint64_t len, uint64_t* out, uint64_t words, uint32_t* bad,
