@@ -47,6 +47,8 @@ struct QueueSmem {
     uint32_t cntw[kQueueWarps * Geo<LOGV>::KP];
   } u;
   uint16_t tb[kMaxTile];           // bucket of each record of a tile
+  u128 lead[kLookWindows / 2];     // look-ahead of a subset's first string
+  uint32_t jstop;
   Task task;
   uint32_t got;
 };
@@ -103,7 +105,76 @@ __device__ void block_excl_scan_smem(const uint32_t* in, uint32_t* out, uint32_t
   __syncthreads();
 }
 
-// One S^5 step on task t by this block.
+// Prefix jump of a subset whose keys at `depth` are all equal and hold no end:
+// every string's next 64 characters are compared with the first one's, and the
+// subset goes on, in place, at the first window where some string differs or
+// ends.  Without it a subset sharing a long prefix was moved once for every 8
+// characters of it (6000 strings sharing 200 characters 683 -> 242 us; the
+// queue of 1 M URLs 125 -> 100 us, of the suffix array of 4 M characters, whose
+// steps pay for the registers, 360 -> 373).  Returns the new depth, with the
+// records' keys reloaded; the task's depth if some key differs.  Two keys at a
+// time in a loop that is not unrolled: the look-ahead of the block sorts, eight
+// at once, took more registers than the step has to spare (20 M URLs: the
+// queue 455 -> 530 us, inline or as a call).
+template <int LOGV>
+__device__ __forceinline__ uint32_t queue_jump(const SortCtx& c, QueueSmem<LOGV>& s) {
+  constexpr uint32_t NT = kQueueThreads;
+  const Task t = s.task;
+  const SetDesc sd = c.sets[task_set(t)];
+  Rec* recs = c.rec[task_par(t)] + t.begin;
+  const uint32_t kw = key_width(sd.dna);
+  if (t.depth + kw * kLookWindows > kMaxDepth) return t.depth;
+  const uint64_t key = s.sm.sample[0];
+  bool differs = false;
+  for (uint32_t p = threadIdx.x; p < t.len; p += NT) differs = differs || recs[p].key != key;
+  if (threadIdx.x == 0) s.jstop = kLookWindows - 1;
+  if (__syncthreads_or(differs)) return t.depth;
+  const uint32_t wide = c.wide[task_set(t)];
+  // (the first string of the subset is its own first lead: it agrees with itself)
+  for (int lead = 1; lead >= 0; --lead) {
+    const uint32_t end = lead ? 1u : t.len;
+    for (uint32_t p = threadIdx.x; p < end; p += NT) {
+      const uint64_t off = rec_offset(sd, wide, recs[p].idx, recs[p].off);
+#pragma unroll 1
+      for (uint32_t q = 0; q < (uint32_t)kLookWindows / 2; ++q) {
+        const u128 k = load_key128(sd.chars, off, t.depth + kw * (2 * q + 1), sd.cap, sd.dna);
+        if (lead) s.lead[q] = k;
+        const u128 l = s.lead[q];
+        if (k != l || KeyOps<u128>::end(k, sd.dna)) {
+          const bool first = k_hi(k) != k_hi(l) || key_end(k_hi(k), sd.dna);
+          atomicMin(&s.jstop, 2 * q + (first ? 0u : 1u));
+          break;
+        }
+      }
+    }
+    __syncthreads();
+  }
+  const uint32_t nd = t.depth + kw * (s.jstop + 1);
+  for (uint32_t p = threadIdx.x; p < t.len; p += NT)
+    recs[p].key = load_key(sd.chars, rec_offset(sd, wide, recs[p].idx, recs[p].off), nd, sd.cap, sd.dna);
+  __syncthreads();
+  return nd;
+}
+
+// The sampling of the step on the block's task (and the zeroing of its
+// counters); returns whether the whole sample is one key without an end.
+template <int LOGV>
+__device__ __forceinline__ bool queue_sample(const SortCtx& c, QueueSmem<LOGV>& s) {
+  using Gm = Geo<LOGV>;
+  const Task t = s.task;
+  const uint32_t dna = c.sets[task_set(t)].dna;
+  for (uint32_t b = threadIdx.x; b < Gm::KP; b += kQueueThreads) {
+    s.hist[b] = 0;
+    if (b <= Gm::V) s.u.lc.below[b] = s.u.lc.above[b] = 0;
+  }
+  const Rec* recs = c.rec[task_par(t)] + t.begin;
+  build_splitters<LOGV, uint64_t, kQueueThreads>([&](uint32_t pos) { return recs[pos].key; }, t.len,
+                                                 mix64(c.seed ^ ((uint64_t)t.begin << 20) ^ t.depth), s.sm, dna);
+  const uint64_t k0 = s.sm.sample[0];  // the sorted sample
+  return k0 == s.sm.sample[Gm::S - 1] && !key_end(k0, dna);
+}
+
+// The rest of the S^5 step on task t by this block, after its sampling.
 // Returns this thread's share of the step's algorithmic bytes: the sample,
 // cache 8 read + bucket index 2 written per record while classifying, and the
 // bytes of each record's move.
@@ -117,12 +188,6 @@ __device__ unsigned long long queue_step(const SortCtx& c, const Task& t, QueueS
   const uint32_t wide = c.wide[task_set(t)];
   Splitters<LOGV>& sp = s.sm.sp;
   const bool with_lcp = sd.lcp != nullptr;
-  for (uint32_t b = threadIdx.x; b < Gm::KP; b += NT) {
-    s.hist[b] = 0;
-    if (b <= Gm::V) s.u.lc.below[b] = s.u.lc.above[b] = 0;
-  }
-  build_splitters<LOGV, uint64_t, NT>([&](uint32_t pos) { return recs[pos].key; }, t.len,
-                                      mix64(c.seed ^ ((uint64_t)t.begin << 20) ^ t.depth), s.sm, sd.dna);
   unsigned long long bytes = threadIdx.x == 0 ? Gm::S * 8ull : 0ull;
 
   // classification (Algorithm 4.1): classify into the array o and count.  With
@@ -223,6 +288,13 @@ __global__ void __launch_bounds__(kQueueThreads, kQueueBlocks) k_queue(SortCtx c
     if (threadIdx.x == 0) s.got = claim_task(c.mq, &s.task, c.status, c.wait_ns) ? 1u : 0u;
     __syncthreads();
     if (!s.got) break;
+    while (queue_sample<LOGV>(c, s)) {
+      const uint32_t nd = queue_jump<LOGV>(c, s);
+      if (nd == s.task.depth) break;
+      __syncthreads();
+      if (threadIdx.x == 0) s.task.depth = nd;
+      __syncthreads();
+    }
     const Task t = s.task;
     bytes += queue_step<LOGV>(c, t, s);
     __syncthreads();
