@@ -62,7 +62,10 @@ __device__ __forceinline__ uint64_t cnt_base(const GenTask& g) {
 // Any depth up to the subset's common prefix is correct: the jump only skips
 // work, and the check on the sample keeps its cost away from subsets that
 // share only the key.
+// The check reads up to kPjChunks times 64 characters of a string, as long as
+// they agree: a round costs several times the check of 64 (PJ_FIGURES).
 constexpr int kPjWindows = 8;        // 64 characters
+constexpr int kPjChunks = 4;
 constexpr uint32_t kPjMinSample = 32;  // sampled agreement that turns the check on
 constexpr uint32_t kPjSampleChecks = 64;  // sampled strings compared (of the sample's S)
 
@@ -72,7 +75,7 @@ template <int LOGV>
 struct BigSplitters {
   Splitters<LOGV, u128> sp;  // wide keys
   uint16_t jump[kJumpSize];
-  uint64_t pj_ref;  // offset of the reference string (the first sampled one)
+  uint64_t pj_ref[kPjChunks * kPjWindows];  // the reference string (the first sampled one) from the depth on
   uint32_t pj_on;   // check every string of the subset
   uint32_t pj_lcp;  // smallest agreement with the reference from the depth (atomicMin)
 };
@@ -101,9 +104,9 @@ __device__ __forceinline__ uint32_t window_lcp(const uint64_t (&w)[kPjWindows], 
   return 8u * kPjWindows;
 }
 
-// Smallest agreement with ref over the strings of items [0, items) taken by
-// this block's threads (off_of(i) gives the string offset of item i), reduced
-// over the block.
+// Smallest agreement with ref (kPjChunks * kPjWindows windows) over the strings
+// of items [0, items) taken by this block's threads (off_of(i) gives the string
+// offset of item i), reduced over the block.
 template <typename OffOf>
 __device__ uint32_t block_min_agreement(const SetDesc& sd, uint32_t depth, uint32_t items, OffOf&& off_of,
                                         const uint64_t* ref, unsigned long long& bytes) {
@@ -111,14 +114,25 @@ __device__ uint32_t block_min_agreement(const SetDesc& sd, uint32_t depth, uint3
   if (threadIdx.x == 0) bmin = 0xFFFFFFFFu;
   __syncthreads();
   uint32_t mn = 0xFFFFFFFFu;
+  uint64_t next = threadIdx.x < items ? off_of(threadIdx.x) : 0ull;  // one string ahead
   for (uint32_t i = threadIdx.x; i < items; i += blockDim.x) {
-    uint64_t w[kPjWindows];
-    load_pj_windows(sd.chars, off_of(i), depth, sd.cap, w);
-    mn = min(mn, window_lcp(w, ref));
-    bytes += 8 + 8 * kPjWindows;  // the record's index and offset, the windows
+    const uint64_t off = next;
+    if (i + blockDim.x < items) next = off_of(i + blockDim.x);
+    bytes += 8;  // the record's index and offset
+    uint32_t l = 0;
+#pragma unroll 1
+    for (int ch = 0; ch < kPjChunks; ++ch) {
+      uint64_t w[kPjWindows];
+      load_pj_windows(sd.chars, off, depth + l, sd.cap, w);
+      const uint32_t m = window_lcp(w, ref + ch * kPjWindows);
+      bytes += 8 * kPjWindows;
+      l += m;
+      if (m < 8u * kPjWindows) break;
+    }
+    mn = min(mn, l);
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mn = min(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, o));
+  __syncwarp();
+  mn = __reduce_min_sync(0xFFFFFFFFu, mn);
   if ((threadIdx.x & 31u) == 0 && mn != 0xFFFFFFFFu) atomicMin(&bmin, mn);
   __syncthreads();
   return bmin;
@@ -321,9 +335,22 @@ __global__ void __launch_bounds__(kSampleThreads<LOGV>) k_big_sample(const BigCt
       __syncthreads();
     }
     if (threadIdx.x == 0) {
-      out[gi].pj_on = one_key && s_min > kPjMinSample ? 1u : 0u;
+      const bool on = one_key && s_min > kPjMinSample;
+      out[gi].pj_on = on ? 1u : 0u;
       out[gi].pj_lcp = 0xFFFFFFFFu;
-      out[gi].pj_ref = ref_off;
+      if (on) {
+        bool ended = false;
+#pragma unroll 1
+        for (int ch = 0; ch < kPjChunks; ++ch) {
+          uint64_t w[kPjWindows];
+          for (int j = 0; j < kPjWindows; ++j) w[j] = 0;
+          if (!ended) load_pj_windows(sd.chars, ref_off, g.t.depth + 8 * kPjWindows * ch, sd.cap, w);
+          for (int j = 0; j < kPjWindows; ++j) {
+            out[gi].pj_ref[ch * kPjWindows + j] = w[j];
+            ended = ended || has_nul(w[j]);
+          }
+        }
+      }
     }
     if (c.classifier == kClassifyUIJ) {
       for (uint32_t p = threadIdx.x; p < kJumpSize; p += blockDim.x)
@@ -343,7 +370,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_big_classify(const BigCtl* __rest
   __shared__ __align__(16) u128 x[Gm::V + 1];
   __shared__ uint32_t hist[Gm::KP];
   __shared__ __align__(16) uint16_t jump[kJumpSize];
-  __shared__ uint64_t ref[kPjWindows];
+  __shared__ uint64_t ref[kPjChunks * kPjWindows];
   __shared__ uint32_t s_g;
   __shared__ uint32_t ts[kTileStartsMax];
   const uint32_t G = ctl->cur.G, tiles = ctl->cur.tiles, R = ctl->cur.R;
@@ -390,11 +417,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_big_classify(const BigCtl* __rest
     if (threadIdx.x == 0) bytes += 4ull * Gm::K;
     if (spl[gi].pj_on) {  // prefix jump: every string's agreement with the reference
       const SetDesc sd = c.sets[task_set(g.t)];
-      if (threadIdx.x == 0) {
-        uint64_t w[kPjWindows];
-        load_pj_windows(sd.chars, spl[gi].pj_ref, g.t.depth, sd.cap, w);
-        for (int j = 0; j < kPjWindows; ++j) ref[j] = w[j];
-      }
+      if (threadIdx.x < kPjChunks * kPjWindows) ref[threadIdx.x] = spl[gi].pj_ref[threadIdx.x];
       __syncthreads();
       const uint2* wids = c.wid[par] + g.t.begin + t0;
       const uint32_t wide = c.wide[task_set(g.t)];
