@@ -301,12 +301,63 @@ constexpr int kLookWindows = 8;  // look-ahead: 8 windows = 64 characters per ro
 // Look-ahead read for the refinement of long common prefixes: the KW windows
 // of 8 characters at depths h, h + 8, ..., h + 8(KW-1) (first character most
 // significant, zero at/after the terminator or the cap), from KW / 2 + 1
-// aligned 16-byte words issued at once (precondition and reads as
-// issue_chars).  Returns how many leading windows are determined: those that
-// lie in the 4 KiB block of byte h, or all of them if the string (or the cap)
-// ends in one of these.
+// aligned 16-byte words (precondition as issue_chars).  The words inside the
+// 4 KiB block of byte h are requested at once; for 1 string in 64 some lie in
+// the next block, which may be read only if the string reaches it: then a
+// second pass reads them all.  (Reading such windows one at a time kept whole
+// warps waiting: 1 M records under a 200-character prefix 635 -> 573 us, batch
+// of 512 sets 2112 -> 2075.  A group of strings that stops its look-ahead at
+// the first block edge any of them meets takes many more of them: 1000 strings
+// sharing 200 characters 17 instead of 4, 352 -> 97 us.)
 template <int KW>
-__device__ __forceinline__ uint32_t load_windows(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap,
+__device__ __forceinline__ void load_windows(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap,
+                                             uint64_t (&w)[KW]) {
+  static_assert(KW % 2 == 0, "whole 16-byte words");
+  constexpr int kWords = KW / 2 + 1;
+#pragma unroll
+  for (int j = 0; j < KW; ++j) w[j] = 0;
+  if (h >= cap) return;
+  const uintptr_t at = (uintptr_t)(chars + off + h);
+  const uint32_t sh = (uint32_t)(at & 15u);
+  const uint32_t inside = 4096u - (uint32_t)(at & 4095u);  // bytes from h inside the block (>= 1)
+  const uint4* p = reinterpret_cast<const uint4*>(at & ~(uintptr_t)15);
+  const uint32_t room = cap - h;
+#pragma unroll 1
+  for (uint32_t limit = inside + sh;; limit = ~0u) {  // second pass: everything again, with the next block's words
+    uint32_t x[4 * kWords];
+#pragma unroll
+    for (int i = 0; i < kWords; ++i) {
+      const uint4 v = 16u * i < limit ? __ldg(p + i) : make_uint4(0, 0, 0, 0);
+      x[4 * i] = v.x;
+      x[4 * i + 1] = v.y;
+      x[4 * i + 2] = v.z;
+      x[4 * i + 3] = v.w;
+    }
+    uint32_t o[2 * KW];
+    take_words<2 * KW>(x, sh, o);
+    uint32_t end = 8u * KW;  // characters before the end of the string, as far as the words show it
+#pragma unroll
+    for (int j = 0; j < KW; ++j) {
+      const uint64_t k = ((uint64_t)o[2 * j] << 32) | o[2 * j + 1];
+      if (end < 8u * j) {
+        w[j] = 0;
+        continue;
+      }
+      const uint32_t keep = min(first_nul(k), room > 8u * j ? room - 8u * j : 0u);
+      w[j] = keep_chars(k, keep);
+      if (keep < 8) end = 8u * j + keep;
+    }
+    // words of the next block read as 0: an end there may be none
+    if (limit == ~0u || inside >= 8u * KW || end < inside || end == room) break;
+  }
+}
+
+// load_windows without the second pass, for the warp sorts, which are short of
+// registers (4 M DNA suffixes: 349 us, 377 with it).  Returns how many leading
+// windows are determined: those that lie in the 4 KiB block of byte h, or all
+// of them if the string (or the cap) ends in one of these.
+template <int KW>
+__device__ __forceinline__ uint32_t load_windows_block(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap,
                                                  uint64_t (&w)[KW]) {
   static_assert(KW % 2 == 0, "whole 16-byte words");
   constexpr int kWords = KW / 2 + 1;
@@ -428,49 +479,29 @@ __device__ __forceinline__ uint64_t load_key(const uint8_t* chars, uint64_t off,
   return dna ? dna_key(chars, off, h, cap) : load_chars8(chars, off, h, cap);
 }
 
-// The KW keys at depths h, h + w, ..., h + (KW - 1) w (w = key_width) and how
-// many of them are determined (all of them for the packed codes, whose buffer
-// is padded; see load_windows for bytes).
+// The KW keys at depths h, h + w, ..., h + (KW - 1) w (w = key_width).
 template <int KW>
-__device__ __forceinline__ uint32_t load_key_windows(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap,
+__device__ __forceinline__ void load_key_windows(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap,
                                                      uint32_t dna, uint64_t (&w)[KW]) {
-  if (!dna) return load_windows<KW>(chars, off, h, cap, w);
+  if (!dna) {
+    load_windows<KW>(chars, off, h, cap, w);
+    return;
+  }
   bool ended = false;
 #pragma unroll
   for (int j = 0; j < KW; ++j) {
     w[j] = ended ? 0ull : dna_key(chars, off, h + kDnaWidth * (uint32_t)j, cap);
     ended = ended || key_end(w[j], 1);
   }
-  return KW;
 }
 
-// The key at depth h, out of line: for windows past the 4 KiB block of a
-// look-ahead, which are rare.
-static __device__ __noinline__ uint64_t load_key_far(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap,
-                                              uint32_t dna) {
-  return load_key(chars, off, h, cap, dna);
-}
-
-// load_key_windows with every window determined: those past the 4 KiB block of
-// the first character (1 string in 64 has some) are read one by one while the
-// string continues.  A group of strings that looks ahead together would
-// otherwise stop at the first block edge any of them meets: 1000 strings
-// sharing 200 characters took 17 look-aheads instead of 4 (352 -> 107 us).  The
-// warp sorts, whose groups are small, do without (their code grew by more than
-// they gained: 4 M DNA suffixes 348 -> 379 us).
+// load_windows_block for both encodings.
 template <int KW>
-__device__ __forceinline__ void load_all_windows(const uint8_t* chars, uint64_t off, uint32_t h, uint32_t cap,
-                                                 uint32_t dna, uint64_t (&w)[KW]) {
-  const uint32_t n = load_key_windows<KW>(chars, off, h, cap, dna, w);
-  bool more = n < (uint32_t)KW;
-  if (more) {
-#pragma unroll
-    for (int j = 0; j < KW; ++j)
-      if (more && (uint32_t)j >= n) {
-        w[j] = load_key_far(chars, off, h + key_width(dna) * (uint32_t)j, cap, dna);
-        more = !key_end(w[j], dna);
-      }
-  }
+__device__ __forceinline__ uint32_t load_key_windows_block(const uint8_t* chars, uint64_t off, uint32_t h,
+                                                           uint32_t cap, uint32_t dna, uint64_t (&w)[KW]) {
+  if (!dna) return load_windows_block<KW>(chars, off, h, cap, w);
+  load_key_windows<KW>(chars, off, h, cap, dna, w);
+  return KW;
 }
 
 // ---------------------------------------------------------------------------

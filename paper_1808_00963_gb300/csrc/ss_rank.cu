@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(64) k_rank_keys(BeginArgs a, RankArgs r) {
   const SetDesc& sd = a.sd;
   const uint64_t off = sd.offsets[i];
   uint64_t w[kRankWords];
-  load_all_windows<kRankWords>(sd.chars, off, 0, sd.cap, sd.dna, w);
+  load_key_windows<kRankWords>(sd.chars, off, 0, sd.cap, sd.dna, w);
   r.keys[2 * i] = make_ulonglong2(w[0], w[1]);
   r.keys[2 * i + 1] = make_ulonglong2(w[2], w[3]);
   r.rank[i] = 0;

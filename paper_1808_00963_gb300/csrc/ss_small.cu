@@ -198,7 +198,7 @@ __device__ uint32_t warp_refine(bool active, uint32_t g0, uint32_t nact, uint64_
     uint64_t w[kLookWindows];
     uint32_t nwin = 0;
     const uint32_t kw = key_width(dna);
-    if (active && open) nwin = load_key_windows<kLookWindows>(chars, off, depth + kw, cap, dna, w);
+    if (active && open) nwin = load_key_windows_block<kLookWindows>(chars, off, depth + kw, cap, dna, w);
     const uint32_t segmask = (next >= 32 ? kFull : ((1u << next) - 1)) & ~((1u << my_start) - 1);
     uint32_t jstop = kLookWindows - 1;
     bool found = false;
@@ -696,7 +696,7 @@ __global__ void __launch_bounds__(NT) k_small_cta(SortCtx c, uint32_t pmax, uint
       uint64_t x[kLookWindows];
       for (uint32_t j0 = 0; j0 < n; j0 += NT) {  // the same code for the leader and the others: it is
         const uint32_t j = j0 + tid;             // run rarely, so fetching it is part of what it costs
-        if (look && j < n) load_all_windows<kLookWindows>(sd.chars, off_at(lo + j), depth + kw, sd.cap, dna, x);
+        if (look && j < n) load_key_windows<kLookWindows>(sd.chars, off_at(lo + j), depth + kw, sd.cap, dna, x);
         __syncwarp();
         if (j == 0) {
 #pragma unroll
