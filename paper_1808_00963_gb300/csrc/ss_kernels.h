@@ -57,19 +57,23 @@ struct BigCtl {
 };
 
 // Rounds of 256 strings in a tile of a round over `total` strings in G
-// subsets: two tiles per SM where there are that many strings, at least
-// kMinTileRounds (a tile's fixed work is its 2^(logv + 1) counters; with a
-// minimum of 8, 100 k strings filled 49 of 152 SMs: classification 17.3 ->
-// 12.8 us, scatter 22.9 -> 15.4 us), at most kMaxTileRounds, and more where
-// the tiles' counters would not fit.  With at most 16 the scatter's shared
-// memory lets three blocks share an SM instead of two (20 M URLs 4820 -> 4415
-// us, 4 M DNA suffixes 1270 -> 1201 us; at most 8: 4401 / 1164 us, but the
-// batch of 512 sets 2637 instead of 2620 us and twice the counters).
-constexpr uint32_t kMinTileRounds = 2, kMaxTileRounds = 16;
+// subsets: kTilesPerSm tiles per SM where there are that many strings (three or
+// four blocks of an SM take tiles as they finish; with two per SM half of the
+// slots had none: 1 M records under a 200-character prefix 572 us, with 6 per SM
+// 531, 9 487, 12 487; 4 M DNA suffixes 1047 / 1044 / 1012 / 1007; 2 M URLs from
+// host memory 1602 / 1545 / 1557 / 1569), at least kMinTileRounds (a tile's
+// fixed work is its 2^(logv + 1) counters; with a minimum of 8, 100 k strings
+// filled 49 of 152 SMs: classification 17.3 -> 12.8 us, scatter 22.9 -> 15.4
+// us), at most kMaxTileRounds, and more where the tiles' counters would not
+// fit.  With at most 16 the scatter's shared memory lets three blocks share an
+// SM instead of two (20 M URLs 4820 -> 4415 us, 4 M DNA suffixes 1270 -> 1201
+// us; at most 8: 4401 / 1164 us, but the batch of 512 sets 2637 instead of 2620
+// us and twice the counters).
+constexpr uint32_t kMinTileRounds = 2, kMaxTileRounds = 16, kTilesPerSm = 9;
 __host__ __device__ inline uint32_t tile_rounds(uint64_t total, uint64_t G, uint32_t sms, uint32_t K,
                                                 uint64_t ncounters_max, uint32_t fixed) {
   if (fixed) return fixed;
-  const uint64_t per = total / ((uint64_t)sms * 2 * 256) + 1;
+  const uint64_t per = total / ((uint64_t)sms * kTilesPerSm * 256) + 1;
   uint32_t R = (uint32_t)(per < kMinTileRounds ? kMinTileRounds : (per > kMaxTileRounds ? kMaxTileRounds : per));
   while (R < 8 && K * (total / (256ull * R) + G) > ncounters_max) ++R;
   return R;
