@@ -215,7 +215,7 @@ enum Ctrl : uint32_t { kCStatus = 0, kCBig0 = 1, kCBig1 = 2, kCHead = 3, kCTail 
 struct Layout {
   size_t ctrl, sets, wide, rec0, rec1, wid0, wid1, bucket_of, big0, big1, gen, spl, counters, partials, gstart,
       gdesc, bigctl, marks, mq_items, mq_ready, sw_items, sc_items, scw_items, rank_keys, rank, total;
-  uint32_t cap_big, cap_mq, cap_sw, cap_sc, cap_scw;
+  uint32_t cap_big, cap_mq, cap_sw, cap_sc, cap_scw, cap_marks;
   uint64_t ncounters_max;
 };
 
@@ -223,11 +223,20 @@ struct Layout {
 // asks for particular distribution steps.
 static bool by_rank(uint64_t n, const Opts& o) { return o.plain_steps && n >= kRankMin && n <= kRankMax; }
 
-static Layout make_layout(uint64_t M, uint32_t num_sets, const Opts& o, bool big, bool rank = false) {
+// Multi-block steps of a sort: none; rounds until no subset is above the big
+// threshold; or one round for the root, whose children all go to the work queue
+// (sorts that may not launch the loop's graph).
+enum class Rounds { kNone, kLoop, kOne };
+
+// limit: bytes the layout may take (a sort with one round sizes its tiles by
+// what its fixed scratch leaves for their counters).
+static Layout make_layout(uint64_t M, uint32_t num_sets, const Opts& o, Rounds rounds, bool rank = false,
+                          size_t limit = ~(size_t)0) {
   Layout L{};
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t at = off; off += align256(bytes); return at; };
-  L.cap_big = big ? (uint32_t)(M / ((uint64_t)o.big_thr + 1) + 2) : 0;
+  const bool big = rounds != Rounds::kNone, one = rounds == Rounds::kOne;
+  L.cap_big = one ? 1u : (big ? (uint32_t)(M / ((uint64_t)o.big_thr + 1) + 2) : 0u);
   // the work queue's ring: more slots than disjoint subsets of > cutoff
   // records can exist, so it never overflows (see WorkQueue)
   L.cap_mq = (uint32_t)std::max<uint64_t>(4096, M / ((uint64_t)o.cutoff + 1) + 1024);
@@ -237,30 +246,24 @@ static Layout make_layout(uint64_t M, uint32_t num_sets, const Opts& o, bool big
   L.cap_sc = (uint32_t)(M / 33 + 2);
   L.cap_scw = (uint32_t)(M / (kSmallCtaNarrowMax + 1) + 2);
   const uint64_t KP = 2ull << o.logv_big;
-  // tiles of the largest round: tile_rounds gives one over all strings the
-  // tile of a GPU of kSizingSms SMs if its counters fit, else up to 8 rounds
-  constexpr uint32_t kSizingSms = 152;
-  const uint32_t R0 = tile_rounds(M, 1, kSizingSms, (2u << o.logv_big) - 1, ~0ull, 0);
-  const uint64_t tiles_max = big ? M / (kBlock * std::min(R0, 8u)) + L.cap_big : 0;
-  L.ncounters_max = big ? KP * (tiles_max + L.cap_big) : 0;
+  // LCP marks of multi-block steps: distinct positions (< M), one per bucket of a single round
+  L.cap_marks = one ? (uint32_t)KP : (big ? (uint32_t)M : 0u);
   L.ctrl = take(kCtrlBytes);
   L.sets = take((size_t)num_sets * sizeof(SetDesc));
   L.wide = take((size_t)num_sets * 4);
   L.rec0 = take(M * sizeof(Rec));
   L.rec1 = take(M * sizeof(Rec));
   L.wid0 = take(big ? M * sizeof(uint2) : 0);  // (idx, off) of the wide records of multi-block subsets
-  L.wid1 = take(big ? M * sizeof(uint2) : 0);
+  L.wid1 = take(big && !one ? M * sizeof(uint2) : 0);
   L.bucket_of = take(M * 2);
   L.big0 = take((size_t)L.cap_big * sizeof(Task));
   L.big1 = take((size_t)L.cap_big * sizeof(Task));
   L.gen = take(2 * (size_t)L.cap_big * sizeof(GenTask));
   L.spl = take((size_t)L.cap_big * big_splitters_bytes(o.logv_big));
-  L.counters = take(L.ncounters_max * 4);
-  L.partials = take((L.ncounters_max / 4096 + 2) * 4);
   L.gstart = take((size_t)L.cap_big * KP * 4);
   L.gdesc = take((size_t)L.cap_big * KP * 4);
   L.bigctl = take(big ? sizeof(BigCtl) : 0);  // a batch's loop control block (plain sorts use the stream's)
-  L.marks = take(big ? M * 4 : 0);             // LCP marks of multi-block steps (distinct positions: < M)
+  L.marks = take((size_t)L.cap_marks * 4);
   L.mq_items = take((size_t)L.cap_mq * sizeof(Task));
   L.mq_ready = take((size_t)L.cap_mq * 4);
   L.sw_items = take(2 * (size_t)L.cap_sw * sizeof(Task));
@@ -268,11 +271,21 @@ static Layout make_layout(uint64_t M, uint32_t num_sets, const Opts& o, bool big
   L.scw_items = take((size_t)L.cap_scw * sizeof(Task));
   L.rank_keys = take(rank ? M * 2 * sizeof(ulonglong2) : 0);
   L.rank = take(rank ? M * 4 : 0);
+  // counters of the largest round: tile_rounds gives one over all strings the
+  // tile of a GPU of kSizingSms SMs if its counters fit, else up to 8 rounds
+  constexpr uint32_t kSizingSms = 152;
+  uint32_t R = std::min(tile_rounds(M, 1, kSizingSms, (uint32_t)KP - 1, ~0ull, 0), 8u);
+  auto counters = [&] { return big ? KP * (M / (kBlock * R) + 2 * (uint64_t)L.cap_big) : 0ull; };
+  auto counter_bytes = [&] { return align256(counters() * 4) + align256((counters() / 4096 + 2) * 4); };
+  while (R < 8 && off + counter_bytes() > limit) ++R;
+  L.ncounters_max = counters();
+  L.counters = take(L.ncounters_max * 4);
+  L.partials = take((L.ncounters_max / 4096 + 2) * 4);
   L.total = off;
   return L;
 }
 
-static SortCtx make_ctx(uint8_t* ws, const Layout& L, uint32_t num_sets, uint32_t total, const Opts& o, bool big) {
+static SortCtx make_ctx(uint8_t* ws, const Layout& L, uint32_t num_sets, uint32_t total, const Opts& o, Rounds rounds) {
   SortCtx c{};
   uint32_t* ctrl = reinterpret_cast<uint32_t*>(ws + L.ctrl);
   c.sets = reinterpret_cast<const SetDesc*>(ws + L.sets);
@@ -299,10 +312,11 @@ static SortCtx make_ctx(uint8_t* ws, const Layout& L, uint32_t num_sets, uint32_
   c.done = ctrl + kCDone;
   c.marks = reinterpret_cast<uint32_t*>(ws + L.marks);
   c.marks_count = ctrl + kCMarks;
-  c.marks_cap = big ? total : 0u;
+  c.marks_cap = L.cap_marks;
   c.small_cutoff = o.cutoff;
   c.big_threshold = o.big_thr;
-  c.big_enabled = big ? 1u : 0u;
+  c.big_enabled = rounds == Rounds::kLoop ? 1u : 0u;
+  c.wide_threshold = rounds == Rounds::kNone ? 0xFFFFFFFFu : o.big_thr;
   c.seed = o.seed;
   c.classifier = o.classifier;
   c.big_cur = 0;
@@ -518,8 +532,9 @@ static ss_status stream_slot(cudaStream_t st, bool create, StreamSlot* out) {
 // descriptors are in place already).  ctl: where the multi-block loop's control
 // block lives (needed when big).
 static ss_status run_sort(uint8_t* ws, const Layout& L, SortCtx c, const Opts& o, const DevInfo& dev,
-                          bool big, cudaStream_t st, const SetDesc* sd, BigCtl* ctl = nullptr) {
+                          Rounds rounds, cudaStream_t st, const SetDesc* sd, BigCtl* ctl = nullptr) {
   const LaunchHook hook{st};
+  const bool big = rounds != Rounds::kNone;
   BeginArgs a{};
   a.ctrl = reinterpret_cast<uint32_t*>(ws + L.ctrl);
   a.ctrl_words = (uint32_t)(kCtrlBytes / 4);
@@ -575,7 +590,9 @@ static ss_status run_sort(uint8_t* ws, const Layout& L, SortCtx c, const Opts& o
     const uint32_t R_max = o.R ? o.R : kMaxTileRounds;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     SS_CUDA(cudaStreamIsCapturing(st, &cs));
-    if (cs == cudaStreamCaptureStatusActive) {
+    if (rounds == Rounds::kOne) {
+      SS_CUDA(launch_big_round(o.logv_big, ctl, R_max, (uint32_t)dev.sms, 0, false, st, hook));
+    } else if (cs == cudaStreamCaptureStatusActive) {
       // the caller is capturing a graph: the loop becomes part of it
       SS_CUDA(add_loop(st, ctl, o.logv_big, R_max, (uint32_t)dev.sms));
     } else if (g_profiling.load() || !g_graph_loop.load()) {
@@ -628,8 +645,8 @@ static ss_status sort_device(const uint8_t* chars, const uint64_t* offsets, uint
   if (!chars || !offsets || !perm) return SS_ERR_INVALID;
   DevInfo dev;
   if ((s = device_info(dev)) != SS_OK) return s;
-  const bool big = n > o.big_thr;
-  const Layout L = make_layout(n, 1, o, big, by_rank(n, o));
+  const Rounds rounds = n > o.big_thr ? Rounds::kLoop : Rounds::kNone;
+  const Layout L = make_layout(n, 1, o, rounds, by_rank(n, o));
   uint8_t* ws = nullptr;
   bool owned = false;
   if (opt && opt->workspace) {
@@ -645,10 +662,10 @@ static ss_status sort_device(const uint8_t* chars, const uint64_t* offsets, uint
     return s;
   }
   SetDesc sd{chars, offsets, perm, lcp, (uint32_t)n, o.cap, 0, dna};
-  SortCtx ctx = make_ctx(ws, L, 1, (uint32_t)n, o, big);
+  SortCtx ctx = make_ctx(ws, L, 1, (uint32_t)n, o, rounds);
   ctx.dna = dna;
   ctx.fold_status = slot.status_dev;  // the device status goes to the stream's status word
-  const ss_status r = run_sort(ws, L, ctx, o, dev, big, st, &sd, slot.ctl);
+  const ss_status r = run_sort(ws, L, ctx, o, dev, rounds, st, &sd, slot.ctl);
   if (g_profiling.load()) read_status(ws, L, st);  // waits: per-kernel times and bytes
   if (owned) cudaFreeAsync(ws, st);
   return r;
@@ -679,6 +696,7 @@ struct ss_batch {
   uint8_t* ws = nullptr;
   bool owned = false;
   bool big = false;  // some set is larger than the multi-block threshold
+  ss::Rounds rounds() const { return big ? ss::Rounds::kLoop : ss::Rounds::kNone; }
   uint32_t num_sets = 0;
   uint32_t total = 0;
   std::vector<ss::SetDesc> sd;  // the set descriptors, written into the workspace by each run
@@ -1048,7 +1066,7 @@ ss_status ss_suffix_array(const uint8_t* text, uint64_t n, uint32_t* out_sa, uin
 size_t ss_workspace_size(uint64_t n, const ss_options* opt) {
   Opts o;
   if (resolve_opts(opt, o) != SS_OK || n >= 0xFFFFFFFFull) return 0;
-  return make_layout(n, 1, o, n > o.big_thr, by_rank(n, o)).total;
+  return make_layout(n, 1, o, n > o.big_thr ? Rounds::kLoop : Rounds::kNone, by_rank(n, o)).total;
 }
 
 ss_status ss_sort_ex(const uint8_t* chars, const uint64_t* offsets, uint64_t n, uint32_t* out_perm,
@@ -1340,7 +1358,7 @@ size_t ss_batch_workspace_size(const ss_set* sets, uint32_t num_sets, const ss_o
   uint64_t total = 0;
   bool big = false;
   if (resolve_opts(opt, o) != SS_OK || batch_geometry(sets, num_sets, o, &total, &big) != SS_OK) return 0;
-  return make_layout(total, num_sets, o, big).total;
+  return make_layout(total, num_sets, o, big ? Rounds::kLoop : Rounds::kNone).total;
 }
 
 ss_status ss_batch_create(const ss_set* sets, uint32_t num_sets, const ss_options* opt, ss_batch** out) {
@@ -1352,7 +1370,7 @@ ss_status ss_batch_create(const ss_set* sets, uint32_t num_sets, const ss_option
   uint64_t total = 0;
   if ((s = batch_geometry(sets, num_sets, b.o, &total, &b.big)) != SS_OK) return s;
   if ((s = device_info(b.dev)) != SS_OK) return s;
-  b.L = make_layout(total, num_sets, b.o, b.big);
+  b.L = make_layout(total, num_sets, b.o, b.rounds());
   if (opt && opt->workspace) {
     if (opt->workspace_bytes < b.L.total) return SS_ERR_INVALID;
     b.ws = static_cast<uint8_t*>(opt->workspace);
@@ -1394,7 +1412,7 @@ ss_status ss_batch_run(ss_batch* b, void* stream) {
     LaunchHook{st}.run("init", [&] { k_set_descs<<<1, kBlock, 0, st>>>(dsets + i0, cnt, ch); });
     if (cudaGetLastError() != cudaSuccess) return SS_ERR_CUDA;
   }
-  SortCtx c = make_ctx(b->ws, b->L, b->num_sets, b->total, b->o, b->big);
+  SortCtx c = make_ctx(b->ws, b->L, b->num_sets, b->total, b->o, b->rounds());
   // the multi-block loop's control block: inside a caller's capture the
   // batch's own (its address goes into the caller's graph); otherwise the
   // stream's, whose loop graph is built once per stream
@@ -1411,7 +1429,7 @@ ss_status ss_batch_run(ss_batch* b, void* stream) {
       ctl = slot.ctl;
     }
   }
-  return run_sort(b->ws, b->L, c, b->o, b->dev, b->big, st, nullptr, ctl);
+  return run_sort(b->ws, b->L, c, b->o, b->dev, b->rounds(), st, nullptr, ctl);
 }
 
 ss_status ss_batch_status(ss_batch* b, void* stream) {
@@ -1505,7 +1523,12 @@ extern "C" ss_status ss_sort_noalloc(const uint8_t* chars, const uint64_t* offse
   if (g_profiling.load()) return SS_ERR_INVALID;  // profiling would create CUDA events
   Opts o;
   if (max_len) o.cap = max_len;
-  const Layout L = make_layout(n, 1, o, false, by_rank(n, o));
+  // One round of multi-block steps where ss_sort would take them (a root of
+  // 20 000 strings took one block 70 us: 20 k random strings 149 -> 131 us, 65 536
+  // 305 -> 145, 20 k URLs 279 -> 198); the rounds after it
+  // would be a graph, whose instantiation may allocate.
+  const Rounds rounds = n > o.big_thr ? Rounds::kOne : Rounds::kNone;
+  const Layout L = make_layout(n, 1, o, rounds, by_rank(n, o), SS_NOALLOC_SCRATCH_BYTES);
   if (L.total > SS_NOALLOC_SCRATCH_BYTES) return SS_ERR_TOO_LARGE;
   DevInfo dev;
   ss_status s = device_info(dev);
@@ -1516,7 +1539,8 @@ extern "C" ss_status ss_sort_noalloc(const uint8_t* chars, const uint64_t* offse
   const SetDesc sd{chars, offsets, out_perm, out_lcp, (uint32_t)n, o.cap, 0, 0};
   // run_sort clears the control words and the queue flags, the only scratch
   // that must start at zero; everything else is written before it is read.
-  s = run_sort(ws, L, make_ctx(ws, L, 1, (uint32_t)n, o, false), o, dev, false, st, &sd);
+  s = run_sort(ws, L, make_ctx(ws, L, 1, (uint32_t)n, o, rounds), o, dev, rounds, st, &sd,
+               reinterpret_cast<BigCtl*>(ws + L.bigctl));
   if (s != SS_OK) return s;
   uint32_t status = 0;
   if (cudaMemcpyAsync(&status, ws + L.ctrl, sizeof(status), cudaMemcpyDeviceToHost, st) != cudaSuccess ||

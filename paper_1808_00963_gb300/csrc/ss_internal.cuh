@@ -134,6 +134,7 @@ struct SortCtx {
   uint32_t small_cutoff;
   uint32_t big_threshold;  // tasks longer than this go to big[] (if big_enabled)
   uint32_t big_enabled;
+  uint32_t wide_threshold; // sets of more strings start with a multi-block step (wide records)
   uint32_t seed;
   uint32_t classifier;     // classification variant (kClassifyUI / UIC / E)
   uint32_t big_cur;        // which big[] list the current step reads

@@ -57,7 +57,8 @@ __global__ void __launch_bounds__(kBlock) k_init(SortCtx c) {
     if (sd.n == 0) continue;
     if (sd.lcp) sd.lcp[0] = 0;
     if (sd.n == 1) sd.perm[0] = 0;
-    else route_task(c, Task{sd.base, sd.n, 0, make_meta(s, 0)}, c.big_cur);
+    else if (c.num_sets > 1 || sd.n <= c.wide_threshold)  // (the host has planned a single set's first round)
+      route_task(c, Task{sd.base, sd.n, 0, make_meta(s, 0)}, c.big_cur);
   }
   __syncwarp();
   for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < c.total; r += stride) {
@@ -66,7 +67,7 @@ __global__ void __launch_bounds__(kBlock) k_init(SortCtx c) {
     const uint32_t i = r - sd.base;
     const uint64_t off = sd.offsets[i];
     if ((off >> 32) && !c.wide[s]) atomicOr(c.wide + s, 1u);
-    if (c.big_enabled && sd.n > c.big_threshold) {  // a multi-block root: wide records
+    if (sd.n > c.wide_threshold) {  // a multi-block root: wide records
       store_wkey(c.rec[0] + r, load_key128(sd.chars, off, 0, sd.cap, sd.dna));
       c.wid[0][r] = make_uint2(i, (uint32_t)off);
       bytes += 48;  // offset 8 + 16 characters read, wide record 24 written
