@@ -269,9 +269,11 @@ static_assert(kWarpPassJumps[kWarpPasses - 1] == 0, "the last pass finishes ever
 // One pass over a list of warp tasks.  With max_jumps > 0, runs with long
 // common prefixes are deferred to the list `out`: their records go back to
 // the record buffer at their current positions, and each run becomes a task.
-// Last: this is the sort's last kernel.
-template <bool Last>
-__global__ void __launch_bounds__(kBlock) k_small_warp(SortCtx c, TaskList list, TaskList out, uint32_t max_jumps) {
+// Last: this is the sort's last kernel.  DNA: the character encoding (with it
+// fixed and at 64 registers, four blocks fit an SM).
+template <bool Last, bool DNA>
+__global__ void __launch_bounds__(kBlock, 4) k_small_warp(SortCtx c, TaskList list, TaskList out, uint32_t max_jumps) {
+  constexpr uint32_t dna = DNA ? 1u : 0u;
   const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
   const uint32_t count = min(*list.count, list.cap);
@@ -288,7 +290,7 @@ __global__ void __launch_bounds__(kBlock) k_small_warp(SortCtx c, TaskList list,
       const uint32_t tdepth = __shfl_sync(kFull, mt.depth, k & 31);
       const uint32_t tmeta = __shfl_sync(kFull, mt.meta, k & 31);
       uint64_t key = 0, off = 0;
-      uint32_t id = 0, cap = kNoCap, dna = 0;
+      uint32_t id = 0, cap = kNoCap;
       const uint8_t* chars = nullptr;
       uint32_t* lcp_g = nullptr;
       uint32_t* perm = nullptr;
@@ -302,7 +304,6 @@ __global__ void __launch_bounds__(kBlock) k_small_warp(SortCtx c, TaskList list,
         off = rec_offset(sd, c.wide[tmeta & 0x7FFFFFFFu], r.idx, r.off);
         cap = sd.cap;
         chars = sd.chars;
-        dna = sd.dna;
         lcp_g = sd.lcp ? sd.lcp + (tb - sd.base) : nullptr;
         perm = sd.perm + (tb - sd.base);
       }
@@ -880,7 +881,7 @@ static cudaError_t launch_small_t(const SortCtx& c, uint32_t pmax, uint32_t sms,
   });
   const uint32_t grid = max(1u, min(sms * 8, (c.total / 2 + kWarps - 1) / kWarps));  // tasks hold at least 2 strings
   if (last) {  // few strings: one pass, there is nothing to gain from packing deferred runs
-    hook.run("small_warp", [&] { k_small_warp<true><<<grid, kBlock, 0, st>>>(c, c.small_warp, c.small_deep, 0u); });
+    hook.run("small_warp", [&] { k_small_warp<true, DNA><<<grid, kBlock, 0, st>>>(c, c.small_warp, c.small_deep, 0u); });
     return cudaGetLastError();
   }
   // the lists alternate: a pass reads one and defers into the other, emptied first
@@ -891,7 +892,7 @@ static cudaError_t launch_small_t(const SortCtx& c, uint32_t pmax, uint32_t sms,
       const cudaError_t e = launch_upload(nullptr, out.count, 4, st, hook);
       if (e != cudaSuccess) return e;
     }
-    hook.run("small_warp", [&] { k_small_warp<false><<<grid, kBlock, 0, st>>>(c, in, out, kWarpPassJumps[p]); });
+    hook.run("small_warp", [&] { k_small_warp<false, DNA><<<grid, kBlock, 0, st>>>(c, in, out, kWarpPassJumps[p]); });
   }
   return cudaGetLastError();
 }
