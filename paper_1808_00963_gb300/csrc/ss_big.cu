@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(kBlock) k_big_emit(BigCtl* ctl, cudaGraphCondi
   }
 }
 
-template <int LOGV>
+template <int LOGV, bool DNA>
 __global__ void __launch_bounds__(kBlock, 3) k_big_scatter(const BigCtl* __restrict__ ctl, uint32_t* __restrict__ work) {
   using Gm = Geo<LOGV>;
   extern __shared__ __align__(16) uint8_t smem[];
@@ -546,7 +546,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_big_scatter(const BigCtl* __restr
         tb, tl, R, base, cntw,
         [&](const uint32_t(&pp)[kWideMoveBatch], const uint32_t(&bb)[kWideMoveBatch],
             const uint32_t(&dd)[kWideMoveBatch]) {
-          bytes += move_batch_wide<kWideMoveBatch>(c, sd, wide, par, src0, depth, desc,
+          bytes += move_batch_wide<kWideMoveBatch, DNA>(c, sd, wide, par, src0, depth, desc,
                                                    [&](uint32_t b) { return bfirst[b]; }, pp, bb, dd);
         });
   }
@@ -697,13 +697,13 @@ cudaError_t launch_big_plan(BigCtl* ctl, cudaStream_t st, const LaunchHook& hook
   return cudaGetLastError();
 }
 
-template <int LOGV>
+template <int LOGV, bool DNA>
 static cudaError_t launch_big_round_t(BigCtl* ctl, uint32_t R_max, uint32_t sms, uint64_t cond, bool use_cond,
                                       cudaStream_t st, const LaunchHook& hook) {
   const size_t smem = big_scatter_smem(LOGV, R_max);
   static bool attr_set = false;
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_big_scatter<LOGV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_big_scatter<LOGV, DNA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)big_scatter_smem(LOGV, kMaxRounds));
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_big_sample<LOGV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -722,15 +722,17 @@ static cudaError_t launch_big_round_t(BigCtl* ctl, uint32_t R_max, uint32_t sms,
   hook.run("big_emit", [&] {
     k_big_emit<LOGV><<<sms * 8, kBlock, 0, st>>>(ctl, (cudaGraphConditionalHandle)cond, use_cond ? 1u : 0u);
   });
-  hook.run("big_scatter", [&] { k_big_scatter<LOGV><<<sms * 3, kBlock, smem, st>>>(ctl, &ctl->mv.next_tile); });
+  hook.run("big_scatter", [&] { k_big_scatter<LOGV, DNA><<<sms * 3, kBlock, smem, st>>>(ctl, &ctl->mv.next_tile); });
   return cudaGetLastError();
 }
 
-cudaError_t launch_big_round(int logv, BigCtl* ctl, uint32_t R_max, uint32_t sms, uint64_t cond_handle, bool use_cond,
-                             cudaStream_t st, const LaunchHook& hook) {
-  switch (logv) {
-    case 8: return launch_big_round_t<8>(ctl, R_max, sms, cond_handle, use_cond, st, hook);
-    case 9: return launch_big_round_t<9>(ctl, R_max, sms, cond_handle, use_cond, st, hook);
+cudaError_t launch_big_round(int logv, bool dna, BigCtl* ctl, uint32_t R_max, uint32_t sms, uint64_t cond_handle,
+                             bool use_cond, cudaStream_t st, const LaunchHook& hook) {
+  switch (2 * logv + (dna ? 1 : 0)) {
+    case 16: return launch_big_round_t<8, false>(ctl, R_max, sms, cond_handle, use_cond, st, hook);
+    case 17: return launch_big_round_t<8, true>(ctl, R_max, sms, cond_handle, use_cond, st, hook);
+    case 18: return launch_big_round_t<9, false>(ctl, R_max, sms, cond_handle, use_cond, st, hook);
+    case 19: return launch_big_round_t<9, true>(ctl, R_max, sms, cond_handle, use_cond, st, hook);
     default: return cudaErrorInvalidValue;  // 2^10 wide splitters exceed static shared memory
   }
 }

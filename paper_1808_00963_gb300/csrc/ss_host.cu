@@ -383,9 +383,10 @@ struct LoopKey {
   int dev;
   const void* ctl;
   int logv;
+  bool dna;
   uint32_t R_max;
   bool operator<(const LoopKey& o) const {
-    return std::tie(dev, ctl, logv, R_max) < std::tie(o.dev, o.ctl, o.logv, o.R_max);
+    return std::tie(dev, ctl, logv, dna, R_max) < std::tie(o.dev, o.ctl, o.logv, o.dna, o.R_max);
   }
 };
 struct LoopGraph {
@@ -417,7 +418,7 @@ static cudaError_t capture_streams(CaptureStreams*& out) {
 // is one round (its emit plans the next one and sets the condition; the first
 // round always runs, the plan for it is in the control block).  Work captured
 // on st afterwards depends on the loop.
-static cudaError_t add_loop(cudaStream_t st, BigCtl* ctl, int logv, uint32_t R_max, uint32_t sms) {
+static cudaError_t add_loop(cudaStream_t st, BigCtl* ctl, int logv, bool dna, uint32_t R_max, uint32_t sms) {
   CaptureStreams* cs = nullptr;
   cudaError_t e = capture_streams(cs);
   if (e != cudaSuccess) return e;
@@ -441,7 +442,7 @@ static cudaError_t add_loop(cudaStream_t st, BigCtl* ctl, int logv, uint32_t R_m
       cudaSuccess)
     return e;
   const LaunchHook bhook{cs->body};
-  cudaError_t e1 = launch_big_round(logv, ctl, R_max, sms, (uint64_t)h, true, cs->body, bhook);
+  cudaError_t e1 = launch_big_round(logv, dna, ctl, R_max, sms, (uint64_t)h, true, cs->body, bhook);
   cudaGraph_t done = nullptr;
   e = cudaStreamEndCapture(cs->body, &done);
   if (e1 != cudaSuccess) return e1;
@@ -450,18 +451,18 @@ static cudaError_t add_loop(cudaStream_t st, BigCtl* ctl, int logv, uint32_t R_m
 }
 
 // The instantiated loop graph for a control block (built on first use).
-static cudaError_t loop_exec(BigCtl* ctl, int logv, uint32_t R_max, uint32_t sms, cudaGraphExec_t* out) {
+static cudaError_t loop_exec(BigCtl* ctl, int logv, bool dna, uint32_t R_max, uint32_t sms, cudaGraphExec_t* out) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> lk(g_loop_mu);
-  LoopGraph& lg = g_loops[LoopKey{dev, ctl, logv, R_max}];
+  LoopGraph& lg = g_loops[LoopKey{dev, ctl, logv, dna, R_max}];
   if (!lg.exec) {
     CaptureStreams* cs = nullptr;
     if ((e = capture_streams(cs)) != cudaSuccess) return e;
     if ((e = cudaStreamBeginCapture(cs->main, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return e;
     t_no_count = true;  // these kernels run once per graph launch; the plan kernels count them
-    cudaError_t e1 = add_loop(cs->main, ctl, logv, R_max, sms);
+    cudaError_t e1 = add_loop(cs->main, ctl, logv, dna, R_max, sms);
     t_no_count = false;
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(cs->main, &g);
@@ -588,26 +589,27 @@ static ss_status run_sort(uint8_t* ws, const Layout& L, SortCtx c, const Opts& o
   if (big) {
     if (c.num_sets > 1) SS_CUDA(launch_big_plan(ctl, st, hook));
     const uint32_t R_max = o.R ? o.R : kMaxTileRounds;
+    const bool dna = c.dna != 0;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     SS_CUDA(cudaStreamIsCapturing(st, &cs));
     if (rounds == Rounds::kOne) {
-      SS_CUDA(launch_big_round(o.logv_big, ctl, R_max, (uint32_t)dev.sms, 0, false, st, hook));
+      SS_CUDA(launch_big_round(o.logv_big, dna, ctl, R_max, (uint32_t)dev.sms, 0, false, st, hook));
     } else if (cs == cudaStreamCaptureStatusActive) {
       // the caller is capturing a graph: the loop becomes part of it
-      SS_CUDA(add_loop(st, ctl, o.logv_big, R_max, (uint32_t)dev.sms));
+      SS_CUDA(add_loop(st, ctl, o.logv_big, dna, R_max, (uint32_t)dev.sms));
     } else if (g_profiling.load() || !g_graph_loop.load()) {
       // launch by launch (timed, or for a profiler): the host runs the rounds, reading each plan
       if (t_down.reserve(64) != SS_OK) return SS_ERR_OOM;
       uint32_t* hG = static_cast<uint32_t*>(t_down.p);
       do {
-        SS_CUDA(launch_big_round(o.logv_big, ctl, R_max, (uint32_t)dev.sms, 0, false, st, hook));
+        SS_CUDA(launch_big_round(o.logv_big, dna, ctl, R_max, (uint32_t)dev.sms, 0, false, st, hook));
         SS_CUDA(cudaMemcpyAsync(hG, &ctl->cur.G, 4, cudaMemcpyDeviceToHost, st));
         SS_CUDA(cudaStreamSynchronize(st));
         collect_profile();
       } while (*hG);
     } else {
       cudaGraphExec_t exec = nullptr;
-      SS_CUDA(loop_exec(ctl, o.logv_big, R_max, (uint32_t)dev.sms, &exec));
+      SS_CUDA(loop_exec(ctl, o.logv_big, dna, R_max, (uint32_t)dev.sms, &exec));
       SS_CUDA(cudaGraphLaunch(exec, st));
     }
   }

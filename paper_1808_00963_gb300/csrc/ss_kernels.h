@@ -96,14 +96,13 @@ cudaError_t launch_big_plan(BigCtl* ctl, cudaStream_t st, const LaunchHook& hook
 // The kernels of one round (they do nothing when its plan holds no subset);
 // with use_cond it also sets the loop graph's condition (1 while big subsets
 // remain).
-cudaError_t launch_big_round(int logv, BigCtl* ctl, uint32_t R_max, uint32_t sms, uint64_t cond_handle, bool use_cond,
-                             cudaStream_t st, const LaunchHook& hook);
+cudaError_t launch_big_round(int logv, bool dna, BigCtl* ctl, uint32_t R_max, uint32_t sms, uint64_t cond_handle,
+                             bool use_cond, cudaStream_t st, const LaunchHook& hook);
 // Kernels the loop graphs of this device have launched so far (their plan
 // kernels count them on the device; reading the count waits for the device).
 uint64_t graph_launch_count();
 
 // Persistent work-queue kernel (single-block S^5 steps).
-size_t queue_smem(int logv);
 cudaError_t queue_occupancy(int logv, int* blocks_per_sm);
 cudaError_t launch_queue(int logv, const SortCtx& c, uint32_t grid, cudaStream_t st, const LaunchHook& hook);
 

@@ -116,13 +116,13 @@ __device__ void block_excl_scan_smem(const uint32_t* in, uint32_t* out, uint32_t
 // time in a loop that is not unrolled: the look-ahead of the block sorts, eight
 // at once, took more registers than the step has to spare (20 M URLs: the
 // queue 455 -> 530 us, inline or as a call).
-template <int LOGV>
+template <int LOGV, bool DNA>
 __device__ __forceinline__ uint32_t queue_jump(const SortCtx& c, QueueSmem<LOGV>& s) {
-  constexpr uint32_t NT = kQueueThreads;
+  constexpr uint32_t NT = kQueueThreads, kDna = DNA ? 1u : 0u;
   const Task t = s.task;
   const SetDesc sd = c.sets[task_set(t)];
   Rec* recs = c.rec[task_par(t)] + t.begin;
-  const uint32_t kw = key_width(sd.dna);
+  const uint32_t kw = key_width(kDna);
   if (t.depth + kw * kLookWindows > kMaxDepth) return t.depth;
   const uint64_t key = s.sm.sample[0];
   bool differs = false;
@@ -137,11 +137,11 @@ __device__ __forceinline__ uint32_t queue_jump(const SortCtx& c, QueueSmem<LOGV>
       const uint64_t off = rec_offset(sd, wide, recs[p].idx, recs[p].off);
 #pragma unroll 1
       for (uint32_t q = 0; q < (uint32_t)kLookWindows / 2; ++q) {
-        const u128 k = load_key128(sd.chars, off, t.depth + kw * (2 * q + 1), sd.cap, sd.dna);
+        const u128 k = load_key128(sd.chars, off, t.depth + kw * (2 * q + 1), sd.cap, kDna);
         if (lead) s.lead[q] = k;
         const u128 l = s.lead[q];
-        if (k != l || KeyOps<u128>::end(k, sd.dna)) {
-          const bool first = k_hi(k) != k_hi(l) || key_end(k_hi(k), sd.dna);
+        if (k != l || KeyOps<u128>::end(k, kDna)) {
+          const bool first = k_hi(k) != k_hi(l) || key_end(k_hi(k), kDna);
           atomicMin(&s.jstop, 2 * q + (first ? 0u : 1u));
           break;
         }
@@ -151,18 +151,18 @@ __device__ __forceinline__ uint32_t queue_jump(const SortCtx& c, QueueSmem<LOGV>
   }
   const uint32_t nd = t.depth + kw * (s.jstop + 1);
   for (uint32_t p = threadIdx.x; p < t.len; p += NT)
-    recs[p].key = load_key(sd.chars, rec_offset(sd, wide, recs[p].idx, recs[p].off), nd, sd.cap, sd.dna);
+    recs[p].key = load_key(sd.chars, rec_offset(sd, wide, recs[p].idx, recs[p].off), nd, sd.cap, kDna);
   __syncthreads();
   return nd;
 }
 
 // The sampling of the step on the block's task (and the zeroing of its
 // counters); returns whether the whole sample is one key without an end.
-template <int LOGV>
+template <int LOGV, bool DNA>
 __device__ __forceinline__ bool queue_sample(const SortCtx& c, QueueSmem<LOGV>& s) {
   using Gm = Geo<LOGV>;
   const Task t = s.task;
-  const uint32_t dna = c.sets[task_set(t)].dna;
+  constexpr uint32_t dna = DNA ? 1u : 0u;
   for (uint32_t b = threadIdx.x; b < Gm::KP; b += kQueueThreads) {
     s.hist[b] = 0;
     if (b <= Gm::V) s.u.lc.below[b] = s.u.lc.above[b] = 0;
@@ -178,10 +178,10 @@ __device__ __forceinline__ bool queue_sample(const SortCtx& c, QueueSmem<LOGV>& 
 // Returns this thread's share of the step's algorithmic bytes: the sample,
 // cache 8 read + bucket index 2 written per record while classifying, and the
 // bytes of each record's move.
-template <int LOGV>
+template <int LOGV, bool DNA>
 __device__ unsigned long long queue_step(const SortCtx& c, const Task& t, QueueSmem<LOGV>& s) {
   using Gm = Geo<LOGV>;
-  constexpr uint32_t NT = kQueueThreads;
+  constexpr uint32_t NT = kQueueThreads, kDna = DNA ? 1u : 0u;
   const SetDesc sd = c.sets[task_set(t)];
   const uint32_t par = task_par(t);
   const Rec* recs = c.rec[par] + t.begin;
@@ -205,11 +205,11 @@ __device__ unsigned long long queue_step(const SortCtx& c, const Task& t, QueueS
         if (!with_lcp || (b & 1u)) return;
         const uint32_t r = b >> 1;
         if (r > 0) {
-          const uint32_t l = key_lcp(k, sp.x[r - 1], sd.dna);
+          const uint32_t l = key_lcp(k, sp.x[r - 1], kDna);
           if (l > s.u.lc.below[r]) atomicMax(&s.u.lc.below[r], l);
         }
         if (r < Gm::V) {
-          const uint32_t l = key_lcp(k, sp.x[r], sd.dna);
+          const uint32_t l = key_lcp(k, sp.x[r], kDna);
           if (l > s.u.lc.above[r]) atomicMax(&s.u.lc.above[r], l);
         }
       });
@@ -233,7 +233,7 @@ __device__ unsigned long long queue_step(const SortCtx& c, const Task& t, QueueS
       const uint32_t pb = last_set_before(s.u.lc.used, some, b);
       if (pb == kNone) continue;
       const uint32_t ra = pb >> 1, rb = (b & 1u) ? b >> 1 : (b >> 1) - 1;
-      uint32_t l = key_lcp(sp.x[ra], sp.x[rb], sd.dna);
+      uint32_t l = key_lcp(sp.x[ra], sp.x[rb], kDna);
       if (!(pb & 1u)) l = min(l, s.u.lc.above[ra]);
       if (!(b & 1u)) l = min(l, s.u.lc.below[b >> 1]);
       sd.lcp[t.begin + s.bstart[b] - sd.base] = t.depth + l;
@@ -242,7 +242,7 @@ __device__ unsigned long long queue_step(const SortCtx& c, const Task& t, QueueS
   }
   for (uint32_t b = threadIdx.x; b < Gm::K; b += NT) {
     const uint32_t size = s.hist[b];
-    s.desc[b] = size ? bucket_desc<LOGV>(b, size, t.depth, sp, sd.dna) : kFin;
+    s.desc[b] = size ? bucket_desc<LOGV>(b, size, t.depth, sp, kDna) : kFin;
     s.hist[b] = t.begin + s.bstart[b];
   }
   __syncthreads();
@@ -263,7 +263,7 @@ __device__ unsigned long long queue_step(const SortCtx& c, const Task& t, QueueS
         s.tb, tl, R, s.hist, s.u.cntw,
         [&](const uint32_t(&pp)[kQueueMoveBatch], const uint32_t(&bb)[kQueueMoveBatch],
             const uint32_t(&dd)[kQueueMoveBatch]) {
-          bytes += move_batch<kQueueMoveBatch>(c, sd, wide, par, src0, t.depth, s.desc,
+          bytes += move_batch<kQueueMoveBatch, DNA>(c, sd, wide, par, src0, t.depth, s.desc,
                                                [&](uint32_t b) { return t.begin + s.bstart[b]; }, pp, bb, dd);
         });
   }
@@ -279,7 +279,9 @@ __device__ unsigned long long queue_step(const SortCtx& c, const Task& t, QueueS
   return bytes;
 }
 
-template <int LOGV>
+// (the character encoding is fixed per instance: at 64 registers the branches on
+// it cost spills, 372 -> 357 us in the suffix array of 4 M characters)
+template <int LOGV, bool DNA>
 __global__ void __launch_bounds__(kQueueThreads, kQueueBlocks) k_queue(SortCtx c) {
   extern __shared__ __align__(16) uint8_t smem[];
   QueueSmem<LOGV>& s = *reinterpret_cast<QueueSmem<LOGV>*>(smem);
@@ -288,15 +290,15 @@ __global__ void __launch_bounds__(kQueueThreads, kQueueBlocks) k_queue(SortCtx c
     if (threadIdx.x == 0) s.got = claim_task(c.mq, &s.task, c.status, c.wait_ns) ? 1u : 0u;
     __syncthreads();
     if (!s.got) break;
-    while (queue_sample<LOGV>(c, s)) {
-      const uint32_t nd = queue_jump<LOGV>(c, s);
+    while (queue_sample<LOGV, DNA>(c, s)) {
+      const uint32_t nd = queue_jump<LOGV, DNA>(c, s);
       if (nd == s.task.depth) break;
       __syncthreads();
       if (threadIdx.x == 0) s.task.depth = nd;
       __syncthreads();
     }
     const Task t = s.task;
-    bytes += queue_step<LOGV>(c, t, s);
+    bytes += queue_step<LOGV, DNA>(c, t, s);
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
@@ -306,62 +308,50 @@ __global__ void __launch_bounds__(kQueueThreads, kQueueBlocks) k_queue(SortCtx c
   account(c, kKQueue, bytes);
 }
 
-template <int LOGV>
+template <int LOGV, bool DNA>
 cudaError_t set_queue_attr() {
-  static cudaError_t e = cudaFuncSetAttribute(k_queue<LOGV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  static cudaError_t e = cudaFuncSetAttribute(k_queue<LOGV, DNA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)sizeof(QueueSmem<LOGV>));
   return e;
 }
 
-}  // namespace
+template <int LOGV>
+cudaError_t occupancy_t(int* blocks_per_sm) {
+  if (cudaError_t e = set_queue_attr<LOGV, false>()) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_queue<LOGV, false>, kQueueThreads,
+                                                       sizeof(QueueSmem<LOGV>));
+}
 
-size_t queue_smem(int logv) {
+template <int LOGV, bool DNA>
+cudaError_t launch_queue_t(const SortCtx& c, uint32_t grid, cudaStream_t st, const LaunchHook& hook) {
+  if (cudaError_t e = set_queue_attr<LOGV, DNA>()) return e;
+  hook.run("queue", [&] { k_queue<LOGV, DNA><<<grid, kQueueThreads, sizeof(QueueSmem<LOGV>), st>>>(c); });
+  return cudaGetLastError();
+}
+
+template <bool DNA>
+cudaError_t launch_queue_d(int logv, const SortCtx& c, uint32_t grid, cudaStream_t st, const LaunchHook& hook) {
   switch (logv) {
-    case 7: return sizeof(QueueSmem<7>);
-    case 8: return sizeof(QueueSmem<8>);
-    case 9: return sizeof(QueueSmem<9>);
-    default: return sizeof(QueueSmem<10>);
+    case 7: return launch_queue_t<7, DNA>(c, grid, st, hook);
+    case 8: return launch_queue_t<8, DNA>(c, grid, st, hook);
+    case 9: return launch_queue_t<9, DNA>(c, grid, st, hook);
+    default: return launch_queue_t<10, DNA>(c, grid, st, hook);
   }
 }
 
+}  // namespace
+
 cudaError_t queue_occupancy(int logv, int* blocks_per_sm) {
   switch (logv) {
-    case 7:
-      if (cudaError_t e = set_queue_attr<7>()) return e;
-      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_queue<7>, kQueueThreads, sizeof(QueueSmem<7>));
-    case 8:
-      if (cudaError_t e = set_queue_attr<8>()) return e;
-      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_queue<8>, kQueueThreads, sizeof(QueueSmem<8>));
-    case 9:
-      if (cudaError_t e = set_queue_attr<9>()) return e;
-      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_queue<9>, kQueueThreads, sizeof(QueueSmem<9>));
-    default:
-      if (cudaError_t e = set_queue_attr<10>()) return e;
-      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_queue<10>, kQueueThreads,
-                                                           sizeof(QueueSmem<10>));
+    case 7: return occupancy_t<7>(blocks_per_sm);
+    case 8: return occupancy_t<8>(blocks_per_sm);
+    case 9: return occupancy_t<9>(blocks_per_sm);
+    default: return occupancy_t<10>(blocks_per_sm);
   }
 }
 
 cudaError_t launch_queue(int logv, const SortCtx& c, uint32_t grid, cudaStream_t st, const LaunchHook& hook) {
-  switch (logv) {
-    case 7:
-      if (cudaError_t e = set_queue_attr<7>()) return e;
-      hook.run("queue", [&] { k_queue<7><<<grid, kQueueThreads, sizeof(QueueSmem<7>), st>>>(c); });
-      break;
-    case 8:
-      if (cudaError_t e = set_queue_attr<8>()) return e;
-      hook.run("queue", [&] { k_queue<8><<<grid, kQueueThreads, sizeof(QueueSmem<8>), st>>>(c); });
-      break;
-    case 9:
-      if (cudaError_t e = set_queue_attr<9>()) return e;
-      hook.run("queue", [&] { k_queue<9><<<grid, kQueueThreads, sizeof(QueueSmem<9>), st>>>(c); });
-      break;
-    default:
-      if (cudaError_t e = set_queue_attr<10>()) return e;
-      hook.run("queue", [&] { k_queue<10><<<grid, kQueueThreads, sizeof(QueueSmem<10>), st>>>(c); });
-      break;
-  }
-  return cudaGetLastError();
+  return c.dna ? launch_queue_d<true>(logv, c, grid, st, hook) : launch_queue_d<false>(logv, c, grid, st, hook);
 }
 
 }  // namespace ss

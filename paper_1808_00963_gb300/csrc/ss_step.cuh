@@ -460,7 +460,7 @@ __device__ void tile_scatter(const uint16_t* tb, uint32_t tl, uint32_t R, uint32
 // + record 16 read (the record carries the string's offset); finished: perm 4
 // (+ lcp 4) written; open: record 16 written, plus 8 characters read when the
 // cache is reloaded.
-template <int MB, typename First>
+template <int MB, bool DNA, typename First>
 __device__ __forceinline__ uint32_t move_batch(const SortCtx& c, const SetDesc& sd, uint32_t wide, uint32_t par,
                                                uint32_t src0, uint32_t depth, const uint32_t* desc,
                                                First&& bucket_first, const uint32_t (&pp)[MB],
@@ -490,7 +490,7 @@ __device__ __forceinline__ uint32_t move_batch(const SortCtx& c, const SetDesc& 
     off[u] = 0;
     if (pp[u] != kInvalid && !(ds[u] & kFin) && (ds[u] & kLow30) != depth) {
       off[u] = rec_offset(sd, wide, id[u], o32[u]);
-      if (!sd.dna) issue_chars(sd.chars, off[u], ds[u] & kLow30, sd.cap, 8, ww[u]);
+      if (!DNA) issue_chars(sd.chars, off[u], ds[u] & kLow30, sd.cap, 8, ww[u]);
     }
   }
 #pragma unroll
@@ -511,7 +511,7 @@ __device__ __forceinline__ uint32_t move_batch(const SortCtx& c, const SetDesc& 
     uint64_t k = key[u];
     bytes += 34;
     if (nd != depth) {
-      k = sd.dna ? dna_key(sd.chars, off[u], nd, sd.cap) : finish_chars8(ww[u], sd.chars, off[u], nd, sd.cap);
+      k = DNA ? dna_key(sd.chars, off[u], nd, sd.cap) : finish_chars8(ww[u], sd.chars, off[u], nd, sd.cap);
       bytes += 8;
     }
     store_rec(c.rec[par ^ 1] + dest, k, id[u], o32[u]);
@@ -530,7 +530,7 @@ __device__ __forceinline__ uint32_t move_batch(const SortCtx& c, const SetDesc& 
 // Returns the algorithmic bytes: bucket index 2 + wide record 24 read;
 // finished: perm 4 (+ lcp 4) written; open: 24 (wide) or 16 (narrow) written,
 // plus 16 (wide) or 8 (narrow) characters read when gathered.
-template <int MB, typename First>
+template <int MB, bool DNA, typename First>
 __device__ __forceinline__ uint32_t move_batch_wide(const SortCtx& c, const SetDesc& sd, uint32_t wide,
                                                     uint32_t par, uint32_t src0, uint32_t depth, const uint32_t* desc,
                                                     First&& bucket_first, const uint32_t (&pp)[MB],
@@ -568,9 +568,9 @@ __device__ __forceinline__ uint32_t move_batch_wide(const SortCtx& c, const SetD
     const uint32_t adv = (d & kLow30) - depth;
     const uint32_t size = bucket_first(bb[u] + 1) - bucket_first(bb[u]);
     to_wide[u] = c.big_enabled && size > c.big_threshold;
-    const bool derive = to_wide[u] ? adv == 0 : (sd.dna ? (adv == 0 || adv == kDnaWidth) : adv <= 8);
+    const bool derive = to_wide[u] ? adv == 0 : (DNA ? (adv == 0 || adv == kDnaWidth) : adv <= 8);
     how[u] = derive ? kKeep : kGather;
-    if (!derive && !sd.dna)
+    if (!derive && !DNA)
       issue_chars(sd.chars, rec_offset(sd, wide, wi[u].x, wi[u].y), d & kLow30, sd.cap, to_wide[u] ? 16 : 8, ww[u]);
   }
 #pragma unroll
@@ -590,7 +590,7 @@ __device__ __forceinline__ uint32_t move_batch_wide(const SortCtx& c, const SetD
     const uint32_t adv = nd - depth;
     u128 k = key[u];
     if (how[u] == kGather) {
-      if (sd.dna) {
+      if (DNA) {
         const uint64_t o = rec_offset(sd, wide, wi[u].x, wi[u].y);
         k = to_wide[u] ? load_key128(sd.chars, o, nd, sd.cap, 1u) : make_k(dna_key(sd.chars, o, nd, sd.cap), 0);
       } else {
@@ -609,7 +609,7 @@ __device__ __forceinline__ uint32_t move_batch_wide(const SortCtx& c, const SetD
     } else {
       bytes += 42;
       // a gathered narrow key is the first half; a kept one is cut out of the wide key
-      const uint64_t nk = how[u] == kGather ? k_hi(k) : (sd.dna ? (adv ? k_lo(k) : k_hi(k)) : narrow_at(k, adv));
+      const uint64_t nk = how[u] == kGather ? k_hi(k) : (DNA ? (adv ? k_lo(k) : k_hi(k)) : narrow_at(k, adv));
       store_rec(c.rec[par ^ 1] + dest, nk, wi[u].x, wi[u].y);
     }
   }
