@@ -788,7 +788,19 @@ ss_status ss_distinguishing(const uint8_t* chars, const uint64_t* offsets, uint6
 
 // ---- K-way LCP merge ------------------------------------------------------------------
 
-static uint32_t merge_step(uint32_t sample_step) { return sample_step ? sample_step : 64; }
+// The default sample step.  A lane merges a piece of at most two steps of
+// records one after the other, each waiting for the next record, so a round
+// takes as long as its longest pieces times the passes over the lanes: the step
+// makes 9/10 as many pieces as the GPU holds lanes, and is never below 3
+// (a sample costs a binary search).  Measured against the fixed step of 64:
+// 20 M URLs in 16 runs 3875 -> 3598 us (136: 3525, 128, one piece more than
+// lanes: 3744), 5 M 1356 -> 1204, 1 M in 8 runs 766 -> 379, 200 k 712 -> 193,
+// 20 k 693 -> 159.
+static uint32_t merge_step(uint32_t sample_step, uint64_t total) {
+  if (sample_step) return sample_step;
+  constexpr uint64_t kPieces = 152ull * kMergeLanesPerSm * 9 / 10;
+  return (uint32_t)std::max<uint64_t>(3, (total + kPieces - 1) / kPieces);
+}
 
 static ss_status merge_geometry(const ss_run* runs, uint32_t num_runs, uint32_t sample_step, uint64_t* total,
                                 uint32_t* S) {
@@ -802,7 +814,7 @@ static ss_status merge_geometry(const ss_run* runs, uint32_t num_runs, uint32_t 
   }
   if (t >= 0xFFFFFFFFull) return SS_ERR_TOO_LARGE;
   *total = t;
-  *S = merge_step(sample_step);
+  *S = merge_step(sample_step, t);
   return SS_OK;
 }
 

@@ -148,6 +148,8 @@ cudaError_t launch_distinguishing(const uint8_t* chars, const uint64_t* offsets,
 // K-way LCP merge of sorted runs (ss_merge.cu): ceil(log2 K) rounds of
 // pairwise LCP merges over 32-byte records.
 constexpr uint32_t kMergeMaxRuns = 64;
+constexpr uint32_t kMergeBlock = 128, kMergeBlocksPerSm = 8;
+constexpr uint32_t kMergeLanesPerSm = kMergeBlock * kMergeBlocksPerSm;
 
 struct MergeRec {
   uint64_t w0, w1;   // the string's characters [h, h + 16), first one most significant

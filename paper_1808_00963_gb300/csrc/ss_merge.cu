@@ -37,7 +37,6 @@ namespace ss {
 
 namespace {
 
-constexpr uint32_t kMergeBlock = 128;
 constexpr uint32_t kNoSample = 0xFFFFFFFFu;
 
 __device__ __forceinline__ uint64_t cache_at(const uint8_t* chars, uint32_t cap, uint64_t off, uint32_t h) {
@@ -245,7 +244,7 @@ __device__ __forceinline__ uint32_t last_sample_below(const MergeRoundArgs& a, u
 // advance of the winner are selects and predicated loads), so lanes diverge
 // only where a comparison has to read past the 16 cached characters; a lane
 // whose piece is done idles until the longest piece of its warp is.
-__global__ void __launch_bounds__(kMergeBlock) k_merge_round(MergeRoundArgs a) {
+__global__ void __launch_bounds__(kMergeBlock, kMergeBlocksPerSm) k_merge_round(MergeRoundArgs a) {
   const uint32_t npairs = (a.ncur + 1) / 2;
   const uint32_t npieces = a.nsamples + npairs;
   const uint32_t lane = lane_id();
