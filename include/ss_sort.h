@@ -266,7 +266,7 @@ size_t ss_merge_workspace_size(const ss_run* runs, uint32_t num_runs, uint32_t s
  *   out_lcp  uint32[n] (device) or NULL: out_lcp[0] = 0, out_lcp[j] = lcp of
  *            the suffixes out_sa[j-1] and out_sa[j].
  * Synchronous: waits for the result (the host reads the number of unsorted
- * suffixes after each round).  Device memory of about 63 bytes per text
+ * suffixes after each round).  Device memory of about 59 bytes per text
  * character is taken from the stream-ordered pool for the call, plus, with
  * an LCP output, 4 bytes per character for every round (the names of each
  * round: an LCP above initial_depth is found by descending through them,

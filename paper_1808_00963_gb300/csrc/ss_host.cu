@@ -934,11 +934,12 @@ ss_status ss_suffix_array(const uint8_t* text, uint64_t n, uint32_t* out_sa, uin
   ss_status s = device_info(dev);
   if (s != SS_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // workspace: offsets, capped LCPs (unless out_lcp holds them), names, group
-  // starts, flags, two compacted position lists, scan totals, and per round
-  // the members, their encoded name pairs, offsets and sorted order / LCPs
+  // workspace: offsets, capped LCPs (unless out_lcp holds them), names, two
+  // lists of unfinished members (positions and groups), the totals of the
+  // naming passes, and per round the members, their second names and new
+  // groups, or their encoded name pairs, offsets and sorted order / LCPs
   const size_t a4 = align256(n * 4), a8 = align256(n * 8);
-  const size_t tot_b = align256(sa_scan_totals(n) * 4);
+  const size_t tot_b = align256(kSaScanBlocks * sizeof(uint2)) + 256;
   const size_t need = a8 + (out_lcp ? 0 : a4) + 7 * a4 + tot_b + align256(n * 11 + 16) + a8;
   uint8_t* ws = nullptr;
   if (cudaMallocAsync(reinterpret_cast<void**>(&ws), need, st) != cudaSuccess) return SS_ERR_OOM;
@@ -947,23 +948,22 @@ ss_status ss_suffix_array(const uint8_t* text, uint64_t n, uint32_t* out_sa, uin
   uint64_t* off = reinterpret_cast<uint64_t*>(take(a8));
   uint32_t* lcp0 = out_lcp ? out_lcp : reinterpret_cast<uint32_t*>(take(a4));
   uint32_t* isa = reinterpret_cast<uint32_t*>(take(a4));
-  uint32_t* gs = reinterpret_cast<uint32_t*>(take(a4));
-  uint32_t* flag = reinterpret_cast<uint32_t*>(take(a4));
   uint32_t* cpos[2] = {reinterpret_cast<uint32_t*>(take(a4)), reinterpret_cast<uint32_t*>(take(a4))};
+  uint32_t* group[2] = {reinterpret_cast<uint32_t*>(take(a4)), reinterpret_cast<uint32_t*>(take(a4))};
   uint32_t* member = reinterpret_cast<uint32_t*>(take(a4));
   uint32_t* perm2 = reinterpret_cast<uint32_t*>(take(a4));
-  uint32_t* tot = reinterpret_cast<uint32_t*>(take(tot_b));
+  uint2* totals = reinterpret_cast<uint2*>(take(tot_b));
   uint8_t* enc = take(align256(n * 11 + 16));
   uint64_t* eoff = reinterpret_cast<uint64_t*>(take(a8));
   uint32_t* lcp2 = reinterpret_cast<uint32_t*>(off);  // the offsets of round 0 are dead by then
   const LaunchHook hook{st};
-  auto grid_for = [&](uint64_t m) {
-    return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((m + 255) / 256, (uint64_t)dev.sms * 32));
-  };
-  auto read_u32 = [&](const uint32_t* d, uint32_t* h) {
-    return cudaMemcpyAsync(h, d, 4, cudaMemcpyDeviceToHost, st) == cudaSuccess &&
-           cudaStreamSynchronize(st) == cudaSuccess;
-  };
+  const uint32_t sms = (uint32_t)dev.sms;
+  // what a naming pass leaves, in host memory: members left, whether a group is large
+  if (t_down.reserve(kCtrlBytes) != SS_OK) {  // (as much as the sorts may ask for: it stays where it is)
+    cudaFreeAsync(ws, st);
+    return SS_ERR_OOM;
+  }
+  volatile uint32_t* result = static_cast<uint32_t*>(t_down.p);
   SaArgs x;
   x.text = text;
   x.n = n;
@@ -971,9 +971,10 @@ ss_status ss_suffix_array(const uint8_t* text, uint64_t n, uint32_t* out_sa, uin
   x.sa = out_sa;
   x.lcp = lcp0;
   x.isa = isa;
-  x.gs = gs;
-  x.flag = flag;
   x.h = h0;
+  x.totals = totals;
+  x.result = static_cast<uint32_t*>(t_down.p);
+  x.listed = reinterpret_cast<uint32_t*>(totals + kSaScanBlocks);
   // with an LCP output: the names after every round, for the LCPs above h0
   std::vector<uint32_t*> snaps;
   auto snapshot = [&]() {
@@ -984,7 +985,7 @@ ss_status ss_suffix_array(const uint8_t* text, uint64_t n, uint32_t* out_sa, uin
     snaps.push_back(q);
     return cudaMemcpyAsync(q, isa, n * 4, cudaMemcpyDeviceToDevice, st) == cudaSuccess;
   };
-  bool ok = sa_launch(SaKernel::kIota, x, grid_for(n), st, hook) == cudaSuccess;
+  bool ok = sa_launch(SaKernel::kIota, x, sms, st, hook) == cudaSuccess;
   // round 0: the string sort by the first h0 characters
   if (ok) {
     ss_options o{};
@@ -996,76 +997,64 @@ ss_status ss_suffix_array(const uint8_t* text, uint64_t n, uint32_t* out_sa, uin
     s = sort_device(text, off, n, out_sa, lcp0, &o, st);
     ok = s == SS_OK;
   }
+  // a naming pass, its outcome, and the names kept for the LCPs
   uint32_t M = 0;
+  bool large = false;
+  auto named = [&](SaKernel k, const SaArgs& a) {
+    result[0] = result[1] = 0;
+    if (sa_launch(k, a, sms, st, hook) != cudaSuccess || !snapshot() || cudaStreamSynchronize(st) != cudaSuccess)
+      return false;
+    M = result[0];
+    large = result[1] != 0;
+    return true;
+  };
+  int cur = 0;
   if (ok) {
-    ok = sa_launch(SaKernel::kHeads0, x, grid_for(n), st, hook) == cudaSuccess &&
-         sa_scan_max(gs, n, tot, st, hook) == cudaSuccess &&
-         sa_launch(SaKernel::kName0, x, grid_for(n), st, hook) == cudaSuccess &&
-         sa_scan_sum(flag, n, tot, st, hook) == cudaSuccess && read_u32(flag + n - 1, &M) && snapshot();
-    SaArgs c = x;
-    c.vals = nullptr;
-    c.out = cpos[0];
-    if (ok && M) ok = sa_launch(SaKernel::kCompact, c, grid_for(n), st, hook) == cudaSuccess;
+    x.out = cpos[0];
+    x.group_out = group[0];
+    ok = named(SaKernel::kNameFirst, x);
   }
   // doubling rounds over the unfinished groups (Observation 8.1)
   uint64_t h = h0;
-  int cur = 0;
   while (ok && s == SS_OK && M > 0) {
     SaArgs r = x;
     r.M = M;
     r.h = (uint32_t)std::min<uint64_t>(h, 0xFFFFFFFFull);
     r.cpos = cpos[cur];
+    r.group = group[cur];
+    r.out = cpos[cur ^ 1];
+    r.group_out = group[cur ^ 1];
     r.member = member;
+    r.second = perm2;
+    r.new_group = lcp2;
     r.enc = enc;
     r.eoff = eoff;
     r.perm2 = perm2;
     r.lcp2 = lcp2;
-    ok = sa_launch(SaKernel::kEncode, r, grid_for(M), st, hook) == cudaSuccess;
-    if (ok) {
-      ss_options o2{};
-      if (M > kRankMax) {  // (smaller sets are ranked by counting)
-        o2.small_cutoff = kSaSmallCutoff;
-        o2.big_threshold = kSaBigThreshold;
+    if (large) {
+      ok = sa_launch(SaKernel::kEncode, r, sms, st, hook) == cudaSuccess;
+      if (ok) {
+        ss_options o2{};
+        if (M > kRankMax) {  // (smaller sets are ranked by counting)
+          o2.small_cutoff = kSaSmallCutoff;
+          o2.big_threshold = kSaBigThreshold;
+        }
+        s = sort_device(enc, eoff, M, perm2, lcp2, &o2, st);
+        ok = s == SS_OK;
       }
-      s = sort_device(enc, eoff, M, perm2, lcp2, &o2, st);
-      ok = s == SS_OK;
     }
-    uint32_t M2 = 0;
-    if (ok)
-      ok = sa_launch(SaKernel::kApply, r, grid_for(M), st, hook) == cudaSuccess &&
-           sa_scan_max(gs, M, tot, st, hook) == cudaSuccess &&
-           sa_launch(SaKernel::kRename, r, grid_for(M), st, hook) == cudaSuccess &&
-           sa_scan_sum(flag, M, tot, st, hook) == cudaSuccess && read_u32(flag + M - 1, &M2) && snapshot();
-    if (ok && M2) {
-      SaArgs c = r;
-      c.n = M;
-      c.vals = cpos[cur];
-      c.out = cpos[cur ^ 1];
-      ok = sa_launch(SaKernel::kCompact, c, grid_for(M), st, hook) == cudaSuccess;
-    }
-    if (ok && M2 && h >= n) ok = false;  // cannot happen: every group is a singleton by depth n
-    M = M2;
+    if (ok) ok = named(large ? SaKernel::kNamePairs : SaKernel::kGroups, r);
+    if (ok && M && h >= n) ok = false;  // cannot happen: every group is a singleton by depth n
     cur ^= 1;
     h *= 2;
   }
-  if (ok && s == SS_OK && out_lcp) {
-    // LCPs of at least h0: list those positions, then one warp each
+  if (ok && s == SS_OK && out_lcp) {  // LCPs of at least h0
     SaArgs l = x;
     l.lcp_out = out_lcp;
+    l.out = cpos[0];
     l.snaps.count = (uint32_t)snaps.size();
     for (size_t k = 0; k < snaps.size(); ++k) l.snaps.p[k] = snaps[k];
-    uint32_t L = 0;
-    ok = sa_launch(SaKernel::kLongFlags, l, grid_for(n), st, hook) == cudaSuccess &&
-         sa_scan_sum(flag, n, tot, st, hook) == cudaSuccess && read_u32(flag + n - 1, &L);
-    if (ok && L) {
-      SaArgs c = x;
-      c.vals = nullptr;
-      c.out = cpos[0];
-      l.cpos = cpos[0];
-      l.M = L;
-      ok = sa_launch(SaKernel::kCompact, c, grid_for(n), st, hook) == cudaSuccess &&
-           sa_launch(SaKernel::kLcp, l, grid_for(32ull * L), st, hook) == cudaSuccess;
-    }
+    ok = sa_launch(SaKernel::kLcp, l, sms, st, hook) == cudaSuccess;
   }
   for (uint32_t* q : snaps) cudaFreeAsync(q, st);
   cudaFreeAsync(ws, st);

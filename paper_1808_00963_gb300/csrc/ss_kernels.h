@@ -202,7 +202,8 @@ cudaError_t launch_layout_check(const uint8_t* chars, uint64_t chars_len, const 
                                 uint32_t* bad, uint32_t sms, cudaStream_t st, const LaunchHook& hook);
 
 // Suffix array by prefix doubling (ss_sa.cu).
-enum class SaKernel { kIota, kHeads0, kName0, kCompact, kEncode, kApply, kRename, kLongFlags, kLcp };
+enum class SaKernel { kIota, kNameFirst, kEncode, kNamePairs, kGroups, kLcp };
+constexpr uint32_t kSaScanBlocks = 1024;  // most blocks of the naming passes (one total each)
 
 // Name arrays of the suffixes after each round (ISA^{h0 2^k}, k = 0..count-1),
 // kept for the LCPs above h0.
@@ -214,20 +215,24 @@ struct SaSnaps {
 
 struct SaArgs {
   const uint8_t* text = nullptr;
-  uint64_t n = 0;             // strings the kernel runs over (suffixes, or members M)
-  uint32_t h = 0;             // current depth (h0 for kHeads0 / kName0 / kLcp)
-  uint32_t M = 0;
+  uint64_t n = 0;                 // suffixes
+  uint32_t h = 0;                 // current depth (h0 for kNameFirst / kLcp)
+  uint32_t M = 0;                 // members of unfinished groups
   uint64_t* off = nullptr;
   uint32_t* sa = nullptr;
   const uint32_t* lcp = nullptr;  // capped LCPs of the first sort
   uint32_t* lcp_out = nullptr;    // final LCP array (holds the capped LCPs on entry)
   uint32_t* isa = nullptr;
-  uint32_t* gs = nullptr;
-  uint32_t* flag = nullptr;       // flags, then their inclusive sum
-  const uint32_t* vals = nullptr;
-  uint32_t* out = nullptr;
-  const uint32_t* cpos = nullptr;
+  const uint32_t* cpos = nullptr;   // suffix array positions of the members, and their groups
+  const uint32_t* group = nullptr;
+  uint32_t* out = nullptr;          // the same for the next round (out: the long LCPs' positions for kLcp)
+  uint32_t* group_out = nullptr;
+  uint2* totals = nullptr;          // kSaScanBlocks
+  uint32_t* result = nullptr;       // host memory: members left, 1 if a group is large
+  uint32_t* listed = nullptr;       // kLcp: how many long LCPs
   uint32_t* member = nullptr;
+  uint32_t* second = nullptr;
+  uint32_t* new_group = nullptr;
   uint8_t* enc = nullptr;
   uint64_t* eoff = nullptr;
   const uint32_t* perm2 = nullptr;
@@ -235,9 +240,6 @@ struct SaArgs {
   SaSnaps snaps{};
 };
 
-size_t sa_scan_totals(uint64_t n);  // entries of the scan's tile-total buffer
-cudaError_t sa_scan_max(uint32_t* a, uint64_t n, uint32_t* tot, cudaStream_t st, const LaunchHook& hook);
-cudaError_t sa_scan_sum(uint32_t* a, uint64_t n, uint32_t* tot, cudaStream_t st, const LaunchHook& hook);
-cudaError_t sa_launch(SaKernel k, const SaArgs& x, uint32_t grid, cudaStream_t st, const LaunchHook& hook);
+cudaError_t sa_launch(SaKernel k, const SaArgs& x, uint32_t sms, cudaStream_t st, const LaunchHook& hook);
 
 }  // namespace ss
