@@ -488,15 +488,26 @@ __global__ void __launch_bounds__(kBlock) k_big_emit(BigCtl* ctl, cudaGraphCondi
   }
 }
 
+// Bound by the latency of the character gathers, each of which holds an L1 line
+// until it is there: the more shared memory a block takes, the fewer gathers
+// are in flight (12 KB more per block, 20 M URLs 4110 -> 4435 us; so the warps'
+// 16-bit counters).  A batch needs two dependent loads, its records and their
+// characters; the records of the next batch are copied to shared memory
+// meanwhile.  Counters of 16 bits and the copies: 20 M URLs 4098 -> 4017 us,
+// 512 sets 2036 -> 2015, 4 M DNA strings 937 -> 930; the copies with 32-bit counters
+// 4408, with three records per lane instead of two 4148 (before the copies).
 template <int LOGV, bool DNA>
 __global__ void __launch_bounds__(kBlock, 3) k_big_scatter(const BigCtl* __restrict__ ctl, uint32_t* __restrict__ work) {
   using Gm = Geo<LOGV>;
   extern __shared__ __align__(16) uint8_t smem[];
-  uint32_t* cntw = reinterpret_cast<uint32_t*>(smem);
-  uint32_t* base = cntw + kWarps * Gm::KP;
+  uint16_t* cntw = reinterpret_cast<uint16_t*>(smem);
+  uint32_t* base = reinterpret_cast<uint32_t*>(cntw + kWarps * Gm::KP);
   uint32_t* desc = base + Gm::KP;
   uint32_t* bfirst = desc + Gm::KP;
-  uint16_t* tb = reinterpret_cast<uint16_t*>(bfirst + Gm::KP);
+  // this lane's slots for the records of the warp's next batch
+  uint4* slot = reinterpret_cast<uint4*>(bfirst + Gm::KP) + threadIdx.x;
+  uint2* wslot = reinterpret_cast<uint2*>(slot + kWideMoveBatch * kBlock - threadIdx.x) + threadIdx.x;
+  uint16_t* tb = reinterpret_cast<uint16_t*>(wslot + kWideMoveBatch * kBlock - threadIdx.x);
   __shared__ uint32_t s_g;
   __shared__ uint32_t ts[kTileStartsMax];
   const uint32_t G = ctl->mv.G, tiles = ctl->mv.tiles, R = ctl->mv.R;
@@ -525,7 +536,22 @@ __global__ void __launch_bounds__(kBlock, 3) k_big_scatter(const BigCtl* __restr
     const uint32_t t0 = tile * T;
     const uint32_t tl = min(T, g.t.len - t0);
     const uint32_t par = task_par(g.t);
-    const uint16_t* bo = c.bucket_of + g.t.begin + t0;
+    const uint32_t src0 = g.t.begin + t0;
+    // records r0 * 32 ... of this warp's part of the tile, on their way to the slots
+    uint32_t ahead = 0;
+    auto fetch = [&](uint32_t r0) {
+#pragma unroll
+      for (uint32_t u = 0; u < (uint32_t)kWideMoveBatch; ++u) {
+        const uint32_t p = (threadIdx.x >> 5) * 32 * R + (r0 + u) * 32 + lane_id();
+        if (r0 + u < R && p < tl) {
+          copy_async<16>(slot + u * kBlock, c.rec[par] + src0 + p);
+          copy_async<8>(wslot + u * kBlock, c.wid[par] + src0 + p);
+        }
+      }
+      copy_async_commit();
+    };
+    fetch(0);
+    const uint16_t* bo = c.bucket_of + src0;
     for (uint32_t p = threadIdx.x; p < tl; p += kBlock) tb[p] = bo[p];
     const uint32_t* sc = ctl->counters + cnt_base(g) + tile;
     for (uint32_t b = threadIdx.x; b < Gm::K; b += kBlock) {
@@ -538,7 +564,6 @@ __global__ void __launch_bounds__(kBlock, 3) k_big_scatter(const BigCtl* __restr
     if (fresh && threadIdx.x == 0) bfirst[Gm::K] = g.t.begin + g.t.len;  // bucket sizes from neighbouring starts
     loaded = gi;
     __syncthreads();
-    const uint32_t src0 = g.t.begin + t0;
     const uint32_t depth = g.t.depth;
     const uint32_t wide = c.wide[task_set(g.t)];
     if (threadIdx.x == 0) bytes += (fresh ? 12ull : 4ull) * Gm::K;  // per-bucket tile offsets (+ descriptors and starts)
@@ -546,7 +571,19 @@ __global__ void __launch_bounds__(kBlock, 3) k_big_scatter(const BigCtl* __restr
         tb, tl, R, base, cntw,
         [&](const uint32_t(&pp)[kWideMoveBatch], const uint32_t(&bb)[kWideMoveBatch],
             const uint32_t(&dd)[kWideMoveBatch]) {
-          bytes += move_batch_wide<kWideMoveBatch, DNA>(c, sd, wide, par, src0, depth, desc,
+          auto load = [&](u128(&key)[kWideMoveBatch], uint2(&wi)[kWideMoveBatch]) {
+            copy_async_wait();
+#pragma unroll
+            for (int u = 0; u < kWideMoveBatch; ++u) {
+              if (pp[u] == kInvalid) continue;
+              key[u] = load_wkey(reinterpret_cast<const Rec*>(slot + u * kBlock));
+              wi[u] = wslot[u * kBlock];
+            }
+            __syncwarp();
+            ahead += kWideMoveBatch;
+            fetch(ahead);
+          };
+          bytes += move_batch_wide<kWideMoveBatch, DNA>(c, sd, wide, par, depth, desc, load,
                                                    [&](uint32_t b) { return bfirst[b]; }, pp, bb, dd);
         });
   }
@@ -689,7 +726,7 @@ size_t big_splitters_bytes(int logv) {
 
 size_t big_scatter_smem(int logv, uint32_t R) {
   const uint32_t KP = 2u << logv;
-  return (size_t)(kWarps * KP + 3 * KP) * 4 + (size_t)kBlock * R * 2;
+  return (size_t)kWarps * KP * 2 + (size_t)3 * KP * 4 + (size_t)kBlock * kWideMoveBatch * 24 + (size_t)kBlock * R * 2;
 }
 
 cudaError_t launch_big_plan(BigCtl* ctl, cudaStream_t st, const LaunchHook& hook) {

@@ -531,6 +531,16 @@ __device__ __forceinline__ uint64_t k_hi(u128 k) { return (uint64_t)(k >> 64); }
 __device__ __forceinline__ uint64_t k_lo(u128 k) { return (uint64_t)k; }
 __device__ __forceinline__ u128 make_k(uint64_t hi, uint64_t lo) { return ((u128)hi << 64) | lo; }
 
+// Copies of N bytes from global to shared memory that the thread waits for with
+// copy_async_wait (its own copies; all groups it has committed).
+template <int N>
+__device__ __forceinline__ void copy_async(void* dst, const void* src) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(N) : "memory");
+}
+__device__ __forceinline__ void copy_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
 __device__ __forceinline__ u128 load_wkey(const Rec* p) {
   const uint4 v = *reinterpret_cast<const uint4*>(p);
   return make_k(((uint64_t)v.y << 32) | v.x, ((uint64_t)v.w << 32) | v.z);

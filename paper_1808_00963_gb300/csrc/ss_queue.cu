@@ -44,7 +44,7 @@ struct QueueSmem {
       uint32_t above[Geo<LOGV>::V + 1];
       uint32_t used[64];           // bit i of word w: bucket 32 w + i is not empty
     } lc;
-    uint32_t cntw[kQueueWarps * Geo<LOGV>::KP];
+    uint16_t cntw[kQueueWarps * Geo<LOGV>::KP];
   } u;
   uint16_t tb[kMaxTile];           // bucket of each record of a tile
   u128 lead[kLookWindows / 2];     // look-ahead of a subset's first string

@@ -395,36 +395,42 @@ __device__ __forceinline__ uint32_t bucket_peers(uint32_t b, bool valid) {
 //   tb[0..tl)    bucket of each record of the tile (shared memory)
 //   base[b]      in: destination of the tile's first record of bucket b;
 //                out: base[b] + number of the tile's records in bucket b
-//   cntw         shared scratch, NT / 32 * KP uint32
+//   cntw         shared scratch, NT / 32 * KP uint16 (4-byte aligned)
 // Warp w owns records [w * 32R, (w + 1) * 32R) of the tile; inside a warp
 // ranks come from the lanes with the same bucket (bucket_peers), so equal
 // buckets keep input order.
 // move(p[], b[], dest[]) is called with MB rounds of one warp at a time
 // (p = kInvalid for lanes without a record).  Ends with __syncthreads().
+// cntw holds what is still to come of a bucket from this warp on, so that 16
+// bits are enough (a record goes to base[b] - left): half the shared memory
+// leaves the multi-block kernel 124 KB of L1 instead of 60.
+static_assert(kMaxTile <= 0xFFFF, "counts within a tile have 16 bits");
 template <int LOGV, uint32_t NT, int MB, typename Move>
 __device__ void tile_scatter(const uint16_t* tb, uint32_t tl, uint32_t R, uint32_t* base,
-                             uint32_t* cntw, Move&& move) {
+                             uint16_t* cntw, Move&& move) {
   using G = Geo<LOGV>;
   constexpr uint32_t kWarps = NT / 32;
   const uint32_t w = threadIdx.x >> 5, lane = lane_id();
-  for (uint32_t i = threadIdx.x; i < kWarps * G::KP; i += NT) cntw[i] = 0;
+  for (uint32_t i = threadIdx.x; i < kWarps * G::KP / 2; i += NT) reinterpret_cast<uint32_t*>(cntw)[i] = 0;
   __syncthreads();
-  uint32_t* mine = cntw + w * G::KP;
+  uint16_t* mine = cntw + w * G::KP;
   const uint32_t p0 = w * 32 * R;
   for (uint32_t r = 0; r < R; ++r) {
     const uint32_t p = p0 + r * 32 + lane;
-    if (p < tl) atomicAdd(&mine[tb[p]], 1u);  // counts only: no need to group equal buckets
+    if (p < tl) {  // counts only: no need to group equal buckets
+      const uint32_t b = tb[p];
+      atomicAdd(reinterpret_cast<uint32_t*>(mine) + (b >> 1), 1u << (16 * (b & 1u)));
+    }
   }
   __syncthreads();
   for (uint32_t b = threadIdx.x; b < G::K; b += NT) {
-    uint32_t run = base[b];
+    uint32_t run = 0;
 #pragma unroll
-    for (uint32_t ww = 0; ww < kWarps; ++ww) {
-      const uint32_t c = cntw[ww * G::KP + b];
-      cntw[ww * G::KP + b] = run;
-      run += c;
+    for (uint32_t ww = kWarps; ww-- > 0;) {
+      run += cntw[ww * G::KP + b];
+      cntw[ww * G::KP + b] = (uint16_t)run;
     }
-    base[b] = run;
+    base[b] += run;
   }
   __syncthreads();
   const uint32_t lt = lanemask_lt();
@@ -438,9 +444,10 @@ __device__ void tile_scatter(const uint16_t* tb, uint32_t tl, uint32_t R, uint32
       const uint32_t b = valid ? tb[p] : 0u;
       const uint32_t peers = bucket_peers<LOGV>(b, valid);
       uint32_t dest = 0;
-      if (valid) dest = mine[b] + __popc(peers & lt);
+      const uint32_t left = mine[b];  // records of the bucket not yet placed, this warp's and the later ones'
+      if (valid) dest = base[b] - left + __popc(peers & lt);
       __syncwarp();
-      if (valid && lane == (uint32_t)(__ffs(peers) - 1)) mine[b] += __popc(peers);
+      if (valid && lane == (uint32_t)(__ffs(peers) - 1)) mine[b] = (uint16_t)(left - __popc(peers));
       __syncwarp();
       pp[u] = valid ? p : kInvalid;
       bb[u] = b;
@@ -527,12 +534,13 @@ __device__ __forceinline__ uint32_t move_batch(const SortCtx& c, const SetDesc& 
 // (bytes), or is the first or second half of it (DNA codes, 0 or 21 deeper),
 // and gathered from the string otherwise.  bucket_first(b) is the position of
 // bucket b's first record (bucket_first(b + 1) - bucket_first(b) its size).
+// load(key, wi) gives the batch's wide keys and (idx, off).
 // Returns the algorithmic bytes: bucket index 2 + wide record 24 read;
 // finished: perm 4 (+ lcp 4) written; open: 24 (wide) or 16 (narrow) written,
 // plus 16 (wide) or 8 (narrow) characters read when gathered.
-template <int MB, bool DNA, typename First>
+template <int MB, bool DNA, typename Load, typename First>
 __device__ __forceinline__ uint32_t move_batch_wide(const SortCtx& c, const SetDesc& sd, uint32_t wide,
-                                                    uint32_t par, uint32_t src0, uint32_t depth, const uint32_t* desc,
+                                                    uint32_t par, uint32_t depth, const uint32_t* desc, Load&& load,
                                                     First&& bucket_first, const uint32_t (&pp)[MB],
                                                     const uint32_t (&bb)[MB], const uint32_t (&dd)[MB]) {
   constexpr uint32_t kSkip = 0, kFinal = 1, kKeep = 2, kGather = 3;  // what a record needs
@@ -543,15 +551,11 @@ __device__ __forceinline__ uint32_t move_batch_wide(const SortCtx& c, const SetD
   uint32_t bytes = 0;
 #pragma unroll
   for (int u = 0; u < MB; ++u) {
-    ds[u] = kFin;
+    ds[u] = pp[u] != kInvalid ? desc[bb[u]] : kFin;
     wi[u] = make_uint2(0, 0);
     key[u] = 0;
-    if (pp[u] != kInvalid) {
-      ds[u] = desc[bb[u]];
-      key[u] = load_wkey(c.rec[par] + src0 + pp[u]);
-      wi[u] = c.wid[par][src0 + pp[u]];
-    }
   }
+  load(key, wi);
   // what each record needs; the characters of every byte-string gather are
   // requested before any of them is used (one memory round trip for the batch)
   CharWords ww[MB];
