@@ -1,5 +1,6 @@
 """The multi-block distribution at its edges: tiles of 8 to 32 rounds that are
-full, ragged or all of one bucket (the largest counts), against the oracle."""
+full, ragged or all of one bucket (the largest counts), and subsets whose common prefix ends
+anywhere in a key, against the oracle."""
 import numpy as np
 import pytest
 
@@ -35,3 +36,22 @@ def test_tile_edges(rounds, extra, kinds):
     rows = words[rng.integers(0, kinds, n)]
     rows[rng.random(n) < 0.2, 17] = 122  # some differ behind the first 16 characters
     check(from_rows(rows), tile_rounds=rounds)
+
+
+@pytest.mark.parametrize("cap", [0, 7, 9, 12, 13, 16, 20])
+@pytest.mark.parametrize("alphabet", [b"ab", b"ACGT", None])
+def test_prefix_ends_inside_the_key(alphabet, cap):
+    # 40 subsets of 500 strings each: the strings of subset k agree in 6 + k % 12
+    # characters (DNA keys: up to three times as many)
+    rng = np.random.default_rng(cap)
+    letters = np.frombuffer(alphabet, np.uint8) if alphabet else np.arange(1, 256, dtype=np.uint8)
+    rows = letters[rng.integers(0, len(letters), (20000, 70))]
+    step = 3 if alphabet == b"ACGT" else 1
+    for k in range(40):
+        share = (6 + k % 12) * step
+        rows[500 * k:500 * (k + 1), :share] = rows[500 * k, :share]
+    rows[rng.random(20000) < 0.1, 11] = 0  # ends inside and before the shared part
+    rows = rows[rng.permutation(20000)]
+    check(from_rows(rows, cap))
+    if alphabet == b"ACGT":
+        check(from_rows(rows, cap), dna=True)
