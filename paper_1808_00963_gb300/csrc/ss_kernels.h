@@ -151,7 +151,7 @@ constexpr uint32_t kMergeMaxRuns = 64;
 constexpr uint32_t kMergeBlock = 128, kMergeBlocksPerSm = 8;
 constexpr uint32_t kMergeLanesPerSm = kMergeBlock * kMergeBlocksPerSm;
 
-struct MergeRec {
+struct alignas(32) MergeRec {
   uint64_t w0, w1;   // the string's characters [h, h + 16), first one most significant
   uint64_t off;      // string offset
   uint32_t idx;      // string index

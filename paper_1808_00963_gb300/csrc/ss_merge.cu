@@ -73,25 +73,23 @@ struct MRec {
 };
 constexpr uint64_t kOffMask = (1ull << 56) - 1;
 
+// A record is one 32-byte sector, read and written as one word of 32 bytes (as
+// two of 16: merge of 16 runs, 20 M URLs, 3632 -> 3609 us; reads that ask L2
+// for the rest of the line change nothing).
 __device__ __forceinline__ MRec load_mrec(const MergeRec* p) {
-  const uint4 a = __ldg(reinterpret_cast<const uint4*>(p));
-  const uint4 b = __ldg(reinterpret_cast<const uint4*>(p) + 1);
   MRec r;
-  r.w0 = ((uint64_t)a.y << 32) | a.x;
-  r.w1 = ((uint64_t)a.w << 32) | a.z;
-  const uint64_t o = ((uint64_t)b.y << 32) | b.x;
+  uint64_t o, ih;
+  asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(r.w0), "=l"(r.w1), "=l"(o), "=l"(ih) : "l"(p));
   r.off = o & kOffMask;
   r.miss = (uint32_t)(o >> 56);
-  r.idx = b.z;
-  r.h = b.w;
+  r.idx = (uint32_t)ih;
+  r.h = (uint32_t)(ih >> 32);
   return r;
 }
 
 __device__ __forceinline__ void store_mrec(MergeRec* p, const MRec& r) {
-  uint4* q = reinterpret_cast<uint4*>(p);
-  const uint64_t o = r.off | ((uint64_t)r.miss << 56);
-  q[0] = make_uint4((uint32_t)r.w0, (uint32_t)(r.w0 >> 32), (uint32_t)r.w1, (uint32_t)(r.w1 >> 32));
-  q[1] = make_uint4((uint32_t)o, (uint32_t)(o >> 32), r.idx, r.h);
+  const uint64_t o = r.off | ((uint64_t)r.miss << 56), ih = ((uint64_t)r.h << 32) | r.idx;
+  asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(r.w0), "l"(r.w1), "l"(o), "l"(ih) : "memory");
 }
 
 // Position (0..15) of the first zero byte of a 16-character cache (first
