@@ -426,7 +426,9 @@ __global__ void __launch_bounds__(kBlock) k_big_emit(BigCtl* ctl, cudaGraphCondi
                                                            uint32_t use_cond) {
   using Gm = Geo<LOGV>;
   constexpr uint32_t kParts = Gm::KP / kBlock;
-  const BigPlan plan = ctl->cur;
+  // (not cur: the last block replaces that one, and blocks that had to wait for
+  // a place on the GPU may start after it)
+  const BigPlan plan = ctl->mv;
   const uint32_t items = plan.G * kParts;
   const uint32_t blocks = max(1u, min(items, gridDim.x));  // blocks with work (or the one that ends the loop)
   if (blockIdx.x >= blocks) return;
@@ -486,11 +488,7 @@ __global__ void __launch_bounds__(kBlock) k_big_emit(BigCtl* ctl, cudaGraphCondi
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  if (threadIdx.x == 0) {
-    ctl->emitted = 0;
-    ctl->mv = plan;
-    ctl->mv.next_tile = 0;
-  }
+  if (threadIdx.x == 0) ctl->emitted = 0;
   const bool more = plan_round(ctl, next_big, ctl->gtbuf[plan.gt == ctl->gtbuf[0] ? 1 : 0]);
   if (use_cond && threadIdx.x == 0) {
     if (plan.G) atomicAdd(&g_graph_launches, (unsigned long long)kBigRoundKernels);
@@ -681,7 +679,12 @@ __global__ void __launch_bounds__(kBlock) k_scan_reduce(const BigCtl* __restrict
 // block finds the offset of its chunk by summing the chunk totals before it
 // (carried from one of its chunks to its next), so no third kernel scans the
 // totals.
-__global__ void __launch_bounds__(kBlock) k_scan_down(const BigCtl* __restrict__ ctl) {
+__global__ void __launch_bounds__(kBlock) k_scan_down(BigCtl* ctl) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {  // the plan for k_big_emit and the scatter
+    BigPlan plan = ctl->cur;
+    plan.next_tile = 0;
+    ctl->mv = plan;
+  }
   const uint64_t n = ctl->cur.ncounters;
   uint32_t* __restrict__ a = ctl->counters;
   const uint32_t* __restrict__ part = ctl->partials;

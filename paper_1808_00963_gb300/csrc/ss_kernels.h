@@ -36,7 +36,8 @@ struct BigPlan {
 // writes the plan of the next round from the list of big subsets this round
 // leaves (a planning kernel before each round took 6-8 us), so rounds follow
 // one another with no host in between (Section 4.2.8: the fully parallel levels need no sequential
-// coordinator).  The scatter, which runs after that, reads the copy in `mv`.
+// coordinator).  k_scan_down copies the plan to `mv`, which k_big_emit and the
+// scatter read: no block may read what another block of its kernel replaces.
 struct BigCtl {
   SortCtx c;
   GenTask* gtbuf[2];      // cap_big tasks each, for two successive rounds
@@ -52,8 +53,8 @@ struct BigCtl {
   uint32_t K;             // buckets per step, 2^(logv + 1) - 1
   uint32_t round;
   uint32_t emitted;       // blocks of the round's k_big_emit that are done
-  BigPlan cur;            // the round's plan, as all its kernels but the scatter read it
-  BigPlan mv;             // the same, for the scatter (k_big_emit has put the next round's into cur by then)
+  BigPlan cur;            // the round's plan, for its kernels before k_big_emit
+  BigPlan mv;             // the same from k_big_emit on, which puts the next round's into cur
 };
 
 // Rounds of 256 strings in a tile of a round over `total` strings in G
