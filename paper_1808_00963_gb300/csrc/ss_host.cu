@@ -4,14 +4,13 @@
 //   1. every string gets a record (cache at depth 0, index) and each set a
 //      root subset;
 //   2. while some subset is larger than the big-task threshold, all such
-//      subsets run one multi-block S^5 step together (the host reads how many
-//      there are after each step, which is the only host synchronisation);
+//      subsets run one multi-block S^5 step together (a CUDA graph loops over
+//      the steps, the host waits for none);
 //   3. one persistent work-queue launch runs single-block S^5 steps until
 //      every remaining subset is at most small_cutoff strings;
 //   4. warps and blocks finish the small subsets;
 //   5. the LCP entries at distribution-step boundaries are resolved.
-// Batches skip step 2 (their launch sequence is fixed, so it can be captured
-// into a CUDA graph).
+// A plain sort of 33..4096 strings is ranked by counting instead of 1 to 3.
 #include <algorithm>
 #include <atomic>
 #include <cstdio>
@@ -230,6 +229,10 @@ enum class Rounds { kNone, kLoop, kOne };
 
 // limit: bytes the layout may take (a sort with one round sizes its tiles by
 // what its fixed scratch leaves for their counters).
+// A layout for more strings is never smaller, so that a workspace made for n
+// strings serves fewer: the counters do not shrink where the tiles grow, and a
+// set a little too large to be ranked by counting has room for the keys of one
+// that is not.
 static Layout make_layout(uint64_t M, uint32_t num_sets, const Opts& o, Rounds rounds, bool rank = false,
                           size_t limit = ~(size_t)0) {
   Layout L{};
@@ -275,13 +278,17 @@ static Layout make_layout(uint64_t M, uint32_t num_sets, const Opts& o, Rounds r
   // tile of a GPU of kSizingSms SMs if its counters fit, else up to 8 rounds
   constexpr uint32_t kSizingSms = 152;
   uint32_t R = std::min(tile_rounds(M, 1, kSizingSms, (uint32_t)KP - 1, ~0ull, 0), 8u);
-  auto counters = [&] { return big ? KP * (M / (kBlock * R) + 2 * (uint64_t)L.cap_big) : 0ull; };
+  // (tiles of R rounds: kTilesPerSm per SM just before R grows)
+  const uint64_t least = one ? 0 : std::min<uint64_t>(M / (kBlock * kMinTileRounds), (uint64_t)kSizingSms * kTilesPerSm);
+  auto counters = [&] { return big ? KP * (std::max<uint64_t>(M / (kBlock * R), least) + 2 * (uint64_t)L.cap_big) : 0ull; };
   auto counter_bytes = [&] { return align256(counters() * 4) + align256((counters() / 4096 + 2) * 4); };
   while (R < 8 && off + counter_bytes() > limit) ++R;
   L.ncounters_max = counters();
   L.counters = take(L.ncounters_max * 4);
   L.partials = take((L.ncounters_max / 4096 + 2) * 4);
   L.total = off;
+  if (num_sets == 1 && !one && !rank && o.plain_steps && M > kRankMax)
+    L.total = std::max(L.total, make_layout(kRankMax, 1, o, Rounds::kNone, true).total);
   return L;
 }
 
@@ -796,10 +803,10 @@ ss_status ss_distinguishing(const uint8_t* chars, const uint64_t* offsets, uint6
 // 20 M URLs in 16 runs 3875 -> 3598 us (136: 3525, 128, one piece more than
 // lanes: 3744), 5 M 1356 -> 1204, 1 M in 8 runs 766 -> 379, 200 k 712 -> 193,
 // 20 k 693 -> 159.
+constexpr uint64_t kMergePieces = 152ull * kMergeLanesPerSm * 9 / 10, kMergeMinStep = 3;
 static uint32_t merge_step(uint32_t sample_step, uint64_t total) {
   if (sample_step) return sample_step;
-  constexpr uint64_t kPieces = 152ull * kMergeLanesPerSm * 9 / 10;
-  return (uint32_t)std::max<uint64_t>(3, (total + kPieces - 1) / kPieces);
+  return (uint32_t)std::max<uint64_t>(kMergeMinStep, (total + kMergePieces - 1) / kMergePieces);
 }
 
 static ss_status merge_geometry(const ss_run* runs, uint32_t num_runs, uint32_t sample_step, uint64_t* total,
@@ -819,17 +826,20 @@ static ss_status merge_geometry(const ss_run* runs, uint32_t num_runs, uint32_t 
 }
 
 // two record buffers (32 bytes per string), the sample cuts of a round, the
-// piece counter
-static size_t merge_ws_bytes(uint64_t total, uint32_t num_runs, uint32_t S) {
+// piece counter.  With the default step room for the most cuts that up to
+// `total` strings have (fewer strings may have more cuts), so that a workspace
+// made for them serves fewer.
+static size_t merge_ws_bytes(uint64_t total, uint32_t num_runs, uint32_t sample_step) {
   if (num_runs <= 1) return 256;
-  return 2 * align256(total * sizeof(MergeRec)) + align256((total / S + num_runs + 1) * 4) + 256;
+  const uint64_t cuts = sample_step ? total / sample_step : std::min(total / kMergeMinStep, kMergePieces);
+  return 2 * align256(total * sizeof(MergeRec)) + align256((cuts + num_runs + 1) * 4) + 256;
 }
 
 size_t ss_merge_workspace_size(const ss_run* runs, uint32_t num_runs, uint32_t sample_step) {
   uint64_t total;
   uint32_t S;
   if (merge_geometry(runs, num_runs, sample_step, &total, &S) != SS_OK) return 0;
-  return merge_ws_bytes(total, num_runs, S);
+  return merge_ws_bytes(total, num_runs, sample_step);
 }
 
 ss_status ss_merge(const uint8_t* chars, const uint64_t* offsets, uint32_t max_len, const ss_run* runs,
@@ -842,7 +852,7 @@ ss_status ss_merge(const uint8_t* chars, const uint64_t* offsets, uint32_t max_l
   if (total == 0) return SS_OK;
   if (!chars || !offsets || !out_perm) return SS_ERR_INVALID;
   if (workspace && (reinterpret_cast<uintptr_t>(workspace) & 255)) return SS_ERR_INVALID;
-  const size_t need = merge_ws_bytes(total, num_runs, S);
+  const size_t need = merge_ws_bytes(total, num_runs, sample_step);
   if (workspace && workspace_bytes < need) return SS_ERR_INVALID;
   DevInfo dev;
   s = device_info(dev);
