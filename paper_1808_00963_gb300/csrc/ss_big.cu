@@ -1,11 +1,12 @@
 // Multi-block S^5 steps: the "fully parallel S^5" of Section 4.2.8 for
 // subsets above the big-task threshold.  All big subsets of one round are
 // processed together: one block samples each subset (SampleJob), every tile
-// of every subset is classified and counted by its own block (CountJob), one
+// of every subset is classified and counted by one block (CountJob), one
 // device-wide prefix sum over the [subset][bucket][tile] counters gives every
 // tile its destination in every bucket (the interleaved prefix sum of
-// Theorem 4.4), one block per subset emits the new subsets, and every tile is
-// redistributed by its own block (DistributeJob).
+// Theorem 4.4), a few blocks per subset emit the new subsets and the last of
+// them plans the next round, and every tile is redistributed by one block
+// (DistributeJob).
 #include "ss_kernels.h"
 #include "ss_step.cuh"
 

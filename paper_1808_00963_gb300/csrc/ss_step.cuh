@@ -1,6 +1,7 @@
 // Building blocks of one Super Scalar String Sample Sort step (Algorithm 4.1),
-// written for a 256-thread block.  Used by the multi-block step kernels and by
-// the persistent single-block kernel.
+// by one block (of 256 threads unless a template argument says otherwise).
+// Used by the multi-block step kernels and by the persistent single-block
+// kernel.
 #pragma once
 
 #include "ss_internal.cuh"
