@@ -28,7 +28,8 @@
  * blocks of at least 4 KiB, so these reads never leave mapped memory.
  *
  * Streams: `stream` is a cudaStream_t passed as void* (NULL = legacy default
- * stream).  All work is enqueued on it.
+ * stream).  All work is enqueued on it.  Several threads may sort on one
+ * stream at the same time (not into one workspace, and not with one batch).
  *
  * Errors: argument errors are returned at once, before any work is enqueued.
  * Errors found on the device (a bounded wait that expired, a string longer

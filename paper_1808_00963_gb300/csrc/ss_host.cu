@@ -17,6 +17,7 @@
 #include <cstring>
 #include <iterator>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <tuple>
@@ -495,29 +496,35 @@ static cudaError_t loop_exec(BigCtl* ctl, int logv, bool dna, uint32_t R_max, ui
 // status into, in pinned host memory that the kernels reach directly (reading
 // it takes no copy and second wait after the wait for the stream; with the
 // fewer launches of k_begin, 1 M URLs 698 -> 653 us), and the multi-block
-// loop's control block in device memory.
+// loop's control block in device memory.  A sort's set-up launch writes the
+// control block and its rounds work on it: whoever enqueues them holds `use`
+// from the one to the last of the others, so that no other thread's sort on
+// the stream comes in between.  Slots are never removed.
 struct StreamSlot {
   uint32_t* status = nullptr;      // host address
   uint32_t* status_dev = nullptr;  // the same word for kernels
   BigCtl* ctl = nullptr;
+  std::mutex use;
 };
 
 static std::mutex g_slot_mu;
-static std::map<std::pair<int, void*>, StreamSlot> g_slots;
+static std::map<std::pair<int, void*>, std::unique_ptr<StreamSlot>> g_slots;
 
-static ss_status stream_slot(cudaStream_t st, bool create, StreamSlot* out) {
-  *out = StreamSlot();
+// The slot of a stream (null: it has none and create is false).
+static ss_status stream_slot(cudaStream_t st, bool create, StreamSlot** out) {
+  *out = nullptr;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return SS_ERR_NO_DEVICE;
   std::lock_guard<std::mutex> lk(g_slot_mu);
   auto key = std::make_pair(dev, static_cast<void*>(st));
   auto it = g_slots.find(key);
   if (it != g_slots.end()) {
-    *out = it->second;
+    *out = it->second.get();
     return SS_OK;
   }
   if (!create) return SS_OK;
-  StreamSlot p;
+  std::unique_ptr<StreamSlot> slot(new StreamSlot);
+  StreamSlot& p = *slot;
   constexpr size_t kStatusBytes = 64;
   if (cudaMalloc(reinterpret_cast<void**>(&p.ctl), sizeof(BigCtl)) != cudaSuccess) return SS_ERR_OOM;
   if (cudaHostAlloc(reinterpret_cast<void**>(&p.status), kStatusBytes, cudaHostAllocMapped | cudaHostAllocPortable) !=
@@ -531,14 +538,15 @@ static ss_status stream_slot(cudaStream_t st, bool create, StreamSlot* out) {
     cudaFree(p.ctl);
     return SS_ERR_CUDA;
   }
-  g_slots[key] = p;
-  *out = p;
+  *out = slot.get();
+  g_slots[key] = std::move(slot);
   return SS_OK;
 }
 
 // Enqueues a sort.  sd: the descriptor of its only set (null: a batch, whose
 // descriptors are in place already).  ctl: where the multi-block loop's control
-// block lives (needed when big).
+// block lives (needed when big).  A stream's control block is the caller's to
+// hold (StreamSlot::use).
 static ss_status run_sort(uint8_t* ws, const Layout& L, SortCtx c, const Opts& o, const DevInfo& dev,
                           Rounds rounds, cudaStream_t st, const SetDesc* sd, BigCtl* ctl = nullptr) {
   const LaunchHook hook{st};
@@ -665,7 +673,7 @@ static ss_status sort_device(const uint8_t* chars, const uint64_t* offsets, uint
     if (cudaMallocAsync(reinterpret_cast<void**>(&ws), L.total, st) != cudaSuccess) return SS_ERR_OOM;
     owned = true;
   }
-  StreamSlot slot;
+  StreamSlot* slot = nullptr;
   if ((s = stream_slot(st, true, &slot)) != SS_OK) {
     if (owned) cudaFreeAsync(ws, st);
     return s;
@@ -673,8 +681,11 @@ static ss_status sort_device(const uint8_t* chars, const uint64_t* offsets, uint
   SetDesc sd{chars, offsets, perm, lcp, (uint32_t)n, o.cap, 0, dna};
   SortCtx ctx = make_ctx(ws, L, 1, (uint32_t)n, o, rounds);
   ctx.dna = dna;
-  ctx.fold_status = slot.status_dev;  // the device status goes to the stream's status word
-  const ss_status r = run_sort(ws, L, ctx, o, dev, rounds, st, &sd, slot.ctl);
+  ctx.fold_status = slot->status_dev;  // the device status goes to the stream's status word
+  std::unique_lock<std::mutex> hold(slot->use, std::defer_lock);
+  if (rounds != Rounds::kNone) hold.lock();
+  const ss_status r = run_sort(ws, L, ctx, o, dev, rounds, st, &sd, slot->ctl);
+  if (hold) hold.unlock();
   if (g_profiling.load()) read_status(ws, L, st);  // waits: per-kernel times and bytes
   if (owned) cudaFreeAsync(ws, st);
   return r;
@@ -683,12 +694,12 @@ static ss_status sort_device(const uint8_t* chars, const uint64_t* offsets, uint
 // Waits for the stream and returns the device status its sorts have left in
 // its status word since it was last read (clearing it).
 static ss_status take_stream_status(cudaStream_t st) {
-  StreamSlot slot;
+  StreamSlot* slot = nullptr;
   stream_slot(st, false, &slot);
   if (cudaStreamSynchronize(st) != cudaSuccess) return SS_ERR_CUDA;
   collect_profile();
-  if (!slot.status) return SS_OK;
-  volatile uint32_t* word = slot.status;
+  if (!slot) return SS_OK;
+  volatile uint32_t* word = slot->status;
   const uint32_t v = *word;
   if (v) *word = 0;
   return map_status(v);
@@ -1430,16 +1441,18 @@ ss_status ss_batch_run(ss_batch* b, void* stream) {
   // batch's own (its address goes into the caller's graph); otherwise the
   // stream's, whose loop graph is built once per stream
   BigCtl* ctl = nullptr;
+  std::unique_lock<std::mutex> hold;
   if (b->big) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) return SS_ERR_CUDA;
     if (cs == cudaStreamCaptureStatusActive) {
       ctl = reinterpret_cast<BigCtl*>(b->ws + b->L.bigctl);
     } else {
-      StreamSlot slot;
+      StreamSlot* slot = nullptr;
       ss_status s = stream_slot(st, true, &slot);
       if (s != SS_OK) return s;
-      ctl = slot.ctl;
+      ctl = slot->ctl;
+      hold = std::unique_lock<std::mutex>(slot->use);
     }
   }
   return run_sort(b->ws, b->L, c, b->o, b->dev, b->rounds(), st, nullptr, ctl);

@@ -1,0 +1,77 @@
+"""What the host code does when several threads sort on one stream, checked on
+a stand-in for the CUDA runtime that logs the launches."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import fake_util
+import paper_1808_00963_gb300 as ss
+
+STREAM = 0x77
+BIG = 20_000  # strings: above the multi-block threshold
+
+
+@pytest.fixture
+def lib(tmp_path):
+    return fake_util.load(tmp_path)
+
+
+class Set:
+    def __init__(self, n):
+        self.n = n
+        self.bufs = [np.zeros(n + 16, np.uint64) for _ in range(4)]
+        self.ptrs = [ctypes.c_void_p(b.ctypes.data) for b in self.bufs]
+
+    def sort(self, lib, stream=STREAM, **opts):
+        chars, offsets, perm, lcp = self.ptrs
+        return lib.ss_sort_ex(chars, offsets, self.n, perm, lcp, ctypes.byref(ss.make_options(**opts)),
+                              ctypes.c_void_p(stream))
+
+    def desc(self):
+        chars, offsets, perm, lcp = (p.value for p in self.ptrs)
+        return ss.SetDesc(chars, offsets, self.n, 0, perm, lcp)
+
+
+def multi_block_parts(lib):
+    """(thread, what) of the launches that use the stream's control block, in order: "begin" writes it, the loop
+    graph or the kernels of a round work on it."""
+    names = {"k_begin": "begin", "k_big_": "round", "k_scan_": "round", "graph": "graph"}
+    return [(tag, kind) for tag, _, stream, what, _ in fake_util.log(lib) if stream == STREAM
+            for part, kind in names.items() if part in what]
+
+
+@pytest.mark.parametrize("graph_loop", [1, 0])
+@pytest.mark.parametrize("second", ["sort", "batch"])
+def test_sorts_of_two_threads_on_one_stream(lib, graph_loop, second):
+    """A sort's multi-block rounds run on the stream's control block, which the sort has written: no other sort of
+    the stream may write it in between."""
+    lib.ss_set_graph_loop(graph_loop)
+    sets = [Set(BIG) for _ in range(2)]
+    assert sets[0].sort(lib) == 0  # the stream's slot and its loop graph
+    batch = ctypes.c_void_p()
+    descs = (ss.SetDesc * 2)(sets[1].desc(), Set(100).desc())
+    assert lib.ss_batch_create(descs, 2, None, ctypes.byref(batch)) == 0
+    lib.fake_delay(b"k_begin", 2000)
+    lib.fake_delay(b"k_big_classify", 500)
+    lib.fake_clear_log()
+
+    def first():
+        lib.fake_set_tag(1)
+        return [sets[0].sort(lib) for _ in range(8)]
+
+    def other():
+        lib.fake_set_tag(2)
+        if second == "batch":
+            return [lib.ss_batch_run(batch, ctypes.c_void_p(STREAM)) for _ in range(8)]
+        return [sets[1].sort(lib) for _ in range(8)]
+
+    assert fake_util.in_threads(first, other) == [[0] * 8] * 2
+    owner = None
+    parts = multi_block_parts(lib)
+    assert sum(kind == "begin" for _, kind in parts) == 16
+    for tag, kind in parts:
+        if kind == "begin":
+            owner = tag
+        assert tag == owner, parts
+    lib.ss_batch_destroy(batch)
