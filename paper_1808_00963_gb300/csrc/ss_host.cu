@@ -699,10 +699,9 @@ static ss_status take_stream_status(cudaStream_t st) {
   if (cudaStreamSynchronize(st) != cudaSuccess) return SS_ERR_CUDA;
   collect_profile();
   if (!slot) return SS_OK;
-  volatile uint32_t* word = slot->status;
-  const uint32_t v = *word;
-  if (v) *word = 0;
-  return map_status(v);
+  // read and cleared in one step: kernels of sorts that other threads have
+  // enqueued since may be adding their bits
+  return map_status(__atomic_exchange_n(slot->status, 0u, __ATOMIC_ACQ_REL));
 }
 
 }  // namespace ss

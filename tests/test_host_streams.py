@@ -75,3 +75,16 @@ def test_sorts_of_two_threads_on_one_stream(lib, graph_loop, second):
             owner = tag
         assert tag == owner, parts
     lib.ss_batch_destroy(batch)
+
+
+def test_status_set_while_it_is_read(lib):
+    """A kernel's error bit that arrives while a thread takes the stream's status word is still reported: by that
+    thread or by the next one, never by none.  (Two bits one after the other, the second with the higher rank: it
+    is reported whether the two are taken together or apart.)"""
+    assert Set(100).sort(lib) == 0
+    take = ctypes.cast(lib.ss_stream_status, ctypes.c_void_p)
+    lib.fake_status_episodes.restype = ctypes.c_uint64
+    lib.fake_status_episodes.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_uint32, ctypes.c_uint32,
+                                         ctypes.c_int, ctypes.c_uint64]
+    timeout, too_deep, too_large = 1 << 1, 1 << 2, 4
+    assert lib.fake_status_episodes(take, STREAM, timeout, too_deep, too_large, 300_000) == 0
