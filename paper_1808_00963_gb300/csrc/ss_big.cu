@@ -748,23 +748,28 @@ cudaError_t launch_big_plan(BigCtl* ctl, cudaStream_t st, const LaunchHook& hook
   return cudaGetLastError();
 }
 
+template <int LOGV>
+static cudaError_t set_big_limits_t() {
+  constexpr cudaFuncAttribute kLimit = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  const int scatter = (int)big_scatter_smem(LOGV, kMaxRounds);
+  cudaError_t e = cudaFuncSetAttribute(k_big_scatter<LOGV, false>, kLimit, scatter);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_big_scatter<LOGV, true>, kLimit, scatter);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_big_sample<LOGV>, kLimit, (int)sizeof(SampleSmem<LOGV, u128>));
+  return e;
+}
+
+cudaError_t set_big_limits() {
+  const cudaError_t e = set_big_limits_t<8>();
+  return e == cudaSuccess ? set_big_limits_t<9>() : e;
+}
+
 template <int LOGV, bool DNA>
 static cudaError_t launch_big_round_t(BigCtl* ctl, uint32_t R_max, uint32_t sms, uint64_t cond, bool use_cond,
                                       cudaStream_t st, const LaunchHook& hook) {
   const size_t smem = big_scatter_smem(LOGV, R_max);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_big_scatter<LOGV, DNA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)big_scatter_smem(LOGV, kMaxRounds));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_big_sample<LOGV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)sizeof(SampleSmem<LOGV, u128>));
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
   // fixed grids (the work of a round is only known on the device): blocks
   // loop over subsets, tiles or counter chunks and return when there are none
-  hook.run("big_sample", [&] { 
+  hook.run("big_sample", [&] {
     k_big_sample<LOGV><<<sms * (2048 / kSampleThreads<LOGV>), kSampleThreads<LOGV>, sizeof(SampleSmem<LOGV, u128>), st>>>(ctl);
   });
   hook.run("big_classify", [&] { k_big_classify<LOGV><<<sms * 8, kBlock, 0, st>>>(ctl, &ctl->cur.next_tile); });

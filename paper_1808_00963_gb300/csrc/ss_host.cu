@@ -123,6 +123,8 @@ static ss_status device_info(DevInfo& out) {
     d.ok = (p.major == 10 && p.minor == 3);
     d.sms = p.multiProcessorCount;
     if (d.ok) {
+      if (set_big_limits() != cudaSuccess || set_queue_limits() != cudaSuccess || set_small_limits() != cudaSuccess)
+        return SS_ERR_CUDA;
       for (int l = 7; l <= 10; ++l) {
         int b = 0;
         if (queue_occupancy(l, &b) != cudaSuccess || b < 1) return SS_ERR_CUDA;
@@ -183,7 +185,7 @@ static ss_status resolve_opts(const ss_options* o, Opts& r) {
     r.R = o->tile_rounds;
   }
   if (o->small_cutoff) {
-    if (o->small_cutoff < 64 || o->small_cutoff > 4096) return SS_ERR_INVALID;
+    if (o->small_cutoff < 64 || o->small_cutoff > kSmallCutoffMax) return SS_ERR_INVALID;
     r.cutoff = o->small_cutoff;
   }
   if (o->big_threshold) r.big_thr = o->big_threshold;

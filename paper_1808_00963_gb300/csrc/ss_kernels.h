@@ -89,6 +89,13 @@ constexpr uint32_t kMaxBigRounds = 1u << 20;
 // prefix-sum kernels, emit and scatter.
 constexpr uint32_t kBigRoundKernels = 6;
 
+// The dynamic shared memory that the kernels of a translation unit may have, at
+// its largest, on the current device (a kernel's limit belongs to a device):
+// called once per device, before the first launch there.
+cudaError_t set_big_limits();
+cudaError_t set_queue_limits();
+cudaError_t set_small_limits();
+
 size_t big_splitters_bytes(int logv);
 size_t big_scatter_smem(int logv, uint32_t R);
 // The plan of the first round from list 0 (for several sets; a single set's
@@ -128,6 +135,7 @@ struct RankArgs {
 cudaError_t launch_rank(const BeginArgs& a, const RankArgs& r, const SortCtx& c, cudaStream_t st,
                         const LaunchHook& hook);
 
+constexpr uint32_t kSmallCutoffMax = 4096;  // largest small_cutoff
 size_t small_cta_smem(uint32_t pmax);
 cudaError_t launch_begin(const BeginArgs& a, cudaStream_t st, const LaunchHook& hook);
 cudaError_t launch_init(const SortCtx& c, cudaStream_t st, const LaunchHook& hook);

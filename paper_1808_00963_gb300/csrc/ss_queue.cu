@@ -308,23 +308,21 @@ __global__ void __launch_bounds__(kQueueThreads, kQueueBlocks) k_queue(SortCtx c
   account(c, kKQueue, bytes);
 }
 
-template <int LOGV, bool DNA>
-cudaError_t set_queue_attr() {
-  static cudaError_t e = cudaFuncSetAttribute(k_queue<LOGV, DNA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)sizeof(QueueSmem<LOGV>));
-  return e;
+template <int LOGV>
+cudaError_t set_limits_t() {
+  constexpr cudaFuncAttribute kLimit = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  const cudaError_t e = cudaFuncSetAttribute(k_queue<LOGV, false>, kLimit, (int)sizeof(QueueSmem<LOGV>));
+  return e == cudaSuccess ? cudaFuncSetAttribute(k_queue<LOGV, true>, kLimit, (int)sizeof(QueueSmem<LOGV>)) : e;
 }
 
 template <int LOGV>
 cudaError_t occupancy_t(int* blocks_per_sm) {
-  if (cudaError_t e = set_queue_attr<LOGV, false>()) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_queue<LOGV, false>, kQueueThreads,
                                                        sizeof(QueueSmem<LOGV>));
 }
 
 template <int LOGV, bool DNA>
 cudaError_t launch_queue_t(const SortCtx& c, uint32_t grid, cudaStream_t st, const LaunchHook& hook) {
-  if (cudaError_t e = set_queue_attr<LOGV, DNA>()) return e;
   hook.run("queue", [&] { k_queue<LOGV, DNA><<<grid, kQueueThreads, sizeof(QueueSmem<LOGV>), st>>>(c); });
   return cudaGetLastError();
 }
@@ -340,6 +338,14 @@ cudaError_t launch_queue_d(int logv, const SortCtx& c, uint32_t grid, cudaStream
 }
 
 }  // namespace
+
+cudaError_t set_queue_limits() {
+  cudaError_t e = set_limits_t<7>();
+  if (e == cudaSuccess) e = set_limits_t<8>();
+  if (e == cudaSuccess) e = set_limits_t<9>();
+  if (e == cudaSuccess) e = set_limits_t<10>();
+  return e;
+}
 
 cudaError_t queue_occupancy(int logv, int* blocks_per_sm) {
   switch (logv) {

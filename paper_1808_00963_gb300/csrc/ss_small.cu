@@ -854,16 +854,16 @@ cudaError_t launch_init(const SortCtx& c, cudaStream_t st, const LaunchHook& hoo
   return cudaGetLastError();
 }
 
+cudaError_t set_small_limits() {
+  constexpr cudaFuncAttribute kLimit = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  const int wide = (int)small_cta_smem(kSmallCutoffMax);
+  const cudaError_t e = cudaFuncSetAttribute(k_small_cta<kSmallWideThreads, false>, kLimit, wide);
+  return e == cudaSuccess ? cudaFuncSetAttribute(k_small_cta<kSmallWideThreads, true>, kLimit, wide) : e;
+}
+
 template <bool DNA>
 static cudaError_t launch_small_t(const SortCtx& c, uint32_t pmax, uint32_t sms, bool last, cudaStream_t st,
                                   const LaunchHook& hook) {
-  static uint32_t attr_pmax = 0;
-  if (pmax > attr_pmax) {
-    cudaError_t e = cudaFuncSetAttribute(k_small_cta<kSmallWideThreads, DNA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)small_cta_smem(pmax));
-    if (e != cudaSuccess) return e;
-    attr_pmax = pmax;
-  }
   // subsets of more than kSmallCtaNarrowMax strings, then smaller ones
   const uint32_t min_count = 2 * sms * kSmallWideBlocks;
   if (pmax > kSmallCtaNarrowMax)

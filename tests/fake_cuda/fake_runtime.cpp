@@ -103,8 +103,9 @@ size_t fake_log(char* out, size_t cap) {
   }
   return text.size();
 }
-// Each time a kernel's shared-memory limit is set below 64 KB, the call takes us.
-void fake_slow_small_attributes(int us) { attr_delay_us = us; }
+// From now on a kernel's shared-memory limit is set late in a call of us microseconds if it is below 64 KB, and early
+// in one of twice that if it is not.
+void fake_slow_attributes(int us) { attr_delay_us = us; }
 void* fake_host_word() { return host_word; }
 
 // `episodes` times: sets bit `low` and then bit `high` of the word, as two
@@ -180,9 +181,13 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void** args, size_t s
 }
 
 cudaError_t cudaFuncSetAttribute(const void* fun, cudaFuncAttribute, int value) {
-  if (value < (64 << 10)) pause_us(attr_delay_us);
-  std::lock_guard<std::mutex> lk(mu);
-  max_smem[{device, fun}] = (size_t)value;
+  const bool small = value < (64 << 10);
+  if (small) pause_us(attr_delay_us);
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    max_smem[{device, fun}] = (size_t)value;
+  }
+  if (!small) pause_us(2 * attr_delay_us);
   return cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void* fun, int, size_t smem, unsigned) {
