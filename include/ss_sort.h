@@ -349,9 +349,8 @@ ss_status ss_sort_batch(const ss_set* sets, uint32_t num_sets, const ss_options*
  *   - The first call on a device looks up the array's device address
  *     (cudaGetSymbolAddress); make that first call before any stream capture.
  *   - All calls share the one array and it keeps the last call's contents
- *     (the call clears what must start at zero).  Calls that overlap on the GPU
- *     race with each other: issue them on one stream, or wait for one to end
- *     before the next starts.
+ *     (the call clears what must start at zero).  Calls of several threads on
+ *     one device take turns: each has its sort ended before the next starts.
  *   - Returns SS_ERR_INVALID while kernel profiling (ss_set_profiling) is on. */
 ss_status ss_sort_noalloc(const uint8_t* chars, const uint64_t* offsets, uint64_t n,
                           uint32_t max_len, uint32_t* out_perm, uint32_t* out_lcp, void* stream);

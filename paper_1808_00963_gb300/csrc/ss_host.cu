@@ -1517,25 +1517,30 @@ namespace ss {
 // until the process exits.
 static __device__ __align__(256) uint8_t g_noalloc_scratch[SS_NOALLOC_SCRATCH_BYTES];
 
+// One device's scratch: its address, and whose call is using it (a call holds
+// `use` until its sort has ended: all calls work in the one array).
 constexpr int kNoAllocMaxDevices = 64;
+struct NoAllocScratch {
+  uint8_t* p = nullptr;
+  std::mutex use;
+};
 static std::mutex g_noalloc_mu;
-static uint8_t* g_noalloc_ptr[kNoAllocMaxDevices] = {nullptr};
+static NoAllocScratch g_noalloc[kNoAllocMaxDevices];
 
-
-// Device address of the scratch on the current device, looked up once per
-// device.  Host code only ever passes this address to kernels: the name
+// The scratch of the current device, its address looked up once per device.
+// Host code only ever passes this address to kernels: the name
 // g_noalloc_scratch in host code is a host-side stand-in, not device memory.
-static ss_status noalloc_scratch(uint8_t** out) {
+static ss_status noalloc_scratch(NoAllocScratch** out) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return SS_ERR_NO_DEVICE;
   if (dev < 0 || dev >= kNoAllocMaxDevices) return SS_ERR_NO_DEVICE;
   std::lock_guard<std::mutex> lk(g_noalloc_mu);
-  if (!g_noalloc_ptr[dev]) {
+  if (!g_noalloc[dev].p) {
     void* p = nullptr;
     if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) return SS_ERR_CUDA;
-    g_noalloc_ptr[dev] = static_cast<uint8_t*>(p);
+    g_noalloc[dev].p = static_cast<uint8_t*>(p);
   }
-  *out = g_noalloc_ptr[dev];
+  *out = &g_noalloc[dev];
   return SS_OK;
 }
 
@@ -1560,8 +1565,10 @@ extern "C" ss_status ss_sort_noalloc(const uint8_t* chars, const uint64_t* offse
   DevInfo dev;
   ss_status s = device_info(dev);
   if (s != SS_OK) return s;
-  uint8_t* ws = nullptr;
-  if ((s = noalloc_scratch(&ws)) != SS_OK) return s;
+  NoAllocScratch* scratch = nullptr;
+  if ((s = noalloc_scratch(&scratch)) != SS_OK) return s;
+  std::lock_guard<std::mutex> hold(scratch->use);
+  uint8_t* const ws = scratch->p;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const SetDesc sd{chars, offsets, out_perm, out_lcp, (uint32_t)n, o.cap, 0, 0};
   // run_sort clears the control words and the queue flags, the only scratch

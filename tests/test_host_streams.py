@@ -88,3 +88,29 @@ def test_status_set_while_it_is_read(lib):
                                          ctypes.c_int, ctypes.c_uint64]
     timeout, too_deep, too_large = 1 << 1, 1 << 2, 4
     assert lib.fake_status_episodes(take, STREAM, timeout, too_deep, too_large, 300_000) == 0
+
+
+def test_noalloc_of_two_threads(lib):
+    """The calls without allocation share one scratch array: a call's launches and its wait come before the next
+    call's first launch, on one stream or on two."""
+    sets = [Set(BIG), Set(300)]
+    for s in sets:
+        assert lib.ss_sort_noalloc(s.ptrs[0], s.ptrs[1], s.n, 0, s.ptrs[2], s.ptrs[3], ctypes.c_void_p(STREAM)) == 0
+    lib.fake_delay(b"k_begin", 1000)
+    lib.fake_delay(b"k_rank_keys", 1000)
+    lib.fake_clear_log()
+
+    def call(tag, s, stream):
+        lib.fake_set_tag(tag)
+        return [lib.ss_sort_noalloc(s.ptrs[0], s.ptrs[1], s.n, 0, s.ptrs[2], s.ptrs[3], ctypes.c_void_p(stream))
+                for _ in range(8)]
+
+    assert fake_util.in_threads(lambda: call(1, sets[0], STREAM), lambda: call(2, sets[1], STREAM),
+                                lambda: call(3, Set(BIG), STREAM + 1)) == [[0] * 8] * 3
+    calls, fresh = 0, True
+    for tag, _, _, what, _ in fake_util.log(lib):
+        if fresh:
+            owner, calls = tag, calls + 1
+        assert tag == owner
+        fresh = what == "wait"
+    assert calls == 24
