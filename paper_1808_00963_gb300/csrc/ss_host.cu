@@ -268,7 +268,7 @@ static Layout make_layout(uint64_t M, uint32_t num_sets, const Opts& o, Rounds r
   L.spl = take((size_t)L.cap_big * big_splitters_bytes(o.logv_big));
   L.gstart = take((size_t)L.cap_big * KP * 4);
   L.gdesc = take((size_t)L.cap_big * KP * 4);
-  L.bigctl = take(big ? sizeof(BigCtl) : 0);  // a batch's loop control block (plain sorts use the stream's)
+  L.bigctl = take(big ? sizeof(BigCtl) : 0);  // the loop's control block of captured sorts (others use the stream's)
   L.marks = take((size_t)L.cap_marks * 4);
   L.mq_items = take((size_t)L.cap_mq * sizeof(Task));
   L.mq_ready = take((size_t)L.cap_mq * 4);
@@ -545,6 +545,26 @@ static ss_status stream_slot(cudaStream_t st, bool create, StreamSlot** out) {
   return SS_OK;
 }
 
+// The control block of a sort's multi-block rounds: the stream's, which *hold
+// keeps for this sort (its loop graph is built once per stream); inside a
+// caller's capture the one in the sort's workspace, since the caller's graph,
+// which gets its address, may be replayed while the stream sorts.
+static ss_status loop_control(uint8_t* ws, const Layout& L, cudaStream_t st, BigCtl** ctl,
+                              std::unique_lock<std::mutex>* hold) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  SS_CUDA(cudaStreamIsCapturing(st, &cs));
+  if (cs == cudaStreamCaptureStatusActive) {
+    *ctl = reinterpret_cast<BigCtl*>(ws + L.bigctl);
+    return SS_OK;
+  }
+  StreamSlot* slot = nullptr;
+  const ss_status s = stream_slot(st, true, &slot);
+  if (s != SS_OK) return s;
+  *hold = std::unique_lock<std::mutex>(slot->use);
+  *ctl = slot->ctl;
+  return SS_OK;
+}
+
 // Enqueues a sort.  sd: the descriptor of its only set (null: a batch, whose
 // descriptors are in place already).  ctl: where the multi-block loop's control
 // block lives (needed when big).  A stream's control block is the caller's to
@@ -684,10 +704,13 @@ static ss_status sort_device(const uint8_t* chars, const uint64_t* offsets, uint
   SortCtx ctx = make_ctx(ws, L, 1, (uint32_t)n, o, rounds);
   ctx.dna = dna;
   ctx.fold_status = slot->status_dev;  // the device status goes to the stream's status word
-  std::unique_lock<std::mutex> hold(slot->use, std::defer_lock);
-  if (rounds != Rounds::kNone) hold.lock();
-  const ss_status r = run_sort(ws, L, ctx, o, dev, rounds, st, &sd, slot->ctl);
-  if (hold) hold.unlock();
+  ss_status r = SS_OK;
+  {
+    BigCtl* ctl = nullptr;
+    std::unique_lock<std::mutex> hold;
+    if (rounds != Rounds::kNone) r = loop_control(ws, L, st, &ctl, &hold);
+    if (r == SS_OK) r = run_sort(ws, L, ctx, o, dev, rounds, st, &sd, ctl);
+  }
   if (g_profiling.load()) read_status(ws, L, st);  // waits: per-kernel times and bytes
   if (owned) cudaFreeAsync(ws, st);
   return r;
@@ -1438,23 +1461,11 @@ ss_status ss_batch_run(ss_batch* b, void* stream) {
     if (cudaGetLastError() != cudaSuccess) return SS_ERR_CUDA;
   }
   SortCtx c = make_ctx(b->ws, b->L, b->num_sets, b->total, b->o, b->rounds());
-  // the multi-block loop's control block: inside a caller's capture the
-  // batch's own (its address goes into the caller's graph); otherwise the
-  // stream's, whose loop graph is built once per stream
   BigCtl* ctl = nullptr;
   std::unique_lock<std::mutex> hold;
   if (b->big) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) return SS_ERR_CUDA;
-    if (cs == cudaStreamCaptureStatusActive) {
-      ctl = reinterpret_cast<BigCtl*>(b->ws + b->L.bigctl);
-    } else {
-      StreamSlot* slot = nullptr;
-      ss_status s = stream_slot(st, true, &slot);
-      if (s != SS_OK) return s;
-      ctl = slot->ctl;
-      hold = std::unique_lock<std::mutex>(slot->use);
-    }
+    const ss_status s = loop_control(b->ws, b->L, st, &ctl, &hold);
+    if (s != SS_OK) return s;
   }
   return run_sort(b->ws, b->L, c, b->o, b->dev, b->rounds(), st, nullptr, ctl);
 }

@@ -114,3 +114,25 @@ def test_noalloc_of_two_threads(lib):
         assert tag == owner
         fresh = what == "wait"
     assert calls == 24
+
+
+def test_captured_sort_has_its_own_control_block(lib):
+    """A captured graph can be replayed on any stream at any time: its rounds run on a control block in the sort's
+    workspace, not on that of the stream it was captured on, where other sorts may be running then."""
+    s = Set(BIG)
+    size = lib.ss_workspace_size(BIG, None)
+    buf = np.zeros(size + 256, np.uint8)
+    ws = (buf.ctypes.data + 255) & ~255
+    opts = dict(workspace=ws, workspace_bytes=size)
+
+    def control_blocks():
+        lib.fake_clear_log()
+        assert s.sort(lib, **opts) == 0
+        return {first for _, _, _, what, first in fake_util.log(lib) if "k_big_" in what}
+
+    plain = control_blocks()  # built with the stream's loop graph
+    assert len(plain) == 1 and not ws <= min(plain) < ws + size
+    lib.fake_capture(STREAM, 1)
+    captured = control_blocks()
+    lib.fake_capture(STREAM, 0)
+    assert len(captured) == 1 and ws <= min(captured) < ws + size
