@@ -358,7 +358,8 @@ constexpr uint32_t kSmallEqual = 64;
 
 template <uint32_t NT>
 struct SmallSplit {
-  uint64_t key[kSmallSample<NT>];           // the sorted sample
+  uint64_t drawn[kSmallSample<NT>];         // the sample
+  uint64_t key[kSmallSample<NT>];           // ... sorted
   uint32_t first[2 * kSmallSample<NT> + 2]; // bucket sizes, then bucket starts
   uint8_t big[2 * kSmallSample<NT> + 2];    // number of a large equality bucket, kNotBig for the others
   uint32_t nbig;
@@ -398,20 +399,30 @@ __device__ __forceinline__ SmallSmem small_smem(uint8_t* smem, uint32_t pmax) {
 // sort): key becomes sorted, pos_out[i] is pos_in[place of the i-th] (null: the
 // place itself).  pos_out must not be pos_in.  Ends with a barrier; the caller
 // has written key before a barrier.
+// The sample is drawn at pseudo-random places, one from each of S equal
+// stretches.  (Evenly spaced places can all hold one key, where the order of
+// the strings has a period: with every 16th of 1024 strings the same key, all
+// other strings shared one bucket.)
 template <uint32_t NT>
 __device__ void small_sort(const SmallSmem& m, SmallSplit<NT>& sp, uint64_t* key, uint32_t n, const uint16_t* pos_in,
-                           uint16_t* pos_out) {
+                           uint16_t* pos_out, uint32_t seed) {
   constexpr uint32_t S = kSmallSample<NT>;
   const uint32_t tid = threadIdx.x, lane = lane_id();
-  // the sample, from evenly spaced places, put in order by counting
+  // the sample, put in order by counting
   for (uint32_t b = tid; b < 2 * S + 2; b += NT) sp.first[b] = 0;
   if (tid == 0) sp.nbig = 0;
+  uint64_t mine = 0;
   if (tid < S) {
-    const uint64_t mine = key[tid * n / S];
+    constexpr uint32_t kStretch = 0xFFFFFFFFu / S + 1;  // 2^32 / S
+    mine = key[__umulhi(tid * kStretch + (uint32_t)mix64(seed + tid) % kStretch, n)];
+    sp.drawn[tid] = mine;
+  }
+  __syncthreads();
+  if (tid < S) {
     uint32_t r = 0;
 #pragma unroll 8
     for (uint32_t i = 0; i < S; ++i) {
-      const uint64_t o = key[i * n / S];  // the same word for every lane
+      const uint64_t o = sp.drawn[i];  // the same word for every lane
       r += (o < mine || (o == mine && i < tid)) ? 1u : 0u;
     }
     sp.key[r] = mine;
@@ -602,7 +613,7 @@ __global__ void __launch_bounds__(NT) k_small_cta(SortCtx c, uint32_t pmax, uint
     // one run: jump over the prefix all its strings share
     bool sorted = s_neq || key_end(k0, dna);
     if (s_neq) {
-      small_sort<NT>(m, split, m.key, n, nullptr, m.pos[0]);
+      small_sort<NT>(m, split, m.key, n, nullptr, m.pos[0], t.begin);
     } else {
       for (uint32_t j = tid; j < n; j += NT) m.pos[0][j] = (uint16_t)j;
       if (tid == 0 && !sorted) {
@@ -733,7 +744,7 @@ __global__ void __launch_bounds__(NT) k_small_cta(SortCtx c, uint32_t pmax, uint
         bytes += 8ull * (jstop + 1);
       }
       __syncthreads();
-      small_sort<NT>(m, split, m.key + lo, n, m.pos[0] + lo, m.pos[1] + lo);
+      small_sort<NT>(m, split, m.key + lo, n, m.pos[0] + lo, m.pos[1] + lo, t.begin + lo + depth);
       for (uint32_t j = tid; j < n; j += NT) m.pos[0][lo + j] = m.pos[1][lo + j];
       __syncthreads();
     }
