@@ -349,19 +349,23 @@ constexpr uint32_t kSmallNarrowThreads = 64, kSmallWideThreads = 256;
 
 // Sampled keys, all of them splitters: 2 * S + 1 buckets (bucket 2r + 1: the
 // keys equal to splitter r; bucket 2r: those between splitters r - 1 and r).
-template <uint32_t NT>
-constexpr uint32_t kSmallSample = NT == kSmallNarrowThreads ? 32 : 64;
+constexpr uint32_t kNarrowSample = 32, kWideSample = 64;
+// Subsets of more than kManySampleAbove strings (a small_cutoff above 1024)
+// take more splitters: a string is compared with its bucket, of 2 n / S strings
+// on average.  60 sets of 4096 strings with 64 splitters 237 us, with 256 124
+// (merge sort before: 133); 2048 strings 110 / 87 (104).
+constexpr uint32_t kManySample = 256, kManySampleAbove = 1024;
 
 // Equality buckets of more strings than this get their places in string order
 // right away instead of a rank by comparing positions.
 constexpr uint32_t kSmallEqual = 64;
 
-template <uint32_t NT>
+template <uint32_t SMAX>
 struct SmallSplit {
-  uint64_t drawn[kSmallSample<NT>];         // the sample
-  uint64_t key[kSmallSample<NT>];           // ... sorted
-  uint32_t first[2 * kSmallSample<NT> + 2]; // bucket sizes, then bucket starts
-  uint8_t big[2 * kSmallSample<NT> + 2];    // number of a large equality bucket, kNotBig for the others
+  uint64_t drawn[SMAX];         // the sample
+  uint64_t key[SMAX];           // ... sorted
+  uint32_t first[2 * SMAX + 2]; // bucket sizes, then bucket starts
+  uint8_t big[2 * SMAX + 2];    // number of a large equality bucket, kNotBig for the others
   uint32_t nbig;
 };
 constexpr uint32_t kNotBig = 255;
@@ -403,18 +407,19 @@ __device__ __forceinline__ SmallSmem small_smem(uint8_t* smem, uint32_t pmax) {
 // stretches.  (Evenly spaced places can all hold one key, where the order of
 // the strings has a period: with every 16th of 1024 strings the same key, all
 // other strings shared one bucket.)
-template <uint32_t NT>
-__device__ void small_sort(const SmallSmem& m, SmallSplit<NT>& sp, uint64_t* key, uint32_t n, const uint16_t* pos_in,
+template <uint32_t NT, uint32_t SMAX>
+__device__ void small_sort(const SmallSmem& m, SmallSplit<SMAX>& sp, uint64_t* key, uint32_t n, const uint16_t* pos_in,
                            uint16_t* pos_out, uint32_t seed) {
-  constexpr uint32_t S = kSmallSample<NT>;
+  static_assert(SMAX <= NT, "a sampled key per thread");
+  const uint32_t S = SMAX > kWideSample && n <= kManySampleAbove ? kWideSample : SMAX;
   const uint32_t tid = threadIdx.x, lane = lane_id();
   // the sample, put in order by counting
   for (uint32_t b = tid; b < 2 * S + 2; b += NT) sp.first[b] = 0;
   if (tid == 0) sp.nbig = 0;
   uint64_t mine = 0;
   if (tid < S) {
-    constexpr uint32_t kStretch = 0xFFFFFFFFu / S + 1;  // 2^32 / S
-    mine = key[__umulhi(tid * kStretch + (uint32_t)mix64(seed + tid) % kStretch, n)];
+    const uint32_t stretch = 0xFFFFFFFFu / S + 1;  // 2^32 / S
+    mine = key[__umulhi(tid * stretch + ((uint32_t)mix64(seed + tid) & (stretch - 1)), n)];
     sp.drawn[tid] = mine;
   }
   __syncthreads();
@@ -440,7 +445,7 @@ __device__ void small_sort(const SmallSmem& m, SmallSplit<NT>& sp, uint64_t* key
   }
   __syncthreads();
   if (tid < 32) {  // bucket starts
-    constexpr uint32_t kPer = (2 * S + 2 + 31) / 32;
+    constexpr uint32_t kPer = (2 * SMAX + 2 + 31) / 32;
     uint32_t v[kPer], sum = 0;
 #pragma unroll
     for (uint32_t u = 0; u < kPer; ++u) {
@@ -538,14 +543,14 @@ __device__ void small_sort(const SmallSmem& m, SmallSplit<NT>& sp, uint64_t* key
 // Each block claims one subset at a time from its launch's counter (subset sizes vary several-fold, so a fixed share
 // per block left many SMs idle at the end); the next subset is claimed, and
 // its task read, while the current one sorts.
-template <uint32_t NT, bool DNA>
+template <uint32_t NT, uint32_t SMAX, bool DNA>
 __global__ void __launch_bounds__(NT) k_small_cta(SortCtx c, uint32_t pmax, uint32_t min_count) {
   constexpr uint32_t dna = DNA ? 1u : 0u;  // the character encoding, fixed per instance
   constexpr uint32_t NW = NT / 32;
   constexpr bool kWide = NT == kSmallWideThreads;
   extern __shared__ __align__(16) uint8_t smem[];
   const SmallSmem m = small_smem(smem, pmax);
-  __shared__ SmallSplit<NT> split;
+  __shared__ SmallSplit<SMAX> split;
   __shared__ uint32_t s_ti, s_open, s_jstop, s_neq, s_runs, s_base;
   __shared__ Task s_task;
   __shared__ uint64_t s_lead[kLookWindows];
@@ -613,7 +618,7 @@ __global__ void __launch_bounds__(NT) k_small_cta(SortCtx c, uint32_t pmax, uint
     // one run: jump over the prefix all its strings share
     bool sorted = s_neq || key_end(k0, dna);
     if (s_neq) {
-      small_sort<NT>(m, split, m.key, n, nullptr, m.pos[0], t.begin);
+      small_sort<NT, SMAX>(m, split, m.key, n, nullptr, m.pos[0], t.begin);
     } else {
       for (uint32_t j = tid; j < n; j += NT) m.pos[0][j] = (uint16_t)j;
       if (tid == 0 && !sorted) {
@@ -744,7 +749,7 @@ __global__ void __launch_bounds__(NT) k_small_cta(SortCtx c, uint32_t pmax, uint
         bytes += 8ull * (jstop + 1);
       }
       __syncthreads();
-      small_sort<NT>(m, split, m.key + lo, n, m.pos[0] + lo, m.pos[1] + lo, t.begin + lo + depth);
+      small_sort<NT, SMAX>(m, split, m.key + lo, n, m.pos[0] + lo, m.pos[1] + lo, t.begin + lo + depth);
       for (uint32_t j = tid; j < n; j += NT) m.pos[0][lo + j] = m.pos[1][lo + j];
       __syncthreads();
     }
@@ -868,8 +873,12 @@ cudaError_t launch_init(const SortCtx& c, cudaStream_t st, const LaunchHook& hoo
 cudaError_t set_small_limits() {
   constexpr cudaFuncAttribute kLimit = cudaFuncAttributeMaxDynamicSharedMemorySize;
   const int wide = (int)small_cta_smem(kSmallCutoffMax);
-  const cudaError_t e = cudaFuncSetAttribute(k_small_cta<kSmallWideThreads, false>, kLimit, wide);
-  return e == cudaSuccess ? cudaFuncSetAttribute(k_small_cta<kSmallWideThreads, true>, kLimit, wide) : e;
+  constexpr uint32_t kNT = kSmallWideThreads;
+  cudaError_t e = cudaFuncSetAttribute(k_small_cta<kNT, kWideSample, false>, kLimit, wide);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_small_cta<kNT, kWideSample, true>, kLimit, wide);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_small_cta<kNT, kManySample, false>, kLimit, wide);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_small_cta<kNT, kManySample, true>, kLimit, wide);
+  return e;
 }
 
 template <bool DNA>
@@ -877,16 +886,18 @@ static cudaError_t launch_small_t(const SortCtx& c, uint32_t pmax, uint32_t sms,
                                   const LaunchHook& hook) {
   // subsets of more than kSmallCtaNarrowMax strings, then smaller ones
   const uint32_t min_count = 2 * sms * kSmallWideBlocks;
-  if (pmax > kSmallCtaNarrowMax)
+  if (pmax > kSmallCtaNarrowMax) {
+    const auto wide = pmax > kManySampleAbove ? k_small_cta<kSmallWideThreads, kManySample, DNA>
+                                              : k_small_cta<kSmallWideThreads, kWideSample, DNA>;
     hook.run("small_cta", [&] {
-      k_small_cta<kSmallWideThreads, DNA>
-          <<<sms * kSmallWideBlocks, kSmallWideThreads, small_cta_smem(pmax), st>>>(c, pmax, min_count);
+      wide<<<sms * kSmallWideBlocks, kSmallWideThreads, small_cta_smem(pmax), st>>>(c, pmax, min_count);
     });
+  }
   const uint32_t narrow_max = min(pmax, kSmallCtaNarrowMax);
   // (so few strings that the wide launch has taken them all: see k_small_cta)
   const bool few = pmax > kSmallCtaNarrowMax && c.total / 33 < min_count;
   if (!few) hook.run("small_cta", [&] {
-    k_small_cta<kSmallNarrowThreads, DNA>
+    k_small_cta<kSmallNarrowThreads, kNarrowSample, DNA>
         <<<sms * kSmallNarrowBlocks, kSmallNarrowThreads, small_cta_smem(narrow_max), st>>>(
             c, narrow_max, pmax > kSmallCtaNarrowMax ? min_count : 0u);
   });

@@ -66,3 +66,24 @@ def test_periodic_order(n, cutoff, period):
             assert np.array_equal(l.cpu().numpy().view(np.uint32), want_l)
         batch.close()
     assert in_order < 1.5 * in_none, (in_order, in_none)
+
+
+def test_large_subsets():
+    # as many strings in subsets of 1024 and of 4096: few enough for every subset to have a block, which then takes
+    # the larger one four times as many steps, most of them short ones; with the same number of splitters for both
+    # a string of the larger one is compared with four times as many others, and it takes 2.7 times as long
+    rng = np.random.default_rng(4)
+    sets = [_rows(rng.integers(97, 123, (4096, LENGTH)).astype(np.uint8)) for _ in range(60)]
+    quarters = [gen.StringSet(s.chars, s.offsets[k:k + 1024].copy()) for s in sets for k in range(0, 4096, 1024)]
+    whole, parts = _us(_batch(sets, 4096)), _us(_batch(quarters, 4096))
+    assert whole < 2 * parts, (whole, parts)
+
+
+@pytest.mark.parametrize("kind", ["letters", "bits"])
+@pytest.mark.parametrize("n", [1023, 1024, 1025, 2047, 2048, 2049, 4095, 4096])
+def test_splitter_counts(n, kind):
+    from gpu_util import assert_parity, gpu_sort
+    lo, hi, length = (97, 123, LENGTH) if kind == "letters" else (97, 99, 10)  # bits: four equal strings each
+    s = _rows(np.random.default_rng(n).integers(lo, hi, (n, length)).astype(np.uint8))
+    assert_parity(s, *gpu_sort(s, small_cutoff=4096))
+    assert_parity(s, *gpu_sort(s, small_cutoff=4096, with_lcp=False))
