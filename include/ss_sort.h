@@ -248,7 +248,7 @@ ss_status ss_merge(const uint8_t* chars, const uint64_t* offsets, uint32_t max_l
                    void* workspace, size_t workspace_bytes, void* stream);
 
 /* Workspace bytes ss_merge needs for these runs: two 32-byte records per
- * string, plus the sample counts (256 for a single run; 0 for invalid
+ * string, plus 8 bytes per sample (256 for a single run; 0 for invalid
  * arguments). */
 size_t ss_merge_workspace_size(const ss_run* runs, uint32_t num_runs, uint32_t sample_step);
 

@@ -194,6 +194,7 @@ struct MergeRoundArgs {
   const MergeRec* src;
   MergeRec* dst;            // null in the last round
   uint32_t* cut;            // per sample: records of the partner run before it
+  uint32_t* cut_lcp;        // ... and its LCP with the one after them
   uint32_t* out_perm;       // last round
   uint32_t* out_lcp;        // last round, may be null
   uint32_t* counter;        // piece counter, zero at launch
