@@ -3,6 +3,7 @@
 // are numbers, and every launch is written to a log, so that tests can check
 // on any machine which launches the host code makes, in which order, from
 // which thread, and under which function attributes.
+#include <algorithm>
 #include <atomic>
 #include <chrono>
 #include <cstdlib>
@@ -25,6 +26,7 @@ std::map<std::pair<int, const void*>, size_t> max_smem;    // per (device, kerne
 std::map<std::string, unsigned> delays_us;                 // by a part of the kernel's name
 std::map<cudaStream_t, cudaGraph_t> capturing;
 std::map<const void*, size_t> allocated;
+size_t live_bytes = 0, peak_bytes = 0;
 std::string text;
 void* host_word = nullptr;
 std::atomic<uintptr_t> next_handle{0x1000};
@@ -61,13 +63,20 @@ cudaError_t allocate(void** p, size_t n) {
   memset(*p, 0, n);
   std::lock_guard<std::mutex> lk(mu);
   allocated[*p] = n;
+  live_bytes += n;
+  peak_bytes = std::max(peak_bytes, live_bytes);
   return cudaSuccess;
 }
 
 cudaError_t release(void* p) {
   {
     std::lock_guard<std::mutex> lk(mu);
-    if (p && !allocated.erase(p)) return fail(cudaErrorInvalidValue);
+    const auto it = allocated.find(p);
+    if (p && it == allocated.end()) return fail(cudaErrorInvalidValue);
+    if (p) {
+      live_bytes -= it->second;
+      allocated.erase(it);
+    }
   }
   free(p);
   return cudaSuccess;
@@ -107,6 +116,13 @@ size_t fake_log(char* out, size_t cap) {
 // in one of twice that if it is not.
 void fake_slow_attributes(int us) { attr_delay_us = us; }
 void* fake_host_word() { return host_word; }
+// Most memory allocated at once since the last call, beyond what is allocated now.
+size_t fake_peak() {
+  std::lock_guard<std::mutex> lk(mu);
+  const size_t over = peak_bytes - live_bytes;
+  peak_bytes = live_bytes;
+  return over;
+}
 
 // `episodes` times: sets bit `low` and then bit `high` of the word, as two
 // kernels of two sorts would, and waits until the word is 0 again.  Meanwhile

@@ -34,6 +34,7 @@ def load(tmp_path):
     lib.fake_log.restype = ctypes.c_size_t
     lib.fake_log.argtypes = [ctypes.c_char_p, ctypes.c_size_t]
     lib.fake_host_word.restype = ctypes.c_void_p
+    lib.fake_peak.restype = ctypes.c_size_t
     lib.fake_capture.argtypes = [ctypes.c_void_p, ctypes.c_int]
     return lib
 
