@@ -248,7 +248,7 @@ ss_status ss_merge(const uint8_t* chars, const uint64_t* offsets, uint32_t max_l
                    void* workspace, size_t workspace_bytes, void* stream);
 
 /* Workspace bytes ss_merge needs for these runs: two 32-byte records per
- * string, plus 8 bytes per sample (256 for a single run; 0 for invalid
+ * string, plus the sample counts (256 for a single run; 0 for invalid
  * arguments). */
 size_t ss_merge_workspace_size(const ss_run* runs, uint32_t num_runs, uint32_t sample_step);
 
@@ -269,13 +269,12 @@ size_t ss_merge_workspace_size(const ss_run* runs, uint32_t num_runs, uint32_t s
  * Synchronous: waits for the result (the host reads the number of unsorted
  * suffixes after each round).  At most about 140 bytes of device memory per
  * text character (and 100 KB) are taken from the stream-ordered pool for the
- * call: 55 (59 without an LCP output) a character throughout, the rest while a round sorts (round 0
- * sorts all suffixes); plus, with an LCP output, 4 bytes per character for
- * every round (the names of each round: an LCP above initial_depth is found by
- * descending through them, O(rounds + initial_depth / 256) per entry however
- * long it is).  Returns
- * SS_ERR_TOO_LARGE for n >= 2^32 - 2, SS_ERR_INVALID for NULL pointers or
- * initial_depth > 2^20. */
+ * call: 55 (59 without an LCP output) a character throughout, the rest while
+ * a round sorts (round 0 sorts all suffixes); plus, with an LCP output, 4 bytes
+ * per character for every round (the names of each round: an LCP above
+ * initial_depth is found by descending through them, O(rounds + initial_depth /
+ * 256) per entry however long it is).  Returns SS_ERR_TOO_LARGE for n >= 2^32 - 2,
+ * SS_ERR_INVALID for NULL pointers or initial_depth > 2^20. */
 ss_status ss_suffix_array(const uint8_t* text, uint64_t n, uint32_t* out_sa, uint32_t* out_lcp,
                           uint32_t initial_depth, void* stream);
 

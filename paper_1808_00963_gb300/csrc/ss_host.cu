@@ -844,6 +844,13 @@ static uint32_t merge_step(uint32_t sample_step, uint64_t total) {
   return (uint32_t)std::max<uint64_t>(kMergeMinStep, (total + kMergePieces - 1) / kMergePieces);
 }
 
+// Where a round keeps its cuts' LCPs (at most one per three strings): where
+// nothing is before the last round has written the order, and in the last
+// round where no records go any more.
+static uint32_t* cut_lcps(uint32_t* order, MergeRec* dst, bool last) {
+  return last ? reinterpret_cast<uint32_t*>(dst) : order;
+}
+
 static ss_status merge_geometry(const ss_run* runs, uint32_t num_runs, uint32_t sample_step, uint64_t* total,
                                 uint32_t* S) {
   if (num_runs == 0 || num_runs > SS_MERGE_MAX_RUNS || !runs) return SS_ERR_INVALID;
@@ -860,14 +867,14 @@ static ss_status merge_geometry(const ss_run* runs, uint32_t num_runs, uint32_t 
   return SS_OK;
 }
 
-// two record buffers (32 bytes per string), the sample cuts of a round and
-// their LCPs, the piece counter.  With the default step room for the most cuts that up to
+// two record buffers (32 bytes per string), the sample cuts of a round, the
+// piece counter.  With the default step room for the most cuts that up to
 // `total` strings have (fewer strings may have more cuts), so that a workspace
 // made for them serves fewer.
 static size_t merge_ws_bytes(uint64_t total, uint32_t num_runs, uint32_t sample_step) {
   if (num_runs <= 1) return 256;
   const uint64_t cuts = sample_step ? total / sample_step : std::min(total / kMergeMinStep, kMergePieces);
-  return 2 * align256(total * sizeof(MergeRec)) + 2 * align256((cuts + num_runs + 1) * 4) + 256;
+  return 2 * align256(total * sizeof(MergeRec)) + align256((cuts + num_runs + 1) * 4) + 256;
 }
 
 size_t ss_merge_workspace_size(const ss_run* runs, uint32_t num_runs, uint32_t sample_step) {
@@ -909,10 +916,8 @@ ss_status ss_merge(const uint8_t* chars, const uint64_t* offsets, uint32_t max_l
   if (own && cudaMallocAsync(reinterpret_cast<void**>(&ws), need, st) != cudaSuccess) return SS_ERR_OOM;
   const size_t recb = align256(total * sizeof(MergeRec));
   MergeRec* rec[2] = {reinterpret_cast<MergeRec*>(ws), reinterpret_cast<MergeRec*>(ws + recb)};
-  const size_t cutb = align256((total / S + K + 1) * 4);
   uint32_t* cut = reinterpret_cast<uint32_t*>(ws + 2 * recb);
-  uint32_t* cut_lcp = reinterpret_cast<uint32_t*>(ws + 2 * recb + cutb);
-  uint32_t* counter = reinterpret_cast<uint32_t*>(ws + 2 * recb + 2 * cutb);
+  uint32_t* counter = reinterpret_cast<uint32_t*>(ws + 2 * recb + align256((total / S + K + 1) * 4));
   const uint32_t cap = max_len ? std::min<uint32_t>(max_len, 1u << 30) : (1u << 30);
   MergePrepArgs pa{};
   pa.chars = chars;
@@ -941,7 +946,7 @@ ss_status ss_merge(const uint8_t* chars, const uint64_t* offsets, uint32_t max_l
     ra.src = rec[cur];
     ra.dst = r + 1 == rounds ? nullptr : rec[cur ^ 1];
     ra.cut = cut;
-    ra.cut_lcp = cut_lcp;
+    ra.cut_lcp = cut_lcps(out_perm, rec[cur ^ 1], r + 1 == rounds);
     ra.out_perm = out_perm;
     ra.out_lcp = out_lcp;
     ra.counter = counter;
@@ -1273,10 +1278,8 @@ static ss_status sort_host_parts(const uint8_t* chars, uint64_t chars_len, const
   const uint32_t sms = (uint32_t)dev.sms;
   const size_t recb = align256(n * sizeof(MergeRec));
   MergeRec* rec[2] = {reinterpret_cast<MergeRec*>(scratch), reinterpret_cast<MergeRec*>(scratch + recb)};
-  const size_t cutb = align256((n / kPipeMinStep + 4) * 4);
   uint32_t* cut = reinterpret_cast<uint32_t*>(scratch + 2 * recb);
-  uint32_t* cut_lcp = reinterpret_cast<uint32_t*>(scratch + 2 * recb + cutb);
-  uint32_t* ctl = reinterpret_cast<uint32_t*>(scratch + 2 * recb + 2 * cutb);
+  uint32_t* ctl = reinterpret_cast<uint32_t*>(scratch + 2 * recb + align256((n / kPipeMinStep + 4) * 4));
   uint32_t* counter = ctl;
   uint32_t* bad = ctl + 1;
   // part p = strings [a[p], a[p + 1]); its characters [b[p], b[p + 1])
@@ -1319,6 +1322,7 @@ static ss_status sort_host_parts(const uint8_t* chars, uint64_t chars_len, const
     for (uint32_t w = 2, lvl = 1; w <= P && (p + 1) % w == 0; w <<= 1, ++lvl) {
       const uint32_t q0 = p + 1 - w;
       MergeRec* dst = w == P ? nullptr : rec[lvl & 1];
+      uint32_t* cut_lcp = cut_lcps(dperm + a[q0], rec[lvl & 1], w == P);
       if (!merge_pair(dchars, doff, cap, rec[(lvl - 1) & 1], dst, (uint32_t)a[q0], (uint32_t)a[q0 + w / 2],
                       (uint32_t)a[p + 1], dperm, dlcp, cut, cut_lcp, counter, sms, st, hook))
         return SS_ERR_CUDA;
@@ -1357,7 +1361,7 @@ ss_status ss_sort_host(const uint8_t* chars, uint64_t chars_len, const uint64_t*
     if (at.type == cudaMemoryTypeDevice) return SS_ERR_INVALID;
   }
   const size_t cb = align256(chars_len + 16), ob = align256(n * 8), pb = align256(n * 4);
-  const size_t scratch = P > 1 ? 2 * align256(n * sizeof(MergeRec)) + 2 * align256((n / kPipeMinStep + 4) * 4) + 256
+  const size_t scratch = P > 1 ? 2 * align256(n * sizeof(MergeRec)) + align256((n / kPipeMinStep + 4) * 4) + 256
                                : 0;
   const size_t need = cb + ob + 2 * pb + scratch;
   uint8_t* d = nullptr;
