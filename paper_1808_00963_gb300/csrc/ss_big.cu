@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(kBlock) k_big_emit(BigCtl* ctl, cudaGraphCondi
           const uint32_t adv = desc - g.t.depth, half = KeyOps<u128>::width(sd.dna) / 2;
           if (adv > half && (adv - half) * 2 <= half) desc = g.t.depth + half;
         }
-        emit_bucket(c, sd, g.t, s, size, desc, next_big, kLcpMark | kLcpWide);
+        emit_bucket(c, sd, g.t, s, size, desc, next_big, true);
         const bool mark = s > 0 && sd.lcp;  // the fix-up at the end visits the listed marks only
         const uint32_t k = warp_slot(c.marks_count, mark);
         if (mark) {

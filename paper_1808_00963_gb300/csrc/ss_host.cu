@@ -1183,7 +1183,6 @@ constexpr uint32_t kPipeAutoParts = 1;
 // Merges of the parts use a sample step between these two, the largest that
 // still gives about 1024 pieces per SM (a piece is merged by one lane).
 constexpr uint32_t kPipeMinStep = 16, kPipeMaxStep = 64;
-static_assert(sizeof(SetDesc) % 4 == 0 && sizeof(GenTask) % 4 == 0, "uploads move whole words");
 
 // A copy stream and its events, per thread and device.
 struct CopyLane {
@@ -1246,7 +1245,7 @@ static bool merge_pair(const uint8_t* chars, const uint64_t* offsets, uint32_t c
   ra.sbase[1] = (mid - lo) / S;
   ra.sbase[2] = ra.sbase[1] + (hi - mid) / S;
   ra.nsamples = ra.sbase[2];
-  return launch_upload(nullptr, counter, sizeof(uint32_t), st, hook) == cudaSuccess &&
+  return launch_zero(counter, 1, st, hook) == cudaSuccess &&
          launch_merge_round(ra, sms, st, hook) == cudaSuccess;
 }
 
@@ -1288,7 +1287,7 @@ static ss_status sort_host_parts(const uint8_t* chars, uint64_t chars_len, const
   b[0] = 0;
   for (uint32_t p = 1; p < P; ++p) b[p] = std::max(b[p - 1], std::min<uint64_t>(offsets[a[p]], chars_len));
   b[P] = chars_len;
-  SS_CUDA(launch_upload(nullptr, ctl, 8, st, hook));
+  SS_CUDA(launch_zero(ctl, 2, st, hook));
   SS_CUDA(cudaEventRecord(lane->start, st));
   SS_CUDA(cudaStreamWaitEvent(lane->cs, lane->start, 0));
   SS_CUDA(cudaMemcpyAsync(doff, offsets, n * 8, cudaMemcpyHostToDevice, lane->cs));

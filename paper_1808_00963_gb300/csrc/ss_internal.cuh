@@ -19,8 +19,7 @@ namespace ss {
 
 constexpr uint32_t kNoCap = 0xFFFFFFFFu;
 constexpr uint32_t kMaxDepth = (1u << 30) - 16;  // deeper strings: SS_ERR_TOO_LARGE
-constexpr uint32_t kLcpMark = 0x80000000u;        // out_lcp[j] = mark | depth: fix up later
-constexpr uint32_t kLcpWide = 0x40000000u;        // ... the two strings differ within 2 keys (a wide step)
+constexpr uint32_t kLcpMark = 0x80000000u;        // out_lcp[j] = mark | depth: the strings differ in the wide keys there
 
 // Device status bits (latched with atomicOr; the host maps them to ss_status).
 constexpr uint32_t kStQueueFull = 1u << 0;
@@ -379,12 +378,7 @@ __device__ __forceinline__ uint32_t load_windows_block(const uint8_t* chars, uin
     x[4 * i + 3] = v.w;
   }
   uint32_t o[2 * KW];
-  {
-    uint32_t y[2 * KW + 4];
-#pragma unroll
-    for (int i = 0; i < 2 * KW + 4; ++i) y[i] = x[i];
-    take_words<2 * KW>(y, sh, o);
-  }
+  take_words<2 * KW>(x, sh, o);
   const uint32_t room = cap - h;
   bool ended = false;
   // most windows hold no end: one test for all of them before any is cut (with

@@ -144,10 +144,9 @@ cudaError_t launch_init(const SortCtx& c, cudaStream_t st, const LaunchHook& hoo
 cudaError_t launch_small(const SortCtx& c, uint32_t pmax, uint32_t sms, bool last, cudaStream_t st,
                          const LaunchHook& hook);
 cudaError_t launch_lcp_fix(const SortCtx& c, uint32_t grid, cudaStream_t st, const LaunchHook& hook);
+// Zeroes a few words with a kernel.
+cudaError_t launch_zero(uint32_t* dst, uint32_t words, cudaStream_t st, const LaunchHook& hook);
 // Packs bytes over {A, C, G, T, 0} into 3-bit codes (dna_key's layout).
-// Copies bytes (a multiple of 4, 4-byte aligned) from pinned host memory
-// with a kernel, or zero-fills dst when host_src is null.
-cudaError_t launch_upload(const void* host_src, void* dst, size_t bytes, cudaStream_t st, const LaunchHook& hook);
 cudaError_t launch_pack_dna(const uint8_t* chars, uint64_t len, uint64_t* out, uint64_t words, uint32_t* bad,
                             uint32_t grid, cudaStream_t st, const LaunchHook& hook);
 cudaError_t launch_distinguishing(const uint8_t* chars, const uint64_t* offsets, uint32_t n, uint32_t cap,

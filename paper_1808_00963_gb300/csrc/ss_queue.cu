@@ -274,7 +274,7 @@ __device__ unsigned long long queue_step(const SortCtx& c, const Task& t, QueueS
   for (uint32_t b = threadIdx.x; b < Gm::K; b += NT) {
     const uint32_t start = s.bstart[b];
     const uint32_t size = s.bstart[b + 1] - start;
-    if (size) emit_bucket(c, sd, t, start, size, s.desc[b], 0, 0u);  // boundary LCPs are written already
+    if (size) emit_bucket(c, sd, t, start, size, s.desc[b], 0, false);  // boundary LCPs are written already
   }
   return bytes;
 }

@@ -260,11 +260,9 @@ __device__ __forceinline__ void pack_rounds(uint32_t nt, uint32_t my_len, Round&
 // Warps take runs of up to 16 consecutive small tasks and pack as many whole
 // tasks as fit into 32 lanes per round.
 constexpr uint32_t kPackChunk = 16;
-// Passes over the warp tasks: look-aheads (64 characters each) a run may take
-// in each pass before it is deferred to the next one (0: no limit).
-constexpr uint32_t kWarpPassJumps[] = {1, 0};
-constexpr uint32_t kWarpPasses = sizeof(kWarpPassJumps) / sizeof(kWarpPassJumps[0]);
-static_assert(kWarpPassJumps[kWarpPasses - 1] == 0, "the last pass finishes every run");
+// Look-aheads (64 characters each) a run may take in the first of the two
+// passes over the warp tasks; then it is left to the second one.
+constexpr uint32_t kFirstPassJumps = 1;
 
 // One pass over a list of warp tasks.  With max_jumps > 0, runs with long
 // common prefixes are deferred to the list `out`: their records go back to
@@ -761,7 +759,7 @@ __global__ void __launch_bounds__(NT) k_small_cta(SortCtx c, uint32_t pmax, uint
 
 // Resolves the boundary marks left by the multi-block steps (listed in
 // c.marks): out_lcp[j] = mark | h means the strings at j-1 and j share exactly
-// their first h characters plus the common prefix of their keys at depth h.
+// their first h characters plus the common prefix of their wide keys at depth h.
 // (The single-block steps write their boundary LCPs themselves.)
 __global__ void __launch_bounds__(kBlock) k_lcp_fix(SortCtx c) {
   const uint32_t stride = gridDim.x * blockDim.x;
@@ -777,20 +775,13 @@ __global__ void __launch_bounds__(kBlock) k_lcp_fix(SortCtx c) {
     const uint32_t v = sd.lcp[j];
     bytes += 8;  // list entry and LCP entry read
     if (j == 0 || !(v & kLcpMark)) continue;
-    const uint32_t h = v & ~(kLcpMark | kLcpWide);
+    const uint32_t h = v & ~kLcpMark;
     const uint32_t pa = sd.perm[j - 1], pb = sd.perm[j];
     if (pa >= sd.n || pb >= sd.n) continue;  // cannot happen after a sort without errors
-    if (v & kLcpWide) {  // a boundary of a multi-block step: the strings differ within its wide key
-      const u128 a = load_key128(sd.chars, sd.offsets[pa], h, sd.cap, sd.dna);
-      const u128 b = load_key128(sd.chars, sd.offsets[pb], h, sd.cap, sd.dna);
-      sd.lcp[j] = h + KeyOps<u128>::lcp(a, b, sd.dna);
-      bytes += 60;  // lcp 4 written; per string: perm 4 + offset 8 + 16 characters read
-    } else {
-      const uint64_t a = load_key(sd.chars, sd.offsets[pa], h, sd.cap, sd.dna);
-      const uint64_t b = load_key(sd.chars, sd.offsets[pb], h, sd.cap, sd.dna);
-      sd.lcp[j] = h + key_lcp(a, b, sd.dna);
-      bytes += 44;  // lcp 4 written; per string: perm 4 + offset 8 + 8 characters read
-    }
+    const u128 a = load_key128(sd.chars, sd.offsets[pa], h, sd.cap, sd.dna);
+    const u128 b = load_key128(sd.chars, sd.offsets[pb], h, sd.cap, sd.dna);
+    sd.lcp[j] = h + KeyOps<u128>::lcp(a, b, sd.dna);
+    bytes += 60;  // lcp 4 written; per string: perm 4 + offset 8 + 16 characters read
   }
   account(c, kKLcpFix, bytes);
 }
@@ -906,16 +897,11 @@ static cudaError_t launch_small_t(const SortCtx& c, uint32_t pmax, uint32_t sms,
     hook.run("small_warp", [&] { k_small_warp<true, DNA><<<grid, kBlock, 0, st>>>(c, c.small_warp, c.small_deep, 0u); });
     return cudaGetLastError();
   }
-  // the lists alternate: a pass reads one and defers into the other, emptied first
-  for (uint32_t p = 0; p < kWarpPasses; ++p) {
-    const TaskList in = (p & 1) ? c.small_deep : c.small_warp;
-    const TaskList out = (p & 1) ? c.small_warp : c.small_deep;
-    if (p > 0 && kWarpPassJumps[p] > 0) {
-      const cudaError_t e = launch_upload(nullptr, out.count, 4, st, hook);
-      if (e != cudaSuccess) return e;
-    }
-    hook.run("small_warp", [&] { k_small_warp<false, DNA><<<grid, kBlock, 0, st>>>(c, in, out, kWarpPassJumps[p]); });
-  }
+  // the second pass takes what the first one has deferred, and defers nothing
+  hook.run("small_warp", [&] {
+    k_small_warp<false, DNA><<<grid, kBlock, 0, st>>>(c, c.small_warp, c.small_deep, kFirstPassJumps);
+  });
+  hook.run("small_warp", [&] { k_small_warp<false, DNA><<<grid, kBlock, 0, st>>>(c, c.small_deep, c.small_warp, 0u); });
   return cudaGetLastError();
 }
 
@@ -931,25 +917,14 @@ cudaError_t launch_pack_dna(const uint8_t* chars, uint64_t len, uint64_t* out, u
   return cudaGetLastError();
 }
 
-// Small host-to-device transfers and zero fills done by a kernel rather than
-// by the copy engines, which a large copy queued on another stream can hold
-// up for milliseconds: src is pinned host memory, which the device reads
-// directly (null: write zeros).
-__global__ void k_upload(const uint32_t* __restrict__ src, uint32_t* __restrict__ dst, uint32_t words) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < words; i += gridDim.x * blockDim.x)
-    dst[i] = src ? src[i] : 0u;
+// A few zero words written by a kernel: a copy engine that works on a large
+// copy queued on another stream would hold a memset up for milliseconds.
+__global__ void k_zero(uint32_t* dst, uint32_t words) {
+  for (uint32_t i = threadIdx.x; i < words; i += blockDim.x) dst[i] = 0u;
 }
 
-cudaError_t launch_upload(const void* host_src, void* dst, size_t bytes, cudaStream_t st, const LaunchHook& hook) {
-  if (bytes == 0) return cudaSuccess;
-  if ((bytes & 3) || (reinterpret_cast<uintptr_t>(dst) & 3) || (reinterpret_cast<uintptr_t>(host_src) & 3) ||
-      bytes >= (4ull << 32))
-    return cudaErrorInvalidValue;
-  const uint32_t words = (uint32_t)(bytes / 4);
-  const uint32_t grid = std::min<uint32_t>((words + kBlock - 1) / kBlock, 1024);
-  hook.run("upload", [&] {
-    k_upload<<<grid, kBlock, 0, st>>>(static_cast<const uint32_t*>(host_src), static_cast<uint32_t*>(dst), words);
-  });
+cudaError_t launch_zero(uint32_t* dst, uint32_t words, cudaStream_t st, const LaunchHook& hook) {
+  hook.run("zero", [&] { k_zero<<<1, 32, 0, st>>>(dst, words); });
   return cudaGetLastError();
 }
 

@@ -621,14 +621,14 @@ __device__ __forceinline__ uint32_t move_batch_wide(const SortCtx& c, const SetD
   return bytes;
 }
 
-// Emits the outcome of one non-empty bucket: its boundary LCP mark (resolved at
-// the end, Section 4.2.8 "LCP Calculation": the LCP with the previous bucket is
-// depth + lcp of the two strings' caches at this depth) and, if it is not
-// finished, a new task.
+// Emits the outcome of one non-empty bucket: its boundary LCP mark, if asked
+// for (resolved at the end, Section 4.2.8 "LCP Calculation": the LCP with the
+// previous bucket is depth + lcp of the two strings' wide keys at this depth)
+// and, if it is not finished, a new task.
 __device__ __forceinline__ void emit_bucket(const SortCtx& c, const SetDesc& sd, const Task& t,
                                             uint32_t start, uint32_t size, uint32_t desc,
-                                            uint32_t next_big, uint32_t mark = kLcpMark) {
-  if (mark && start > 0 && sd.lcp) sd.lcp[t.begin + start - sd.base] = mark | t.depth;
+                                            uint32_t next_big, bool mark) {
+  if (mark && start > 0 && sd.lcp) sd.lcp[t.begin + start - sd.base] = kLcpMark | t.depth;
   if (!(desc & kFin)) {
     Task ch{t.begin + start, size, desc & kLow30, make_meta(task_set(t), task_par(t) ^ 1)};
     route_task(c, ch, next_big);
