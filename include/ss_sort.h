@@ -98,9 +98,9 @@ typedef struct ss_options {
                                   sorted while part p + 1 is still being
                                   copied; the sorted parts are LCP-merged
                                   (Section 4.3).  0 or 1 = copy everything,
-                                  then sort (the default: over a host link
-                                  as fast as the sort, the parts' sorts and
-                                  merges cost more than the overlap saves);
+                                  then sort (the default: over a fast host
+                                  link the parts' sorts and merges cost about
+                                  what the overlap saves, or more);
                                   else a power of two <= 16.  Ignored
                                   elsewhere.                                  */
     uint32_t wait_limit_us;    /* bound, in microseconds, on every device-side

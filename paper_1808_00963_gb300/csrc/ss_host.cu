@@ -835,9 +835,13 @@ ss_status ss_distinguishing(const uint8_t* chars, const uint64_t* offsets, uint6
 // takes as long as its longest pieces times the passes over the lanes: the step
 // makes 9/10 as many pieces as the GPU holds lanes, and is never below 3
 // (a sample costs a binary search).  Measured against the fixed step of 64:
-// 20 M URLs in 16 runs 3875 -> 3598 us (136: 3525, 128, one piece more than
-// lanes: 3744), 5 M 1356 -> 1204, 1 M in 8 runs 766 -> 379, 200 k 712 -> 193,
-// 20 k 693 -> 159.
+// 20 M URLs in 16 runs 3875 -> 3598 us, 5 M 1356 -> 1204, 1 M in 8 runs 766 ->
+// 379, 200 k 712 -> 193, 20 k 693 -> 159.  5/10, 8/10, 9/10 and 10/10 of the
+// lanes: 20 M URLs 4231 / 3660 / 3598 / 3480 us, 8 M random strings in 16 runs
+// 1705 / 1516 / 1497 / 1453, 1 M URLs in 8 390 / 377 / 391 / 395, 500 k random
+// strings in 8 201 / 209 / 219 / 221.  (9/10 dates from pieces that read their
+// first strings again: a step of 128, one piece past the lanes, then took 3744
+// us on 20 M URLs, one of 143 3598.)
 constexpr uint64_t kMergePieces = 152ull * kMergeLanesPerSm * 9 / 10, kMergeMinStep = 3;
 static uint32_t merge_step(uint32_t sample_step, uint64_t total) {
   if (sample_step) return sample_step;
@@ -970,9 +974,10 @@ ss_status ss_merge(const uint8_t* chars, const uint64_t* offsets, uint32_t max_l
 // The suffix array's own sorts (the capped sort of all suffixes and the rounds'
 // pair sorts) hand subsets of up to 128 strings to the block sorts and keep
 // subsets of up to 32768 on single-block steps: the subsets of a text's
-// suffixes after the first characters are many and small, and on a GB300 these
-// two settings took the 4M-character DNA-like text from 2.44 to 2.16 ms
-// (1024 / 8192, the plain sort's defaults; 256 / 32768 gave 2.18 ms).
+// suffixes after the first characters are many and small.  The 4 M-character
+// DNA-like text takes 1102 us with them, 1212 with 1024 / 8192, the plain sort's
+// defaults, 1208 with 128 / 8192, 1096 with 1024 / 32768, 1072 with 256 / 32768
+// (texts of one repeated block, Fibonacci and unary ones the same within 3 %).
 constexpr uint32_t kSaSmallCutoff = 128;
 constexpr uint32_t kSaBigThreshold = 32768;
 
@@ -1176,9 +1181,10 @@ ss_status ss_sort_dna(const uint8_t* chars, uint64_t chars_len, const uint64_t* 
 // ---- host buffers ------------------------------------------------------------------
 
 // With the default (0) the whole set is copied, then sorted: on the GB300's
-// host link (about 210 GB/s) sorting the parts and merging them costs more
-// than the overlap saves (20 M URL-like strings: 13.5 ms in one piece, 14.5 /
-// 16.0 / 20.4 ms in 2 / 4 / 8 parts).
+// host link (about 210 GB/s) sorting the parts and merging them costs about
+// what the overlap saves for the largest sets and more for others (in one piece
+// / 2 / 4 / 8 parts: 20 M URL-like strings 11.5 / 11.2 / 11.1 / 13.0 ms, 2 M 1.56
+// / 1.88 / 2.72 / 4.43, 200 k 0.52 / 0.95 / 1.28 / 2.42).
 constexpr uint32_t kPipeAutoParts = 1;
 // Merges of the parts use a sample step between these two, the largest that
 // still gives about 1024 pieces per SM (a piece is merged by one lane).
@@ -1577,9 +1583,11 @@ extern "C" ss_status ss_sort_noalloc(const uint8_t* chars, const uint64_t* offse
   Opts o;
   if (max_len) o.cap = max_len;
   // One round of multi-block steps where ss_sort would take them (a root of
-  // 20 000 strings took one block 70 us: 20 k random strings 149 -> 131 us, 65 536
-  // 305 -> 145, 20 k URLs 279 -> 198); the rounds after it
-  // would be a graph, whose instantiation may allocate.
+  // 20 000 strings takes one block 70 us); the rounds after it would be a graph,
+  // whose instantiation may allocate.  Without / with the round: random strings
+  // 10 k 121 / 137 us, 16 k 132 / 139, 20 k 157 / 138, 65 536 310 / 160; URLs
+  // 8193 156 / 150, 10 k 174 / 160, 20 k 267 / 207: URLs gain from the first size
+  // on, random strings from about 17 000.
   const Rounds rounds = n > o.big_thr ? Rounds::kOne : Rounds::kNone;
   const Layout L = make_layout(n, 1, o, rounds, by_rank(n, o), SS_NOALLOC_SCRATCH_BYTES);
   if (L.total > SS_NOALLOC_SCRATCH_BYTES) return SS_ERR_TOO_LARGE;

@@ -67,9 +67,9 @@ struct BigCtl {
 // filled 49 of 152 SMs: classification 17.3 -> 12.8 us, scatter 22.9 -> 15.4
 // us), at most kMaxTileRounds, and more where the tiles' counters would not
 // fit.  With at most 16 the scatter's shared memory lets three blocks share an
-// SM instead of two (20 M URLs 4820 -> 4415 us, 4 M DNA suffixes 1270 -> 1201
-// us; at most 8: 4401 / 1164 us, but the batch of 512 sets 2637 instead of 2620
-// us and twice the counters).
+// SM instead of two; with 8 there are twice the counters (at most 8 / 16 / 32:
+// 20 M URLs 4065 / 4020 / 4255 us, 512 sets 1992 / 1973 / 2016, 4 M DNA suffixes
+// 940 / 948 / 954, 10 M random strings 1579 / 1600 / 1704).
 constexpr uint32_t kMinTileRounds = 2, kMaxTileRounds = 16, kTilesPerSm = 9;
 __host__ __device__ inline uint32_t tile_rounds(uint64_t total, uint64_t G, uint32_t sms, uint32_t K,
                                                 uint64_t ncounters_max, uint32_t fixed) {

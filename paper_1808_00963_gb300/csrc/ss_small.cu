@@ -2,15 +2,15 @@
 //
 // A subset of at most small_cutoff strings with a common prefix of `depth`
 // characters is finished by one block (33..cutoff strings) or one warp (2..32)
-// without further distribution steps: its records are sorted by
-// (segment, cache, index) in shared memory or registers; runs of equal caches
-// without a terminator are refined by reloading their caches 8 characters
-// deeper and sorting again (the recursion of the equality buckets of
-// Section 4.2.2, done in place).  This replaces the paper's sequential base
-// cases (caching multikey quicksort and insertion sort, Section 4.2.8) with
-// sorting networks that suit a warp or a block.  LCPs between neighbours are
-// computed from the caches as they are separated (Section 4.2.3, "LCP via
-// XOR").
+// without further distribution steps.  A block splits the subset once by a
+// sample of its caches and ranks every string by counting within its bucket; a
+// warp sorts its strings by (segment, cache, index) with a network in
+// registers.  Runs of equal caches without a terminator are refined by
+// reloading their caches deeper and sorting again (the recursion of the
+// equality buckets of Section 4.2.2, done in place).  This replaces the paper's
+// sequential base cases (caching multikey quicksort and insertion sort,
+// Section 4.2.8).  LCPs between neighbours are computed from the caches as they
+// are separated (Section 4.2.3, "LCP via XOR").
 #include "ss_kernels.h"
 #include "ss_step.cuh"
 
