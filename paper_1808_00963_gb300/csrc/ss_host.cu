@@ -744,13 +744,25 @@ struct ss_batch {
   uint32_t num_sets = 0;
   uint32_t total = 0;
   std::vector<ss::SetDesc> sd;  // the set descriptors, written into the workspace by each run
+  // A thread that asks for a stream's status may be reading the workspace when
+  // another one destroys the plan: it keeps the plan alive and holds `use`, and
+  // finds ws null if it came too late.
+  std::mutex use;
+  std::shared_ptr<ss_batch> self;  // the handle's own reference, until ss_batch_destroy
 };
 
 using namespace ss;
 
 // Last asynchronous run enqueued on each stream (for ss_stream_status).
 static std::mutex g_stream_mu;
-static std::map<void*, ss_batch*> g_stream_last;
+static std::map<void*, std::shared_ptr<ss_batch>> g_stream_last;
+
+// Waits for the stream and returns the status a plan's last run has left (SS_OK
+// if the plan has been destroyed).
+static ss_status batch_status(ss_batch& b, cudaStream_t st) {
+  std::lock_guard<std::mutex> hold(b.use);
+  return b.num_sets && b.ws ? read_status(b.ws, b.L, st) : SS_OK;
+}
 
 extern "C" {
 
@@ -1428,7 +1440,8 @@ size_t ss_batch_workspace_size(const ss_set* sets, uint32_t num_sets, const ss_o
 ss_status ss_batch_create(const ss_set* sets, uint32_t num_sets, const ss_options* opt, ss_batch** out) {
   if (!out) return SS_ERR_INVALID;
   *out = nullptr;
-  ss_batch b;
+  std::shared_ptr<ss_batch> plan(new ss_batch);
+  ss_batch& b = *plan;
   ss_status s = resolve_opts(opt, b.o);
   if (s != SS_OK) return s;
   uint64_t total = 0;
@@ -1454,7 +1467,8 @@ ss_status ss_batch_create(const ss_set* sets, uint32_t num_sets, const ss_option
   }
   b.num_sets = num_sets;
   b.total = (uint32_t)total;
-  *out = new ss_batch(b);
+  b.self = plan;
+  *out = plan.get();
   return SS_OK;
 }
 
@@ -1463,7 +1477,7 @@ ss_status ss_batch_run(ss_batch* b, void* stream) {
   if (b->num_sets == 0) return SS_OK;
   {
     std::lock_guard<std::mutex> lk(g_stream_mu);
-    g_stream_last[stream] = b;
+    g_stream_last[stream] = b->self;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // the set descriptors, as kernel parameters (no staging copy to wait for,
@@ -1488,8 +1502,7 @@ ss_status ss_batch_run(ss_batch* b, void* stream) {
 
 ss_status ss_batch_status(ss_batch* b, void* stream) {
   if (!b) return SS_ERR_INVALID;
-  if (b->num_sets == 0) return SS_OK;
-  return read_status(b->ws, b->L, static_cast<cudaStream_t>(stream));
+  return batch_status(*b, static_cast<cudaStream_t>(stream));
 }
 
 ss_status ss_batch_destroy(ss_batch* b) {
@@ -1497,15 +1510,17 @@ ss_status ss_batch_destroy(ss_batch* b) {
   {
     std::lock_guard<std::mutex> lk(g_stream_mu);
     for (auto it = g_stream_last.begin(); it != g_stream_last.end();)
-      it = (it->second == b) ? g_stream_last.erase(it) : std::next(it);
+      it = (it->second.get() == b) ? g_stream_last.erase(it) : std::next(it);
   }
+  const std::shared_ptr<ss_batch> last = std::move(b->self);  // the plan goes with its last reader
+  std::lock_guard<std::mutex> hold(b->use);
   if (b->owned) cudaFree(b->ws);
-  delete b;
+  b->ws = nullptr;
   return SS_OK;
 }
 
 ss_status ss_stream_status(void* stream) {
-  ss_batch* b = nullptr;
+  std::shared_ptr<ss_batch> b;
   {
     std::lock_guard<std::mutex> lk(g_stream_mu);
     auto it = g_stream_last.find(stream);
@@ -1514,7 +1529,7 @@ ss_status ss_stream_status(void* stream) {
   // the sorts' status word of the stream, then the last batch run on it
   const ss_status s = take_stream_status(static_cast<cudaStream_t>(stream));
   if (s != SS_OK || !b) return s;
-  return ss_batch_status(b, stream);
+  return batch_status(*b, static_cast<cudaStream_t>(stream));
 }
 
 ss_status ss_sort_batch(const ss_set* sets, uint32_t num_sets, const ss_options* opt, void* stream) {

@@ -26,7 +26,7 @@ std::map<std::pair<int, const void*>, size_t> max_smem;    // per (device, kerne
 std::map<std::string, unsigned> delays_us;                 // by a part of the kernel's name
 std::map<cudaStream_t, cudaGraph_t> capturing;
 std::map<const void*, size_t> allocated;
-size_t live_bytes = 0, peak_bytes = 0;
+size_t live_bytes = 0, peak_bytes = 0, stray_copies = 0;
 std::string text;
 void* host_word = nullptr;
 std::atomic<uintptr_t> next_handle{0x1000};
@@ -116,6 +116,11 @@ size_t fake_log(char* out, size_t cap) {
 // in one of twice that if it is not.
 void fake_slow_attributes(int us) { attr_delay_us = us; }
 void* fake_host_word() { return host_word; }
+// Copies from addresses that are in no allocation (device memory that has been freed), which were left out.
+size_t fake_stray_copies() {
+  std::lock_guard<std::mutex> lk(mu);
+  return stray_copies;
+}
 // Most memory allocated at once since the last call, beyond what is allocated now.
 size_t fake_peak() {
   std::lock_guard<std::mutex> lk(mu);
@@ -248,7 +253,15 @@ cudaError_t cudaHostGetDevicePointer(void** d, void* h, unsigned) {
 cudaError_t cudaFree(void* p) { return release(p); }
 cudaError_t cudaFreeAsync(void* p, cudaStream_t) { return release(p); }
 cudaError_t cudaFreeHost(void* p) { return release(p); }
-cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind kind, cudaStream_t) {
+  std::lock_guard<std::mutex> lk(mu);
+  if (kind == cudaMemcpyDeviceToHost) {
+    auto it = allocated.upper_bound(s);
+    if (it == allocated.begin() || (const char*)s + n > (const char*)(--it)->first + it->second) {
+      ++stray_copies;
+      return cudaSuccess;
+    }
+  }
   memmove(d, s, n);
   return cudaSuccess;
 }
@@ -288,8 +301,13 @@ cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
 }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t st) {
-  std::lock_guard<std::mutex> lk(mu);
-  log_line("wait", st, nullptr);
+  unsigned us;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    log_line("wait", st, nullptr);
+    us = delays_us.count("wait") ? delays_us["wait"] : 0;
+  }
+  pause_us(us);
   return cudaSuccess;
 }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }

@@ -1,6 +1,7 @@
 """What the host code does when several threads sort on one stream, checked on
 a stand-in for the CUDA runtime that logs the launches."""
 import ctypes
+import time
 
 import numpy as np
 import pytest
@@ -136,3 +137,27 @@ def test_captured_sort_has_its_own_control_block(lib):
     captured = control_blocks()
     lib.fake_capture(STREAM, 0)
     assert len(captured) == 1 and ws <= min(captured) < ws + size
+
+
+def test_batch_destroyed_while_its_stream_is_asked(lib):
+    """The status of a stream includes that of the last batch run on it, which another thread may destroy while the
+    stream is waited for: its workspace, gone by then, is not read."""
+    stop = []
+    descs = (ss.SetDesc * 2)(Set(50).desc(), Set(100).desc())
+
+    def run():
+        for _ in range(100):
+            batch = ctypes.c_void_p()
+            assert lib.ss_batch_create(descs, 2, None, ctypes.byref(batch)) == 0
+            assert lib.ss_batch_run(batch, ctypes.c_void_p(STREAM)) == 0
+            time.sleep(0.001)
+            assert lib.ss_batch_destroy(batch) == 0
+        stop.append(True)
+        return True
+
+    def ask():
+        return {lib.ss_stream_status(ctypes.c_void_p(STREAM)) for _ in iter(lambda: bool(stop), True)}
+
+    lib.fake_delay(b"wait", 1500)
+    assert fake_util.in_threads(run, ask, ask) == [True, {0}, {0}]
+    assert lib.fake_stray_copies() == 0
