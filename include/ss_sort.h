@@ -161,8 +161,8 @@ size_t ss_workspace_size(uint64_t n, const ss_options* opt);
  * sort parts independently, then K-way LCP-merge them).  That needs the
  * strings packed in index order (string i lies in [offsets[i],
  * offsets[i + 1]) with its terminator at offsets[i + 1] - 1, the last one
- * ending at chars_len - 1), which is checked on the device once all bytes
- * are in; a set that is not packed that way (overlapping strings, gaps,
+ * ending at chars_len - 1), which is checked on the device part by part;
+ * a set that is not packed that way (overlapping strings, gaps,
  * another order) is then sorted again as a whole, with the same result.
  * offsets must then be host-readable memory (SS_ERR_INVALID for a device
  * pointer).  The extra device memory of the parts is 64 bytes per string. */

@@ -1274,10 +1274,11 @@ static bool merge_pair(const uint8_t* chars, const uint64_t* offsets, uint32_t c
 // 32-byte merge records, and adjacent runs are LCP-merged as soon as both
 // exist (a binary tree, the last level writing the outputs).  This needs
 // every part's strings inside its own stretch of chars (strings packed in
-// index order), which k_layout_check verifies on the device once everything
-// has arrived; a set that fails is sorted again as a whole (the parts'
-// results are discarded).  Returns SS_OK with *done = false when the layout
-// check failed.
+// index order), which k_layout_check verifies on the device before each part is
+// sorted; a set that fails is sorted again as a whole (the parts' results are
+// discarded, and from the failing part on they are of empty strings).  Returns
+// SS_OK with *done = false when the layout check failed; the offsets on the
+// device are then not the caller's any more.
 static ss_status sort_host_parts(const uint8_t* chars, uint64_t chars_len, const uint64_t* offsets, uint64_t n,
                                  uint32_t P, uint8_t* dchars, uint64_t* doff, uint32_t* dperm, uint32_t* dlcp,
                                  uint8_t* scratch, const Opts& o, const ss_options* opt, const DevInfo& dev,
@@ -1320,6 +1321,7 @@ static ss_status sort_host_parts(const uint8_t* chars, uint64_t chars_len, const
   for (uint32_t p = 0; p < P; ++p) {
     SS_CUDA(cudaStreamWaitEvent(st, lane->chunk[p], 0));
     const uint32_t lo = (uint32_t)a[p], np = (uint32_t)(a[p + 1] - a[p]);
+    SS_CUDA(launch_layout_check(dchars, b[p + 1], doff + lo, np, chars_len, bad, sms, st, hook));
     s = sort_device(dchars, doff + lo, np, dperm + lo, dlcp + lo, opt, st);
     if (s != SS_OK) return s;
     MergePrepArgs pa{};
@@ -1345,7 +1347,6 @@ static ss_status sort_host_parts(const uint8_t* chars, uint64_t chars_len, const
         return SS_ERR_CUDA;
     }
   }
-  SS_CUDA(launch_layout_check(dchars, chars_len, doff, (uint32_t)n, bad, sms, st, hook));
   if (t_down.reserve(256) != SS_OK) return SS_ERR_OOM;
   uint32_t* hbad = static_cast<uint32_t*>(t_down.p);
   SS_CUDA(cudaMemcpyAsync(hbad, bad, 4, cudaMemcpyDeviceToHost, st));
@@ -1395,8 +1396,8 @@ ss_status ss_sort_host(const uint8_t* chars, uint64_t chars_len, const uint64_t*
     r = sort_host_parts(chars, chars_len, offsets, n, P, dchars, doff, dperm, dlcp, d + cb + ob + 2 * pb, o, opt,
                         dev, st, &done);
   if (r == SS_OK && !done) {
-    if (P == 1 && (cudaMemcpyAsync(dchars, chars, chars_len, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-                   cudaMemcpyAsync(doff, offsets, n * 8, cudaMemcpyHostToDevice, st) != cudaSuccess))
+    if ((P == 1 && cudaMemcpyAsync(dchars, chars, chars_len, cudaMemcpyHostToDevice, st) != cudaSuccess) ||
+        cudaMemcpyAsync(doff, offsets, n * 8, cudaMemcpyHostToDevice, st) != cudaSuccess)
       r = SS_ERR_CUDA;
     if (r == SS_OK) r = sort_device(dchars, doff, n, dperm, out_lcp ? dlcp : nullptr, opt, st);
   }

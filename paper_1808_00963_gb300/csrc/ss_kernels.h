@@ -206,8 +206,9 @@ cudaError_t launch_merge_round(const MergeRoundArgs& a, uint32_t sms, cudaStream
 cudaError_t launch_merge_copy(const uint32_t* perm, const uint32_t* lcp, uint32_t n, uint32_t* out_perm,
                               uint32_t* out_lcp, uint32_t sms, cudaStream_t st, const LaunchHook& hook);
 // Sets *bad unless every string i lies in [offsets[i], offsets[i + 1]) with
-// its terminator at offsets[i + 1] - 1 (the last one ending at chars_len - 1).
-cudaError_t launch_layout_check(const uint8_t* chars, uint64_t chars_len, const uint64_t* offsets, uint32_t n,
+// its terminator at offsets[i + 1] - 1 (the last one ending at end - 1).  If
+// *bad is set, by this call or before it, all offsets become `empty`.
+cudaError_t launch_layout_check(const uint8_t* chars, uint64_t end, uint64_t* offsets, uint32_t n, uint64_t empty,
                                 uint32_t* bad, uint32_t sms, cudaStream_t st, const LaunchHook& hook);
 
 // Suffix array by prefix doubling (ss_sa.cu).

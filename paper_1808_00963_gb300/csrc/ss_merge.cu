@@ -437,18 +437,28 @@ __global__ void k_merge_copy(const uint32_t* __restrict__ perm, const uint32_t* 
 }
 
 // Strings packed one after the other in index order: string i starts after
-// string i - 1's terminator.  A set that passes can be sorted in parts while
-// later parts are still being copied (each part's strings lie in its own
-// stretch of chars).
-__global__ void k_layout_check(const uint8_t* __restrict__ chars, uint64_t chars_len,
-                               const uint64_t* __restrict__ offsets, uint32_t n, uint32_t* bad) {
+// string i - 1's terminator.  A set of such strings can be sorted in parts while
+// later parts are still being copied: the n strings of a part end before `end`,
+// the first character after its stretch of chars, and only characters before
+// that are read here.
+__global__ void k_layout_check(const uint8_t* __restrict__ chars, uint64_t end, const uint64_t* __restrict__ offsets,
+                               uint32_t n, uint32_t* bad) {
   bool ok = true;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const uint64_t o = offsets[i];
-    const uint64_t e = i + 1 < n ? offsets[i + 1] : chars_len;
-    ok = ok && o < e && e <= chars_len && chars[e - 1] == 0;
+    const uint64_t e = i + 1 < n ? offsets[i + 1] : end;
+    ok = ok && o < e && e <= end && chars[e - 1] == 0;
   }
   if (__syncthreads_or(!ok) && threadIdx.x == 0) *bad = 1u;
+}
+
+// After a part that is not packed that way, its strings and those of the later
+// parts may reach into characters that are still being copied.  Sorts and
+// merges follow their keys and LCPs without checks, so they get empty strings
+// instead: the results are discarded anyway.
+__global__ void k_layout_guard(uint64_t* offsets, uint32_t n, uint64_t empty, const uint32_t* bad) {
+  if (!*bad) return;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) offsets[i] = empty;
 }
 
 uint32_t grid_for(uint64_t items, uint32_t block, uint32_t sms, uint32_t per_sm) {
@@ -482,10 +492,11 @@ cudaError_t launch_merge_copy(const uint32_t* perm, const uint32_t* lcp, uint32_
   return cudaGetLastError();
 }
 
-cudaError_t launch_layout_check(const uint8_t* chars, uint64_t chars_len, const uint64_t* offsets, uint32_t n,
+cudaError_t launch_layout_check(const uint8_t* chars, uint64_t end, uint64_t* offsets, uint32_t n, uint64_t empty,
                                 uint32_t* bad, uint32_t sms, cudaStream_t st, const LaunchHook& hook) {
-  hook.run("layout_check",
-           [&] { k_layout_check<<<grid_for(n, 256, sms, 8), 256, 0, st>>>(chars, chars_len, offsets, n, bad); });
+  const uint32_t grid = grid_for(n, 256, sms, 8);
+  hook.run("layout_check", [&] { k_layout_check<<<grid, 256, 0, st>>>(chars, end, offsets, n, bad); });
+  hook.run("layout_check", [&] { k_layout_guard<<<grid, 256, 0, st>>>(offsets, n, empty, bad); });
   return cudaGetLastError();
 }
 

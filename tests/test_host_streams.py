@@ -161,3 +161,20 @@ def test_batch_destroyed_while_its_stream_is_asked(lib):
     lib.fake_delay(b"wait", 1500)
     assert fake_util.in_threads(run, ask, ask) == [True, {0}, {0}]
     assert lib.fake_stray_copies() == 0
+
+
+@pytest.mark.parametrize("parts", [2, 4, 16])
+def test_parts_are_checked_before_they_are_sorted(lib, parts):
+    """A part of a host set is sorted while the characters of later ones are on their way.  Strings that reach into
+    those must not be read: each part's layout is checked, and such strings left out, before its sort begins."""
+    s = Set(BIG * parts)
+    chars = np.zeros(s.n * 2, np.uint8)
+    offsets = np.arange(s.n, dtype=np.uint64) * 2
+    lib.fake_clear_log()
+    o = ss.make_options(host_parts=parts)
+    assert lib.ss_sort_host(chars.ctypes.data, chars.size, offsets.ctypes.data, s.n, s.ptrs[2], s.ptrs[3],
+                            ctypes.byref(o), ctypes.c_void_p(STREAM)) == 0
+    names = {"k_layout_check": "check", "k_layout_guard": "guard", "k_begin": "sort", "k_merge_prep": "records"}
+    order = [kind for _, _, stream, what, _ in fake_util.log(lib) if stream == STREAM
+             for part, kind in names.items() if part in what]
+    assert order == ["check", "guard", "sort", "records"] * parts
