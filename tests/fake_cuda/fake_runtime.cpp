@@ -28,6 +28,7 @@ std::map<cudaStream_t, cudaGraph_t> capturing;
 std::map<const void*, size_t> allocated;
 size_t live_bytes = 0, peak_bytes = 0, stray_copies = 0;
 std::string text;
+bool logging = true;
 void* host_word = nullptr;
 std::atomic<uintptr_t> next_handle{0x1000};
 std::atomic<int> attr_delay_us{0};
@@ -49,6 +50,7 @@ T handle() {
 }
 
 void log_line(const std::string& what, cudaStream_t st, const void* p) {
+  if (!logging) return;
   text += std::to_string(tag) + " " + std::to_string(device) + " " + std::to_string((uintptr_t)st) + " " + what + " " +
           std::to_string((uintptr_t)p) + "\n";
 }
@@ -137,6 +139,10 @@ uint64_t fake_status_episodes(int (*take)(void*), void* stream, uint32_t low, ui
                               uint64_t episodes) {
   uint32_t* word = static_cast<uint32_t*>(host_word);
   std::atomic<uint64_t> done{0};
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    logging = false;  // millions of takes
+  }
   std::thread setter([&] {
     uint32_t r = 1;
     for (uint64_t e = 0; e < episodes; ++e) {
@@ -145,13 +151,18 @@ uint64_t fake_status_episodes(int (*take)(void*), void* stream, uint32_t low, ui
       for (volatile uint32_t k = 0, n = r >> 23; k < n; k = k + 1) {
       }
       __atomic_fetch_or(word, high, __ATOMIC_ACQ_REL);
-      while (__atomic_load_n(word, __ATOMIC_ACQUIRE)) {
-      }
+      for (uint32_t k = 0; __atomic_load_n(word, __ATOMIC_ACQUIRE); ++k)
+        if (k > 1000) std::this_thread::yield();
       done.fetch_add(1);
     }
   });
   uint64_t seen = 0;
-  while (done.load() < episodes) seen += take(stream) == high_status ? 1 : 0;
+  for (uint32_t idle = 0; done.load() < episodes;) {
+    const int status = take(stream);
+    seen += status == high_status ? 1 : 0;
+    idle = status ? 0 : idle + 1;
+    if (idle > 1000) std::this_thread::yield();
+  }
   setter.join();
   return episodes - seen;
 }
